@@ -155,151 +155,153 @@ FD_HD void floor_adj3(const R Q[3], R fscale, R flb, R Qb[3]) {
   for (int k = 0; k < 3; ++k) Qb[k] += ab[k] * sgn0(Q[k]);
 }
 
-// 13/3 t^2 + u^2 with t = a - b - x h, u = 2 (a - b) - x h (the sub-stencil
-// with an averaged gradient, App. C): adds to ab, bb, xb
-FD_HD void is_grad_adj(R a, R b, R x, R h, R ISb, R& ab, R& bb, R& xb) {
-  const R t = a - b - x * h, u = 2.0 * (a - b) - x * h;
-  const R tb = (26.0 / 3.0) * t * ISb, ub = 2.0 * u * ISb;
-  ab += tb + 2.0 * ub;
-  bb -= tb + 2.0 * ub;
-  xb -= h * (tb + ub);
-}
 // 13/12 t^2 + u^2 / 4 for given t and u: returns (tb, ub)
 FD_HD void is_three_adj(R t, R u, R ISb, R& tb, R& ub) {
   tb = (13.0 / 6.0) * t * ISb;
   ub = 0.5 * u * ISb;
 }
 
+// 13/3 t^2 + u^2 with t = b - xh, u = 2 b - xh (the sub-stencil with an
+// averaged gradient, App. C): adds to bb, xhb
+FD_HD void is_grad_adj(R b, R xh, R ISb, R& bb, R& xhb) {
+  const R t = b - xh, u = 2.0 * b - xh;
+  const R tb = (26.0 / 3.0) * t * ISb, ub = 2.0 * u * ISb;
+  bb += tb + 2.0 * ub;
+  xhb -= tb + ub;
+}
+
 // adjoint of recon_interface (FP64, path-function floor from fscale as in
 // geno_floor_of): output adjoints vlb, dlb, chilb, vrb, drb, chirb -> Qb[4],
-// Qxb[4] (added)
+// Qxb[4] (added).  As the forward: everything in the differences b_k, and no
+// indicators on a side that the FP32 screen finds saturated.
 FD_HD void recon_interface_adj(const GenoK<R>& g, const R Q[4], const R Qx[4], R h, R ih, R vlb, R dlb, R chilb,
                                R vrb, R drb, R chirb, R Qb[4], R Qxb[4], R fscale = 0.0) {
   const R c64 = 1.0 / 64.0, c30 = 1.0 / 30.0;
-  const R fl = geno_floor_of(s_max(s_max(s_abs(Q[0]), s_abs(Q[1])), s_max(s_abs(Q[2]), s_abs(Q[3]))), fscale);
-  R flb = 0.0;
-  const R PHx = -((Q[0] + 45.0 * Q[1] - 45.0 * Q[2] - Q[3]) * ih + 9.0 * (Qx[1] + Qx[2])) * c30;
-  const R dq12 = (Q[2] - Q[1]) * ih;
-  R PHxb = 0.0, dq12b = 0.0;
-  // ---- left (App. C1) ----
-  {
-    const R PH = ((7.0 * Q[0] + 35.0 * Q[1] + 21.0 * Q[2] + Q[3]) + (Qx[0] + 22.0 * Qx[1] - 7.0 * Qx[2]) * h) * c64;
-    const R q[3] = {(-5.0 * Q[0] + 9.0 * Q[1] - 3.0 * Qx[0] * h) * 0.25, (-Q[0] + 6.0 * Q[1] + 3.0 * Q[2]) * 0.125,
-                    (3.0 * Q[1] + 6.0 * Q[2] - Q[3]) * 0.125};
-    const R qx0 = (-3.0 * Q[0] + 3.0 * Q[1]) * ih - 2.0 * Qx[0];
-    R t = Q[1] - Q[0] - Qx[0] * h, u = 2.0 * (Q[1] - Q[0]) - Qx[0] * h;
-    R IS[3];
-    IS[0] = (13.0 / 3.0) * t * t + u * u;
-    const R t1 = Q[0] - 2.0 * Q[1] + Q[2], u1 = Q[2] - Q[0];
-    IS[1] = (13.0 / 12.0) * t1 * t1 + 0.25 * u1 * u1;
-    const R t2 = Q[1] - 2.0 * Q[2] + Q[3], u2 = 3.0 * Q[1] - 4.0 * Q[2] + Q[3];
-    IS[2] = (13.0 / 12.0) * t2 * t2 + 0.25 * u2 * u2;
-    R PHb = 0.0, qb[3] = {0.0, 0.0, 0.0}, qx0b = 0.0, ISb[3] = {0.0, 0.0, 0.0};
-    geno_blend_adj(g, g.d_iface, IS, fl, PH, PHx, q, qx0, dq12, vlb, dlb, chilb, PHb, PHxb, qb, qx0b, dq12b, ISb,
-                   flb);
-    // PH
-    Qb[0] += 7.0 * c64 * PHb; Qb[1] += 35.0 * c64 * PHb; Qb[2] += 21.0 * c64 * PHb; Qb[3] += c64 * PHb;
-    Qxb[0] += h * c64 * PHb; Qxb[1] += 22.0 * h * c64 * PHb; Qxb[2] -= 7.0 * h * c64 * PHb;
-    // q0..q2, qx0
-    Qb[0] += -1.25 * qb[0] - 0.125 * qb[1] - 3.0 * ih * qx0b;
-    Qb[1] += 2.25 * qb[0] + 0.75 * qb[1] + 0.375 * qb[2] + 3.0 * ih * qx0b;
-    Qb[2] += 0.375 * qb[1] + 0.75 * qb[2];
-    Qb[3] -= 0.125 * qb[2];
-    Qxb[0] += -0.75 * h * qb[0] - 2.0 * qx0b;
-    // IS
-    is_grad_adj(Q[1], Q[0], Qx[0], h, ISb[0], Qb[1], Qb[0], Qxb[0]);
-    R tb, ub;
-    is_three_adj(t1, u1, ISb[1], tb, ub);
-    Qb[0] += tb - ub; Qb[1] -= 2.0 * tb; Qb[2] += tb + ub;
-    is_three_adj(t2, u2, ISb[2], tb, ub);
-    Qb[1] += tb + 3.0 * ub; Qb[2] -= 2.0 * tb + 4.0 * ub; Qb[3] += tb + ub;
+  const R b0 = Q[1] - Q[0], b1 = Q[2] - Q[1], b2 = Q[3] - Q[2];
+  bool smooth_l = g.linear, smooth_r = g.linear;
+  if (!g.linear && fscale == 0.0) screen_iface(g, b0, b1, b2, Qx[0], Qx[3], screen_h(h), smooth_l, smooth_r);
+  R b0b = 0.0, b1b = 0.0, b2b = 0.0, PHxb = 0.0, PHlb = 0.0, PHrb = 0.0;
+  if (smooth_l) {
+    PHlb = vlb;
+    PHxb += dlb;
   }
-  // ---- right (App. C2, formulas for interface j+1/2) ----
-  {
-    const R PH = ((Q[0] + 21.0 * Q[1] + 35.0 * Q[2] + 7.0 * Q[3]) + (7.0 * Qx[1] - 22.0 * Qx[2] - Qx[3]) * h) * c64;
-    const R q[3] = {(-5.0 * Q[3] + 9.0 * Q[2] + 3.0 * Qx[3] * h) * 0.25, (-Q[3] + 6.0 * Q[2] + 3.0 * Q[1]) * 0.125,
-                    (-Q[0] + 6.0 * Q[1] + 3.0 * Q[2]) * 0.125};
-    const R qx0 = (-3.0 * Q[2] + 3.0 * Q[3]) * ih - 2.0 * Qx[3];
-    R IS[3];
-    const R t0 = Q[2] - Q[3] + Qx[3] * h, u0 = 2.0 * (Q[3] - Q[2]) - Qx[3] * h;
-    IS[0] = (13.0 / 3.0) * t0 * t0 + u0 * u0;
-    const R t1 = Q[1] - 2.0 * Q[2] + Q[3], u1 = Q[3] - Q[1];
-    IS[1] = (13.0 / 12.0) * t1 * t1 + 0.25 * u1 * u1;
-    const R t2 = Q[0] - 2.0 * Q[1] + Q[2], u2 = 3.0 * Q[2] - 4.0 * Q[1] + Q[0];
-    IS[2] = (13.0 / 12.0) * t2 * t2 + 0.25 * u2 * u2;
-    R PHb = 0.0, qb[3] = {0.0, 0.0, 0.0}, qx0b = 0.0, ISb[3] = {0.0, 0.0, 0.0};
-    geno_blend_adj(g, g.d_iface, IS, fl, PH, PHx, q, qx0, dq12, vrb, drb, chirb, PHb, PHxb, qb, qx0b, dq12b, ISb,
-                   flb);
-    Qb[0] += c64 * PHb; Qb[1] += 21.0 * c64 * PHb; Qb[2] += 35.0 * c64 * PHb; Qb[3] += 7.0 * c64 * PHb;
-    Qxb[1] += 7.0 * h * c64 * PHb; Qxb[2] -= 22.0 * h * c64 * PHb; Qxb[3] -= h * c64 * PHb;
-    Qb[3] += -1.25 * qb[0] - 0.125 * qb[1] + 3.0 * ih * qx0b;
-    Qb[2] += 2.25 * qb[0] + 0.75 * qb[1] + 0.375 * qb[2] - 3.0 * ih * qx0b;
-    Qb[1] += 0.375 * qb[1] + 0.75 * qb[2];
-    Qb[0] -= 0.125 * qb[2];
-    Qxb[3] += 0.75 * h * qb[0] - 2.0 * qx0b;
-    // IS0: t = Q2 - Q3 + Qx3 h = (Q2) - (Q3) - (-Qx3) h, u = 2 (Q3 - Q2) - Qx3 h
-    {
-      const R tb0 = (26.0 / 3.0) * t0 * ISb[0], ub0 = 2.0 * u0 * ISb[0];
-      Qb[2] += tb0 - 2.0 * ub0;
-      Qb[3] += -tb0 + 2.0 * ub0;
-      Qxb[3] += h * tb0 - h * ub0;
+  if (smooth_r) {
+    PHrb = vrb;
+    PHxb += drb;
+  }
+  if (!smooth_l || !smooth_r) {
+    const R PHx = (b0 + b2 + 46.0 * b1) * (ih * c30) - 0.3 * (Qx[1] + Qx[2]);
+    const R fl = geno_floor_of(s_max(s_max(s_abs(Q[0]), s_abs(Q[1])), s_max(s_abs(Q[2]), s_abs(Q[3]))), fscale);
+    const R dq12 = b1 * ih, t01 = b1 - b0, t12 = b2 - b1;
+    const R s01 = (13.0 / 12.0) * t01 * t01, s12 = (13.0 / 12.0) * t12 * t12;
+    R flb = 0.0, dq12b = 0.0, t01b = 0.0, t12b = 0.0, tb, ub;
+    // ---- left (App. C1) ----
+    if (!smooth_l) {
+      const R PH = (22.0 * b1 + b2 - 7.0 * b0 + (Qx[0] + 22.0 * Qx[1] - 7.0 * Qx[2]) * h) * c64;
+      const R xh = Qx[0] * h, u1 = b0 + b1, u2 = b2 - 3.0 * b1;
+      const R q[3] = {1.25 * b0 - 0.75 * xh, 0.125 * b0 + 0.375 * b1, 0.625 * b1 - 0.125 * b2};
+      const R t = b0 - xh, u = 2.0 * b0 - xh;
+      const R IS[3] = {(13.0 / 3.0) * t * t + u * u, s01 + 0.25 * u1 * u1, s12 + 0.25 * u2 * u2};
+      R qb[3] = {0.0, 0.0, 0.0}, qx0b = 0.0, ISb[3] = {0.0, 0.0, 0.0}, xhb = 0.0;
+      geno_blend_adj(g, g.d_iface, IS, fl, PH, PHx, q, 3.0 * b0 * ih - 2.0 * Qx[0], dq12, vlb, dlb, chilb, PHlb,
+                     PHxb, qb, qx0b, dq12b, ISb, flb);
+      b0b += 1.25 * qb[0] + 0.125 * qb[1] + 3.0 * ih * qx0b;
+      b1b += 0.375 * qb[1] + 0.625 * qb[2];
+      b2b -= 0.125 * qb[2];
+      xhb -= 0.75 * qb[0];
+      is_grad_adj(b0, xh, ISb[0], b0b, xhb);
+      is_three_adj(t01, u1, ISb[1], tb, ub);
+      t01b += tb; b0b += ub; b1b += ub;
+      is_three_adj(t12, u2, ISb[2], tb, ub);
+      t12b += tb; b2b += ub; b1b -= 3.0 * ub;
+      Qxb[0] += h * xhb - 2.0 * qx0b;
     }
-    R tb, ub;
-    is_three_adj(t1, u1, ISb[1], tb, ub);
-    Qb[1] += tb - ub; Qb[2] -= 2.0 * tb; Qb[3] += tb + ub;
-    is_three_adj(t2, u2, ISb[2], tb, ub);
-    Qb[0] += tb + ub; Qb[1] -= 2.0 * tb + 4.0 * ub; Qb[2] += tb + 3.0 * ub;
+    // ---- right (App. C2, formulas for interface j+1/2) ----
+    if (!smooth_r) {
+      const R PH = (7.0 * b2 - 22.0 * b1 - b0 + (7.0 * Qx[1] - 22.0 * Qx[2] - Qx[3]) * h) * c64;
+      const R xh = Qx[3] * h, u1 = b1 + b2, u2 = b0 - 3.0 * b1;
+      const R q[3] = {0.75 * xh - 1.25 * b2, -(0.125 * b2 + 0.375 * b1), 0.125 * b0 - 0.625 * b1};
+      const R t = b2 - xh, u = 2.0 * b2 - xh;
+      const R IS[3] = {(13.0 / 3.0) * t * t + u * u, s12 + 0.25 * u1 * u1, s01 + 0.25 * u2 * u2};
+      R qb[3] = {0.0, 0.0, 0.0}, qx0b = 0.0, ISb[3] = {0.0, 0.0, 0.0}, xhb = 0.0;
+      geno_blend_adj(g, g.d_iface, IS, fl, PH, PHx, q, 3.0 * b2 * ih - 2.0 * Qx[3], dq12, vrb, drb, chirb, PHrb,
+                     PHxb, qb, qx0b, dq12b, ISb, flb);
+      b2b += 3.0 * ih * qx0b - 1.25 * qb[0] - 0.125 * qb[1];
+      b1b -= 0.375 * qb[1] + 0.625 * qb[2];
+      b0b += 0.125 * qb[2];
+      xhb += 0.75 * qb[0];
+      is_grad_adj(b2, xh, ISb[0], b2b, xhb);
+      is_three_adj(t12, u1, ISb[1], tb, ub);
+      t12b += tb; b1b += ub; b2b += ub;
+      is_three_adj(t01, u2, ISb[2], tb, ub);
+      t01b += tb; b0b += ub; b1b -= 3.0 * ub;
+      Qxb[3] += h * xhb - 2.0 * qx0b;
+    }
+    b1b += t01b - t12b + ih * dq12b;
+    b0b -= t01b;
+    b2b += t12b;
+    floor_adj4(Q, fscale, flb, Qb);
   }
-  // shared PHx and dq12
-  Qb[0] -= c30 * ih * PHxb; Qb[1] -= 45.0 * c30 * ih * PHxb; Qb[2] += 45.0 * c30 * ih * PHxb; Qb[3] += c30 * ih * PHxb;
-  Qxb[1] -= 9.0 * c30 * PHxb; Qxb[2] -= 9.0 * c30 * PHxb;
-  Qb[2] += ih * dq12b;
-  Qb[1] -= ih * dq12b;
-  floor_adj4(Q, fscale, flb, Qb);
+  // values relative to Q1 (left) and Q2 (right), shared derivative
+  const R hl = c64 * PHlb, hr = c64 * PHrb, hx = ih * c30 * PHxb;
+  b0b += hx - 7.0 * hl - hr;
+  b1b += 46.0 * hx + 22.0 * (hl - hr);
+  b2b += hx + hl + 7.0 * hr;
+  Qxb[0] += h * hl;
+  Qxb[1] += h * (22.0 * hl + 7.0 * hr) - 0.3 * PHxb;
+  Qxb[2] -= h * (7.0 * hl + 22.0 * hr) + 0.3 * PHxb;
+  Qxb[3] -= h * hr;
+  Qb[0] -= b0b;
+  Qb[1] += vlb + b0b - b1b;
+  Qb[2] += vrb + b1b - b2b;
+  Qb[3] += b2b;
 }
 
 // adjoint of recon_node (FP64, floor from fscale): rb -> Qb[3], Qxb[3] (added)
 FD_HD void recon_node_adj(const GenoK<R>& g, const R Q[3], const R Qx[3], R h, R ih, R rb, R Qb[3], R Qxb[3],
                           R fscale = 0.0) {
   const R c30 = 1.0 / 30.0;
-  const R PHx = (9.0 * (Q[0] - Q[2]) * ih + (Qx[0] + 46.0 * Qx[1] + Qx[2])) * c30;
-  const R qx[3] = {(Q[2] - Q[0]) * 0.5 * ih, 2.0 * (Q[1] - Q[0]) * ih - Qx[0], 2.0 * (Q[2] - Q[1]) * ih - Qx[2]};
-  const R t0 = Q[0] - 2.0 * Q[1] + Q[2], u0 = Q[2] - Q[0];
-  R IS[3];
-  IS[0] = (13.0 / 12.0) * t0 * t0 + 0.25 * u0 * u0;
-  R t = Q[1] - Q[0] - Qx[0] * h, u = 2.0 * (Q[1] - Q[0]) - Qx[0] * h;
-  IS[1] = (13.0 / 3.0) * t * t + u * u;
-  t = Q[2] - Q[1] - Qx[2] * h;
-  u = 2.0 * (Q[2] - Q[1]) - Qx[2] * h;
-  IS[2] = (13.0 / 3.0) * t * t + u * u;
-  R PHxb = 0.0, qxb[3] = {0.0, 0.0, 0.0}, ISb[3] = {0.0, 0.0, 0.0}, flb = 0.0;
-  const R fl = geno_floor_of(s_max(s_abs(Q[1]), s_max(s_abs(Q[0]), s_abs(Q[2]))), fscale);
-  const R chi = geno_chi(g, IS[0], IS[1], IS[2], fl);
-  if (chi == 1.0) {
-    PHxb = rb;
-  } else {
-    R w[3];
-    geno_weights(g, g.d_node, IS[0], IS[1], IS[2], w);
-    const R PLx = w[0] * qx[0] + w[1] * qx[1] + w[2] * qx[2];
-    PHxb = chi * rb;
-    const R PLxb = (1.0 - chi) * rb;
-    const R wb[3] = {PLxb * qx[0], PLxb * qx[1], PLxb * qx[2]};
-    for (int k = 0; k < 3; ++k) qxb[k] = PLxb * w[k];
-    geno_weights_adj(g, g.d_node, IS, wb, ISb);
-    geno_chi_adj(g, IS, fl, rb * (PHx - PLx), ISb, flb);
+  const R b0 = Q[1] - Q[0], b1 = Q[2] - Q[1], b = b0 + b1;
+  R PHxb = rb, b0b = 0.0, b1b = 0.0, bb = 0.0;
+  if (!g.linear && !(fscale == 0.0 && screen_node(g, b0, b1, Qx[0], Qx[2], screen_h(h)))) {
+    const R x0 = Qx[0] * h, x2 = Qx[2] * h, t = b1 - b0;
+    const R t1 = b0 - x0, u1 = 2.0 * b0 - x0, t2 = b1 - x2, u2 = 2.0 * b1 - x2;
+    const R IS[3] = {(13.0 / 12.0) * t * t + 0.25 * b * b, (13.0 / 3.0) * t1 * t1 + u1 * u1,
+                     (13.0 / 3.0) * t2 * t2 + u2 * u2};
+    const R fl = geno_floor_of(s_max(s_abs(Q[1]), s_max(s_abs(Q[0]), s_abs(Q[2]))), fscale);
+    const R chi = geno_chi(g, IS[0], IS[1], IS[2], fl);
+    if (chi != 1.0) {
+      R ISb[3] = {0.0, 0.0, 0.0}, flb = 0.0, w[3], x0b = 0.0, x2b = 0.0, tb, ub;
+      const R PHx = (Qx[0] + 46.0 * Qx[1] + Qx[2]) * c30 - (0.3 * ih) * b;
+      const R qx[3] = {0.5 * b * ih, 2.0 * b0 * ih - Qx[0], 2.0 * b1 * ih - Qx[2]};
+      geno_weights(g, g.d_node, IS[0], IS[1], IS[2], w);
+      const R PLx = w[0] * qx[0] + w[1] * qx[1] + w[2] * qx[2];
+      PHxb = chi * rb;
+      const R PLxb = (1.0 - chi) * rb;
+      const R wb[3] = {PLxb * qx[0], PLxb * qx[1], PLxb * qx[2]};
+      geno_weights_adj(g, g.d_node, IS, wb, ISb);
+      geno_chi_adj(g, IS, fl, rb * (PHx - PLx), ISb, flb);
+      floor_adj3(Q, fscale, flb, Qb);
+      bb += 0.5 * ih * PLxb * w[0];
+      b0b += 2.0 * ih * PLxb * w[1];
+      b1b += 2.0 * ih * PLxb * w[2];
+      Qxb[0] -= PLxb * w[1];
+      Qxb[2] -= PLxb * w[2];
+      is_three_adj(t, b, ISb[0], tb, ub);
+      b1b += tb; b0b -= tb; bb += ub;
+      is_grad_adj(b0, x0, ISb[1], b0b, x0b);
+      is_grad_adj(b1, x2, ISb[2], b1b, x2b);
+      Qxb[0] += h * x0b;
+      Qxb[2] += h * x2b;
+    }
   }
-  floor_adj3(Q, fscale, flb, Qb);
-  Qb[0] += 9.0 * c30 * ih * PHxb;
-  Qb[2] -= 9.0 * c30 * ih * PHxb;
+  bb -= 0.3 * ih * PHxb;
   Qxb[0] += c30 * PHxb; Qxb[1] += 46.0 * c30 * PHxb; Qxb[2] += c30 * PHxb;
-  Qb[2] += 0.5 * ih * qxb[0]; Qb[0] -= 0.5 * ih * qxb[0];
-  Qb[1] += 2.0 * ih * qxb[1]; Qb[0] -= 2.0 * ih * qxb[1]; Qxb[0] -= qxb[1];
-  Qb[2] += 2.0 * ih * qxb[2]; Qb[1] -= 2.0 * ih * qxb[2]; Qxb[2] -= qxb[2];
-  R tb, ub;
-  is_three_adj(t0, u0, ISb[0], tb, ub);
-  Qb[0] += tb - ub; Qb[1] -= 2.0 * tb; Qb[2] += tb + ub;
-  is_grad_adj(Q[1], Q[0], Qx[0], h, ISb[1], Qb[1], Qb[0], Qxb[0]);
-  is_grad_adj(Q[2], Q[1], Qx[2], h, ISb[2], Qb[2], Qb[1], Qxb[2]);
+  b0b += bb;
+  b1b += bb;
+  Qb[0] -= b0b;
+  Qb[1] += b0b - b1b;
+  Qb[2] += b1b;
 }
 
 // Adjoint of the reconstruction of one 4-point line in conservative
