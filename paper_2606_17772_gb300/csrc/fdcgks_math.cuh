@@ -977,4 +977,15 @@ FD_HD R compact_flux(int variant, R chi, R Fim, R Fi0, R Fip, R Fn0, R Fn1) {
   return (R(1) - chi) * Flow + chi * Fbar;
 }
 
+// Difference of the compact fluxes at j+1/2 and j-1/2 over the node j.
+// Fi = {F_{j-3/2}, F_{j-1/2}, F_{j+1/2}, F_{j+3/2}}, Fn = {F_{j-1}, F_j, F_{j+1}}.
+// SMOOTH: both interfaces take the high-order flux (chi = 1), whose difference
+// is (F_{j+3/2} - F_{j-3/2} + 45 (F_{j+1/2} - F_{j-1/2}) - 9 (F_{j+1} - F_{j-1}))/30,
+// 6 operations instead of the two blended fluxes' 22.
+template <bool SMOOTH, class R>
+FD_HD R compact_flux_diff(int variant, R chim, R chip, R Fmm, R Fm, R Fp, R Fpp, R Nm, R N0, R Np) {
+  if (SMOOTH) return (R(45) * (Fp - Fm) + (Fpp - Fmm) - R(9) * (Np - Nm)) * R(1.0 / 30.0);
+  return compact_flux(variant, chip, Fm, Fp, Fpp, N0, Np) - compact_flux(variant, chim, Fmm, Fm, Fp, Nm, N0);
+}
+
 }  // namespace fdk
