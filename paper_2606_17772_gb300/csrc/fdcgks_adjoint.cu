@@ -40,8 +40,7 @@
 
 namespace fdk {
 // the forward FP64 kernels are instantiated in fdcgks_fp64.cu
-extern template cudaError_t launch_nodal<double>(const KArgs<double>&, cudaStream_t);
-extern template cudaError_t launch_points<double>(const KArgs<double>&, cudaStream_t);
+extern template cudaError_t launch_points<double>(const KArgs<double>&, bool, cudaStream_t);
 extern template cudaError_t launch_update<double>(const KArgs<double>&, int, cudaStream_t);
 }  // namespace fdk
 
@@ -68,7 +67,7 @@ __device__ __noinline__ void recon_adj_call(const GenoK<double>& g, const double
 // ---------------------------------------------------------------------------
 // point map adjoint: inputs are the 64 values (2 lines x 4 entries x (4 W +
 // 4 gradients along the line)) the point reads; outputs its 50 values.
-// Reverse order of point_compute: W~ assembly (linear) <- two kinetic solves
+// Reverse order of point_compute_pair: W~ assembly (linear) <- two kinetic solves
 // <- tangential derivatives (means) <- two line reconstructions, each step
 // by its hand-written reverse pass (fdcgks_reverse.cuh).  fscale > 0 (mixed
 // contexts): GENO's path function takes the FP32 path's rounding floor
@@ -90,7 +89,7 @@ __global__ void __launch_bounds__(128) point_vjp_kernel(KArgs<double> a, const d
     any = any || ah[k] != 0.0;
   }
   if (!any) return;
-  const PointLines pl = point_lines<TYPE>(L, i, j);
+  const PointLines pl = point_lines(L, TYPE, i, j);
   auto addr = [&](int s) -> long {
     const int l = s / 32, e = (s / 8) % 4, f = s % 8;
     const int field = f < 4 ? f : pl.gfield[l] + (f - 4);
@@ -504,8 +503,7 @@ cudaError_t forward_step(const Work& w, double dt, const double* in, double* out
   for (int stage = 0; stage < 2; ++stage) {
     KArgs<double> a = stage_args(w, dt, stage);
     if ((e = fill_ghosts_fwd(w, const_cast<double*>(a.Sr))) != cudaSuccess) return e;
-    if ((e = launch_nodal<double>(a, s)) != cudaSuccess) return e;
-    if ((e = launch_points<double>(a, s)) != cudaSuccess) return e;
+    if ((e = launch_points<double>(a, true, s)) != cudaSuccess) return e;
     if ((e = launch_update<double>(a, stage == 0 ? UPD_STAGE1 : UPD_STAGE2, s)) != cudaSuccess) return e;
   }
   if (out != w.Snext) e = cudaMemcpyAsync(out, w.Snext, w.fs, cudaMemcpyDeviceToDevice, s);

@@ -435,6 +435,18 @@ static void stage_state(fdcgks_t c, int mode, KArgs<float>& a) {
   a.Gb_lo = c->Gb_lo;
 }
 
+// Whether a stage's nodes and points go out in one launch.  FP64: always; the
+// short nodal items fill the points' last wave (vortex, ms per step, apart and
+// merged: 33^2 0.304, 0.213; 128^2 0.675, 0.568; 512^2 4.90, 4.73; 1024^2 17.90,
+// 17.86).  Mixed: while launches and partly empty waves weigh more than the
+// nodal work's lower occupancy at the points' register count (33^2 0.067, 0.053;
+// 128^2 0.072, 0.064; 256^2 0.111, 0.108; 320^2 0.146, 0.142; 384^2 0.190,
+// 0.194; 1024^2 1.12, 1.27).
+template <class R>
+static bool stage_merged(const Layout& L) {
+  return sizeof(R) == sizeof(double) || (long)L.nx * L.ny <= 100000;
+}
+
 template <class R>
 static fdcgks_status run_stage(fdcgks_t c, double dt, int mode, double* const* op) {
   KArgs<R> a = make_args<R>(c, dt, nullptr, nullptr, mode != UPD_STAGE2);
@@ -444,16 +456,20 @@ static fdcgks_status run_stage(fdcgks_t c, double dt, int mode, double* const* o
   CUDA_TRY(c, prof_mark(c, KC_GHOST, false));
   if (op)
     for (int k = 0; k < 8; ++k) a.op[k] = op[k];
-  CUDA_TRY(c, prof_mark(c, KC_NODAL, true));
-  CUDA_TRY(c, launch_nodal<R>(a, c->stream));
-  CUDA_TRY(c, prof_mark(c, KC_NODAL, false));
+  // nodes and points in one launch, unless they are timed apart
+  const bool apart = c->profiling || !stage_merged<R>(c->L);
+  if (apart) {
+    CUDA_TRY(c, prof_mark(c, KC_NODAL, true));
+    CUDA_TRY(c, launch_nodal<R>(a, c->stream));
+    CUDA_TRY(c, prof_mark(c, KC_NODAL, false));
+  }
   CUDA_TRY(c, prof_mark(c, KC_POINTS, true));
-  CUDA_TRY(c, launch_points<R>(a, c->stream));
+  CUDA_TRY(c, launch_points<R>(a, !apart, c->stream));
   CUDA_TRY(c, prof_mark(c, KC_POINTS, false));
   CUDA_TRY(c, prof_mark(c, KC_UPDATE, true));
   CUDA_TRY(c, launch_update<R>(a, mode, c->stream));
   CUDA_TRY(c, prof_mark(c, KC_UPDATE, false));
-  c->launches += 6;   // 2 ghost passes, nodal, 2 point types, update
+  c->launches += apart ? 5 : 4;   // 2 ghost passes, nodes and points, update
   return FDCGKS_OK;
 }
 

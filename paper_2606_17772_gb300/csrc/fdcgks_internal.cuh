@@ -314,7 +314,7 @@ cudaError_t launch_split_ff(const double* S, float* hi, float* lo, long n, cudaS
 cudaError_t launch_join_ff(const float* hi, const float* lo, double* S, long n, cudaStream_t s);
 
 template <class R> cudaError_t launch_nodal(const KArgs<R>& a, cudaStream_t s);
-template <class R> cudaError_t launch_points(const KArgs<R>& a, cudaStream_t s);
+template <class R> cudaError_t launch_points(const KArgs<R>& a, bool nodal, cudaStream_t s);
 template <class R> cudaError_t launch_update(const KArgs<R>& a, int mode, cudaStream_t s);
 
 // component-level batches (device arrays), for parity tests of the kernels' arithmetic

@@ -10,48 +10,24 @@
 #include "fdcgks_internal.cuh"
 
 // Tuning knobs of the interface-point kernel (defaults are the tuned values):
-// FDK_POINT_MINB   minimum resident blocks per SM in the launch bounds
-//                  (caps registers per thread), per compute type
-// FDK_UPDATE_MINB_F32, FDK_NODAL_MINB_F32  the same for the FP32 update and
-//                  nodal kernels (the FP64 kernels are FP64-pipe bound and
+// FDK_UPDATE_MINB_F32, FDK_NODAL_MINB_F32  minimum resident blocks per SM in
+//                  the launch bounds (caps registers per thread) of the FP32
+//                  update and nodal kernels (the FP64 kernels are FP64-pipe bound and
 //                  are left uncapped).  1024^2 vortex, ms per mixed step:
 //                  update 4, 5, 6, 8 gave 0.448, 0.411, 0.382, 0.437; nodal
 //                  5, 6, 8, 10, 12, 16 gave 0.303, 0.264, 0.234, 0.221, 0.225,
 //                  0.332
-// FDK_SOLVE_NOINLINE  1: the kinetic solve is an out-of-line function called
-//                  twice (one code copy per kernel), 0: inlined twice
-#ifndef FDK_POINT_MINB_F64
-#define FDK_POINT_MINB_F64 1
-#endif
-#ifndef FDK_POINT_MINB_F32
-#define FDK_POINT_MINB_F32 4
-#endif
 #ifndef FDK_UPDATE_MINB_F32
 #define FDK_UPDATE_MINB_F32 6
 #endif
 #ifndef FDK_NODAL_MINB_F32
 #define FDK_NODAL_MINB_F32 10
 #endif
-#ifndef FDK_SOLVE_NOINLINE_F64
-#define FDK_SOLVE_NOINLINE_F64 1
-#endif
-#ifndef FDK_SOLVE_NOINLINE_F32
-#define FDK_SOLVE_NOINLINE_F32 1
-#endif
-// FDK_POINT_PAIR_F32 / _F64  1: two threads per interface point (one line and
-//                  one solve each, coupled by warp shuffles; point_pair_kernel),
-//                  0: one thread per point (point_kernel).  On the 1024^2 vortex
-//                  the pair form takes the mixed point phase from 1.019 to
-//                  0.903 ms per step and the FP64 one from 32.06 to 31.41 ms
+// FDK_STAGE_THREADS_F64  block size of the FP64 stage kernel (below; 32 and 128:
+//                  33^2 0.213 and 0.227 ms per step, 512^2 4.73 and 4.78)
 // FDK_POINT_PAIR_MINB_F32 / _F64  minimum resident blocks per SM of the pair
 //                  kernel (FP32 without preload: 2, 3, 4, 5 gave 1.43, 1.06,
 //                  0.915, 0.903 ms; with preload 4 and 5 give 0.822 and 0.840)
-#ifndef FDK_POINT_PAIR_F32
-#define FDK_POINT_PAIR_F32 1
-#endif
-#ifndef FDK_POINT_PAIR_F64
-#define FDK_POINT_PAIR_F64 1
-#endif
 #ifndef FDK_POINT_PAIR_MINB_F32
 #define FDK_POINT_PAIR_MINB_F32 4
 #endif
@@ -66,6 +42,9 @@
 //                  smooth data it is short enough (512^2 vortex, point phase per
 //                  step: mixed 0.153 -> 0.146 ms, FP64 4.25 -> 4.20 ms against
 //                  one out-of-line copy per kernel)
+#ifndef FDK_STAGE_THREADS_F64
+#define FDK_STAGE_THREADS_F64 32
+#endif
 #ifndef FDK_PAIR_PRELOAD_F32
 #define FDK_PAIR_PRELOAD_F32 1
 #endif
@@ -74,27 +53,15 @@ namespace fdk {
 
 template <class R> struct PointTune;
 template <> struct PointTune<double> {
-  static constexpr int minb = FDK_POINT_MINB_F64;
   static constexpr int update_minb = 1;
   static constexpr int nodal_minb = 1;
-  static constexpr bool noinline = FDK_SOLVE_NOINLINE_F64;
-  static constexpr bool pair = FDK_POINT_PAIR_F64;
   static constexpr int pair_minb = FDK_POINT_PAIR_MINB_F64;
 };
 template <> struct PointTune<float> {
-  static constexpr int minb = FDK_POINT_MINB_F32;
   static constexpr int update_minb = FDK_UPDATE_MINB_F32;
   static constexpr int nodal_minb = FDK_NODAL_MINB_F32;
-  static constexpr bool noinline = FDK_SOLVE_NOINLINE_F32;
-  static constexpr bool pair = FDK_POINT_PAIR_F32;
   static constexpr int pair_minb = FDK_POINT_PAIR_MINB_F32;
 };
-
-template <class R>
-__device__ __noinline__ void iface_solve_call(const GasK<R>& gas, int normal, const R* Wl, const R* Wr, const R* Wln,
-                                             const R* Wrn, const R* Wt, bool want_n, IfaceOut<R>& o) {
-  iface_solve(gas, normal, Wl, Wr, Wln, Wrn, Wt, want_n, o);
-}
 
 // ---------------------------------------------------------------------------
 // nodal reconstruction and flux (Sec. 4 item 2; Sec. 2.1 nodal fluxes)
@@ -268,64 +235,6 @@ FD_HD void recon_line_char(const GenoK<R>& geno, R gm1, int normal, LD ld, int l
   positivity_fix(ld, l, vl, dl, vr, dr, chi);
 }
 
-// One virtual-interface point: the two line reconstructions (with the
-// safeguard), the tangential derivatives, the two kinetic solves and the W~
-// combination.  ld(l, e, f) as for recon_line_ld, line 0 being the
-// primary-grid line (normal TYPE, spacing h[TYPE]) and line 1 the dual-grid
-// line (normal 1 - TYPE); st(k, v): output k (PO_* of solve 0, NPS + PO_* of
-// solve 1; F and W~ values only when wn).  Shared by the kernel and its adjoint.
-template <class R, int TYPE, bool CHAR = false, class LD, class ST>
-FD_HD void point_compute(const GenoK<R>& geno, const GasK<R>& gas, const R h[2], const R ih[2], bool wn, LD ld,
-                         ST st) {
-  const int n0 = TYPE;        // normal of the primary-grid solve
-  R l0v[4], l0d[4], r0v[4], r0d[4], chi0;
-  R l1v[4], l1d[4], r1v[4], r1d[4], chi1;
-  if constexpr (CHAR) {
-    recon_line_char(geno, gas.gm1, n0, ld, 0, h[n0], ih[n0], l0v, l0d, r0v, r0d, chi0);
-    recon_line_char(geno, gas.gm1, 1 - n0, ld, 1, h[1 - n0], ih[1 - n0], l1v, l1d, r1v, r1d, chi1);
-  } else {
-    recon_line_ld(geno, ld, 0, h[n0], ih[n0], l0v, l0d, r0v, r0d, chi0);
-    recon_line_ld(geno, ld, 1, h[1 - n0], ih[1 - n0], l1v, l1d, r1v, r1d, chi1);
-  }
-  // tangential derivative of each solve: mean of the other line's l/r derivatives
-  R t0[4], t1[4];
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    t0[c] = R(0.5) * (l1d[c] + r1d[c]);
-    t1[c] = R(0.5) * (l0d[c] + r0d[c]);
-  }
-  IfaceOut<R> o0, o1;
-  if constexpr (PointTune<R>::noinline) {
-    iface_solve_call(gas, n0, l0v, r0v, l0d, r0d, t0, wn, o0);
-    iface_solve_call(gas, 1 - n0, l1v, r1v, l1d, r1d, t1, wn, o1);
-  } else {
-    iface_solve(gas, n0, l0v, r0v, l0d, r0d, t0, wn, o0);
-    iface_solve(gas, 1 - n0, l1v, r1v, l1d, r1d, t1, wn, o1);
-  }
-  // W~ of Eq. (eq:W-model-2d): half of the own solve plus a quarter of each side of the other
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    R m1t = R(0.25) * (o1.Wlt[c] + o1.Wrt[c]), m0t = R(0.25) * (o0.Wlt[c] + o0.Wrt[c]);
-    st(PO_FT + c, o0.Ft[c]);
-    st(PO_WLT + c, R(0.5) * o0.Wlt[c] + m1t);
-    st(PO_WRT + c, R(0.5) * o0.Wrt[c] + m1t);
-    st(NPS + PO_FT + c, o1.Ft[c]);
-    st(NPS + PO_WLT + c, R(0.5) * o1.Wlt[c] + m0t);
-    st(NPS + PO_WRT + c, R(0.5) * o1.Wrt[c] + m0t);
-    if (wn) {
-      R m1 = R(0.25) * (o1.Wl[c] + o1.Wr[c]), m0 = R(0.25) * (o0.Wl[c] + o0.Wr[c]);
-      st(PO_F + c, o0.F[c]);
-      st(PO_WL + c, R(0.5) * o0.Wl[c] + m1);
-      st(PO_WR + c, R(0.5) * o0.Wr[c] + m1);
-      st(NPS + PO_F + c, o1.F[c]);
-      st(NPS + PO_WL + c, R(0.5) * o1.Wl[c] + m0);
-      st(NPS + PO_WR + c, R(0.5) * o1.Wr[c] + m0);
-    }
-  }
-  st(PO_CHI, chi0);
-  st(NPS + PO_CHI, chi1);
-}
-
 // Where the lines of point (i, j) lie in the padded state: entry e of line l
 // is at base[l] + e * stride[l] of grid l (primary 0, dual 1), its gradient
 // along the line in fields gfield[l]..gfield[l] + 3.
@@ -333,10 +242,9 @@ struct PointLines {
   long base[2], stride[2];
   int gfield[2];
 };
-template <int TYPE>
-FD_HD PointLines point_lines(const Layout& L, int i, int j) {
+FD_HD PointLines point_lines(const Layout& L, int type, int i, int j) {
   PointLines p;
-  if (TYPE == 0) {
+  if (type == 0) {
     // primary nodes (i-1..i+2, j) along x; dual nodes (i+1, j-1..j+2) along y
     p.base[0] = cell(L, i - 1, j); p.stride[0] = 1; p.gfield[0] = 4;
     p.base[1] = cell(L, i + 1, j - 1); p.stride[1] = L.pitch; p.gfield[1] = 8;
@@ -353,47 +261,24 @@ FD_HD PointLines point_lines(const Layout& L, int i, int j) {
 // TYPE 0 = point A (i+1/2, j): primary x-interface, dual y-interface of dual column i+1
 // TYPE 1 = point B (i, j+1/2): primary y-interface, dual x-interface of dual row j+1
 // ---------------------------------------------------------------------------
-template <class R, int TYPE, bool CHAR = false>
-__device__ __forceinline__ void point_body(const KArgs<R>& a, int i, int j) {
-  const Layout& L = a.L;
-  const int imax = TYPE == 0 ? L.nx : L.nxd;
-  const int jmax = TYPE == 0 ? L.nyd : L.ny;
-  if (i < -2 || j < -2 || i > imax || j > jmax) return;
-  const PointLines pl = point_lines<TYPE>(L, i, j);
-  const R* S = a.Sr;
-  R* P = (TYPE == 0 ? a.PA : a.PB) + pcell(L, i, j);
-  const long pp = L.pplane;
-  point_compute<R, TYPE, CHAR>(
-      a.geno, a.gas, a.h, a.ih, a.want_n != 0,
-      [&](int l, int e, int f) -> R {
-        const int field = f < 4 ? f : pl.gfield[l] + (f - 4);
-        return S[((long)l * NFLD + field) * L.plane + pl.base[l] + e * pl.stride[l]];
-      },
-      [&](int k, R v) { P[(long)k * pp] = v; });
-}
-
-template <class R, int TYPE, bool CHAR>
-__global__ void __launch_bounds__(128, PointTune<R>::minb) point_kernel(KArgs<R> a) {
-  point_body<R, TYPE, CHAR>(a, blockIdx.x * blockDim.x + threadIdx.x - 2,
-                            blockIdx.y * blockDim.y + threadIdx.y - 2);
-}
-
+// Two threads per point (lanes 2k and 2k + 1 of a warp): lane parity l
+// reconstructs line l and runs solve l (l = 0 the primary-grid line and solve
+// with normal `type`, spacing h[type]; l = 1 the dual-grid ones with the other
+// normal).  What couples the two solves of a point travels between the
+// partner lanes by warp shuffles: the tangential derivative of each solve (the
+// mean of the other line's l/r derivatives) and the other solve's quarter in
+// W~ (Eq. eq:W-model-2d).  One thread with both solves needs a call frame in
+// local memory (1024^2 vortex, point phase per step: 1.019 ms mixed and
+// 32.06 ms FP64 against 0.903 and 31.41 ms for the pair when it was brought
+// in).  ld(l, e, f) as for recon_line_ld; st(k, v): output k of this lane's
+// solve (PO_*; F and W~ values only when wn).  mask: the lanes of the warp
+// that take part (pairs are valid together).
 // ---------------------------------------------------------------------------
-// The same point with two threads (lanes 2k and 2k + 1 of a warp): lane
-// parity l reconstructs line l and runs solve l (l = 0 the primary-grid solve
-// with normal TYPE, l = 1 the dual-grid solve).  What couples the two solves
-// of a point travels between the partner lanes by warp shuffles: the
-// tangential derivative of each solve (the mean of the other line's l/r
-// derivatives) and the other solve's quarter in W~ (Eq. eq:W-model-2d).
-// Each thread holds one line and one solve instead of two, so the solve runs
-// inline without a local-memory call frame; the arithmetic is point_compute's,
-// in the same order.  mask: the lanes of the warp that take part (pairs are
-// valid together).
-// ---------------------------------------------------------------------------
-template <class R, int TYPE, bool CHAR, class LD, class ST>
+template <class R, bool CHAR, class LD, class ST>
 __device__ __forceinline__ void point_compute_pair(const GenoK<R>& geno, const GasK<R>& gas, const R h[2],
-                                                   const R ih[2], bool wn, int l, unsigned mask, LD ld, ST st) {
-  const int n = l == 0 ? TYPE : 1 - TYPE;   // normal of this lane's solve
+                                                   const R ih[2], bool wn, int type, int l, unsigned mask, LD ld,
+                                                   ST st) {
+  const int n = l == 0 ? type : 1 - type;   // normal of this lane's solve
   R lv[4], ldv[4], rv[4], rdv[4], chi;
   if constexpr (CHAR)
     recon_line_char(geno, gas.gm1, n, ld, l, h[n], ih[n], lv, ldv, rv, rdv, chi);
@@ -420,18 +305,18 @@ __device__ __forceinline__ void point_compute_pair(const GenoK<R>& geno, const G
   st(PO_CHI, chi);
 }
 
-// one thread of a point pair: point (i, j), line / solve l
-template <class R, int TYPE, bool CHAR>
-__device__ __forceinline__ void point_pair_body(const KArgs<R>& a, int i, int j, int l) {
+// one thread of a point pair: point (i, j) of the type, line / solve l
+template <class R, bool CHAR>
+__device__ __forceinline__ void point_pair_body(const KArgs<R>& a, int type, int i, int j, int l) {
   const Layout& L = a.L;
-  const int imax = TYPE == 0 ? L.nx : L.nxd;
-  const int jmax = TYPE == 0 ? L.nyd : L.ny;
+  const int imax = type == 0 ? L.nx : L.nxd;
+  const int jmax = type == 0 ? L.nyd : L.ny;
   const bool valid = !(i < -2 || j < -2 || i > imax || j > jmax);
   const unsigned mask = __ballot_sync(0xffffffffu, valid);
   if (!valid) return;
-  const PointLines pl = point_lines<TYPE>(L, i, j);
+  const PointLines pl = point_lines(L, type, i, j);
   const R* S = a.Sr;
-  R* P = (TYPE == 0 ? a.PA : a.PB) + pcell(L, i, j) + (long)l * NPS * L.pplane;
+  R* P = (type == 0 ? a.PA : a.PB) + pcell(L, i, j) + (long)l * NPS * L.pplane;
   const long pp = L.pplane;
   auto st = [&](int k, R v) { P[(long)k * pp] = v; };
   auto gl = [&](int ll, int e, int f) -> R {
@@ -445,21 +330,69 @@ __device__ __forceinline__ void point_pair_body(const KArgs<R>& a, int i, int j,
   for (int e = 0; e < 4; ++e)
 #pragma unroll
     for (int f = 0; f < 8; ++f) xl[e * 8 + f] = gl(l, e, f);
-  point_compute_pair<R, TYPE, CHAR>(a.geno, a.gas, a.h, a.ih, a.want_n != 0, l, mask,
-                                    [&](int, int e, int f) -> R { return xl[e * 8 + f]; }, st);
+  point_compute_pair<R, CHAR>(a.geno, a.gas, a.h, a.ih, a.want_n != 0, type, l, mask,
+                              [&](int, int e, int f) -> R { return xl[e * 8 + f]; }, st);
   } else {
-    point_compute_pair<R, TYPE, CHAR>(a.geno, a.gas, a.h, a.ih, a.want_n != 0, l, mask, gl, st);
+    point_compute_pair<R, CHAR>(a.geno, a.gas, a.h, a.ih, a.want_n != 0, type, l, mask, gl, st);
   }
 #else
-  point_compute_pair<R, TYPE, CHAR>(a.geno, a.gas, a.h, a.ih, a.want_n != 0, l, mask, gl, st);
+  point_compute_pair<R, CHAR>(a.geno, a.gas, a.h, a.ih, a.want_n != 0, type, l, mask, gl, st);
 #endif
 }
 
-// block (32, 4): 16 points per warp row, two lanes each
-template <class R, int TYPE, bool CHAR>
-__global__ void __launch_bounds__(128, PointTune<R>::pair_minb) point_pair_kernel(KArgs<R> a) {
-  point_pair_body<R, TYPE, CHAR>(a, blockIdx.x * (blockDim.x / 2) + (threadIdx.x >> 1) - 2,
-                                 blockIdx.y * blockDim.y + threadIdx.y - 2, threadIdx.x & 1);
+// Both point types and, if `nodal` is set, the nodal work of a stage in one
+// launch (the three are independent).  FP64: items are dealt out linearly
+// (A pairs, B pairs, nodes) to blocks of one warp, since the FP64 pipe needs
+// one warp per scheduler and nothing else: no tile is partly empty, the last
+// wave is one warp deep, and the short nodal items fill it.  Mixed: tiles of
+// 16 x 4 points (32 x 4 nodes) in blocks of 128, whose rows share lines in L1.
+struct StageGrid {
+  int nA, nB, nN0, nN1;   // items (FP64) or blocks (mixed) of each kind
+  int wA, wB, w0, w1;     // items or blocks per row
+};
+
+template <class R> struct StageTune;
+template <> struct StageTune<double> { static constexpr int threads = FDK_STAGE_THREADS_F64; };
+template <> struct StageTune<float> { static constexpr int threads = 128; };
+
+template <class R, bool CHAR, bool NODAL>
+__global__ void __launch_bounds__(StageTune<R>::threads, PointTune<R>::pair_minb * 128 / StageTune<R>::threads)
+    stage_kernel(KArgs<R> a, StageGrid G) {
+  const int T = StageTune<R>::threads;
+  if constexpr (IsF32<R>::v) {
+    int b = blockIdx.x;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    if (b < G.nA + G.nB) {
+      const int type = b < G.nA ? 0 : 1;
+      if (type) b -= G.nA;
+      const int w = type ? G.wB : G.wA, by = b / w, bx = b - by * w;
+      point_pair_body<R, CHAR>(a, type, bx * 16 + (tx >> 1) - 2, by * 4 + ty - 2, tx & 1);
+    } else if constexpr (NODAL) {
+      b -= G.nA + G.nB;
+      const int g = b < G.nN0 ? 0 : 1;
+      if (g) b -= G.nN0;
+      const int w = g ? G.w1 : G.w0, by = b / w, bx = b - by * w;
+      nodal_body(a, g, bx * 32 + tx - 1, by * 4 + ty - 1);
+    }
+  } else {
+    // whole warps take points or nodes: the point items are padded to a warp
+    const int q = blockIdx.x * T + threadIdx.x;
+    const int np = 2 * (G.nA + G.nB), npp = (np + 31) / 32 * 32;
+    if (q < npp) {
+      int p = q >> 1;
+      const int type = p < G.nA ? 0 : 1;
+      if (type) p -= G.nA;
+      const int w = type ? G.wB : G.wA, j = p / w;
+      point_pair_body<R, CHAR>(a, type, q < np ? p - j * w - 2 : -3, j - 2, q & 1);
+    } else if constexpr (NODAL) {
+      int n = q - npp;
+      if (n >= G.nN0 + G.nN1) return;
+      const int g = n < G.nN0 ? 0 : 1;
+      if (g) n -= G.nN0;
+      const int w = g ? G.w1 : G.w0, j = n / w;
+      nodal_body(a, g, n - j * w - 1, j - 1);
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -523,39 +456,39 @@ __device__ __forceinline__ void node_operator(const KArgs<R>& a, int g, int i, i
     };
     if (chixm == R(1) && chix0 == R(1) && chiym == R(1) && chiy0 == R(1)) components(std::true_type());
     else components(std::false_type());
-    return;
-  }
+  } else {
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const R* nF = NF + (long)c * L.plane;
-    const R* nG = NF + (long)(4 + c) * L.plane;
-    const R* nFt = NF + (long)(8 + c) * L.plane;
-    const R* nGt = NF + (long)(12 + c) * L.plane;
-    const R* pF = PX + (long)(PO_F + c) * pp;
-    const R* pFt = PX + (long)(PO_FT + c) * pp;
-    const R* qF = PY + (long)(PO_F + c) * pp;
-    const R* qFt = PY + (long)(PO_FT + c) * pp;
-    {
-      R fp = compact_flux(fv, chix0, pFt[xm1], pFt[x0], pFt[xp1], nFt[cN], nFt[cN + 1]);
-      R fm = compact_flux(fv, chixm, pFt[xm2], pFt[xm1], pFt[x0], nFt[cN - 1], nFt[cN]);
-      R gp = compact_flux(fv, chiy0, qFt[ym1], qFt[y0], qFt[yp1], nGt[cN], nGt[cN + L.pitch]);
-      R gm = compact_flux(fv, chiym, qFt[ym2], qFt[ym1], qFt[y0], nGt[cN - L.pitch], nGt[cN]);
-      o.Lt[c] = -(fp - fm) * ihx - (gp - gm) * ihy;
+    for (int c = 0; c < 4; ++c) {
+      const R* nF = NF + (long)c * L.plane;
+      const R* nG = NF + (long)(4 + c) * L.plane;
+      const R* nFt = NF + (long)(8 + c) * L.plane;
+      const R* nGt = NF + (long)(12 + c) * L.plane;
+      const R* pF = PX + (long)(PO_F + c) * pp;
+      const R* pFt = PX + (long)(PO_FT + c) * pp;
+      const R* qF = PY + (long)(PO_F + c) * pp;
+      const R* qFt = PY + (long)(PO_FT + c) * pp;
+      {
+        R fp = compact_flux(fv, chix0, pFt[xm1], pFt[x0], pFt[xp1], nFt[cN], nFt[cN + 1]);
+        R fm = compact_flux(fv, chixm, pFt[xm2], pFt[xm1], pFt[x0], nFt[cN - 1], nFt[cN]);
+        R gp = compact_flux(fv, chiy0, qFt[ym1], qFt[y0], qFt[yp1], nGt[cN], nGt[cN + L.pitch]);
+        R gm = compact_flux(fv, chiym, qFt[ym2], qFt[ym1], qFt[y0], nGt[cN - L.pitch], nGt[cN]);
+        o.Lt[c] = -(fp - fm) * ihx - (gp - gm) * ihy;
+      }
+      o.L[c] = R(0);
+      o.gbx[c] = R(0);
+      o.gby[c] = R(0);
+      if (want_n) {
+        R fp = compact_flux(fv, chix0, pF[xm1], pF[x0], pF[xp1], nF[cN], nF[cN + 1]);
+        R fm = compact_flux(fv, chixm, pF[xm2], pF[xm1], pF[x0], nF[cN - 1], nF[cN]);
+        R gp = compact_flux(fv, chiy0, qF[ym1], qF[y0], qF[yp1], nG[cN], nG[cN + L.pitch]);
+        R gm = compact_flux(fv, chiym, qF[ym2], qF[ym1], qF[y0], nG[cN - L.pitch], nG[cN]);
+        o.L[c] = -(fp - fm) * ihx - (gp - gm) * ihy;
+        o.gbx[c] = (PX[(PO_WL + c) * pp + x0] - PX[(PO_WR + c) * pp + xm1]) * ihx;
+        o.gby[c] = (PY[(PO_WL + c) * pp + y0] - PY[(PO_WR + c) * pp + ym1]) * ihy;
+      }
+      o.gtx[c] = (PX[(PO_WLT + c) * pp + x0] - PX[(PO_WRT + c) * pp + xm1]) * ihx;
+      o.gty[c] = (PY[(PO_WLT + c) * pp + y0] - PY[(PO_WRT + c) * pp + ym1]) * ihy;
     }
-    o.L[c] = R(0);
-    o.gbx[c] = R(0);
-    o.gby[c] = R(0);
-    if (want_n) {
-      R fp = compact_flux(fv, chix0, pF[xm1], pF[x0], pF[xp1], nF[cN], nF[cN + 1]);
-      R fm = compact_flux(fv, chixm, pF[xm2], pF[xm1], pF[x0], nF[cN - 1], nF[cN]);
-      R gp = compact_flux(fv, chiy0, qF[ym1], qF[y0], qF[yp1], nG[cN], nG[cN + L.pitch]);
-      R gm = compact_flux(fv, chiym, qF[ym2], qF[ym1], qF[y0], nG[cN - L.pitch], nG[cN]);
-      o.L[c] = -(fp - fm) * ihx - (gp - gm) * ihy;
-      o.gbx[c] = (PX[(PO_WL + c) * pp + x0] - PX[(PO_WR + c) * pp + xm1]) * ihx;
-      o.gby[c] = (PY[(PO_WL + c) * pp + y0] - PY[(PO_WR + c) * pp + ym1]) * ihy;
-    }
-    o.gtx[c] = (PX[(PO_WLT + c) * pp + x0] - PX[(PO_WRT + c) * pp + xm1]) * ihx;
-    o.gty[c] = (PY[(PO_WLT + c) * pp + y0] - PY[(PO_WRT + c) * pp + ym1]) * ihy;
   }
 }
 
@@ -755,27 +688,35 @@ cudaError_t launch_nodal(const KArgs<R>& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// interface points, with the nodal work in the same launch if nodal is set
 template <class R>
-cudaError_t launch_points(const KArgs<R>& a, cudaStream_t s) {
-  dim3 b(32, 4);
-  if constexpr (PointTune<R>::pair) {
-    const dim3 bp(16, 4);   // points per block; the block itself is (32, 4) threads
-    const dim3 gA = grid2(a.L.nx + 3, a.L.nyd + 3, bp, 1), gB = grid2(a.L.nxd + 3, a.L.ny + 3, bp, 1);
-    if (a.recon_vars) point_pair_kernel<R, 0, true><<<gA, b, 0, s>>>(a);
-    else point_pair_kernel<R, 0, false><<<gA, b, 0, s>>>(a);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (a.recon_vars) point_pair_kernel<R, 1, true><<<gB, b, 0, s>>>(a);
-    else point_pair_kernel<R, 1, false><<<gB, b, 0, s>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_points(const KArgs<R>& a, bool nodal, cudaStream_t s) {
+  const Layout& L = a.L;
+  StageGrid G;
+  const int T = StageTune<R>::threads;
+  long blocks;
+  if (IsF32<R>::v) {
+    auto up = [](int n, int b) { return (n + b - 1) / b; };
+    G.wA = up(L.nx + 3, 16); G.nA = G.wA * up(L.nyd + 3, 4);
+    G.wB = up(L.nxd + 3, 16); G.nB = G.wB * up(L.ny + 3, 4);
+    G.w0 = up(L.nx + 2, 32); G.nN0 = G.w0 * up(L.ny + 2, 4);
+    G.w1 = up(L.nxd + 2, 32); G.nN1 = G.w1 * up(L.nyd + 2, 4);
+    blocks = (long)G.nA + G.nB + (nodal ? G.nN0 + G.nN1 : 0);
+  } else {
+    G.wA = L.nx + 3; G.nA = G.wA * (L.nyd + 3);
+    G.wB = L.nxd + 3; G.nB = G.wB * (L.ny + 3);
+    G.w0 = L.nx + 2; G.nN0 = G.w0 * (L.ny + 2);
+    G.w1 = L.nxd + 2; G.nN1 = G.w1 * (L.nyd + 2);
+    const long np = (2L * G.nA + 2L * G.nB + 31) / 32 * 32;
+    blocks = (np + (nodal ? (long)G.nN0 + G.nN1 : 0) + T - 1) / T;
   }
-  const dim3 gA = grid2(a.L.nx + 3, a.L.nyd + 3, b, 1), gB = grid2(a.L.nxd + 3, a.L.ny + 3, b, 1);
-  if (a.recon_vars) point_kernel<R, 0, true><<<gA, b, 0, s>>>(a);
-  else point_kernel<R, 0, false><<<gA, b, 0, s>>>(a);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if (a.recon_vars) point_kernel<R, 1, true><<<gB, b, 0, s>>>(a);
-  else point_kernel<R, 1, false><<<gB, b, 0, s>>>(a);
+  if (a.recon_vars) {
+    if (nodal) stage_kernel<R, true, true><<<(unsigned)blocks, T, 0, s>>>(a, G);
+    else stage_kernel<R, true, false><<<(unsigned)blocks, T, 0, s>>>(a, G);
+  } else {
+    if (nodal) stage_kernel<R, false, true><<<(unsigned)blocks, T, 0, s>>>(a, G);
+    else stage_kernel<R, false, false><<<(unsigned)blocks, T, 0, s>>>(a, G);
+  }
   return cudaGetLastError();
 }
 
@@ -858,7 +799,7 @@ cudaError_t launch_recon_batch(const GenoK<R>& g, int kind, double h, int n, con
 
 #define FDK_INSTANTIATE(R)                                                                                  \
   template cudaError_t launch_nodal<R>(const KArgs<R>&, cudaStream_t);                                     \
-  template cudaError_t launch_points<R>(const KArgs<R>&, cudaStream_t);                                    \
+  template cudaError_t launch_points<R>(const KArgs<R>&, bool, cudaStream_t);                                    \
   template cudaError_t launch_update<R>(const KArgs<R>&, int, cudaStream_t);                               \
   template cudaError_t launch_iface_batch<R>(const GasK<R>&, int, int, const double*, double*, cudaStream_t); \
   template cudaError_t launch_nodal_batch<R>(const GasK<R>&, int, const double*, double*, cudaStream_t);   \
