@@ -395,8 +395,8 @@ __global__ void __launch_bounds__(128) update_adj_kernel(KArgs<double> a, int st
 // ---------------------------------------------------------------------------
 // ghost fill: forward (as the library's) and its adjoint
 // ---------------------------------------------------------------------------
-__global__ void ghost_fwd_kernel(double* S, Layout L, int bc0, int bc1, int dir) {
-  ghost_body(S, L, bc0, bc1, dir, blockIdx.z, blockIdx.x * blockDim.x + threadIdx.x);
+__global__ void ghost_fwd_kernel(double* S, Layout L, GhostPlain K) {
+  ghost_fill(S, L, K, blockIdx.z, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 __global__ void ghost_adj_kernel(double* Sa, Layout L, int bc0, int bc1, int dir) {
@@ -437,12 +437,10 @@ struct Work {
 
 cudaError_t fill_ghosts_fwd(const Work& w, double* S) {
   const Layout& L = w.v.L;
-  const int tx = (L.ny > L.nyd ? L.ny : L.nyd) * 2 * GH;
-  ghost_fwd_kernel<<<dim3((tx + 127) / 128, 1, 2), 128, 0, w.v.stream>>>(S, L, w.v.p.bc[0], w.v.p.bc[1], 0);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  const int ty = ((L.nx > L.nxd ? L.nx : L.nxd) + 2 * GH) * 2 * GH;
-  ghost_fwd_kernel<<<dim3((ty + 127) / 128, 1, 2), 128, 0, w.v.stream>>>(S, L, w.v.p.bc[2], w.v.p.bc[3], 1);
+  GhostPlain K;
+  for (int k = 0; k < 4; ++k) K.bc[k] = w.v.p.bc[k];
+  const int n = ghost_count(std::max(L.nx, L.nxd), std::max(L.ny, L.nyd));
+  ghost_fwd_kernel<<<dim3((n + 127) / 128, 1, 2), 128, 0, w.v.stream>>>(S, L, K);
   return cudaGetLastError();
 }
 

@@ -122,19 +122,13 @@ const char* fdk::check_params(const fdcgks_params* p) {
 static size_t rsize(const fdcgks_params& p) { return p.precision == FDCGKS_MIXED ? sizeof(float) : sizeof(double); }
 
 // ---------------------------------------------------------------------------
-// ghost fill: periodic wrap, mirror (symmetry / no-slip) or constant
-// extrapolation (transmissive); x pass over interior rows, then y pass over
-// all columns so that corners are filled consistently
+// ghost fill: periodic wrap, mirror (symmetry / no-slip), constant
+// extrapolation (transmissive) or a fixed state, all ghosts of both grids in
+// one launch (ghost_fill)
 // ---------------------------------------------------------------------------
-template <class T>
-__global__ void ghost_kernel(T* S, Layout L, int bc0, int bc1, int dir) {
-  int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  ghost_body(S, L, bc0, bc1, dir, blockIdx.z, idx);
-}
-
-template <class T>
-__global__ void ghost_sides_kernel(T* S, Layout L, GhostSides gs, int dir) {
-  ghost_body_sides(S, L, gs, dir, blockIdx.z, blockIdx.x * blockDim.x + threadIdx.x);
+template <class T, class KINDS>
+__global__ void ghost_kernel(T* S, Layout L, KINDS K) {
+  ghost_fill(S, L, K, blockIdx.z, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // split sides evaluated at time t
@@ -145,7 +139,7 @@ static GhostSides ghost_sides(fdcgks_t c, double t) {
     const fdcgks_side& sd = c->sides[k];
     gs.split[k] = std::fma(sd.split_speed, t, sd.split0);
     for (int q = 0; q < 2; ++q) {
-      gs.kind[k][q] = sd.kind[q];
+      gs.kinds[k][q] = sd.kind[q];
       const double* pr = sd.prim[q];
       gs.W[k][q][0] = pr[0];
       gs.W[k][q][1] = pr[0] * pr[1];
@@ -164,20 +158,14 @@ static GhostSides ghost_sides(fdcgks_t c, double t) {
 template <class T>
 static cudaError_t fill_ghosts(fdcgks_t c, T* S, double t) {
   const Layout& L = c->L;
-  int tx = (L.ny > L.nyd ? L.ny : L.nyd) * 2 * GH;
-  int ty = ((L.nx > L.nxd ? L.nx : L.nxd) + 2 * GH) * 2 * GH;
+  const dim3 grid((ghost_count(std::max(L.nx, L.nxd), std::max(L.ny, L.nyd)) + 127) / 128, 1, 2);
   if (c->has_sides) {
-    const GhostSides gs = ghost_sides(c, t);
-    ghost_sides_kernel<T><<<dim3((tx + 127) / 128, 1, 2), 128, 0, c->stream>>>(S, L, gs, 0);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    ghost_sides_kernel<T><<<dim3((ty + 127) / 128, 1, 2), 128, 0, c->stream>>>(S, L, gs, 1);
-    return cudaGetLastError();
+    ghost_kernel<<<grid, 128, 0, c->stream>>>(S, L, ghost_sides(c, t));
+  } else {
+    GhostPlain K;
+    for (int k = 0; k < 4; ++k) K.bc[k] = c->p.bc[k];
+    ghost_kernel<<<grid, 128, 0, c->stream>>>(S, L, K);
   }
-  ghost_kernel<T><<<dim3((tx + 127) / 128, 1, 2), 128, 0, c->stream>>>(S, L, c->p.bc[0], c->p.bc[1], 0);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  ghost_kernel<T><<<dim3((ty + 127) / 128, 1, 2), 128, 0, c->stream>>>(S, L, c->p.bc[2], c->p.bc[3], 1);
   return cudaGetLastError();
 }
 
@@ -469,7 +457,7 @@ static fdcgks_status run_stage(fdcgks_t c, double dt, int mode, double* const* o
   CUDA_TRY(c, prof_mark(c, KC_UPDATE, true));
   CUDA_TRY(c, launch_update<R>(a, mode, c->stream));
   CUDA_TRY(c, prof_mark(c, KC_UPDATE, false));
-  c->launches += apart ? 5 : 4;   // 2 ghost passes, nodes and points, update
+  c->launches += apart ? 4 : 3;   // ghosts, nodes and points, update
   return FDCGKS_OK;
 }
 

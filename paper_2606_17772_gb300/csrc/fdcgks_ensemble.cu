@@ -103,10 +103,13 @@ __global__ void __launch_bounds__(ENS_THREADS, (EnsMinB<R, PH>::v)) ens_phase_ke
       __syncthreads();
       const int li = threadIdx.x & ((1 << q.lbx) - 1), lj = threadIdx.x >> q.lbx;
       const int i = (tl.z << q.lbx) + li, j = tl.w * (ENS_THREADS >> q.lbx) + lj;
-      if (PH == PH_GHOSTX) {
-        ghost_body(const_cast<R*>(sa.Sr), sa.L, sa.bc[0], sa.bc[1], 0, tl.y, tl.z * ENS_THREADS + threadIdx.x);
-      } else if (PH == PH_GHOSTY) {
-        ghost_body(const_cast<R*>(sa.Sr), sa.L, sa.bc[2], sa.bc[3], 1, tl.y, tl.z * ENS_THREADS + threadIdx.x);
+      if (PH == PH_GHOSTX || PH == PH_GHOSTY) {
+        // x ghosts of the interior rows, then the y ghosts (ghost_fill's items in two launches)
+        GhostPlain K;
+        for (int k = 0; k < 4; ++k) K.bc[k] = sa.bc[k];
+        const int nx6 = 2 * GH * (tl.y == 0 ? sa.L.ny : sa.L.nyd), idx = tl.z * ENS_THREADS + threadIdx.x;
+        if (PH == PH_GHOSTY || idx < nx6)
+          ghost_fill(const_cast<R*>(sa.Sr), sa.L, K, tl.y, PH == PH_GHOSTX ? idx : nx6 + idx);
       } else if (PH == PH_NODAL) {
         nodal_body(sa, tl.y, i - 1, j - 1);
       } else if (PH == PH_POINTS) {

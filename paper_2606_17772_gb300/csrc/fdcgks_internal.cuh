@@ -129,7 +129,8 @@ struct KArgs {
   double* op[8];         // operator outputs (Lp, Ltp, gbp, gtp, Ld, Ltd, gbd, gtd), interior layout
 };
 
-// Ghost layers of one grid g of a padded state (W, x- and y-gradients):
+// Ghost layers of one grid g of a padded state (W, x- and y-gradients), as the
+// adjoint folds them back (the forward fill is ghost_fill below):
 // periodic wrap, mirror (symmetry: normal momentum odd; no-slip: both momenta
 // odd; gradients take the field's parity times -1 along the mirror normal) or
 // constant extrapolation with zero gradients (transmissive).  Work item idx
@@ -169,77 +170,102 @@ FD_HD void ghost_sign(int b, int dir, int c, int& sW, int& sgx, int& sgy) {
   sgy = dir == 1 ? -sW : sW;
 }
 
-// copy the source node into the ghost node with the parities of kind b
+// Kinds of the four sides (x-low, x-high, y-low, y-high) as params.bc gives
+// them, and as split sides (fdcgks_set_sides) evaluated at one stage time:
+// kind of each part, the split position along the side, the fixed conservative
+// states, the node geometry for the coordinate along the side.  kind(side, g,
+// t): the boundary kind at row or column t of grid g (part: which part).
+struct GhostPlain {
+  int bc[4];
+  FD_HD int kind(int side, int, int, int& part) const { part = 0; return bc[side]; }
+  FD_HD double fixed(int, int, int) const { return 0.0; }
+};
+struct GhostSides {
+  int kinds[4][2];
+  double split[4];
+  double W[4][2][4];
+  double x0, y0, hx, hy;
+  // coordinate along the side of the ghost's row (x sides) or column (y
+  // sides), a single-rounded fused product like the split point, so that a
+  // node lying on the split is classified independently of contraction
+  FD_HD int kind(int side, int g, int t, int& part) const {
+    const double pos = t + (g == 0 ? 0.5 : 0.0);
+    const double coord = side < 2 ? fma(pos, hy, y0) : fma(pos, hx, x0);
+    part = coord < split[side] ? 0 : 1;
+    return kinds[side][part];
+  }
+  FD_HD double fixed(int side, int part, int c) const { return W[side][part][c]; }
+};
+
+// index inside [0, n) that the ghost index takes its value from under kind b
+FD_HD int ghost_source(int b, int g, int n, int ghost) {
+  if (b == 0) return ((ghost % n) + n) % n;                       // periodic, also for n < GH
+  if (b == 1 || b == 4) return ghost < 0 ? 0 : n - 1;             // transmissive (fixed: not read)
+  if (g == 0) return ghost < 0 ? -ghost - 1 : 2 * n - 1 - ghost;  // mirror about the boundary line
+  return ghost < 0 ? -ghost : 2 * n - 2 - ghost;
+}
+
+#ifdef __CUDACC__
+// the boundary kind b along direction dir applied to one component's values
 template <class T>
-__device__ __forceinline__ void ghost_apply(T* Sg, const Layout& L, int b, int dir, long gc, long sc) {
+__device__ __forceinline__ void ghost_rule(int b, int dir, int c, double fixed, T& w, T& gx, T& gy) {
+  if (b == 0) return;
+  if (b == 1 || b == 4) {
+    if (b == 4) w = (T)fixed;
+    gx = 0;
+    gy = 0;
+    return;
+  }
+  int sW, sgx, sgy;
+  ghost_sign(b, dir, c, sW, sgx, sgy);
+  w *= (T)sW;
+  gx *= (T)sgx;
+  gy *= (T)sgy;
+}
+
+// Number of ghost nodes of a grid: three columns either side of the interior
+// rows, three rows above and below all columns (corners included).
+FD_HD int ghost_count(int nxg, int nyg) { return 2 * GH * (nyg + nxg + 2 * GH); }
+
+// Ghost node idx of grid g.  A corner's value is its row's y-ghost of an
+// x-ghost; both rules are applied here in that order to the interior value, so
+// one pass over all ghosts reads interior nodes only and needs no second
+// launch behind the x ghosts (and writes nothing that another item reads).
+template <class T, class KINDS>
+__device__ __forceinline__ void ghost_fill(T* S, const Layout& L, const KINDS& K, int g, int idx) {
+  const int nxg = g == 0 ? L.nx : L.nxd, nyg = g == 0 ? L.ny : L.nyd;
+  if (idx >= ghost_count(nxg, nyg)) return;
+  const bool ypart = idx >= 2 * GH * nyg;
+  if (ypart) idx -= 2 * GH * nyg;
+  const int t = idx / (2 * GH) - (ypart ? GH : 0);   // row (x ghosts) or column (y ghosts)
+  const int k = idx % (2 * GH), n = ypart ? nyg : nxg;
+  const int ghost = k < GH ? -1 - k : n - GH + k;    // -1, -2, -3, n, n + 1, n + 2
+  const int i = ypart ? t : ghost, j = ypart ? ghost : t;
+  int by = 0, bx = 0, py = 0, px = 0, sy = 0, sx = 0, is = i, js = j;
+  if (ypart) {
+    sy = j < 0 ? 2 : 3;
+    by = K.kind(sy, g, i, py);
+    js = ghost_source(by, g, nyg, j);
+  }
+  const bool xg = i < 0 || i >= nxg;
+  if (xg) {
+    sx = i < 0 ? 0 : 1;
+    bx = K.kind(sx, g, js, px);
+    is = ghost_source(bx, g, nxg, i);
+  }
+  T* Sg = S + (long)g * NFLD * L.plane;
+  const long sc = cell(L, is, js), gc = cell(L, i, j);
+#pragma unroll
   for (int c = 0; c < 4; ++c) {
-    int sW, sgx, sgy;
-    ghost_sign(b, dir, c, sW, sgx, sgy);
-    T w = Sg[(long)c * L.plane + sc];
-    T gx = Sg[(long)(4 + c) * L.plane + sc];
-    T gy = Sg[(long)(8 + c) * L.plane + sc];
-    if (b == 1) {
-      gx = 0;
-      gy = 0;
-    } else if (b != 0) {
-      w *= (T)sW;
-      gx *= (T)sgx;
-      gy *= (T)sgy;
-    }
+    T w = Sg[(long)c * L.plane + sc], gx = Sg[(long)(4 + c) * L.plane + sc], gy = Sg[(long)(8 + c) * L.plane + sc];
+    if (xg) ghost_rule(bx, 0, c, K.fixed(sx, px, c), w, gx, gy);
+    if (ypart) ghost_rule(by, 1, c, K.fixed(sy, py, c), w, gx, gy);
     Sg[(long)c * L.plane + gc] = w;
     Sg[(long)(4 + c) * L.plane + gc] = gx;
     Sg[(long)(8 + c) * L.plane + gc] = gy;
   }
 }
-
-template <class T>
-__device__ __forceinline__ void ghost_body(T* S, const Layout& L, int bc0, int bc1, int dir, int g, int idx) {
-  long gc, sc;
-  int b;
-  if (!ghost_map(L, bc0, bc1, dir, g, idx, gc, sc, b)) return;
-  ghost_apply(S + (long)g * NFLD * L.plane, L, b, dir, gc, sc);
-}
-
-// Split sides (fdcgks_set_sides), at one stage time: kind of each part, the
-// split position along the side, the fixed conservative states, the node
-// geometry for the coordinate along the side.
-struct GhostSides {
-  int kind[4][2];
-  double split[4];
-  double W[4][2][4];
-  double x0, y0, hx, hy;
-};
-
-template <class T>
-__device__ __forceinline__ void ghost_body_sides(T* S, const Layout& L, const GhostSides& gs, int dir, int g,
-                                                 int idx) {
-  const int nxg = g == 0 ? L.nx : L.nxd, nyg = g == 0 ? L.ny : L.nyd;
-  const int tcount = dir == 0 ? nyg : nxg + 2 * GH;
-  if (idx < 0 || idx >= tcount * 2 * GH) return;
-  const int side = (idx / GH) % 2;
-  const int t = idx / (2 * GH) + (dir == 0 ? 0 : -GH);
-  const int sd = 2 * dir + side;
-  // coordinate along the side of the ghost's row (x sides) or column (y
-  // sides), a single-rounded fused product like the split point, so that a
-  // node lying on the split is classified independently of contraction
-  const double pos = t + (g == 0 ? 0.5 : 0.0);
-  const double coord = dir == 0 ? fma(pos, gs.hy, gs.y0) : fma(pos, gs.hx, gs.x0);
-  const int part = coord < gs.split[sd] ? 0 : 1;
-  const int kind = gs.kind[sd][part];
-  long gc, sc;
-  int b;
-  if (!ghost_map(L, kind, kind, dir, g, idx, gc, sc, b)) return;
-  T* Sg = S + (long)g * NFLD * L.plane;
-  if (kind == 4) {   // FIXED
-    for (int c = 0; c < 4; ++c) {
-      Sg[(long)c * L.plane + gc] = (T)gs.W[sd][part][c];
-      Sg[(long)(4 + c) * L.plane + gc] = 0;
-      Sg[(long)(8 + c) * L.plane + gc] = 0;
-    }
-    return;
-  }
-  ghost_apply(Sg, L, b, dir, gc, sc);
-}
+#endif
 
 enum { UPD_STAGE1 = 0, UPD_STAGE2 = 1, UPD_OPERATOR = 2 };
 
