@@ -38,8 +38,10 @@ struct fdcgks_ctx {
   void* PA = nullptr;       // point outputs [50][pplane]
   void* PB = nullptr;
   int* flag = nullptr;      // device flags
-  double* red = nullptr;    // reduction scratch
-  int red_blocks = 0;
+  struct CflRes* res = nullptr;   // CFL maxima (device), zero between calls
+  float2* est = nullptr;          // CFL screening maxima [red_blocks]
+  double* res_host = nullptr;     // the two maxima, pinned host memory written by the device
+  int red_blocks = 0;             // most blocks of the CFL reduction
   bool has_state = false;
   // kernel-class timing with CUDA events on the context stream (optional)
   int profiling = 0;
@@ -247,7 +249,7 @@ struct StatePair {
   __device__ float est(long k) const { return hi[k]; }
 };
 
-// Work split of the CFL passes: the rows of both grids (primary first), each
+// Work split of the CFL reduction: the rows of both grids (primary first), each
 // cut into segments of CFL_SEG nodes; an item is one segment of one row.
 // The FP32 constants of the screening go with it.
 const int CFL_SEG = 1024;
@@ -271,7 +273,7 @@ __device__ __forceinline__ void cfl_item(const CflGrid& G, int it, F f) {
   for (int i = seg * CFL_SEG + threadIdx.x; i < i1; i += blockDim.x) f(base + cell(L, i, j));
 }
 
-// block-wide maxima of two values (>= 0) into thread 0; blockDim.x <= 1024
+// block-wide maxima of two values (>= 0), in every thread; blockDim.x <= 1024
 template <class T>
 __device__ __forceinline__ void block_max2(T& a, T& b, T* sa, T* sb) {
   for (int o = 16; o > 0; o >>= 1) {
@@ -281,15 +283,13 @@ __device__ __forceinline__ void block_max2(T& a, T& b, T* sa, T* sb) {
   const int w = threadIdx.x / 32;
   if ((threadIdx.x & 31) == 0) { sa[w] = a; sb[w] = b; }
   __syncthreads();
-  if (threadIdx.x == 0)
-    for (int k = 1; k < (int)(blockDim.x / 32); ++k) { a = fmax(a, sa[k]); b = fmax(b, sb[k]); }
+  for (int k = 0; k < (int)(blockDim.x / 32); ++k) { a = fmax(a, sa[k]); b = fmax(b, sb[k]); }
 }
 
-// First pass: the largest reliable FP32 estimates (cfl_estimate_f) of the
-// rate and of nu over all nodes, folded into mxf[0..1] (zeroed before) with
-// atomicMax on the bit patterns (non-negative floats order as their bits).
+// First pass of large grids: per-block maxima of the reliable FP32 estimates
+// (cfl_estimate_f) of the rate and of nu.
 template <class ST>
-__global__ void cfl_screen_kernel(ST S, CflGrid G, int items, unsigned* mxf) {
+__global__ void cfl_screen_kernel(ST S, CflGrid G, int items, float2* est) {
   __shared__ float sa[32], sb[32];
   float mr = 0.0f, mn = 0.0f;
   const long P = G.L.plane;
@@ -305,31 +305,46 @@ __global__ void cfl_screen_kernel(ST S, CflGrid G, int items, unsigned* mxf) {
       }
     });
   block_max2(mr, mn, sa, sb);
-  if (threadIdx.x == 0) {
-    if (mr > 0.0f) atomicMax(mxf, __float_as_uint(mr));
-    if (mn > 0.0f) atomicMax(mxf + 1, __float_as_uint(mn));
-  }
+  if (threadIdx.x == 0) est[blockIdx.x] = make_float2(mr, mn);
 }
 
-// Second pass: per-block maxima of the FP64 rate and nu, evaluated (from the
-// FP64 entries or the joined pairs) only at nodes whose estimate is
-// unreliable or within CFL_SCREEN_MARGIN of the first pass's maxima; the
-// maxima are exactly those of evaluating every node.
-template <class ST>
-__global__ void cfl_kernel(ST S, CflGrid G, int items, const unsigned* mxf, double* out) {
+// The maxima of the FP64 rate and nu (from the FP64 entries or the joined
+// pairs): of every node (ALL), or, given the first pass's nest maxima, of the
+// nodes whose estimate is unreliable or within CFL_SCREEN_MARGIN of the
+// largest; the maxima are exactly those of evaluating every node.  res: the
+// maxima as bit patterns (>= 0, ordered as their values) and the blocks done;
+// the last block to finish writes them to out (pinned host memory) and leaves
+// res zeroed for the next call, so the call needs neither a clear nor a copy.
+struct CflRes {
+  unsigned long long rate, nu;
+  unsigned done;
+};
+template <class ST, bool ALL>
+__global__ void cfl_kernel(ST S, CflGrid G, int items, const float2* est, int nest, CflRes* res, double* out) {
+  __shared__ float fa[32], fb[32];
   __shared__ double sa[32], sb[32];
-  double rate = 0.0, numax = 0.0;
   const long P = G.L.plane;
-  const float mr = __uint_as_float(mxf[0]), mn = __uint_as_float(mxf[1]);
-  const float tr = mr * (1.0f - CFL_SCREEN_MARGIN);
-  const float tn = mn > 0.0f ? mn * (1.0f - CFL_SCREEN_MARGIN) : INFINITY;   // mu = 0: nu never decides
+  float tr = 0.0f, tn = INFINITY;
+  if (!ALL) {
+    float mr = 0.0f, mn = 0.0f;
+    for (int k = threadIdx.x; k < nest; k += blockDim.x) {
+      mr = fmaxf(mr, est[k].x);
+      mn = fmaxf(mn, est[k].y);
+    }
+    block_max2(mr, mn, fa, fb);
+    tr = mr * (1.0f - CFL_SCREEN_MARGIN);
+    if (mn > 0.0f) tn = mn * (1.0f - CFL_SCREEN_MARGIN);   // mu = 0: nu never decides
+  }
+  double rate = 0.0, numax = 0.0;
   for (int it = blockIdx.x; it < items; it += gridDim.x)
     cfl_item(G, it, [&](long c0) {
-      float rt, nu;
-      bool ok;
-      cfl_estimate_f(S.est(c0), S.est(c0 + P), S.est(c0 + 2 * P), S.est(c0 + 3 * P), G.gf, G.muf, G.ihxf, G.ihyf,
-                     G.sum != 0, rt, nu, ok);
-      if (ok && rt < tr && nu < tn) return;
+      if (!ALL) {
+        float rt, nu;
+        bool ok;
+        cfl_estimate_f(S.est(c0), S.est(c0 + P), S.est(c0 + 2 * P), S.est(c0 + 3 * P), G.gf, G.muf, G.ihxf, G.ihyf,
+                       G.sum != 0, rt, nu, ok);
+        if (ok && rt < tr && nu < tn) return;
+      }
       const double r = S(c0), ru = S(c0 + P), rv = S(c0 + 2 * P), E = S(c0 + 3 * P);
       if (G.sum)
         cfl_rates_sum(r, ru, rv, E, G.gamma, G.mu, G.ihx, G.ihy, rate, numax);
@@ -337,11 +352,21 @@ __global__ void cfl_kernel(ST S, CflGrid G, int items, const unsigned* mxf, doub
         cfl_rates(r, ru, rv, E, G.gamma, G.mu, G.ihx, G.ihy, rate, numax);
     });
   block_max2(rate, numax, sa, sb);
-  if (threadIdx.x == 0) {
-    out[2 * blockIdx.x] = rate;
-    out[2 * blockIdx.x + 1] = numax;
-  }
+  if (threadIdx.x != 0) return;
+  if (rate > 0.0) atomicMax(&res->rate, (unsigned long long)__double_as_longlong(rate));
+  if (numax > 0.0) atomicMax(&res->nu, (unsigned long long)__double_as_longlong(numax));
+  __threadfence();
+  if (atomicAdd(&res->done, 1u) + 1u < gridDim.x) return;
+  __threadfence();
+  out[0] = __longlong_as_double((long long)atomicExch(&res->rate, 0ull));
+  out[1] = __longlong_as_double((long long)atomicExch(&res->nu, 0ull));
+  res->done = 0;
 }
+
+// Nodes (both grids) up to which the maxima are taken in one FP64 pass: about
+// 35 slots of the FP64 pipe a node, 2.4 us at 40000 nodes over 152 SMs, where
+// the FP32 screen's second launch costs about 3 us
+const long CFL_ALL_NODES = 40000;
 
 // ---------------------------------------------------------------------------
 // optional timing of kernel classes (events recorded around each launch group)
@@ -500,6 +525,23 @@ fdcgks_status fdk::ctx_replay_step(fdcgks_t c, double dt, const double* in, doub
   return FDCGKS_OK;
 }
 
+template <class ST>
+static cudaError_t launch_cfl(fdcgks_t c, const ST& st, const CflGrid& G, int items) {
+  const int blocks = std::min(items, c->red_blocks);
+  const Layout& L = c->L;
+  if ((long)L.nx * L.ny + (long)L.nxd * L.nyd <= CFL_ALL_NODES) {
+    cfl_kernel<ST, true><<<blocks, 256, 0, c->stream>>>(st, G, items, nullptr, 0, c->res, c->res_host);
+    c->launches += 1;
+    return cudaGetLastError();
+  }
+  cfl_screen_kernel<<<blocks, 256, 0, c->stream>>>(st, G, items, c->est);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  cfl_kernel<ST, false><<<blocks, 256, 0, c->stream>>>(st, G, items, c->est, blocks, c->res, c->res_host);
+  c->launches += 2;
+  return cudaGetLastError();
+}
+
 // ---------------------------------------------------------------------------
 // C entry points
 // ---------------------------------------------------------------------------
@@ -526,9 +568,10 @@ void fdcgks_destroy(fdcgks_t c) {
   delete[] c->ev;
   delete[] c->ev_class;
   void* bufs[] = {c->S, c->S2, c->Sf, c->Slo, c->S2f, c->Acc_hi, c->Acc_lo, c->Gb_hi, c->Gb_lo,
-                  c->Wacc, c->gB, c->NF, c->PA, c->PB, c->flag, c->red};
+                  c->Wacc, c->gB, c->NF, c->PA, c->PB, c->flag, c->res, c->est};
   for (void* b : bufs)
     if (b) cudaFree(b);
+  if (c->res_host) cudaFreeHost(c->res_host);
   delete c;
 }
 
@@ -576,10 +619,11 @@ fdcgks_status fdcgks_create(const fdcgks_params* p, fdcgks_t* out) {
     }
   }
   c->red_blocks = 1024;
-  // per-block maxima, then the two screening maxima (2 unsigned in one more double)
-  if (cudaMalloc((void**)&c->red, sizeof(double) * (2 * c->red_blocks + 1)) != cudaSuccess) {
+  if (cudaMalloc((void**)&c->res, sizeof(CflRes)) != cudaSuccess ||
+      cudaMalloc((void**)&c->est, sizeof(float2) * c->red_blocks) != cudaSuccess ||
+      cudaHostAlloc((void**)&c->res_host, 2 * sizeof(double), cudaHostAllocMapped) != cudaSuccess) {
     fdcgks_destroy(c);
-    return fail(nullptr, FDCGKS_ERR_NOMEM, "cudaMalloc of the reduction scratch failed");
+    return fail(nullptr, FDCGKS_ERR_NOMEM, "allocation of the reduction scratch failed");
   }
   // zero everything once so that ghost corners and unused entries are defined
   cudaError_t e = cudaSuccess;
@@ -588,6 +632,7 @@ fdcgks_status fdcgks_create(const fdcgks_params* p, fdcgks_t* out) {
   if (c->Sf) e = e == cudaSuccess ? cudaMemsetAsync(c->Sf, 0, sizeof(float) * 2 * NFLD * L.plane, c->stream) : e;
   if (c->S2f) e = e == cudaSuccess ? cudaMemsetAsync(c->S2f, 0, sizeof(float) * 2 * NFLD * L.plane, c->stream) : e;
   e = e == cudaSuccess ? cudaMemsetAsync(c->flag, 0, sizeof(int) * 4, c->stream) : e;
+  e = e == cudaSuccess ? cudaMemsetAsync(c->res, 0, sizeof(CflRes), c->stream) : e;
   e = e == cudaSuccess ? cudaStreamSynchronize(c->stream) : e;
   if (e != cudaSuccess) {
     fdcgks_destroy(c);
@@ -777,36 +822,12 @@ static fdcgks_status cfl_dt_impl(fdcgks_t c, double cfl, int sum, double* dt_out
   G.sum = sum;
   const long items = (long)(c->L.ny + c->L.nyd) * G.segs;
   if (items > INT_MAX) return fail(c, FDCGKS_ERR_ARG, "grid too large for the CFL reduction");
-  unsigned* mxf = (unsigned*)(c->red + 2 * c->red_blocks);
   CUDA_TRY(c, prof_mark(c, KC_CFL, true));
-  CUDA_TRY(c, cudaMemsetAsync(mxf, 0, 2 * sizeof(unsigned), c->stream));
-  if (c->Sf) {
-    const StatePair st{c->Sf, c->Slo};
-    cfl_screen_kernel<<<c->red_blocks, 256, 0, c->stream>>>(st, G, (int)items, mxf);
-    CUDA_TRY(c, cudaGetLastError());
-    cfl_kernel<<<c->red_blocks, 256, 0, c->stream>>>(st, G, (int)items, mxf, c->red);
-  } else {
-    const StateF64 st{c->S};
-    cfl_screen_kernel<<<c->red_blocks, 256, 0, c->stream>>>(st, G, (int)items, mxf);
-    CUDA_TRY(c, cudaGetLastError());
-    cfl_kernel<<<c->red_blocks, 256, 0, c->stream>>>(st, G, (int)items, mxf, c->red);
-  }
-  CUDA_TRY(c, cudaGetLastError());
-  c->launches += 2;
+  CUDA_TRY(c, c->Sf ? launch_cfl(c, StatePair{c->Sf, c->Slo}, G, (int)items)
+                    : launch_cfl(c, StateF64{c->S}, G, (int)items));
   CUDA_TRY(c, prof_mark(c, KC_CFL, false));
-  double* h = new double[2 * c->red_blocks];
-  cudaError_t e = cudaMemcpyAsync(h, c->red, sizeof(double) * 2 * c->red_blocks, cudaMemcpyDeviceToHost, c->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  if (e != cudaSuccess) {
-    delete[] h;
-    return fail(c, FDCGKS_ERR_CUDA, "cfl reduction: %s", cudaGetErrorString(e));
-  }
-  double rate = 0.0, numax = 0.0;
-  for (int b = 0; b < c->red_blocks; ++b) {
-    rate = std::fmax(rate, h[2 * b]);
-    numax = std::fmax(numax, h[2 * b + 1]);
-  }
-  delete[] h;
+  CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  const double rate = ((volatile double*)c->res_host)[0], numax = ((volatile double*)c->res_host)[1];
   if (!(rate > 0.0) || !std::isfinite(rate)) return fail(c, FDCGKS_ERR_NONPHYSICAL, "no finite wave speed");
   double dt = cfl / rate;
   if (numax > 0.0) {
