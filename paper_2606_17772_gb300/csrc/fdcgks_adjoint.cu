@@ -542,29 +542,6 @@ cudaError_t adjoint_step(const Work& w, double dt, const double* Aout, double* A
   return cudaSuccess;
 }
 
-// dense [4][ny][nx] / [2][4][ny][nx] <-> padded planes of one grid
-cudaError_t dense_copy(const Work& w, double* pad, const double* Wsrc, const double* Gsrc, double* Wdst,
-                       double* Gdst, int g) {
-  const Layout& L = w.v.L;
-  const int nxg = g == 0 ? L.nx : L.nxd, nyg = g == 0 ? L.ny : L.nyd;
-  const long NN = (long)nxg * nyg;
-  for (int f = 0; f < NFLD; ++f) {
-    double* p = pad + ((long)g * NFLD + f) * L.plane + cell(L, 0, 0);
-    cudaError_t e;
-    if (Wsrc) {
-      const double* src = f < 4 ? Wsrc + f * NN : Gsrc + (f - 4) * NN;
-      e = cudaMemcpy2DAsync(p, sizeof(double) * L.pitch, src, sizeof(double) * nxg, sizeof(double) * nxg, nyg,
-                            cudaMemcpyDeviceToDevice, w.v.stream);
-    } else {
-      double* dst = f < 4 ? Wdst + f * NN : Gdst + (f - 4) * NN;
-      e = cudaMemcpy2DAsync(dst, sizeof(double) * nxg, p, sizeof(double) * L.pitch, sizeof(double) * nxg, nyg,
-                            cudaMemcpyDeviceToDevice, w.v.stream);
-    }
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
 fdcgks_status afail(fdcgks_t c, fdcgks_status s, const char* what, cudaError_t e = cudaSuccess) {
   char m[400];
   if (e != cudaSuccess) snprintf(m, sizeof(m), "%s: %s", what, cudaGetErrorString(e));
@@ -648,8 +625,9 @@ extern "C" fdcgks_status fdcgks_vjp_steps(fdcgks_t ctx, double dt, int nsteps, i
     // adjoint of the final state
     double* Aout = w.A0;
     double* Ain = w.A1;
-    if ((r = dense_copy(w, Aout, aWp, aGp, nullptr, nullptr, 0)) != cudaSuccess ||
-        (r = dense_copy(w, Aout, aWd, aGd, nullptr, nullptr, 1)) != cudaSuccess)
+    const DenseState seed{{const_cast<double*>(aWp), const_cast<double*>(aWd)},
+                          {const_cast<double*>(aGp), const_cast<double*>(aGd)}};
+    if ((r = launch_load(seed, L, 0.0, Aout, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s)) != cudaSuccess)
       return afail(ctx, FDCGKS_ERR_CUDA, "adjoint seed", r);
     // reverse sweep, one checkpoint segment at a time
     for (int k = nck - 1; k >= 0; --k) {
@@ -666,8 +644,7 @@ extern "C" fdcgks_status fdcgks_vjp_steps(fdcgks_t ctx, double dt, int nsteps, i
         std::swap(Aout, Ain);
       }
     }
-    if ((r = dense_copy(w, Aout, nullptr, nullptr, gWp, gGp, 0)) != cudaSuccess ||
-        (r = dense_copy(w, Aout, nullptr, nullptr, gWd, gGd, 1)) != cudaSuccess)
+    if ((r = launch_store(DenseState{{gWp, gWd}, {gGp, gGd}}, L, Aout, nullptr, nullptr, s)) != cudaSuccess)
       return afail(ctx, FDCGKS_ERR_CUDA, "gradient copy", r);
     if (mixed && (fs = ctx_load_padded(ctx, w.fin)) != FDCGKS_OK) return fs;
     if ((r = cudaStreamSynchronize(s)) != cudaSuccess) return afail(ctx, FDCGKS_ERR_CUDA, "adjoint", r);

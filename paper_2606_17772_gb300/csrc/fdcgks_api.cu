@@ -40,7 +40,7 @@ struct fdcgks_ctx {
   int* flag = nullptr;      // device flags
   struct CflRes* res = nullptr;   // CFL maxima (device), zero between calls
   float2* est = nullptr;          // CFL screening maxima [red_blocks]
-  double* res_host = nullptr;     // the two maxima, pinned host memory written by the device
+  double* res_host = nullptr;     // pinned host memory the device writes: the two maxima, set_state's verdict
   int red_blocks = 0;             // most blocks of the CFL reduction
   bool has_state = false;
   // kernel-class timing with CUDA events on the context stream (optional)
@@ -199,25 +199,79 @@ static cudaError_t join_state(fdcgks_t c) {
 }
 
 // ---------------------------------------------------------------------------
-// state validation and CFL reduction
+// loading, validation and reading of a state; CFL reduction
 // ---------------------------------------------------------------------------
-__global__ void validate_kernel(const double* S, Layout L, double gamma, int* flag) {
+// One thread per node and its 12 values: a warp reads and writes 32
+// consecutive entries of one field at a time.  At 1024^2 a load moves 604 MB
+// (mixed: dense state in, FP64 copy and pairs out), against 24 pitched copies,
+// a split and a validation pass that moved 1.4 GB in 27 launches.
+__global__ void load_kernel(DenseState d, Layout L, double gamma, double* S, float* hi, float* lo, int* bad, int* clear,
+                            double* t0, double* t1) {
   const int g = blockIdx.z;
   const int nxg = g == 0 ? L.nx : L.nxd, nyg = g == 0 ? L.ny : L.nyd;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-  if (i >= nxg || j >= nyg) return;
-  const double* Sg = S + (long)g * NFLD * L.plane;
-  const long c0 = cell(L, i, j);
-  double r = Sg[c0], mu_ = Sg[L.plane + c0], mv_ = Sg[2 * L.plane + c0], E = Sg[3 * L.plane + c0];
-  double p = (gamma - 1.0) * (E - 0.5 * (mu_ * mu_ + mv_ * mv_) / r);
-  bool ok = r > 0.0 && p > 0.0 && r < INFINITY && p < INFINITY;
-  for (int f = 4; f < NFLD; ++f) ok = ok && fabs(Sg[(long)f * L.plane + c0]) < INFINITY;
-  if (!ok) atomicOr(flag, 1);
+  if (blockIdx.x == 0 && blockIdx.y == 0 && g == 0 && threadIdx.x == 0) {
+    if (clear) *clear = 0;
+    if (t0) *t0 = 0.0;
+    if (t1) *t1 = 0.0;
+  }
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nxg) return;
+  const long NN = (long)nxg * nyg, o0 = (long)g * NFLD * L.plane;
+  for (int j = blockIdx.y; j < nyg; j += gridDim.y) {
+    const long k = (long)j * nxg + i, c0 = o0 + cell(L, i, j);
+    double v[NFLD];
+#pragma unroll
+    for (int f = 0; f < NFLD; ++f) v[f] = f < 4 ? d.W[g][f * NN + k] : d.G[g][(f - 4) * NN + k];
+    if (bad) {
+      const double p = (gamma - 1.0) * (v[3] - 0.5 * (v[1] * v[1] + v[2] * v[2]) / v[0]);
+      bool ok = v[0] > 0.0 && p > 0.0 && v[0] < INFINITY && p < INFINITY;
+#pragma unroll
+      for (int f = 4; f < NFLD; ++f) ok = ok && fabs(v[f]) < INFINITY;
+      if (!ok) *bad = 1;
+    }
+#pragma unroll
+    for (int f = 0; f < NFLD; ++f) {
+      const long o = c0 + (long)f * L.plane;
+      if (S) S[o] = v[f];
+      if (hi) {
+        const float h = (float)v[f];
+        hi[o] = h;
+        lo[o] = (float)(v[f] - (double)h);
+      }
+    }
+  }
+}
+__global__ void store_kernel(DenseState d, Layout L, const double* S, const float* hi, const float* lo) {
+  const int g = blockIdx.z;
+  const int nxg = g == 0 ? L.nx : L.nxd, nyg = g == 0 ? L.ny : L.nyd;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nxg) return;
+  const long NN = (long)nxg * nyg, o0 = (long)g * NFLD * L.plane;
+  for (int j = blockIdx.y; j < nyg; j += gridDim.y) {
+    const long k = (long)j * nxg + i, c0 = o0 + cell(L, i, j);
+    double v[NFLD];
+#pragma unroll
+    for (int f = 0; f < NFLD; ++f) {
+      const long o = c0 + (long)f * L.plane;
+      v[f] = hi ? (double)hi[o] + (double)lo[o] : S[o];
+    }
+#pragma unroll
+    for (int f = 0; f < NFLD; ++f) (f < 4 ? d.W[g][f * NN + k] : d.G[g][(f - 4) * NN + k]) = v[f];
+  }
 }
 
-cudaError_t fdk::launch_validate(const double* S, const Layout& L, double gamma, int* flag, cudaStream_t s) {
-  const int mx = L.nx > L.nxd ? L.nx : L.nxd, my = L.ny > L.nyd ? L.ny : L.nyd;
-  validate_kernel<<<dim3((mx + 127) / 128, my, 2), 128, 0, s>>>(S, L, gamma, flag);
+static dim3 dense_grid(const Layout& L) {
+  const int mx = std::max(L.nx, L.nxd), my = std::max(L.ny, L.nyd);
+  return dim3((unsigned)((mx + 127) / 128), (unsigned)std::min(my, 65535), 2);
+}
+cudaError_t fdk::launch_load(const DenseState& d, const Layout& L, double gamma, double* S, float* hi, float* lo,
+                             int* bad, int* clear, double* t0, double* t1, cudaStream_t s) {
+  load_kernel<<<dense_grid(L), 128, 0, s>>>(d, L, gamma, S, hi, lo, bad, clear, t0, t1);
+  return cudaGetLastError();
+}
+cudaError_t fdk::launch_store(const DenseState& d, const Layout& L, const double* S, const float* hi, const float* lo,
+                              cudaStream_t s) {
+  store_kernel<<<dense_grid(L), 128, 0, s>>>(d, L, S, hi, lo);
   return cudaGetLastError();
 }
 
@@ -621,7 +675,7 @@ fdcgks_status fdcgks_create(const fdcgks_params* p, fdcgks_t* out) {
   c->red_blocks = 1024;
   if (cudaMalloc((void**)&c->res, sizeof(CflRes)) != cudaSuccess ||
       cudaMalloc((void**)&c->est, sizeof(float2) * c->red_blocks) != cudaSuccess ||
-      cudaHostAlloc((void**)&c->res_host, 2 * sizeof(double), cudaHostAllocMapped) != cudaSuccess) {
+      cudaHostAlloc((void**)&c->res_host, 3 * sizeof(double), cudaHostAllocMapped) != cudaSuccess) {
     fdcgks_destroy(c);
     return fail(nullptr, FDCGKS_ERR_NOMEM, "allocation of the reduction scratch failed");
   }
@@ -651,68 +705,26 @@ fdcgks_status fdcgks_dims(fdcgks_t c, int* nx, int* ny, int* nxd, int* nyd) {
   return FDCGKS_OK;
 }
 
-// copy one interior field plane between a dense [ny][nx] array and the padded layout
-static cudaError_t copy_field(fdcgks_t c, double* dev_plane, const double* src, double* dst, int nxg, int nyg,
-                              bool to_dev, int on_device) {
-  const Layout& L = c->L;
-  double* d0 = dev_plane + cell(L, 0, 0);
-  cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : (to_dev ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost);
-  if (to_dev)
-    return cudaMemcpy2DAsync(d0, sizeof(double) * L.pitch, src, sizeof(double) * nxg, sizeof(double) * nxg, nyg, k,
-                             c->stream);
-  return cudaMemcpy2DAsync(dst, sizeof(double) * nxg, d0, sizeof(double) * L.pitch, sizeof(double) * nxg, nyg, k,
-                           c->stream);
-}
-
-// Dense state [grid][field][nyg][nxg] (the four caller arrays back to back:
-// Wp, Gp, Wd, Gd) <-> the padded layout of both grids, on the device.
-// blockIdx.z = grid * NFLD + field; rows strided over gridDim.y.
-__global__ void dense_padded_kernel(double* dense, double* S, Layout L, int to_padded) {
-  const int g = blockIdx.z / NFLD, f = blockIdx.z % NFLD;
-  const int nxg = g == 0 ? L.nx : L.nxd, nyg = g == 0 ? L.ny : L.nyd;
-  const long goff = g == 0 ? 0 : (long)NFLD * L.nx * L.ny;
-  double* Sf = S + ((long)g * NFLD + f) * L.plane;
-  for (int j = blockIdx.y; j < nyg; j += gridDim.y) {
-    double* d = dense + goff + ((long)f * nyg + j) * nxg;
-    double* p = Sf + cell(L, 0, j);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nxg; i += gridDim.x * blockDim.x) {
-      if (to_padded) p[i] = d[i];
-      else d[i] = p[i];
-    }
-  }
-}
-
-// Host state <-> device: the whole state in four contiguous copies through a
-// dense staging area (the point-output buffer, free between steps), and one
-// kernel between the staging area and the padded layout; contiguous copies
-// run at the host link's full rate where per-row (pitched) copies do not.
-// Returns false (nothing done) when the staging area is too small.
-static bool staged_size_ok(fdcgks_t c) {
-  const Layout& L = c->L;
-  const size_t need = sizeof(double) * NFLD * ((size_t)L.nx * L.ny + (size_t)L.nxd * L.nyd);
-  return need <= rsize(c->p) * NPT * (size_t)L.pplane;
-}
-
-static cudaError_t launch_dense_padded(fdcgks_t c, double* dense, int to_padded) {
-  const Layout& L = c->L;
-  const int mx = std::max(L.nx, L.nxd), my = std::max(L.ny, L.nyd);
-  const dim3 grid((unsigned)std::min((mx + 255) / 256, 64), (unsigned)std::min(my, 65535), 2 * NFLD);
-  dense_padded_kernel<<<grid, 256, 0, c->stream>>>(dense, c->S, L, to_padded);
-  return cudaGetLastError();
+// The state at host pointers as a dense state on the device: four contiguous
+// areas in the point-output buffer, which is free between steps (192 bytes a
+// primary and dual node pair against its 200 or 400 bytes a point).
+// Contiguous copies run at the host link's full rate where per-row (pitched)
+// copies do not.
+static DenseState staged(fdcgks_t c) {
+  const long N0 = (long)c->L.nx * c->L.ny, N1 = (long)c->L.nxd * c->L.nyd;
+  double* st = (double*)c->PA;
+  return DenseState{{st, st + NFLD * N0}, {st + 4 * N0, st + NFLD * N0 + 4 * N1}};
 }
 
 static cudaError_t host_state_copy(fdcgks_t c, double* const* host, bool to_dev) {
   const Layout& L = c->L;
-  double* st = (double*)c->PA;
-  const long N0 = (long)L.nx * L.ny, N1 = (long)L.nxd * L.nyd;
-  const long off[4] = {0, 4 * N0, NFLD * N0, NFLD * N0 + 4 * N1};
-  const long len[4] = {4 * N0, 8 * N0, 4 * N1, 8 * N1};
+  const DenseState d = staged(c);
+  double* const dev[4] = {d.W[0], d.G[0], d.W[1], d.G[1]};
+  const long N0 = (long)L.nx * L.ny, N1 = (long)L.nxd * L.nyd, len[4] = {4 * N0, 8 * N0, 4 * N1, 8 * N1};
   cudaError_t e = cudaSuccess;
-  if (!to_dev) e = launch_dense_padded(c, st, 0);
   for (int k = 0; k < 4 && e == cudaSuccess; ++k)
-    e = to_dev ? cudaMemcpyAsync(st + off[k], host[k], sizeof(double) * len[k], cudaMemcpyHostToDevice, c->stream)
-               : cudaMemcpyAsync(host[k], st + off[k], sizeof(double) * len[k], cudaMemcpyDeviceToHost, c->stream);
-  if (to_dev && e == cudaSuccess) e = launch_dense_padded(c, st, 1);
+    e = to_dev ? cudaMemcpyAsync(dev[k], host[k], sizeof(double) * len[k], cudaMemcpyHostToDevice, c->stream)
+               : cudaMemcpyAsync(host[k], dev[k], sizeof(double) * len[k], cudaMemcpyDeviceToHost, c->stream);
   return e;
 }
 
@@ -720,33 +732,19 @@ fdcgks_status fdcgks_set_state(fdcgks_t c, const double* Wp, const double* Gp, c
                                int on_device) {
   if (!c) return fail(nullptr, FDCGKS_ERR_ARG, "ctx is NULL");
   if (!Wp || !Gp || !Wd || !Gd) return fail(c, FDCGKS_ERR_ARG, "NULL state pointer");
-  const Layout& L = c->L;
-  if (!on_device && staged_size_ok(c)) {
-    double* const host[4] = {const_cast<double*>(Wp), const_cast<double*>(Gp), const_cast<double*>(Wd),
-                             const_cast<double*>(Gd)};
-    CUDA_TRY(c, host_state_copy(c, host, true));
-  } else {
-    const double* srcW[2] = {Wp, Wd};
-    const double* srcG[2] = {Gp, Gd};
-    for (int g = 0; g < 2; ++g) {
-      int nxg = g == 0 ? L.nx : L.nxd, nyg = g == 0 ? L.ny : L.nyd;
-      long NN = (long)nxg * nyg;
-      double* Sg = c->S + (long)g * NFLD * L.plane;
-      for (int f = 0; f < NFLD; ++f) {
-        const double* src = f < 4 ? srcW[g] + f * NN : srcG[g] + (f - 4) * NN;
-        CUDA_TRY(c, copy_field(c, Sg + (long)f * L.plane, src, nullptr, nxg, nyg, true, on_device));
-      }
-    }
+  double* const src[4] = {const_cast<double*>(Wp), const_cast<double*>(Gp), const_cast<double*>(Wd),
+                          const_cast<double*>(Gd)};
+  DenseState d{{src[0], src[2]}, {src[1], src[3]}};
+  if (!on_device) {
+    CUDA_TRY(c, host_state_copy(c, src, true));
+    d = staged(c);
   }
-  if (c->Sf) CUDA_TRY(c, launch_split_ff(c->S, c->Sf, c->Slo, 2L * NFLD * L.plane, c->stream));
-  CUDA_TRY(c, cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream));
-  CUDA_TRY(c, launch_validate(c->S, L, c->p.gamma, c->flag, c->stream));
-  int h = 0;
-  CUDA_TRY(c, cudaMemcpyAsync(&h, c->flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  volatile int* bad = (volatile int*)(c->res_host + 2);
+  *bad = 0;
+  CUDA_TRY(c, launch_load(d, c->L, c->p.gamma, c->S, c->Sf, c->Slo, (int*)bad, c->flag, nullptr, nullptr, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  if (h) {
+  if (*bad) {
     c->has_state = false;
-    CUDA_TRY(c, cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream));
     return fail(c, FDCGKS_ERR_NONPHYSICAL, "state has non-positive or non-finite density/pressure");
   }
   c->has_state = true;
@@ -758,25 +756,13 @@ fdcgks_status fdcgks_get_state(fdcgks_t c, double* Wp, double* Gp, double* Wd, d
   if (!c) return fail(nullptr, FDCGKS_ERR_ARG, "ctx is NULL");
   if (!c->has_state) return fail(c, FDCGKS_ERR_STATE, "no state loaded");
   if (!Wp || !Gp || !Wd || !Gd) return fail(c, FDCGKS_ERR_ARG, "NULL state pointer");
-  const Layout& L = c->L;
-  CUDA_TRY(c, join_state(c));
-  if (!on_device && staged_size_ok(c)) {
-    double* const host[4] = {Wp, Gp, Wd, Gd};
-    CUDA_TRY(c, host_state_copy(c, host, false));
-  } else {
-    double* dstW[2] = {Wp, Wd};
-    double* dstG[2] = {Gp, Gd};
-    for (int g = 0; g < 2; ++g) {
-      int nxg = g == 0 ? L.nx : L.nxd, nyg = g == 0 ? L.ny : L.nyd;
-      long NN = (long)nxg * nyg;
-      double* Sg = c->S + (long)g * NFLD * L.plane;
-      for (int f = 0; f < NFLD; ++f) {
-        double* dst = f < 4 ? dstW[g] + f * NN : dstG[g] + (f - 4) * NN;
-        CUDA_TRY(c, copy_field(c, Sg + (long)f * L.plane, nullptr, dst, nxg, nyg, false, on_device));
-      }
-    }
+  double* const dst[4] = {Wp, Gp, Wd, Gd};
+  const DenseState d = on_device ? DenseState{{Wp, Wd}, {Gp, Gd}} : staged(c);
+  CUDA_TRY(c, launch_store(d, c->L, c->S, c->Sf, c->Slo, c->stream));
+  if (!on_device) {
+    CUDA_TRY(c, host_state_copy(c, dst, false));
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   }
-  if (!on_device) CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   return FDCGKS_OK;
 }
 

@@ -334,8 +334,8 @@ struct fdcgks_ens {
   unsigned long long* mx = nullptr;
   unsigned* mxf = nullptr;
   int* heads = nullptr;
-  int* vflag = nullptr;
-  double* staging = nullptr;              // FP64 padded state of the largest member
+  int* vflag = nullptr;                   // pinned host memory: set_state's verdict, written by the device
+  double* staging = nullptr;              // room for the largest member's dense state (host copies)
   // per member: padded FP64 state S (FP64 path) or the float-float pair (mixed)
   std::vector<double*> S;
   std::vector<float*> Shi, Slo;
@@ -718,13 +718,35 @@ fdcgks_status time_config(fdcgks_ens_t e, int steps, double* ms) {
 // ---------------------------------------------------------------------------
 extern "C" {
 
+// member m's dense state at host pointers, staged on the device in four
+// contiguous areas
+static DenseState staged(fdcgks_ens_t e, int m) {
+  const long N0 = (long)e->L[m].nx * e->L[m].ny, N1 = (long)e->L[m].nxd * e->L[m].nyd;
+  double* st = e->staging;
+  return DenseState{{st, st + NFLD * N0}, {st + 4 * N0, st + NFLD * N0 + 4 * N1}};
+}
+static cudaError_t host_copy(fdcgks_ens_t e, int m, const DenseState& h, bool to_dev) {
+  const DenseState d = staged(e, m);
+  cudaError_t r = cudaSuccess;
+  for (int g = 0; g < 2 && r == cudaSuccess; ++g) {
+    const Layout& L = e->L[m];
+    const size_t b = sizeof(double) * 4 * (g == 0 ? (size_t)L.nx * L.ny : (size_t)L.nxd * L.nyd);
+    const cudaMemcpyKind k = to_dev ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost;
+    r = cudaMemcpyAsync(to_dev ? d.W[g] : h.W[g], to_dev ? h.W[g] : d.W[g], b, k, e->stream);
+    if (r == cudaSuccess)
+      r = cudaMemcpyAsync(to_dev ? d.G[g] : h.G[g], to_dev ? h.G[g] : d.G[g], 2 * b, k, e->stream);
+  }
+  return r;
+}
+
 void fdcgks_ens_destroy(fdcgks_ens_t e) {
   if (!e) return;
   drop_graphs(e);
   void* bufs[] = {e->arena, e->args, e->meta, e->mstat, e->time, e->last_dt, e->fixed_dt, e->cfl,
-                  e->mx, e->mxf, e->heads, e->vflag, e->staging, e->tiles};
+                  e->mx, e->mxf, e->heads, e->staging, e->tiles};
   for (void* b : bufs)
     if (b) cudaFree(b);
+  if (e->vflag) cudaFreeHost(e->vflag);
   if (e->stream) cudaStreamDestroy(e->stream);
   delete e;
 }
@@ -810,14 +832,15 @@ fdcgks_status fdcgks_ens_create(const fdcgks_params* params, int count, fdcgks_e
       {(void**)&e->mx, sizeof(unsigned long long) * 2 * count},
       {(void**)&e->mxf, sizeof(unsigned) * 2 * count},
       {(void**)&e->heads, sizeof(int) * N_COUNTERS},
-      {(void**)&e->vflag, sizeof(int)},
-      {(void**)&e->staging, mixed ? sizeof(double) * 2 * NFLD * max_plane : 0},
+      {(void**)&e->staging, sizeof(double) * 2 * NFLD * max_plane},
   };
   for (auto& a : allocs) {
     if (!a.bytes) continue;
     if ((r = cudaMalloc(a.ptr, a.bytes)) != cudaSuccess)
       return bail(r == cudaErrorMemoryAllocation ? FDCGKS_ERR_NOMEM : FDCGKS_ERR_CUDA, "ensemble buffers", r);
   }
+  if ((r = cudaHostAlloc((void**)&e->vflag, sizeof(int), cudaHostAllocMapped)) != cudaSuccess)
+    return bail(r == cudaErrorMemoryAllocation ? FDCGKS_ERR_NOMEM : FDCGKS_ERR_CUDA, "ensemble buffers", r);
   // argument blocks and constants
   e->h_args.assign(ab * 2 * count, 0);
   std::vector<MemberMeta> meta(count);
@@ -869,30 +892,15 @@ fdcgks_status fdcgks_ens_set_state(fdcgks_ens_t e, int m, const double* Wp, cons
   if (!Wp || !Gp || !Wd || !Gd) return efail(e, FDCGKS_ERR_ARG, "NULL state pointer");
   const Layout& L = e->L[m];
   const bool mixed = e->precision == FDCGKS_MIXED;
-  double* S = mixed ? e->staging : e->S[m];
-  const double* srcW[2] = {Wp, Wd};
-  const double* srcG[2] = {Gp, Gd};
-  const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   e->has_state[m] = 0;
-  for (int g = 0; g < 2; ++g) {
-    const int nxg = g == 0 ? L.nx : L.nxd, nyg = g == 0 ? L.ny : L.nyd;
-    const long NN = (long)nxg * nyg;
-    for (int f = 0; f < NFLD; ++f) {
-      const double* src = f < 4 ? srcW[g] + f * NN : srcG[g] + (f - 4) * NN;
-      double* dst = S + ((long)g * NFLD + f) * L.plane + cell(L, 0, 0);
-      ENS_TRY(e, cudaMemcpy2DAsync(dst, sizeof(double) * L.pitch, src, sizeof(double) * nxg, sizeof(double) * nxg,
-                                   nyg, kind, e->stream));
-    }
-  }
-  if (mixed) ENS_TRY(e, launch_split_ff(S, e->Shi[m], e->Slo[m], 2L * NFLD * L.plane, e->stream));
-  ENS_TRY(e, cudaMemsetAsync(e->vflag, 0, sizeof(int), e->stream));
-  ENS_TRY(e, launch_validate(S, L, e->p[m].gamma, e->vflag, e->stream));
-  ENS_TRY(e, cudaMemsetAsync(e->mstat + m, 0, sizeof(int), e->stream));
-  ENS_TRY(e, cudaMemsetAsync(e->time + m, 0, sizeof(double), e->stream));
-  ENS_TRY(e, cudaMemsetAsync(e->last_dt + m, 0, sizeof(double), e->stream));
-  int h = 0;
-  ENS_TRY(e, cudaMemcpyAsync(&h, e->vflag, sizeof(int), cudaMemcpyDeviceToHost, e->stream));
+  DenseState d{{const_cast<double*>(Wp), const_cast<double*>(Wd)}, {const_cast<double*>(Gp), const_cast<double*>(Gd)}};
+  if (!on_device) ENS_TRY(e, host_copy(e, m, d, true));
+  *(volatile int*)e->vflag = 0;
+  ENS_TRY(e, launch_load(on_device ? d : staged(e, m), L, e->p[m].gamma, mixed ? nullptr : e->S[m],
+                         mixed ? e->Shi[m] : nullptr, mixed ? e->Slo[m] : nullptr, e->vflag, e->mstat + m, e->time + m,
+                         e->last_dt + m, e->stream));
   ENS_TRY(e, cudaStreamSynchronize(e->stream));
+  const int h = *(volatile int*)e->vflag;
   if (h) return efail(e, FDCGKS_ERR_NONPHYSICAL, "member %d: state has non-positive or non-finite density/pressure", m);
   e->has_state[m] = 1;
   return FDCGKS_OK;
@@ -904,25 +912,11 @@ fdcgks_status fdcgks_ens_get_state(fdcgks_ens_t e, int m, double* Wp, double* Gp
   if (st != FDCGKS_OK) return st;
   if (!e->has_state[m]) return efail(e, FDCGKS_ERR_STATE, "member %d has no state loaded", m);
   if (!Wp || !Gp || !Wd || !Gd) return efail(e, FDCGKS_ERR_ARG, "NULL state pointer");
-  const Layout& L = e->L[m];
-  double* S = e->S[m];
-  if (e->precision == FDCGKS_MIXED) {
-    S = e->staging;
-    ENS_TRY(e, launch_join_ff(e->Shi[m], e->Slo[m], S, 2L * NFLD * L.plane, e->stream));
-  }
-  double* dstW[2] = {Wp, Wd};
-  double* dstG[2] = {Gp, Gd};
-  const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  for (int g = 0; g < 2; ++g) {
-    const int nxg = g == 0 ? L.nx : L.nxd, nyg = g == 0 ? L.ny : L.nyd;
-    const long NN = (long)nxg * nyg;
-    for (int f = 0; f < NFLD; ++f) {
-      double* dst = f < 4 ? dstW[g] + f * NN : dstG[g] + (f - 4) * NN;
-      const double* src = S + ((long)g * NFLD + f) * L.plane + cell(L, 0, 0);
-      ENS_TRY(e, cudaMemcpy2DAsync(dst, sizeof(double) * nxg, src, sizeof(double) * L.pitch, sizeof(double) * nxg,
-                                   nyg, kind, e->stream));
-    }
-  }
+  const bool mixed = e->precision == FDCGKS_MIXED;
+  const DenseState d{{Wp, Wd}, {Gp, Gd}};
+  ENS_TRY(e, launch_store(on_device ? d : staged(e, m), e->L[m], e->S[m], mixed ? e->Shi[m] : nullptr,
+                          mixed ? e->Slo[m] : nullptr, e->stream));
+  if (!on_device) ENS_TRY(e, host_copy(e, m, d, false));
   ENS_TRY(e, cudaStreamSynchronize(e->stream));
   return FDCGKS_OK;
 }

@@ -332,10 +332,25 @@ inline GasK<R> make_gas(const fdcgks_params& p, double dt) {
 }
 
 
-// whole-plane helpers of the host runtime (fdcgks_api.cu), on stream s:
-// positivity/finiteness check of the interior of an FP64 state (sets bit 0 of
-// *flag), and the FP64 <-> float-float conversion of n entries
-cudaError_t launch_validate(const double* S, const Layout& L, double gamma, int* flag, cudaStream_t s);
+// A state in the caller's layout: W [4][ny][nx] and gradients [2][4][ny][nx]
+// of both grids, device pointers.
+struct DenseState {
+  double* W[2];
+  double* G[2];
+};
+
+// whole-state helpers of the host runtime (fdcgks_api.cu), on stream s.
+// launch_load: a dense state into the padded layout, as FP64 (S, unless null)
+// and/or as float-float pairs (hi, lo, unless null), in one pass.  With
+// `bad` given, every node is checked (positive finite density and pressure,
+// finite gradients) and *bad is set to 1 where one fails; *clear, *t0 and *t1
+// are set to 0 (each unless null).  launch_store: the interior of a padded
+// state (S, or the pairs if hi is given) back to the dense layout.
+cudaError_t launch_load(const DenseState& d, const Layout& L, double gamma, double* S, float* hi, float* lo, int* bad,
+                        int* clear, double* t0, double* t1, cudaStream_t s);
+cudaError_t launch_store(const DenseState& d, const Layout& L, const double* S, const float* hi, const float* lo,
+                         cudaStream_t s);
+// FP64 <-> float-float conversion of n entries
 cudaError_t launch_split_ff(const double* S, float* hi, float* lo, long n, cudaStream_t s);
 cudaError_t launch_join_ff(const float* hi, const float* lo, double* S, long n, cudaStream_t s);
 
