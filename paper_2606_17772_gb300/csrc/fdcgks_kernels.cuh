@@ -152,11 +152,16 @@ FD_HD void positivity_fix(LD ld, int l, R vl[4], R dl[4], R vr[4], R dr[4], R& c
 // Reconstruct one 4-point line at its virtual interface (between entries 1
 // and 2), with the safeguard above.  ld(l, e, f) = field f (0-3 W, 4-7 the
 // averaged gradient along the line) of entry e (0-3) of line l.
-template <class R, class LD>
+// D1: component 2 is 0 throughout (the one-dimensional gas).
+template <bool D1 = false, class R, class LD>
 FD_HD void recon_line_ld(const GenoK<R>& geno, LD ld, int l, R h, R ih, R vl[4], R dl[4], R vr[4], R dr[4],
                          R& chi) {
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
+    if (D1 && c == 2) {
+      vl[c] = dl[c] = vr[c] = dr[c] = R(0);
+      continue;
+    }
     R Q[4] = {ld(l, 0, c), ld(l, 1, c), ld(l, 2, c), ld(l, 3, c)};
     R Qx[4] = {ld(l, 0, 4 + c), ld(l, 1, 4 + c), ld(l, 2, 4 + c), ld(l, 3, 4 + c)};
     R cl, cr;
@@ -174,7 +179,7 @@ FD_HD void recon_line_ld(const GenoK<R>& geno, LD ld, int l, R h, R ih, R vl[4],
 // values and derivatives mapped back with R; chi of the flux is the smaller
 // of the two acoustic fields' (Sec. 3.2).  A non-physical mean state falls
 // back to conservative components.
-template <class R, class LD>
+template <bool D1 = false, class R, class LD>
 FD_HD void recon_line_char(const GenoK<R>& geno, R gm1, int normal, LD ld, int l, R h, R ih, R vl[4], R dl[4],
                            R vr[4], R dr[4], R& chi) {
   const int in = normal == 0 ? 1 : 2, it = normal == 0 ? 2 : 1;
@@ -186,7 +191,7 @@ FD_HD void recon_line_char(const GenoK<R>& geno, R gm1, int normal, LD ld, int l
   const R q2 = u * u + v * v;
   const R p = gm1 * (E - R(0.5) * r * q2);
   if (!(r > R(0)) || !(p > R(0))) {
-    recon_line_ld(geno, ld, l, h, ih, vl, dl, vr, dr, chi);
+    recon_line_ld<D1>(geno, ld, l, h, ih, vl, dl, vr, dr, chi);
     return;
   }
   const R c = s_sqrt((gm1 + R(1)) * p * ir), ic = s_div(R(1), c), H = (E + p) * ir;
@@ -202,12 +207,17 @@ FD_HD void recon_line_char(const GenoK<R>& geno, R gm1, int normal, LD ld, int l
   R cvl[4], cdl[4], cvr[4], cdr[4], cl[4], cr[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
+    if (D1 && k == 2) {   // shear
+      cvl[k] = cdl[k] = cvr[k] = cdr[k] = R(0);
+      continue;
+    }
     R Q[4], Qx[4];
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       R a = R(0), b = R(0);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
+        if (D1 && j == 2) continue;
         a += Lm[k][j] * ld(l, m, perm[j]);
         b += Lm[k][j] * ld(l, m, 4 + perm[j]);
       }
@@ -219,8 +229,10 @@ FD_HD void recon_line_char(const GenoK<R>& geno, R gm1, int normal, LD ld, int l
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     R a = R(0), b = R(0), d = R(0), e = R(0);
+    if (!D1 || j != 2)
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
+      if (D1 && k == 2) continue;
       a += Rm[j][k] * cvl[k];
       b += Rm[j][k] * cvr[k];
       d += Rm[j][k] * cdl[k];

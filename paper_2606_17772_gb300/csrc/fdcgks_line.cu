@@ -17,10 +17,13 @@
 // ordering makes each block's global-memory writes visible to the others.
 // A single line then runs at the FP64 rate of several SMs instead of one.  The line's working arrays stay in global memory (L2-resident for
 // the line sizes of Sec. 5); the per-node device functions are the 2-D
-// path's: the line reconstruction of the 2-D interface points with the
-// y-momentum set to zero, the x-normal kinetic solve with V = 0 and no
-// tangential variation (the 1-D BGK gas is the 2-D one restricted so), and
-// the nodal solve with W_y = 0.  The compute type R is FP64, or FP32 (the
+// path's restricted to the 1-D BGK gas (the 2-D one with V = 0 and no
+// y-variation): the line reconstruction, the x-normal kinetic solve and the
+// nodal solve with every term in V and the y-derivatives dropped at compile
+// time (D1), which the compiler cannot drop by itself because 0 * x is not 0
+// for every x; the second stage computes and stores time derivatives only (608
+// FP64 lines of 400 nodes, 10 steps, bound by the FP64 pipe: 22.3 -> 17.3 ms;
+// one 200-node line, 21 steps: 3.26 -> 2.87 ms).  The compute type R is FP64, or FP32 (the
 // mixed path: reconstruction, kinetic solves and compact fluxes in FP32 with
 // the 2-D mixed path's FP64 time coefficients, the interface and nodal
 // outputs stored in FP32); the state, its stage copy and the S2O4
@@ -111,9 +114,10 @@ __device__ void line_ghosts(const LineArgs<R>& a, double* B) {
   }
 }
 
-// interface solves (k = -2..n) and nodal fluxes (j = -1..n) of buffer B
+// interface solves (k = -2..n) and nodal fluxes (j = -1..n) of buffer B;
+// want_n = false (second stage): the time derivatives only
 template <class R>
-__device__ void line_fluxes(const LineArgs<R>& a, const GasK<R>& gas, const double* B, R* P, R* NF) {
+__device__ void line_fluxes(const LineArgs<R>& a, const GasK<R>& gas, bool want_n, const double* B, R* P, R* NF) {
   const int ni = a.n + 3, nn = a.n + 2;
   const R h = (R)a.h, ih = (R)a.ih;
   for (int idx = lt_index(a); idx < ni + nn; idx += lt_count(a)) {
@@ -126,26 +130,28 @@ __device__ void line_fluxes(const LineArgs<R>& a, const GasK<R>& gas, const doub
         return (R)B[((f < 4 ? 0 : 3) + c) * a.np + GH + (k - 1 + e)];
       };
       R vl[4], dl[4], vr[4], dr[4], chi;
-      if (a.recon_vars) recon_line_char(a.geno, gas.gm1, 0, ld, 0, h, ih, vl, dl, vr, dr, chi);
-      else recon_line_ld(a.geno, ld, 0, h, ih, vl, dl, vr, dr, chi);
+      if (a.recon_vars) recon_line_char<true>(a.geno, gas.gm1, 0, ld, 0, h, ih, vl, dl, vr, dr, chi);
+      else recon_line_ld<true>(a.geno, ld, 0, h, ih, vl, dl, vr, dr, chi);
       const R zero[4] = {R(0), R(0), R(0), R(0)};
       IfaceOut<R> o;
-      iface_solve(gas, 0, vl, vr, dl, dr, zero, true, o);
+      iface_solve_x<true>(gas, vl, vr, dl, dr, zero, want_n, o);
       R* q = P + idx;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const int s = slot4(c);
-        q[(0 + c) * ni] = o.F[s];
+        if (want_n) {
+          q[(0 + c) * ni] = o.F[s];
+          q[(6 + c) * ni] = o.Wl[s];
+          q[(9 + c) * ni] = o.Wr[s];
+        }
         q[(3 + c) * ni] = o.Ft[s];
-        q[(6 + c) * ni] = o.Wl[s];
-        q[(9 + c) * ni] = o.Wr[s];
         q[(12 + c) * ni] = o.Wlt[s];
         q[(15 + c) * ni] = o.Wrt[s];
       }
       q[18 * ni] = chi;
     } else {
       const int j = idx - ni - 1;   // node j: value and GENO x-derivative
-      R W[4] = {R(0), R(0), R(0), R(0)}, Wx[4] = {R(0), R(0), R(0), R(0)}, Wy[4] = {R(0), R(0), R(0), R(0)};
+      R W[4] = {R(0), R(0), R(0), R(0)}, Wx[4] = {R(0), R(0), R(0), R(0)};
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const double* w = B + c * a.np + GH + j;
@@ -154,11 +160,11 @@ __device__ void line_fluxes(const LineArgs<R>& a, const GasK<R>& gas, const doub
         W[slot4(c)] = q[1];
         Wx[slot4(c)] = recon_node(a.geno, q, gx, h, ih);
       }
-      R F[4], G[4], Ft[4], Gt[4];
-      nodal_flux(gas, W, Wx, Wy, F, G, Ft, Gt);
+      R F[4], Ft[4];
+      nodal_flux_1d(gas, W, Wx, F, Ft, want_n);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        NF[c * nn + j + 1] = F[slot4(c)];
+        if (want_n) NF[c * nn + j + 1] = F[slot4(c)];
         NF[(3 + c) * nn + j + 1] = Ft[slot4(c)];
       }
     }
@@ -172,23 +178,26 @@ __device__ void line_update(const LineArgs<R>& a, int mode, int stage, double dt
                             const double* Bin, double* Bout, double* A, int line, int* flag) {
   const int ni = a.n + 3, nn = a.n + 2;
   const R ih = (R)a.ih;
+  const double dt26 = dt * dt / 6.0, dt23 = dt * dt / 3.0;
   for (int j = lt_index(a); j < a.n; j += lt_count(a)) {
     const R chip = P[18 * ni + j + 2], chim = P[18 * ni + j + 1];
     double L[3], Lt[3], gb[3], gt[3];
+    // FP64: the short form of the flux difference where both interfaces are
+    // smooth (as the 2-D update)
+    const bool smooth = !IsF32<R>::v && chip == R(1) && chim == R(1);
+    auto div = [&](const R* F, const R* nF) -> double {
+      if (smooth)
+        return (double)(-compact_flux_diff<true>(a.fv, chim, chip, F[j], F[j + 1], F[j + 2], F[j + 3], nF[j],
+                                                 nF[j + 1], nF[j + 2]) * ih);
+      return (double)(-compact_flux_diff<false>(a.fv, chim, chip, F[j], F[j + 1], F[j + 2], F[j + 3], nF[j],
+                                                nF[j + 1], nF[j + 2]) * ih);
+    };
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const R* F = P + c * ni;
-      const R* Ft = P + (3 + c) * ni;
-      const R* nF = NF + c * nn;
-      const R* nFt = NF + (3 + c) * nn;
       // interface k + 1/2 sits at P index k + 2, node k at NF index k + 1
-      const R fp = compact_flux(a.fv, chip, F[j + 1], F[j + 2], F[j + 3], nF[j + 1], nF[j + 2]);
-      const R fm = compact_flux(a.fv, chim, F[j], F[j + 1], F[j + 2], nF[j], nF[j + 1]);
-      const R ftp = compact_flux(a.fv, chip, Ft[j + 1], Ft[j + 2], Ft[j + 3], nFt[j + 1], nFt[j + 2]);
-      const R ftm = compact_flux(a.fv, chim, Ft[j], Ft[j + 1], Ft[j + 2], nFt[j], nFt[j + 1]);
-      L[c] = (double)(-(fp - fm) * ih);
-      Lt[c] = (double)(-(ftp - ftm) * ih);
-      gb[c] = (double)((P[(6 + c) * ni + j + 2] - P[(9 + c) * ni + j + 1]) * ih);
+      L[c] = stage == 0 ? div(P + c * ni, NF + c * nn) : 0.0;
+      Lt[c] = div(P + (3 + c) * ni, NF + (3 + c) * nn);
+      gb[c] = stage == 0 ? (double)((P[(6 + c) * ni + j + 2] - P[(9 + c) * ni + j + 1]) * ih) : 0.0;
       gt[c] = (double)((P[(12 + c) * ni + j + 2] - P[(15 + c) * ni + j + 1]) * ih);
     }
     if (mode == LINE_OPERATOR) {
@@ -208,12 +217,12 @@ __device__ void line_update(const LineArgs<R>& a, int mode, int stage, double dt
       if (stage == 0) {
         const double Wn = Bin[c * a.np + GH + j];
         W[c] = Wn + 0.5 * dt * L[c] + 0.125 * dt * dt * Lt[c];
-        A[c * a.n + j] = Wn + dt * L[c] + dt * dt / 6.0 * Lt[c];
+        A[c * a.n + j] = Wn + dt * L[c] + dt26 * Lt[c];
         const double base = a.grad_base ? Bin[(3 + c) * a.np + GH + j] : gb[c];
         A[(3 + c) * a.n + j] = base;
         Bout[(3 + c) * a.np + GH + j] = base + 0.5 * dt * gt[c];
       } else {
-        W[c] = A[c * a.n + j] + dt * dt / 3.0 * Lt[c];
+        W[c] = A[c * a.n + j] + dt23 * Lt[c];
         Bout[(3 + c) * a.np + GH + j] = A[(3 + c) * a.n + j] + dt * gt[c];
       }
       Bout[c * a.np + GH + j] = W[c];
@@ -270,7 +279,7 @@ __device__ void line_stage(const LineArgs<R>& a, const GasK<R>& gas, int mode, i
                            double* Bout, R* P, R* NF, double* A, int line, int* flag) {
   line_ghosts(a, Bin);
   line_sync(a);
-  line_fluxes(a, gas, Bin, P, NF);
+  line_fluxes(a, gas, stage == 0, Bin, P, NF);
   line_sync(a);
   line_update(a, mode, stage, dt, P, NF, Bin, Bout, A, line, flag);
   line_sync(a);
@@ -285,8 +294,10 @@ __device__ __forceinline__ void gas_set_dt(GasK<R>& gas, double dt) {
   gas.inv_dt_r = (R)(1.0 / dt);
 }
 
+// 2 (FP64) and 4 (mixed) blocks a SM: 3 FP64 blocks spill (608 lines of 400
+// nodes, 10 steps: 17.3 and 20.2 ms), 3 mixed blocks 1.92 ms against 1.23
 template <class R>
-__global__ void __launch_bounds__(LT) line_kernel(LineArgs<R> a, int mode, double dt_fixed, int nsteps, double t_end,
+__global__ void __launch_bounds__(LT, (IsF32<R>::v ? 4 : 2)) line_kernel(LineArgs<R> a, int mode, double dt_fixed, int nsteps, double t_end,
                                                   double cfl, int max_steps) {
   const int b = blockIdx.x / a.cs;
   const bool lead = blockIdx.x % a.cs == 0 && threadIdx.x == 0;

@@ -595,6 +595,8 @@ FD_HD TimeCoef<TW> time_coef(TW tau, TW dt, TW inv_dt) {
 // so a slope-weighted moment is a polynomial in u alone.  Whole-space moments
 // (the equilibrium state g0 and the compatibility conditions) are then the
 // Euler flux, its time derivative and the Navier-Stokes stress and heat flux.
+// D1: the one-dimensional gas, V = 0 and no y-derivatives; component 2 is
+// neither read nor written.
 // ---------------------------------------------------------------------------
 
 // conservative W with its primitive variables; th = p/rho, en = rho E/rho
@@ -602,15 +604,15 @@ template <class R>
 struct GasState {
   R rho, ir, U, V, p, th, en;
 };
-template <class R>
+template <bool D1 = false, class R>
 FD_HD GasState<R> gas_state(const R W[4], R gm1) {
   GasState<R> g;
   g.rho = W[0];
   g.ir = s_div(R(1), W[0]);
   g.U = W[1] * g.ir;
-  g.V = W[2] * g.ir;
+  g.V = D1 ? R(0) : W[2] * g.ir;
   g.en = W[3] * g.ir;
-  g.p = gm1 * (W[3] - R(0.5) * W[0] * (g.U * g.U + g.V * g.V));
+  g.p = gm1 * (W[3] - R(0.5) * W[0] * (D1 ? g.U * g.U : g.U * g.U + g.V * g.V));
   g.th = g.p * g.ir;
   return g;
 }
@@ -621,20 +623,32 @@ struct PrimGrad {
   R d, u, v, t;
 };
 // from the derivative D of the conservative variables
-template <class R>
+template <bool D1 = false, class R>
 FD_HD PrimGrad<R> prim_grad(const GasState<R>& g, R gm1, const R D[4]) {
   PrimGrad<R> q;
   q.d = D[0] * g.ir;
   q.u = D[1] * g.ir - g.U * q.d;
-  q.v = D[2] * g.ir - g.V * q.d;
-  q.t = gm1 * (D[3] * g.ir - g.en * q.d - g.U * q.u - g.V * q.v);
+  if (D1) {
+    q.v = R(0);
+    q.t = gm1 * (D[3] * g.ir - g.en * q.d - g.U * q.u);
+  } else {
+    q.v = D[2] * g.ir - g.V * q.d;
+    q.t = gm1 * (D[3] * g.ir - g.en * q.d - g.U * q.u - g.V * q.v);
+  }
   return q;
 }
 // time derivative from the x- and y-derivatives (compatibility
 // <(a u + b v + A) psi> = 0: the Euler equations)
-template <class R>
+template <bool D1 = false, class R>
 FD_HD PrimGrad<R> prim_rate(const GasState<R>& g, R gm1, const PrimGrad<R>& x, const PrimGrad<R>& y) {
   PrimGrad<R> q;
+  if (D1) {
+    q.d = -(g.U * x.d + x.u);
+    q.u = -(g.U * x.u + g.th * x.d + x.t);
+    q.v = R(0);
+    q.t = -(g.U * x.t + gm1 * g.th * x.u);
+    return q;
+  }
   const R div = x.u + y.v;
   q.d = -(g.U * x.d + g.V * y.d + div);
   q.u = -(g.U * x.u + g.V * y.u + g.th * x.d + x.t);
@@ -643,36 +657,46 @@ FD_HD PrimGrad<R> prim_rate(const GasState<R>& g, R gm1, const PrimGrad<R>& x, c
   return q;
 }
 // derivative of the conservative variables; hN = (K + 2)/2; rt = rho theta'
-template <class R>
+template <bool D1 = false, class R>
 FD_HD void cons_rate(const GasState<R>& g, R hN, const PrimGrad<R>& q, R W[4], R& rt) {
-  const R ru = g.rho * q.u, rv = g.rho * q.v;
+  const R ru = g.rho * q.u;
   rt = g.rho * q.t;
   W[0] = g.rho * q.d;
   W[1] = g.U * W[0] + ru;
+  if (D1) {
+    W[3] = g.en * W[0] + g.U * ru + hN * rt;
+    return;
+  }
+  const R rv = g.rho * q.v;
   W[2] = g.V * W[0] + rv;
   W[3] = g.en * W[0] + g.U * ru + g.V * rv + hN * rt;
 }
 // Euler x-flux of g and its derivative for the derivative (q, Wq, rt) of g
-template <class R>
+template <bool D1 = false, class R>
 FD_HD void euler_flux(const GasState<R>& g, const R W[4], R F[4]) {
   F[0] = W[1];
   F[1] = g.U * W[1] + g.p;
-  F[2] = g.V * W[1];
+  if (!D1) F[2] = g.V * W[1];
   F[3] = g.U * (W[3] + g.p);
 }
-template <class R>
+template <bool D1 = false, class R>
 FD_HD void euler_flux_rate(const GasState<R>& g, const R W[4], const PrimGrad<R>& q, const R Wq[4], R rt, R F[4]) {
   const R pq = g.th * Wq[0] + rt;
   F[0] = Wq[1];
   F[1] = g.U * Wq[1] + W[1] * q.u + pq;
-  F[2] = g.V * Wq[1] + W[1] * q.v;
+  if (!D1) F[2] = g.V * Wq[1] + W[1] * q.v;
   F[3] = q.u * (W[3] + g.p) + g.U * (Wq[3] + pq);
 }
 // rho <u psi (a u + b v + A)>: minus the Navier-Stokes stress and heat flux
 // over the collision time (the density component is 0)
-template <class R>
+template <bool D1 = false, class R>
 FD_HD void stress_flux(const GasState<R>& g, R K, R gm1, const PrimGrad<R>& x, const PrimGrad<R>& y, R S[4]) {
   S[0] = R(0);
+  if (D1) {
+    S[1] = g.p * ((R(2) - gm1) * x.u);
+    S[3] = g.U * S[1] + (R(0.5) * K + R(2)) * g.p * x.t;
+    return;
+  }
   S[1] = g.p * (R(2) * x.u - gm1 * (x.u + y.v));
   S[2] = g.p * (x.v + y.u);
   S[3] = g.U * S[1] + g.V * S[2] + (R(0.5) * K + R(2)) * g.p * x.t;
@@ -710,7 +734,7 @@ FD_HD void half_moments(const GasState<R>& g, int sign, R sl, R M[7]) {
   }
 }
 
-template <class R>
+template <bool D1 = false, class R>
 FD_HD void half_side(const GasState<R>& g, R N, R ith, const PrimGrad<R>& gx, const PrimGrad<R>& gy,
                      const PrimGrad<R>& gt, HalfSide<R>& s) {
   s.rho = g.rho;
@@ -721,47 +745,57 @@ FD_HD void half_side(const GasState<R>& g, R N, R ith, const PrimGrad<R>& gx, co
   // integral over c and xi)
   const R ta = gx.t * ith, a3 = ta * ith, a1 = gx.u * ith - g.U * a3;
   const R a0 = gx.d - R(0.5) * ta - g.U * a1 - cU * a3;
-  const R tb = gy.t * ith, b3 = tb * ith, b1 = gy.u * ith - g.U * b3;
-  const R b0 = gy.d - R(0.5) * tb - g.U * b1 - cU * b3;
-  s.e0 = g.V * b0 + gy.v;
-  s.e1 = a0 + g.V * b1;
-  s.e2 = a1 + R(0.5) * g.V * b3;
   s.e3 = R(0.5) * a3;
-  s.X0 = g.V * (s.Nh * tb) + g.th * gy.v;
   s.X1 = s.Nh * ta;
-  s.c0 = g.V * gy.v + g.th * (b0 + tb);
-  s.c1 = gx.v + g.th * b1;
-  s.c2 = R(0.5) * tb;
+  if (D1) {
+    s.e1 = a0;
+    s.e2 = a1;
+  } else {
+    const R tb = gy.t * ith, b3 = tb * ith, b1 = gy.u * ith - g.U * b3;
+    const R b0 = gy.d - R(0.5) * tb - g.U * b1 - cU * b3;
+    s.e0 = g.V * b0 + gy.v;
+    s.e1 = a0 + g.V * b1;
+    s.e2 = a1 + R(0.5) * g.V * b3;
+    s.X0 = g.V * (s.Nh * tb) + g.th * gy.v;
+    s.c0 = g.V * gy.v + g.th * (b0 + tb);
+    s.c1 = gx.v + g.th * b1;
+    s.c2 = R(0.5) * tb;
+  }
   const R tA = gt.t * ith, A3 = tA * ith;
   s.Ae1 = gt.u * ith - g.U * A3;
   s.Ae0 = gt.d - R(0.5) * tA - g.U * s.Ae1 - cU * A3;
   s.Ae2 = R(0.5) * A3;
   s.AX0 = s.Nh * tA;
-  s.Ac0 = gt.v;
+  if (!D1) s.Ac0 = gt.v;
 }
 
 // adds rho <psi s> to Wm and rho <u psi s> to F for s = k3 + k4 D + k5 A
-template <class R>
+template <bool D1 = false, class R>
 FD_HD void half_flux(const HalfSide<R>& s, R k3, R k4, R k5, R F[4], R Wm[4]) {
   const R q3 = s.rho * k3, q4 = s.rho * k4, q5 = s.rho * k5;
-  const R e0 = q3 + q4 * s.e0 + q5 * s.Ae0, e1 = q4 * s.e1 + q5 * s.Ae1, e2 = q4 * s.e2 + q5 * s.Ae2;
+  const R e0 = D1 ? q3 + q5 * s.Ae0 : q3 + q4 * s.e0 + q5 * s.Ae0, e1 = q4 * s.e1 + q5 * s.Ae1, e2 = q4 * s.e2 + q5 * s.Ae2;
   const R e3 = q4 * s.e3;
-  const R X0 = q4 * s.X0 + q5 * s.AX0, X1 = q4 * s.X1;
-  const R c0 = q4 * s.c0 + q5 * s.Ac0, c1 = q4 * s.c1, c2 = q4 * s.c2;
+  const R X0 = D1 ? q5 * s.AX0 : q4 * s.X0 + q5 * s.AX0, X1 = q4 * s.X1;
   const R* M = s.M;
   R T[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) T[k] = e0 * M[k] + e1 * M[k + 1] + e2 * M[k + 2] + e3 * M[k + 3];
-  const R C0 = c0 * M[0] + c1 * M[1] + c2 * M[2], C1 = c0 * M[1] + c1 * M[2] + c2 * M[3];
   const R E0 = R(0.5) * T[2] + s.Nh * T[0] + X0 * M[0] + X1 * M[1];
   const R E1 = R(0.5) * T[3] + s.Nh * T[1] + X0 * M[1] + X1 * M[2];
-  const R hV = R(0.5) * s.V;
   Wm[0] += T[0];
   Wm[1] += T[1];
-  Wm[2] += C0 + s.V * T[0];
-  Wm[3] += E0 + s.V * (C0 + hV * T[0]);
   F[0] += T[1];
   F[1] += T[2];
+  if (D1) {
+    Wm[3] += E0;
+    F[3] += E1;
+    return;
+  }
+  const R c0 = q4 * s.c0 + q5 * s.Ac0, c1 = q4 * s.c1, c2 = q4 * s.c2;
+  const R C0 = c0 * M[0] + c1 * M[1] + c2 * M[2], C1 = c0 * M[1] + c1 * M[2] + c2 * M[3];
+  const R hV = R(0.5) * s.V;
+  Wm[2] += C0 + s.V * T[0];
+  Wm[3] += E0 + s.V * (C0 + hV * T[0]);
   F[2] += C1 + s.V * T[1];
   F[3] += E1 + s.V * (C1 + hV * T[1]);
 }
@@ -788,11 +822,11 @@ struct IfaceOut {
   R F[4], Ft[4], Wl[4], Wr[4], Wlt[4], Wrt[4];
 };
 
-template <class R>
+template <bool D1 = false, class R>
 FD_HD void iface_solve_x(const GasK<R>& gas, const R Wl[4], const R Wr[4], const R Wln[4], const R Wrn[4],
                          const R Wt[4], bool want_n, IfaceOut<R>& o) {
   const R K = gas.K, gm1 = gas.gm1, N = K + R(1), hN = R(0.5) * K + R(1);
-  const GasState<R> gl = gas_state(Wl, gm1), gr = gas_state(Wr, gm1);
+  const GasState<R> gl = gas_state<D1>(Wl, gm1), gr = gas_state<D1>(Wr, gm1);
   HalfSide<R> sl, sr;
   const R ql = s_rsqrt(R(2) * gl.th), qr = s_rsqrt(R(2) * gr.th);   // sqrt(lambda)
   half_moments(gl, +1, ql, sl.M);
@@ -804,33 +838,39 @@ FD_HD void iface_solve_x(const GasK<R>& gas, const R Wl[4], const R Wr[4], const
     const R ml = gl.rho * sl.M[0], mr = gr.rho * sr.M[0];
     W0[0] = ml + mr;
     W0[1] = gl.rho * sl.M[1] + gr.rho * sr.M[1];
-    W0[2] = gl.V * ml + gr.V * mr;
-    W0[3] = R(0.5) * (gl.rho * (sl.M[2] + N * gl.th * sl.M[0] + gl.V * gl.V * sl.M[0]) +
-                      gr.rho * (sr.M[2] + N * gr.th * sr.M[0] + gr.V * gr.V * sr.M[0]));
+    if (D1) {
+      W0[2] = R(0);
+      W0[3] = R(0.5) * (gl.rho * (sl.M[2] + N * gl.th * sl.M[0]) + gr.rho * (sr.M[2] + N * gr.th * sr.M[0]));
+    } else {
+      W0[2] = gl.V * ml + gr.V * mr;
+      W0[3] = R(0.5) * (gl.rho * (sl.M[2] + N * gl.th * sl.M[0] + gl.V * gl.V * sl.M[0]) +
+                        gr.rho * (sr.M[2] + N * gr.th * sr.M[0] + gr.V * gr.V * sr.M[0]));
+    }
   }
-  const GasState<R> g0 = gas_state(W0, gm1);
+  const GasState<R> g0 = gas_state<D1>(W0, gm1);
 
   // gradients (x: normal, y: tangential) and time derivatives of each state
   R x1[4], Wlq[4], Wrq[4], W0q[4], rt;
   {
-    const PrimGrad<R> gx = prim_grad(gl, gm1, Wln), gy = prim_grad(gl, gm1, Wt), gt = prim_rate(gl, gm1, gx, gy);
-    half_side(gl, N, R(2) * ql * ql, gx, gy, gt, sl);
-    cons_rate(gl, hN, gt, Wlq, rt);
+    const PrimGrad<R> gx = prim_grad<D1>(gl, gm1, Wln), gy = prim_grad<D1>(gl, gm1, Wt), gt = prim_rate<D1>(gl, gm1, gx, gy);
+    half_side<D1>(gl, N, R(2) * ql * ql, gx, gy, gt, sl);
+    cons_rate<D1>(gl, hN, gt, Wlq, rt);
   }
   {
-    const PrimGrad<R> gx = prim_grad(gr, gm1, Wrn), gy = prim_grad(gr, gm1, Wt), gt = prim_rate(gr, gm1, gx, gy);
-    half_side(gr, N, R(2) * qr * qr, gx, gy, gt, sr);
-    cons_rate(gr, hN, gt, Wrq, rt);
+    const PrimGrad<R> gx = prim_grad<D1>(gr, gm1, Wrn), gy = prim_grad<D1>(gr, gm1, Wt), gt = prim_rate<D1>(gr, gm1, gx, gy);
+    half_side<D1>(gr, N, R(2) * qr * qr, gx, gy, gt, sr);
+    cons_rate<D1>(gr, hN, gt, Wrq, rt);
   }
   R FE[4], FQ[4], FS[4];   // g0: Euler flux, its time derivative, stress
   {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) x1[k] = R(0.5) * (Wln[k] + Wrn[k]);
-    const PrimGrad<R> gx = prim_grad(g0, gm1, x1), gy = prim_grad(g0, gm1, Wt), gt = prim_rate(g0, gm1, gx, gy);
-    cons_rate(g0, hN, gt, W0q, rt);
-    euler_flux(g0, W0, FE);
-    euler_flux_rate(g0, W0, gt, W0q, rt, FQ);
-    stress_flux(g0, K, gm1, gx, gy, FS);
+    for (int k = 0; k < 4; ++k)
+      if (!D1 || k != 2) x1[k] = R(0.5) * (Wln[k] + Wrn[k]);
+    const PrimGrad<R> gx = prim_grad<D1>(g0, gm1, x1), gy = prim_grad<D1>(g0, gm1, Wt), gt = prim_rate<D1>(g0, gm1, gx, gy);
+    cons_rate<D1>(g0, hN, gt, W0q, rt);
+    euler_flux<D1>(g0, W0, FE);
+    euler_flux_rate<D1>(g0, W0, gt, W0q, rt, FQ);
+    stress_flux<D1>(g0, K, gm1, gx, gy, FS);
   }
 
   // collision time and time coefficients: FP64 with expm1 where they cancel
@@ -860,19 +900,23 @@ FD_HD void iface_solve_x(const GasK<R>& gas, const R Wl[4], const R Wr[4], const
   // <psi (a0 u + b0 v)> = -W0q and <psi A0> = W0q (compatibility); the fluxes
   // of the two terms are FS - FQ and FQ
   R F[4], We[4];
+  auto used = [](int k) { return !D1 || k != 2; };
+  if (D1) F[2] = We[2] = R(0);
   if (want_n) {
     const R kq = cn[2] - cn[1];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
+      if (!used(k)) continue;
       F[k] = cn[0] * FE[k] + kq * FQ[k] + cn[1] * FS[k];
       We[k] = cn[0] * W0[k] + kq * W0q[k];
     }
-    half_flux(sr, cn[3], cn[4], cn[5], F, We);
-    half_flux(sl, cn[3], cn[4], cn[5], F, We);
+    half_flux<D1>(sr, cn[3], cn[4], cn[5], F, We);
+    half_flux<D1>(sl, cn[3], cn[4], cn[5], F, We);
     // Prandtl-number correction of the energy flux
     if (gas.prfix != R(0)) F[3] += gas.prfix * heat_flux_x(F, We, g0.U, g0.V);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
+      if (!used(k)) continue;
       // interface flow variables, Eq. (eq:W-model) with tau_0 = tau
       o.F[k] = F[k];
       o.Wl[k] = e1 * We[k] + E * Wl[k];
@@ -882,14 +926,16 @@ FD_HD void iface_solve_x(const GasK<R>& gas, const R Wl[4], const R Wr[4], const
   const R kq = ct[2] - ct[1];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
+    if (!used(k)) continue;
     F[k] = ct[0] * FE[k] + kq * FQ[k] + ct[1] * FS[k];
     We[k] = ct[0] * W0[k] + kq * W0q[k];
   }
-  half_flux(sl, ct[3], ct[4], ct[5], F, We);
-  half_flux(sr, ct[3], ct[4], ct[5], F, We);
+  half_flux<D1>(sl, ct[3], ct[4], ct[5], F, We);
+  half_flux<D1>(sr, ct[3], ct[4], ct[5], F, We);
   if (gas.prfix != R(0)) F[3] += gas.prfix * heat_flux_x(F, We, g0.U, g0.V);
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
+    if (!used(k)) continue;
     // the one-sided time derivatives are W_t = -rho <(a u + b v) psi>
     o.Ft[k] = F[k];
     o.Wlt[k] = e1 * We[k] + E * Wlq[k];
@@ -964,6 +1010,27 @@ FD_HD void nodal_flux(const GasK<R>& gas, const R W[4], const R Wx[4], const R W
 #pragma unroll
   for (int k = 1; k < 4; ++k) x[k] = x[k] - tau * y[k];
   G[0] = x[0]; G[1] = x[2]; G[2] = x[1]; G[3] = x[3];
+}
+
+// The x-flux of nodal_flux for the one-dimensional gas (V = 0, no
+// y-derivative); component 2 is neither read nor written.
+template <class R>
+FD_HD void nodal_flux_1d(const GasK<R>& gas, const R W[4], const R Wx[4], R F[4], R Ft[4], bool want_n) {
+  const R K = gas.K, gm1 = gas.gm1;
+  const GasState<R> g = gas_state<true>(W, gm1);
+  const PrimGrad<R> gx = prim_grad<true>(g, gm1, Wx), gt = prim_rate<true>(g, gm1, gx, gx);
+  R Wq[4], rt, x[4];
+  cons_rate<true>(g, R(0.5) * K + R(1), gt, Wq, rt);
+  const R qf = gas.prfix * (R(0.5) * K + R(2)) * g.p;
+  euler_flux_rate<true>(g, W, gt, Wq, rt, Ft);
+  Ft[3] += qf * gt.u;
+  if (!want_n) return;
+  const R tau = gas.c1_r * gas.dt_r + gas.mu_r * s_div(R(1), g.p);   // c1 dt + mu/p
+  euler_flux<true>(g, W, F);
+  stress_flux<true>(g, K, gm1, gx, gx, x);
+  x[3] += qf * gx.t;
+  F[1] = F[1] - tau * x[1];
+  F[3] = F[3] - tau * x[3];
 }
 
 // ---------------------------------------------------------------------------
