@@ -97,6 +97,8 @@ FD_HD float s_erfc_e(float x, float ex2) { (void)ex2; return erfcf(x); }
 template <class R> struct TanhSat;
 template <> struct TanhSat<double> { static constexpr double z = 19.5; };
 template <> struct TanhSat<float> { static constexpr float z = 9.5f; };
+// and, in FP64, the value from which it does: e^(-2z) = 2^-54, z = 27 ln 2
+const double GENO_SAT64 = 18.715;
 
 // ---------------------------------------------------------------------------
 // constants of one run, in compute precision
@@ -152,10 +154,10 @@ FD_HD R geno_floor(R qmax) {
 // Sufficient test for tanh(C alpha) rounding to 1, which smooth data pass:
 // alpha = 2 aH/(aH + aL) with aH >= 1, so C alpha > z wherever
 // aL = 1 + (tau/(ISL + eps))^r < 2C/z - 1.  C = 20; the bounds on
-// tau/(ISL + eps) are the r-th roots of 2C/z - 2 (1/19.5 in FP64, 2.2105 in
-// FP32), rounded down.  It takes a product where the quotients of the path
+// tau/(ISL + eps) are the r-th roots of 2C/z - 2 (0.13732 in FP64, where z =
+// GENO_SAT64, 2.2105 in FP32), rounded down.  It takes a product where the quotients of the path
 // function take divisions (FP32) or 14 more FP64 operations.
-template <class R> struct GenoSmooth { static constexpr double c2 = 0.226455, c3 = 0.371510; };
+template <class R> struct GenoSmooth { static constexpr double c2 = 0.370560, c3 = 0.515910; };
 template <> struct GenoSmooth<float> { static constexpr float c2 = 1.48670f, c3 = 1.30260f; };
 template <class R>
 FD_HD bool geno_smooth(R tau, R ISL, R ea, int r) {
@@ -177,17 +179,19 @@ FD_HD R geno_chi(const GenoK<R>& g, R IS0, R IS1, R IS2, R floor = R(0)) {
     R aL = R(1) + rpow(s_div(tau, ISL + ea), g.r);
     alpha = s_div(R(2) * aH, aH + aL);
   } else {
-    // alpha = 2 aH/(aH + aL), aH = 1 + (tau/h)^r, aL = 1 + (tau/l)^r, written
-    // over the common denominator h^r l^r; tanh(C alpha) rounds to 1 when
-    // C alpha > z_sat, which is tested before dividing.  A floor is added to
-    // eps_a only when one is given (the FP64 linearisation of a mixed run)
+    // tanh(C alpha) with alpha = 2 aH/(aH + aL), aH = 1 + (tau/h)^r, aL = 1 +
+    // (tau/l)^r, over the common denominator h^r l^r; tanh z as
+    // (1 - e^-2z)/(1 + e^-2z), one exponential and two reciprocals (tanh(C) is
+    // 1).  A floor is added to eps_a only when one is given (the FP64
+    // linearisation of a mixed run)
     R ea = g.eps_a;
     if (floor != R(0)) ea = ea + floor;
-    R hr = rpow(ISH + ea, g.r), lr = rpow(ISL + ea, g.r), tr = rpow(tau, g.r);
-    R num = R(2) * (hr + tr) * lr;
-    R den = (hr + tr) * lr + (lr + tr) * hr;
-    if (g.C * num > R(TanhSat<R>::z) * den) return g.inv_tanhC;
-    alpha = num / den;
+    const R hr = rpow(ISH + ea, g.r), lr = rpow(ISL + ea, g.r), tr = rpow(tau, g.r);
+    const R a = (hr + tr) * lr, b = (lr + tr) * hr;
+    const R z = (R(2) * g.C) * (a * (R(1) / (a + b)));
+    if (z > R(GENO_SAT64)) return g.inv_tanhC;
+    const R e = s_exp(R(-2) * z);
+    return (R(1) - e) * (R(1) / (R(1) + e));
   }
   R z = g.C * alpha;
   // tanh(z) is exactly 1 in this precision above the saturation point
@@ -195,8 +199,11 @@ FD_HD R geno_chi(const GenoK<R>& g, R IS0, R IS1, R IS2, R floor = R(0)) {
   return s_tanh(z) * g.inv_tanhC;
 }
 
+// Weights of the three sub-stencils up to the factor returned (FP64: the
+// reciprocal of their sum, which is applied once to what they weight; FP32:
+// 1, the weights are normalised, which keeps their range).
 template <class R>
-FD_HD void geno_weights(const GenoK<R>& g, const R d[3], R IS0, R IS1, R IS2, R w[3]) {
+FD_HD R geno_weights(const GenoK<R>& g, const R d[3], R IS0, R IS1, R IS2, R w[3]) {
   R e0 = IS0 + g.eps_w, e1 = IS1 + g.eps_w, e2 = IS2 + g.eps_w;
   R s0 = e0 * e0, s1 = e1 * e1, s2 = e2 * e2;
   if (IsF32<R>::v) {
@@ -205,14 +212,13 @@ FD_HD void geno_weights(const GenoK<R>& g, const R d[3], R IS0, R IS1, R IS2, R 
     w[0] = t0 * inv;
     w[1] = t1 * inv;
     w[2] = t2 * inv;
-  } else {
-    // d_k/s_k normalised = d_k P_k / sum_m d_m P_m with P_k the product of the other two s
-    R t0 = d[0] * s1 * s2, t1 = d[1] * s0 * s2, t2 = d[2] * s0 * s1;
-    R inv = R(1) / (t0 + t1 + t2);
-    w[0] = t0 * inv;
-    w[1] = t1 * inv;
-    w[2] = t2 * inv;
+    return R(1);
   }
+  // d_k/s_k normalised = d_k P_k / sum_m d_m P_m with P_k the product of the other two s
+  w[0] = d[0] * (s1 * s2);
+  w[1] = d[1] * (s0 * s2);
+  w[2] = d[2] * (s0 * s1);
+  return R(1) / (w[0] + (w[1] + w[2]));
 }
 
 // The floor of an FP64 evaluation: (fscale max|Q|)^2 when fscale is given
@@ -253,7 +259,7 @@ FD_HD float est_f32(double x) {
 FD_HD bool geno_smooth_est(float I0, float I1, float I2, float ea, int r) {
   const float lo = fminf(I0, fminf(I1, I2)), hi = fmaxf(I0, fmaxf(I1, I2));
   const float tau = fabsf(0.5f * (I1 + I2) - I0);
-  return tau + 2e-4f * hi < (r == 3 ? 0.37150f : 0.22644f) * (0.9999f * lo + ea);
+  return tau + 2e-4f * hi < (r == 3 ? 0.51585f : 0.37050f) * (0.9999f * lo + ea);
 }
 FD_HD float is_grad_est(float b, float xh) {   // the sub-stencil with an averaged gradient
   const float t = b - xh, u = 2.0f * b - xh;
@@ -327,12 +333,12 @@ FD_HD void recon_interface(const GenoK<R>& g, const R Q[4], const R Qx[4], R h, 
     chil = chi;
     if (chi != R(1)) {
       R w[3];
-      geno_weights(g, g.d_iface, IS0, IS1, IS2, w);
+      const R om = (R(1) - chi) * geno_weights(g, g.d_iface, IS0, IS1, IS2, w);
       const R PL = w[0] * (R(1.25) * b0 - R(0.75) * xh) + w[1] * (R(0.125) * b0 + R(0.375) * b1) +
                    w[2] * (R(0.625) * b1 - R(0.125) * b2);
       const R PLx = w[0] * (R(3) * b0 * ih - R(2) * Qx[0]) + (w[1] + w[2]) * (b1 * ih);
-      vl = Q[1] + (chi * PHl + (R(1) - chi) * PL);
-      dl = chi * PHx + (R(1) - chi) * PLx;
+      vl = Q[1] + (chi * PHl + om * PL);
+      dl = chi * PHx + om * PLx;
     }
   }
   // ---- right state (App. C2, formulas for interface j+1/2) ----
@@ -348,12 +354,12 @@ FD_HD void recon_interface(const GenoK<R>& g, const R Q[4], const R Qx[4], R h, 
     chir = chi;
     if (chi != R(1)) {
       R w[3];
-      geno_weights(g, g.d_iface, IS0, IS1, IS2, w);
+      const R om = (R(1) - chi) * geno_weights(g, g.d_iface, IS0, IS1, IS2, w);
       const R PL = w[0] * (R(0.75) * xh - R(1.25) * b2) - w[1] * (R(0.125) * b2 + R(0.375) * b1) +
                    w[2] * (R(0.125) * b0 - R(0.625) * b1);
       const R PLx = w[0] * (R(3) * b2 * ih - R(2) * Qx[3]) + (w[1] + w[2]) * (b1 * ih);
-      vr = Q[2] + (chi * PHr + (R(1) - chi) * PL);
-      dr = chi * PHx + (R(1) - chi) * PLx;
+      vr = Q[2] + (chi * PHr + om * PL);
+      dr = chi * PHx + om * PLx;
     }
   }
 }
@@ -387,9 +393,9 @@ FD_HD R recon_node(const GenoK<R>& g, const R Q[3], const R Qx[3], R h, R ih, R 
       geno_chi(g, IS0, IS1, IS2, geno_floor_of(s_max(s_abs(Q[1]), s_max(s_abs(Q[0]), s_abs(Q[2]))), fscale));
   if (chi == R(1)) return PHx;
   R w[3];
-  geno_weights(g, g.d_node, IS0, IS1, IS2, w);
+  const R om = (R(1) - chi) * geno_weights(g, g.d_node, IS0, IS1, IS2, w);
   const R PLx = w[0] * (R(0.5) * b * ih) + w[1] * (R(2) * b0 * ih - Qx[0]) + w[2] * (R(2) * b1 * ih - Qx[2]);
-  return chi * PHx + (R(1) - chi) * PLx;
+  return chi * PHx + om * PLx;
 }
 
 // ---------------------------------------------------------------------------

@@ -51,13 +51,11 @@ FD_HD void geno_chi_adj(const GenoK<R>& g, const R IS[3], R fl, R chib, R ISb[3]
   if (fl != 0.0) ea = ea + fl;
   const R H = ISH + ea, Lo = ISL + ea;
   const R hr = rpow(H, g.r), lr = rpow(Lo, g.r), tr = rpow(tau, g.r);
-  const R A = (hr + tr) * lr, B = (lr + tr) * hr;
-  const R num = 2.0 * A, den = A + B;
-  if (g.C * num > R(TanhSat<R>::z) * den) return;   // saturated: chi constant
-  const R alpha = num / den, z = g.C * alpha;
-  if (z > R(TanhSat<R>::z)) return;
-  const R th = s_tanh(z);
-  const R alphab = chib * g.inv_tanhC * (1.0 - th * th) * g.C;
+  const R A = (hr + tr) * lr, B = (lr + tr) * hr, den = A + B;
+  const R z = (2.0 * g.C) * (A * (1.0 / den));
+  if (z > R(GENO_SAT64)) return;   // saturated: chi constant
+  const R e = s_exp(-2.0 * z), ie = 1.0 / (1.0 + e);
+  const R alphab = chib * (4.0 * e * ie * ie) * g.C;
   // alpha = 2 A / (A + B)
   const R Ab = alphab * 2.0 * B / (den * den), Bb = -alphab * 2.0 * A / (den * den);
   const R hrb = Ab * lr + Bb * (lr + tr), lrb = Ab * (hr + tr) + Bb * hr, trb = (Ab * lr + Bb * hr);
@@ -109,7 +107,8 @@ FD_HD void geno_blend_adj(const GenoK<R>& g, const R dk[3], const R IS[3], R fl,
     return;
   }
   R w[3];
-  geno_weights(g, dk, IS[0], IS[1], IS[2], w);
+  const R inv = geno_weights(g, dk, IS[0], IS[1], IS[2], w);
+  for (int k = 0; k < 3; ++k) w[k] *= inv;
   const R PL = w[0] * q[0] + w[1] * q[1] + w[2] * q[2];
   const R PLx = w[0] * qx0 + (w[1] + w[2]) * dq12;
   const R chib_t = chib + vb * (PH - PL) + db * (PHx - PLx);
@@ -274,7 +273,8 @@ FD_HD void recon_node_adj(const GenoK<R>& g, const R Q[3], const R Qx[3], R h, R
       R ISb[3] = {0.0, 0.0, 0.0}, flb = 0.0, w[3], x0b = 0.0, x2b = 0.0, tb, ub;
       const R PHx = (Qx[0] + 46.0 * Qx[1] + Qx[2]) * c30 - (0.3 * ih) * b;
       const R qx[3] = {0.5 * b * ih, 2.0 * b0 * ih - Qx[0], 2.0 * b1 * ih - Qx[2]};
-      geno_weights(g, g.d_node, IS[0], IS[1], IS[2], w);
+      const R inv = geno_weights(g, g.d_node, IS[0], IS[1], IS[2], w);
+      for (int k = 0; k < 3; ++k) w[k] *= inv;
       const R PLx = w[0] * qx[0] + w[1] * qx[1] + w[2] * qx[2];
       PHxb = chi * rb;
       const R PLxb = (1.0 - chi) * rb;
