@@ -590,6 +590,48 @@ FD_HD TimeCoef<TW> time_coef(TW tau, TW dt, TW inv_dt) {
   return t;
 }
 
+// The same for x = dt/tau <= 1, for the FP32 path without FP64: inserting
+// exp(-y) = sum (-y)^n/n! in the integrals, every term that cancels drops out
+// and four power series in x remain,
+//   cn0 = x^2 p0,  cn1 = dt x p1,  cn2 = -dt x p0,
+//   ct0 = x (1 - x r0)/dt,  ct1 = x s0,  ct2 = x r0,
+//   p0 = sum_{n>=3} (-1)^n (4/2^n - 1)/n! x^(n-3),  p1 the same times (n - 2),
+//   r0 = -sum_{n>=3} (-1)^n 4 (1 - 2/2^n)/n! x^(n-3),  s0 = -r0's terms times (n - 2),
+// each dominated by its first term, so that Horner's rule keeps them within
+// about an ulp of FP32; terms to n = 11 (the next is below 1e-8 of the sum).
+template <class R>
+FD_HD TimeCoef<R> time_coef_small(R x, R tau, R dt, R inv_dt) {
+  const int NC = 9;   // n = 3..11
+  R p0 = R(0), p1 = R(0), r0 = R(0), s0 = R(0);
+#pragma unroll
+  for (int n = NC + 2; n >= 3; --n) {
+    double f = 1.0, h = 1.0;   // n!, 2^-n
+    for (int k = 1; k <= n; ++k) { f *= k; h *= 0.5; }
+    const double sg = n % 2 ? -1.0 : 1.0, a = sg * (4.0 * h - 1.0) / f, b = sg * 4.0 * (1.0 - 2.0 * h) / f;
+    p0 = p0 * x + R(a);
+    p1 = p1 * x + R(a * (n - 2));
+    r0 = r0 * x + R(-b);
+    s0 = s0 * x + R(b * (n - 2));
+  }
+  TimeCoef<R> t;
+  const R xdt = x * dt, q0 = R(1) - x * r0;
+  t.cn[0] = x * x * p0;
+  t.cn[1] = xdt * p1;
+  t.cn[2] = -xdt * p0;
+  t.ct[0] = x * q0 * inv_dt;
+  t.ct[1] = x * s0;
+  t.ct[2] = x * r0;
+  t.cn[3] = R(1) - t.cn[0];
+  t.ct[3] = -t.ct[0];
+  t.cn[4] = -tau - t.cn[1];
+  t.ct[4] = -t.ct[1];
+  t.cn[5] = -tau - t.cn[2];
+  t.ct[5] = q0;
+  t.e1 = -s_expm1(-x);
+  t.E = R(1) - t.e1;
+  return t;
+}
+
 // ---------------------------------------------------------------------------
 // Closed-form moments.  A slope a = (d ln g) of a Maxwellian is fixed by the
 // gradients of its primitive variables; with c = v - V the tangential
@@ -846,7 +888,7 @@ FD_HD void iface_solve_x(const GasK<R>& gas, const R Wl[4], const R Wr[4], const
     W0[1] = gl.rho * sl.M[1] + gr.rho * sr.M[1];
     if (D1) {
       W0[2] = R(0);
-      W0[3] = R(0.5) * (gl.rho * (sl.M[2] + N * gl.th * sl.M[0]) + gr.rho * (sr.M[2] + N * gr.th * sr.M[0]));
+      W0[3] = R(0.5) * (gl.rho * sl.M[2] + gr.rho * sr.M[2] + N * (gl.p * sl.M[0] + gr.p * sr.M[0]));
     } else {
       W0[2] = gl.V * ml + gr.V * mr;
       W0[3] = R(0.5) * (gl.rho * (sl.M[2] + N * gl.th * sl.M[0] + gl.V * gl.V * sl.M[0]) +
@@ -880,13 +922,21 @@ FD_HD void iface_solve_x(const GasK<R>& gas, const R Wl[4], const R Wr[4], const
   }
 
   // collision time and time coefficients: FP64 with expm1 where they cancel
-  // (dt/tau small); in the FP32 path, FP32 where dt/tau > 4
+  // (dt/tau small); in the FP32 path FP32 where dt/tau > 4, where they do not,
+  // and where dt/tau <= 1, from series that do not (viscous runs lie there: the
+  // 85 slots of the FP64 pipe cost more than the rest of the FP32 solve)
   typedef typename Wide<R>::T TW;
   R cn[6], ct[6], E, e1;
   R ip0r = s_div(R(1), g0.p);
   R taur = gas.c1_r * gas.dt_r + gas.mu_r * ip0r + gas.c2_r * gas.dt_r * s_div(s_abs(gl.p - gr.p), gl.p + gr.p);
   if (IsF32<R>::v && gas.dt_r > R(TIME_COEF_FP32_RATIO) * taur) {
     TimeCoef<R> tc = time_coef(taur, gas.dt_r, gas.inv_dt_r);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) { cn[k] = tc.cn[k]; ct[k] = tc.ct[k]; }
+    E = tc.E;
+    e1 = tc.e1;
+  } else if (IsF32<R>::v && !(gas.dt_r > taur)) {
+    TimeCoef<R> tc = time_coef_small(s_div(gas.dt_r, taur), taur, gas.dt_r, gas.inv_dt_r);
 #pragma unroll
     for (int k = 0; k < 6; ++k) { cn[k] = tc.cn[k]; ct[k] = tc.ct[k]; }
     E = tc.E;
