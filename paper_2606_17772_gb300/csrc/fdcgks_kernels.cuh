@@ -182,10 +182,16 @@ FD_HD void recon_line_ld(const GenoK<R>& geno, LD ld, int l, R h, R ih, R vl[4],
 template <bool D1 = false, class R, class LD>
 FD_HD void recon_line_char(const GenoK<R>& geno, R gm1, int normal, LD ld, int l, R h, R ih, R vl[4], R dl[4],
                            R vr[4], R dr[4], R& chi) {
-  const int in = normal == 0 ? 1 : 2, it = normal == 0 ? 2 : 1;
-  const int perm[4] = {0, in, it, 3};
+  // component j of (rho, m_n, m_t, E) of an entry's values (f0 = 0) or
+  // gradients (f0 = 4): a select between the two momenta, not an index, so that
+  // values held in registers stay there
+  const bool sw = normal != 0;
+  auto comp = [&](int e, int f0, int j) -> R {
+    return j == 1 ? (sw ? ld(l, e, f0 + 2) : ld(l, e, f0 + 1))
+                  : j == 2 ? (sw ? ld(l, e, f0 + 1) : ld(l, e, f0 + 2)) : ld(l, e, f0 + j);
+  };
   const R r = R(0.5) * (ld(l, 1, 0) + ld(l, 2, 0));
-  const R mn = R(0.5) * (ld(l, 1, in) + ld(l, 2, in)), mt = R(0.5) * (ld(l, 1, it) + ld(l, 2, it));
+  const R mn = R(0.5) * (comp(1, 0, 1) + comp(2, 0, 1)), mt = R(0.5) * (comp(1, 0, 2) + comp(2, 0, 2));
   const R E = R(0.5) * (ld(l, 1, 3) + ld(l, 2, 3));
   const R ir = s_div(R(1), r), u = mn * ir, v = mt * ir;
   const R q2 = u * u + v * v;
@@ -218,31 +224,32 @@ FD_HD void recon_line_char(const GenoK<R>& geno, R gm1, int normal, LD ld, int l
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         if (D1 && j == 2) continue;
-        a += Lm[k][j] * ld(l, m, perm[j]);
-        b += Lm[k][j] * ld(l, m, 4 + perm[j]);
+        a += Lm[k][j] * comp(m, 0, j);
+        b += Lm[k][j] * comp(m, 4, j);
       }
       Q[m] = a;
       Qx[m] = b;
     }
     recon_interface(geno, Q, Qx, h, ih, cvl[k], cdl[k], cl[k], cvr[k], cdr[k], cr[k]);
   }
+  R tvl[4], tdl[4], tvr[4], tdr[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    R a = R(0), b = R(0), d = R(0), e = R(0);
-    if (!D1 || j != 2)
+    tvl[j] = tdl[j] = tvr[j] = tdr[j] = R(0);
+    if (D1 && j == 2) continue;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       if (D1 && k == 2) continue;
-      a += Rm[j][k] * cvl[k];
-      b += Rm[j][k] * cvr[k];
-      d += Rm[j][k] * cdl[k];
-      e += Rm[j][k] * cdr[k];
+      tvl[j] += Rm[j][k] * cvl[k];
+      tvr[j] += Rm[j][k] * cvr[k];
+      tdl[j] += Rm[j][k] * cdl[k];
+      tdr[j] += Rm[j][k] * cdr[k];
     }
-    vl[perm[j]] = a;
-    vr[perm[j]] = b;
-    dl[perm[j]] = d;
-    dr[perm[j]] = e;
   }
+  swap_uv(tvl, vl, sw);
+  swap_uv(tdl, dl, sw);
+  swap_uv(tvr, vr, sw);
+  swap_uv(tdr, dr, sw);
   chi = s_min(s_min(cl[0], cr[0]), s_min(cl[3], cr[3]));
   positivity_fix(ld, l, vl, dl, vr, dr, chi);
 }
