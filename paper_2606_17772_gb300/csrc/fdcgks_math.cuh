@@ -462,130 +462,6 @@ FD_HD R recon_node(const GenoK<R>& g, const R Q[3], const R Qx[3], R h, R ih, R 
 }
 
 // ---------------------------------------------------------------------------
-// Maxwellian moments (App. A1).  Tables hold normalized moments <u^n>, <v^n>,
-// <xi^{2c}> of g / rho; half-space tables restrict u to one sign.
-// ---------------------------------------------------------------------------
-template <class R>
-struct Maxw {
-  R rho, U, V, lam;
-  R ir;    // 1/rho
-  R p;     // pressure rho/(2 lam)
-  R i2l;   // 1/(2 lam) = p/rho
-};
-
-// conservative W -> Maxwellian; rho E = rho (U^2 + V^2 + (K+2)/(2 lam))/2,
-// so p = (gamma - 1)(rho E - rho (U^2+V^2)/2) and lam = rho/(2 p)
-template <class R>
-FD_HD Maxw<R> maxw_from_W(const R W[4], R gm1) {
-  Maxw<R> g;
-  g.rho = W[0];
-  g.ir = s_div(R(1), W[0]);
-  g.U = W[1] * g.ir;
-  g.V = W[2] * g.ir;
-  g.p = gm1 * (W[3] - R(0.5) * W[0] * (g.U * g.U + g.V * g.V));
-  g.i2l = g.p * g.ir;
-  g.lam = s_div(R(0.5), g.i2l);
-  return g;
-}
-
-const int NT = 7;   // moment orders 0..6
-
-template <class R>
-struct Tab {
-  R u[NT], v[NT], xi[3];
-};
-
-template <class R>
-FD_HD void recur(R m, R i2l, R* t) {
-  // <c^{n+2}> = m <c^{n+1}> + (n+1)/(2 lam) <c^n>
-#pragma unroll
-  for (int n = 0; n + 2 < NT; ++n) t[n + 2] = m * t[n + 1] + R(n + 1) * i2l * t[n];
-}
-
-// full-space tables of g
-template <class R>
-FD_HD void tab_full(const Maxw<R>& g, R K, Tab<R>& T) {
-  R i2l = g.i2l;
-  T.u[0] = R(1); T.u[1] = g.U;
-  T.v[0] = R(1); T.v[1] = g.V;
-  recur(g.U, i2l, T.u);
-  recur(g.V, i2l, T.v);
-  T.xi[0] = R(1);
-  T.xi[1] = K * i2l;
-  T.xi[2] = K * (K + R(2)) * i2l * i2l;
-}
-
-// u-half-space tables (sign +1: u > 0, -1: u < 0), sharing v and xi with T
-template <class R>
-FD_HD void tab_half(const Maxw<R>& g, int sign, const Tab<R>& full, Tab<R>& H) {
-  R i2l = g.i2l;
-  R sl = s_sqrt(g.lam);
-  R isl = sl * (R(2) * i2l);                   // 1/sqrt(lam)
-  R e = s_exp(-g.lam * g.U * g.U);
-  const R isqpi = R(0.56418958354775628695);   // 1/sqrt(pi)
-  H.u[0] = R(0.5) * s_erfc_e(-R(sign) * sl * g.U, e);
-  H.u[1] = g.U * H.u[0] + R(sign) * R(0.5) * e * isqpi * isl;
-  recur(g.U, i2l, H.u);
-#pragma unroll
-  for (int n = 0; n < NT; ++n) H.v[n] = full.v[n];
-  H.xi[0] = full.xi[0]; H.xi[1] = full.xi[1]; H.xi[2] = full.xi[2];
-}
-
-template <int a, int b, int c, class R>
-FD_HD R mm(const Tab<R>& T) { return T.u[a] * T.v[b] * T.xi[c]; }
-
-// <u^a v^b xi^{2c} psi>, psi = (1, u, v, (u^2+v^2+xi^2)/2)
-template <int a, int b, int c, class R>
-FD_HD void mpsi(const Tab<R>& T, R o[4]) {
-  o[0] = mm<a, b, c>(T);
-  o[1] = mm<a + 1, b, c>(T);
-  o[2] = mm<a, b + 1, c>(T);
-  o[3] = R(0.5) * (mm<a + 2, b, c>(T) + mm<a, b + 2, c>(T) + mm<a, b, c + 1>(T));
-}
-
-// <s u^a v^b psi> for a slope polynomial s = s0 + s1 u + s2 v + s3 psi_4,
-// psi_4 = (u^2 + v^2 + xi^2)/2.  The moments factor, <u^p v^q xi^2m> =
-// u[p] v[q] xi[m], so with h = s3/2 the slope-weighted moment is
-//   <s u^p v^q> = v[q] U(p) + u[p] V(q),
-//   U(p) = (s0 + h xi[1]) u[p] + s1 u[p+1] + h u[p+2],  V(q) = s2 v[q+1] + h v[q+2],
-//   <s u^p v^q xi^2> = xi[1] (v[q] U'(p) + u[p] V(q)) + h xi[2] u[p] v[q],
-//   U'(p) = s0 u[p] + s1 u[p+1] + h u[p+2],
-// and the psi components are <s u^a v^b (1, u, v)> and half the sum of
-// <s u^(a+2) v^b>, <s u^a v^(b+2)> and <s u^a v^b xi^2>.
-template <int p, class R>
-FD_HD R slope_u(const Tab<R>& T, R c0, R s1, R h) { return c0 * T.u[p] + s1 * T.u[p + 1] + h * T.u[p + 2]; }
-template <int q, class R>
-FD_HD R slope_v(const Tab<R>& T, R s2, R h) { return s2 * T.v[q + 1] + h * T.v[q + 2]; }
-template <int p, int q, class R>
-FD_HD R slope_uv(const Tab<R>& T, R c0, const R s[4], R h) {
-  return T.v[q] * slope_u<p>(T, c0, s[1], h) + T.u[p] * slope_v<q>(T, s[2], h);
-}
-
-template <int a, int b, class R>
-FD_HD void mslope(const Tab<R>& T, const R s[4], R o[4]) {
-  const R h = R(0.5) * s[3];
-  const R c0 = s[0] + h * T.xi[1];
-  const R sx = T.xi[1] * (T.v[b] * slope_u<a>(T, s[0], s[1], h) + T.u[a] * slope_v<b>(T, s[2], h)) +
-               h * T.xi[2] * T.u[a] * T.v[b];
-  o[0] = slope_uv<a, b>(T, c0, s, h);
-  o[1] = slope_uv<a + 1, b>(T, c0, s, h);
-  o[2] = slope_uv<a, b + 1>(T, c0, s, h);
-  o[3] = R(0.5) * (slope_uv<a + 2, b>(T, c0, s, h) + slope_uv<a, b + 2>(T, c0, s, h) + sx);
-}
-
-// slope s with <s psi> = r (r = dW / rho), closed form of the 4x4 moment system
-template <class R>
-FD_HD void slope_solve(const Maxw<R>& g, R K, R c4K, const R r[4], R s[4]) {
-  R q = g.U * g.U + g.V * g.V + (K + R(2)) * g.i2l;
-  R Ah = r[1] - g.U * r[0];
-  R Ch = r[2] - g.V * r[0];
-  R B = R(2) * r[3] - q * r[0];
-  s[3] = c4K * g.lam * g.lam * (B - R(2) * g.U * Ah - R(2) * g.V * Ch);
-  s[2] = R(2) * g.lam * Ch - g.V * s[3];
-  s[1] = R(2) * g.lam * Ah - g.U * s[3];
-  s[0] = r[0] - g.U * s[1] - g.V * s[2] - R(0.5) * s[3] * q;
-}
-
 // heat flux of the energy equation relative to (U0, V0) from the moments
 // F = int u psi f and W = int psi f of one distribution (x-normal)
 template <class R>
@@ -593,13 +469,6 @@ FD_HD R heat_flux_x(const R F[4], const R W[4], R U0, R V0) {
   return F[3] - U0 * W[3] - U0 * F[1] - V0 * F[2] + (R(1.5) * U0 * U0 + R(0.5) * V0 * V0) * W[1] +
          U0 * V0 * W[2] - R(0.5) * U0 * (U0 * U0 + V0 * V0) * W[0];
 }
-// same for the y-normal flux G = int v psi f
-template <class R>
-FD_HD R heat_flux_y(const R G[4], const R W[4], R U0, R V0) {
-  return G[3] - V0 * W[3] - V0 * G[2] - U0 * G[1] + (R(1.5) * V0 * V0 + R(0.5) * U0 * U0) * W[2] +
-         U0 * V0 * W[1] - R(0.5) * V0 * (U0 * U0 + V0 * V0) * W[0];
-}
-
 // ---------------------------------------------------------------------------
 // Time coefficients of the interface distribution, integrated over
 // [0, delta] for delta = dt/2 and dt and fitted to f^n + t f_t^n (App. A1).

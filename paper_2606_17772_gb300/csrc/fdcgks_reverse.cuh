@@ -361,227 +361,270 @@ FD_HD void recon_line_adj(const GenoK<R>& g, const R* x, R h, R ih, const R vb[4
 }
 
 // ---------------------------------------------------------------------------
-// Maxwellian moments (App. A1)
+// Closed-form moments (gas_state, prim_grad, prim_rate, cons_rate, euler_flux,
+// euler_flux_rate, stress_flux, half_moments, half_side, half_flux): each
+// reverse adds the adjoints of its inputs, given those of its outputs.  A
+// state's or gradient's adjoint is kept in the struct of the value itself.
 // ---------------------------------------------------------------------------
-struct MaxwB {
-  R rho, ir, U, V, p, i2l, lam;
-};
-FD_HD MaxwB maxw_zero() {
-  MaxwB b;
-  b.rho = b.ir = b.U = b.V = b.p = b.i2l = b.lam = 0.0;
-  return b;
+typedef GasState<R> Gas;
+typedef PrimGrad<R> Grad;
+FD_HD Gas gas_zero() { return Gas{0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0}; }
+FD_HD Grad grad_zero() { return Grad{0.0, 0.0, 0.0, 0.0}; }
+
+FD_HD void gas_state_adj(const R W[4], R gm1, const Gas& g, const Gas& gb, R Wb[4]) {
+  const R pb = gm1 * (gb.p + gb.th * g.ir);                    // th = p ir, p = gm1 (W3 - W0 (U^2 + V^2)/2)
+  const R Ub = gb.U - W[0] * g.U * pb, Vb = gb.V - W[0] * g.V * pb;
+  const R irb = gb.ir + gb.th * g.p + gb.en * W[3] + Ub * W[1] + Vb * W[2];
+  Wb[0] += gb.rho - 0.5 * (g.U * g.U + g.V * g.V) * pb - irb * g.ir * g.ir;
+  Wb[1] += Ub * g.ir;
+  Wb[2] += Vb * g.ir;
+  Wb[3] += pb + gb.en * g.ir;
 }
 
-struct TabB {
-  R u[NT], v[NT], xi[3];
-};
-FD_HD TabB tab_zero() {
-  TabB b;
-  for (int k = 0; k < NT; ++k) b.u[k] = b.v[k] = 0.0;
-  b.xi[0] = b.xi[1] = b.xi[2] = 0.0;
-  return b;
+FD_HD void prim_grad_adj(const Gas& g, R gm1, const R D[4], const Grad& q, const Grad& qb, Gas& gb, R Db[4]) {
+  const R tb = gm1 * qb.t, ub = qb.u - g.U * tb, vb = qb.v - g.V * tb;
+  const R db = qb.d - g.en * tb - g.V * vb - g.U * ub;
+  gb.en -= q.d * tb;
+  gb.U -= q.u * tb + q.d * ub;
+  gb.V -= q.v * tb + q.d * vb;
+  gb.ir += D[0] * db + D[1] * ub + D[2] * vb + D[3] * tb;
+  Db[0] += g.ir * db;
+  Db[1] += g.ir * ub;
+  Db[2] += g.ir * vb;
+  Db[3] += g.ir * tb;
 }
 
-// W -> Maxwellian, given the adjoints gb of the Maxwellian's fields: Wb += ...
-FD_HD void maxw_from_W_adj(const R W[4], R gm1, const Maxw<R>& g, MaxwB gb, R Wb[4]) {
-  gb.i2l += -gb.lam * g.lam / g.i2l;                    // lam = 1/2 / i2l
-  gb.p += gb.i2l * g.ir;                                // i2l = p ir
-  gb.ir += gb.i2l * g.p;
-  Wb[3] += gm1 * gb.p;                                  // p = gm1 (W3 - W0 (U^2 + V^2)/2)
-  Wb[0] -= 0.5 * gm1 * (g.U * g.U + g.V * g.V) * gb.p;
-  gb.U -= gm1 * W[0] * g.U * gb.p;
-  gb.V -= gm1 * W[0] * g.V * gb.p;
-  Wb[1] += gb.U * g.ir;                                 // U = W1 ir, V = W2 ir
-  Wb[2] += gb.V * g.ir;
-  gb.ir += gb.U * W[1] + gb.V * W[2];
-  Wb[0] += gb.rho - gb.ir * g.ir * g.ir;                // rho = W0, ir = 1/W0
+FD_HD void prim_rate_adj(const Gas& g, R gm1, const Grad& x, const Grad& y, const Grad& qb, Gas& gb, Grad& xb,
+                         Grad& yb) {
+  const R div = x.u + y.v, divb = qb.d + gm1 * g.th * qb.t;
+  gb.U -= qb.d * x.d + qb.u * x.u + qb.v * x.v + qb.t * x.t;
+  gb.V -= qb.d * y.d + qb.u * y.u + qb.v * y.v + qb.t * y.t;
+  gb.th -= qb.u * x.d + qb.v * y.d + gm1 * div * qb.t;
+  xb.d -= g.U * qb.d + g.th * qb.u;
+  xb.u -= g.U * qb.u + divb;
+  xb.v -= g.U * qb.v;
+  xb.t -= g.U * qb.t + qb.u;
+  yb.d -= g.V * qb.d + g.th * qb.v;
+  yb.u -= g.V * qb.u;
+  yb.v -= g.V * qb.v + divb;
+  yb.t -= g.V * qb.t + qb.v;
 }
 
-// t[n+2] = m t[n+1] + (n+1) i2l t[n], run backwards
-FD_HD void recur_adj(R m, R i2l, const R* t, R* tb, R& mb, R& i2lb) {
-  for (int n = NT - 3; n >= 0; --n) {
-    const R b = tb[n + 2];
-    tb[n + 1] += m * b;
-    tb[n] += R(n + 1) * i2l * b;
-    mb += t[n + 1] * b;
-    i2lb += R(n + 1) * t[n] * b;
+// W = cons_rate(g, q), rt = rho q.t; the adjoints Wb and rtb
+FD_HD void cons_rate_adj(const Gas& g, R hN, const Grad& q, const R W[4], const R Wb[4], R rtb, Gas& gb, Grad& qb) {
+  const R w0b = Wb[0] + g.U * Wb[1] + g.V * Wb[2] + g.en * Wb[3];
+  const R rub = Wb[1] + g.U * Wb[3], rvb = Wb[2] + g.V * Wb[3], tb = rtb + hN * Wb[3];
+  gb.U += W[0] * Wb[1] + g.rho * q.u * Wb[3];
+  gb.V += W[0] * Wb[2] + g.rho * q.v * Wb[3];
+  gb.en += W[0] * Wb[3];
+  gb.rho += q.d * w0b + q.u * rub + q.v * rvb + q.t * tb;
+  qb.d += g.rho * w0b;
+  qb.u += g.rho * rub;
+  qb.v += g.rho * rvb;
+  qb.t += g.rho * tb;
+}
+
+FD_HD void euler_flux_adj(const Gas& g, const R W[4], const R Fb[4], Gas& gb, R Wb[4]) {
+  Wb[1] += Fb[0] + g.U * Fb[1] + g.V * Fb[2];
+  Wb[3] += g.U * Fb[3];
+  gb.U += W[1] * Fb[1] + (W[3] + g.p) * Fb[3];
+  gb.V += W[1] * Fb[2];
+  gb.p += Fb[1] + g.U * Fb[3];
+}
+
+FD_HD void euler_flux_rate_adj(const Gas& g, const R W[4], const Grad& q, const R Wq[4], R rt, const R Fb[4], Gas& gb,
+                               R Wb[4], Grad& qb, R Wqb[4], R& rtb) {
+  const R pq = g.th * Wq[0] + rt, pqb = Fb[1] + g.U * Fb[3], Ep = W[3] + g.p;
+  gb.U += Wq[1] * Fb[1] + (Wq[3] + pq) * Fb[3];
+  gb.V += Wq[1] * Fb[2];
+  gb.p += q.u * Fb[3];
+  gb.th += Wq[0] * pqb;
+  Wb[1] += q.u * Fb[1] + q.v * Fb[2];
+  Wb[3] += q.u * Fb[3];
+  qb.u += W[1] * Fb[1] + Ep * Fb[3];
+  qb.v += W[1] * Fb[2];
+  Wqb[0] += g.th * pqb;
+  Wqb[1] += Fb[0] + g.U * Fb[1] + g.V * Fb[2];
+  Wqb[3] += g.U * Fb[3];
+  rtb += pqb;
+}
+
+FD_HD void stress_flux_adj(const Gas& g, R K, R gm1, const Grad& x, const Grad& y, const R Sb[4], Gas& gb, Grad& xb,
+                           Grad& yb) {
+  const R A = 2.0 * x.u - gm1 * (x.u + y.v), B = x.v + y.u, c = 0.5 * K + 2.0;
+  const R s1 = Sb[1] + g.U * Sb[3], s2 = Sb[2] + g.V * Sb[3], s1p = g.p * s1, s2p = g.p * s2;
+  gb.U += g.p * A * Sb[3];
+  gb.V += g.p * B * Sb[3];
+  gb.p += A * s1 + B * s2 + c * x.t * Sb[3];
+  xb.u += (2.0 - gm1) * s1p;
+  yb.v -= gm1 * s1p;
+  xb.v += s2p;
+  yb.u += s2p;
+  xb.t += c * g.p * Sb[3];
+}
+
+// half_moments with sl = 1/sqrt(2 theta): Mb -> U, theta (Mb is used up)
+FD_HD void half_moments_adj(const Gas& g, int sign, R sl, const R M[7], R Mb[7], Gas& gb) {
+  for (int n = 4; n >= 0; --n) {
+    const R b = Mb[n + 2], nb = R(n + 1) * b;
+    Mb[n + 1] += g.U * b;
+    Mb[n] += g.th * nb;
+    gb.U += M[n + 1] * b;
+    gb.th += M[n] * nb;
   }
+  // M1 = U M0 + sign e sl theta/sqrt(pi), M0 = erfc(-sign x)/2, e = exp(-x^2), x = sl U
+  const R x = sl * g.U, sg = R(sign), c = 0.56418958354775628695, b1 = Mb[1];
+  R e, ec;
+  exp_erfc(x, e, ec);
+  const R ce = c * e, m0b = Mb[0] + g.U * b1;
+  const R xb = sg * (ce * m0b - 2.0 * x * ce * (sl * g.th) * b1);
+  const R slb = sg * ce * g.th * b1 + g.U * xb;
+  gb.U += M[0] * b1 + sl * xb;
+  gb.th += sg * ce * sl * b1 - sl * sl * sl * slb;
 }
 
-FD_HD void tab_full_adj(const Maxw<R>& g, R K, const Tab<R>& T, TabB& Tb, MaxwB& gb) {
-  recur_adj(g.U, g.i2l, T.u, Tb.u, gb.U, gb.i2l);
-  recur_adj(g.V, g.i2l, T.v, Tb.v, gb.V, gb.i2l);
-  gb.U += Tb.u[1];
-  gb.V += Tb.v[1];
-  gb.i2l += K * Tb.xi[1] + 2.0 * K * (K + 2.0) * g.i2l * Tb.xi[2];
+// one slope s0, s1, s3 = t/theta (t = q.t/theta) of half_side: the adjoints of
+// t, s0 (its integrated form), s1 and s3
+FD_HD void slope_adj(const Gas& g, R ith, R cU, const Grad& q, R t, R s1, R s3, R tb, R s0b, R s1b, R s3b, Gas& gb,
+                     R& cUb, R& ithb, Grad& qb) {
+  qb.d += s0b;
+  tb -= 0.5 * s0b;
+  s1b -= g.U * s0b;
+  s3b -= cU * s0b + g.U * s1b;
+  cUb -= s3 * s0b;
+  gb.U -= s1 * s0b + s3 * s1b;
+  qb.u += ith * s1b;
+  tb += ith * s3b;
+  qb.t += ith * tb;
+  ithb += q.u * s1b + t * s3b + q.t * tb;
 }
 
-FD_HD void tab_half_adj(const Maxw<R>& g, int sign, const Tab<R>& H, TabB& Hb, TabB& fullb, MaxwB& gb) {
-  const R sl = s_sqrt(g.lam), isl = sl * (2.0 * g.i2l), e = s_exp(-g.lam * g.U * g.U);
-  const R isqpi = 0.56418958354775628695;
-  const R sg = R(sign);
-  recur_adj(g.U, g.i2l, H.u, Hb.u, gb.U, gb.i2l);
-  // H.u1 = U H.u0 + sign e isl / (2 sqrt(pi))
-  const R b1 = Hb.u[1];
-  gb.U += b1 * H.u[0];
-  const R u0b = Hb.u[0] + b1 * g.U;
-  const R eb = sg * 0.5 * isqpi * isl * b1;
-  R islb = sg * 0.5 * e * isqpi * b1;
-  // H.u0 = erfc(z)/2, z = -sign sl U, d erfc/dz = -2 e^{-z^2}/sqrt(pi), e^{-z^2} = e
-  const R zb = -u0b * isqpi * e;
-  R slb = -zb * sg * g.U;
-  gb.U -= zb * sg * sl;
-  // e = exp(-lam U^2)
-  gb.lam -= eb * e * g.U * g.U;
-  gb.U -= 2.0 * eb * e * g.lam * g.U;
-  // isl = 2 sl i2l
-  slb += islb * 2.0 * g.i2l;
-  gb.i2l += islb * 2.0 * sl;
-  gb.lam += slb * 0.5 / sl;   // sl = sqrt(lam)
-  for (int n = 0; n < NT; ++n) fullb.v[n] += Hb.v[n];
-  for (int n = 0; n < 3; ++n) fullb.xi[n] += Hb.xi[n];
+// sb: adjoints of half_side's outputs (M unused; rho and V go to the state)
+FD_HD void half_side_adj(const Gas& g, R N, R ith, const Grad& gx, const Grad& gy, const Grad& gt,
+                         const HalfSide<R>& s, const HalfSide<R>& sb, Gas& gb, Grad& xb, Grad& yb, Grad& tb) {
+  const R cU = 0.5 * g.U * g.U, V = g.V, th = g.th, Nh = s.Nh;
+  const R ta = gx.t * ith, a3 = ta * ith, a1 = s.e2 - 0.5 * V * (gy.t * ith * ith);
+  const R tb_ = gy.t * ith, b3 = tb_ * ith, b1 = gy.u * ith - g.U * b3;
+  const R b0 = gy.d - 0.5 * tb_ - g.U * b1 - cU * b3;
+  const R tA = gt.t * ith, A3 = tA * ith;
+  R cUb = 0.0, ithb = 0.0;
+  const R Nhb = sb.Nh + tA * sb.AX0 + V * tb_ * sb.X0 + ta * sb.X1;
+  gb.rho += sb.rho;
+  gb.V += sb.V + b0 * sb.e0 + b1 * sb.e1 + 0.5 * b3 * sb.e2 + Nh * tb_ * sb.X0 + gy.v * sb.c0;
+  gb.th += gy.v * sb.X0 + (b0 + tb_) * sb.c0 + b1 * sb.c1 + 0.5 * N * Nhb;
+  xb.v += sb.c1;
+  yb.v += sb.e0 + th * sb.X0 + V * sb.c0;
+  tb.v += sb.Ac0;
+  slope_adj(g, ith, cU, gt, tA, s.Ae1, A3, Nh * sb.AX0, sb.Ae0, sb.Ae1, 0.5 * sb.Ae2, gb, cUb, ithb, tb);
+  slope_adj(g, ith, cU, gx, ta, a1, a3, Nh * sb.X1, sb.e1, sb.e2, 0.5 * sb.e3, gb, cUb, ithb, xb);
+  slope_adj(g, ith, cU, gy, tb_, b1, b3, V * Nh * sb.X0 + th * sb.c0 + 0.5 * sb.c2, V * sb.e0 + th * sb.c0,
+            V * sb.e1 + th * sb.c1, 0.5 * V * sb.e2, gb, cUb, ithb, yb);
+  gb.U += g.U * cUb;
+  gb.th -= ith * ith * ithb;
 }
 
-template <int a, int b, int c>
-FD_HD void mm_adj(const Tab<R>& T, R ob, TabB& Tb) {
-  Tb.u[a] += ob * T.v[b] * T.xi[c];
-  Tb.v[b] += ob * T.u[a] * T.xi[c];
-  Tb.xi[c] += ob * T.u[a] * T.v[b];
-}
-
-template <int a, int b, int c>
-FD_HD void mpsi_adj(const Tab<R>& T, const R ob[4], TabB& Tb) {
-  mm_adj<a, b, c>(T, ob[0], Tb);
-  mm_adj<a + 1, b, c>(T, ob[1], Tb);
-  mm_adj<a, b + 1, c>(T, ob[2], Tb);
-  mm_adj<a + 2, b, c>(T, 0.5 * ob[3], Tb);
-  mm_adj<a, b + 2, c>(T, 0.5 * ob[3], Tb);
-  mm_adj<a, b, c + 1>(T, 0.5 * ob[3], Tb);
-}
-
-// o = <s u^a v^b psi> (mslope, factored form): sb += ..., Tb += ...
-// Forward, with h = s3/2, c0 = s0 + h xi[1]:
-//   U(p) = c0 u[p] + s1 u[p+1] + h u[p+2],  V(q) = s2 v[q+1] + h v[q+2],
-//   S(p,q) = v[q] U(p) + u[p] V(q),  U'(a) = s0 u[a] + s1 u[a+1] + h u[a+2],
-//   Sx = xi[1] (v[b] U'(a) + u[a] V(b)) + h xi[2] u[a] v[b],
-//   o = (S(a,b), S(a+1,b), S(a,b+1), (S(a+2,b) + S(a,b+2) + Sx)/2).
-// Reverse: the weights of the S terms give the adjoints of U, V and the
-// tables; those of U, U', V give the adjoints of the slope and the tables.
-template <int a, int b>
-FD_HD void mslope_adj(const Tab<R>& T, const R s[4], const R ob[4], TabB& Tb, R sb[4]) {
-  const R h = 0.5 * s[3], x1 = T.xi[1], x2 = T.xi[2];
-  const R c0 = s[0] + h * x1;
-  R U[3], V[3];                                   // U(a + k), V(b + k)
+// half_flux for the weights k[0..2] = (k3, k4, k5): the adjoints Fb, Wb of the
+// sums it adds to -> those of the side (into sb, M's included) and of k
+FD_HD void half_flux_adj(const HalfSide<R>& s, const R k[3], const R Fb[4], const R Wb[4], HalfSide<R>& sb, R kb[3]) {
+  const R q3 = s.rho * k[0], q4 = s.rho * k[1], q5 = s.rho * k[2];
+  const R e[4] = {q3 + q4 * s.e0 + q5 * s.Ae0, q4 * s.e1 + q5 * s.Ae1, q4 * s.e2 + q5 * s.Ae2, q4 * s.e3};
+  const R X0 = q4 * s.X0 + q5 * s.AX0, X1 = q4 * s.X1;
+  const R c0 = q4 * s.c0 + q5 * s.Ac0, c1 = q4 * s.c1, c2 = q4 * s.c2;
+  const R* M = s.M;
+  const R V = s.V, hV2 = 0.5 * V * V;
+  const R T0 = e[0] * M[0] + e[1] * M[1] + e[2] * M[2] + e[3] * M[3];
+  const R T1 = e[0] * M[1] + e[1] * M[2] + e[2] * M[3] + e[3] * M[4];
+  const R C0 = c0 * M[0] + c1 * M[1] + c2 * M[2], C1 = c0 * M[1] + c1 * M[2] + c2 * M[3];
+  const R E0b = Wb[3], E1b = Fb[3], C0b = Wb[2] + V * Wb[3], C1b = Fb[2] + V * Fb[3];
+  const R Tb[4] = {Wb[0] + V * Wb[2] + hV2 * Wb[3] + s.Nh * E0b,
+                   Wb[1] + Fb[0] + V * Fb[2] + hV2 * Fb[3] + s.Nh * E1b, Fb[1] + 0.5 * E0b, 0.5 * E1b};
+  sb.V += T0 * Wb[2] + (C0 + V * T0) * Wb[3] + T1 * Fb[2] + (C1 + V * T1) * Fb[3];
+  sb.Nh += T0 * E0b + T1 * E1b;
+  const R X0b = M[0] * E0b + M[1] * E1b, X1b = M[1] * E0b + M[2] * E1b;
+  const R c0b = M[0] * C0b + M[1] * C1b, c1b = M[1] * C0b + M[2] * C1b, c2b = M[2] * C0b + M[3] * C1b;
+  sb.M[0] += X0 * E0b + c0 * C0b;
+  sb.M[1] += X1 * E0b + X0 * E1b + c1 * C0b + c0 * C1b;
+  sb.M[2] += X1 * E1b + c2 * C0b + c1 * C1b;
+  sb.M[3] += c2 * C1b;
+  R eb[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    U[k] = c0 * T.u[a + k] + s[1] * T.u[a + k + 1] + h * T.u[a + k + 2];
-    V[k] = s[2] * T.v[b + k + 1] + h * T.v[b + k + 2];
-  }
-  const R Up = s[0] * T.u[a] + s[1] * T.u[a + 1] + h * T.u[a + 2];
-  R Ub[3] = {0.0, 0.0, 0.0}, Vb[3] = {0.0, 0.0, 0.0}, c0b = 0.0, hb = 0.0, Upb = 0.0;
-  // S(a + dp, b + dq) with weight w
-  auto S_adj = [&](int dp, int dq, R w) {
-    Ub[dp] += w * T.v[b + dq];
-    Tb.v[b + dq] += w * U[dp];
-    Tb.u[a + dp] += w * V[dq];
-    Vb[dq] += w * T.u[a + dp];
-  };
-  const R w3 = 0.5 * ob[3];
-  S_adj(0, 0, ob[0]);
-  S_adj(1, 0, ob[1]);
-  S_adj(0, 1, ob[2]);
-  S_adj(2, 0, w3);
-  S_adj(0, 2, w3);
-  // Sx with weight w3
-  {
-    const R inner = T.v[b] * Up + T.u[a] * V[0];
-    Tb.xi[1] += w3 * inner;
-    const R wi = w3 * x1;
-    Upb += wi * T.v[b];
-    Tb.v[b] += wi * Up;
-    Tb.u[a] += wi * V[0];
-    Vb[0] += wi * T.u[a];
-    const R uv = T.u[a] * T.v[b];
-    hb += w3 * x2 * uv;
-    Tb.xi[2] += w3 * h * uv;
-    Tb.u[a] += w3 * h * x2 * T.v[b];
-    Tb.v[b] += w3 * h * x2 * T.u[a];
-  }
-  // U(a + k), V(b + k), U'(a)
+  for (int t = 0; t < 4; ++t)
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    c0b += Ub[k] * T.u[a + k];
-    sb[1] += Ub[k] * T.u[a + k + 1];
-    hb += Ub[k] * T.u[a + k + 2];
-    Tb.u[a + k] += Ub[k] * c0;
-    Tb.u[a + k + 1] += Ub[k] * s[1];
-    Tb.u[a + k + 2] += Ub[k] * h;
-    sb[2] += Vb[k] * T.v[b + k + 1];
-    hb += Vb[k] * T.v[b + k + 2];
-    Tb.v[b + k + 1] += Vb[k] * s[2];
-    Tb.v[b + k + 2] += Vb[k] * h;
-  }
-  sb[0] += Upb * T.u[a];
-  sb[1] += Upb * T.u[a + 1];
-  hb += Upb * T.u[a + 2];
-  Tb.u[a] += Upb * s[0];
-  Tb.u[a + 1] += Upb * s[1];
-  Tb.u[a + 2] += Upb * h;
-  // c0 = s0 + h xi[1], h = s3 / 2
-  sb[0] += c0b;
-  hb += c0b * x1;
-  Tb.xi[1] += c0b * h;
-  sb[3] += 0.5 * hb;
+    for (int m = 0; m < 4; ++m) {
+      eb[m] += M[t + m] * Tb[t];
+      sb.M[t + m] += e[m] * Tb[t];
+    }
+  sb.e0 += q4 * eb[0];
+  sb.e1 += q4 * eb[1];
+  sb.e2 += q4 * eb[2];
+  sb.e3 += q4 * eb[3];
+  sb.X0 += q4 * X0b;
+  sb.X1 += q4 * X1b;
+  sb.c0 += q4 * c0b;
+  sb.c1 += q4 * c1b;
+  sb.c2 += q4 * c2b;
+  sb.Ae0 += q5 * eb[0];
+  sb.Ae1 += q5 * eb[1];
+  sb.Ae2 += q5 * eb[2];
+  sb.AX0 += q5 * X0b;
+  sb.Ac0 += q5 * c0b;
+  const R q4b = s.e0 * eb[0] + s.e1 * eb[1] + s.e2 * eb[2] + s.e3 * eb[3] + s.X0 * X0b + s.X1 * X1b + s.c0 * c0b +
+                s.c1 * c1b + s.c2 * c2b;
+  const R q5b = s.Ae0 * eb[0] + s.Ae1 * eb[1] + s.Ae2 * eb[2] + s.AX0 * X0b + s.Ac0 * c0b;
+  sb.rho += k[0] * eb[0] + k[1] * q4b + k[2] * q5b;
+  kb[0] += s.rho * eb[0];
+  kb[1] += s.rho * q4b;
+  kb[2] += s.rho * q5b;
 }
 
-// s = slope_solve(g, r): sb -> rb, gb (added)
-FD_HD void slope_solve_adj(const Maxw<R>& g, R K, R c4K, const R r[4], const R s[4], const R sb_in[4], MaxwB& gb,
-                           R rb[4]) {
-  const R q = g.U * g.U + g.V * g.V + (K + 2.0) * g.i2l;
-  const R Ah = r[1] - g.U * r[0], Ch = r[2] - g.V * r[0], B = 2.0 * r[3] - q * r[0];
-  const R X = B - 2.0 * g.U * Ah - 2.0 * g.V * Ch;
-  R s1b = sb_in[1], s2b = sb_in[2], s3b = sb_in[3], qb = 0.0, Ahb = 0.0, Chb = 0.0;
-  // s0 = r0 - U s1 - V s2 - s3 q / 2
-  const R s0b = sb_in[0];
-  rb[0] += s0b;
-  gb.U -= s0b * s[1];
-  gb.V -= s0b * s[2];
-  s1b -= s0b * g.U;
-  s2b -= s0b * g.V;
-  s3b -= 0.5 * s0b * q;
-  qb -= 0.5 * s0b * s[3];
-  // s1 = 2 lam Ah - U s3, s2 = 2 lam Ch - V s3
-  gb.lam += 2.0 * (Ah * s1b + Ch * s2b);
-  Ahb += 2.0 * g.lam * s1b;
-  Chb += 2.0 * g.lam * s2b;
-  gb.U -= s[3] * s1b;
-  gb.V -= s[3] * s2b;
-  s3b -= g.U * s1b + g.V * s2b;
-  // s3 = c4K lam^2 X
-  gb.lam += 2.0 * c4K * g.lam * X * s3b;
-  const R Xb = c4K * g.lam * g.lam * s3b;
-  const R Bb = Xb;
-  gb.U -= 2.0 * Ah * Xb;
-  Ahb -= 2.0 * g.U * Xb;
-  gb.V -= 2.0 * Ch * Xb;
-  Chb -= 2.0 * g.V * Xb;
-  // B = 2 r3 - q r0, Ch = r2 - V r0, Ah = r1 - U r0
-  rb[3] += 2.0 * Bb;
-  qb -= r[0] * Bb;
-  rb[0] -= q * Bb;
-  rb[2] += Chb;
-  gb.V -= r[0] * Chb;
-  rb[0] -= g.V * Chb;
-  rb[1] += Ahb;
-  gb.U -= r[0] * Ahb;
-  rb[0] -= g.U * Ahb;
-  // q = U^2 + V^2 + (K + 2) i2l
-  gb.U += 2.0 * g.U * qb;
-  gb.V += 2.0 * g.V * qb;
-  gb.i2l += (K + 2.0) * qb;
+FD_HD void half_side_zero(HalfSide<R>& s) {
+  for (int n = 0; n < 7; ++n) s.M[n] = 0.0;
+  s.rho = s.V = s.Nh = s.e0 = s.e1 = s.e2 = s.e3 = s.X0 = s.X1 = s.c0 = s.c1 = s.c2 = 0.0;
+  s.Ae0 = s.Ae1 = s.Ae2 = s.AX0 = s.Ac0 = 0.0;
 }
 
-// heat flux of the energy flux relative to (U0, V0), x-normal and y-normal:
+// one side of the interface solve: everything that hangs on W (state), D (its
+// normal derivative) and Dt (the tangential one)
+struct SideFwd {
+  Gas g;
+  Grad x, y, t;
+  R sl, Wq[4], rt;
+  HalfSide<R> s;
+};
+FD_HD void side_fwd(const R W[4], const R D[4], const R Dt[4], int sign, R K, R gm1, SideFwd& f) {
+  f.g = gas_state(W, gm1);
+  f.sl = s_rsqrt(2.0 * f.g.th);
+  half_moments(f.g, sign, f.sl, f.s.M);
+  f.x = prim_grad(f.g, gm1, D);
+  f.y = prim_grad(f.g, gm1, Dt);
+  f.t = prim_rate(f.g, gm1, f.x, f.y);
+  half_side(f.g, K + 1.0, 2.0 * f.sl * f.sl, f.x, f.y, f.t, f.s);
+  cons_rate(f.g, 0.5 * K + 1.0, f.t, f.Wq, f.rt);
+}
+// sb: adjoint of the half-space quantities, Wqb of W_t, W0b of the equilibrium
+// state rho (M0, M1, V M0, (M2 + (N theta + V^2) M0)/2) summed over the sides
+FD_HD void side_adj(const R W[4], const R D[4], const R Dt[4], int sign, R K, R gm1, const SideFwd& f, HalfSide<R>& sb,
+                    const R Wqb[4], const R W0b[4], Gas& gb, R Wb[4], R Db[4], R Dtb[4]) {
+  const Gas& g = f.g;
+  const R* M = f.s.M;
+  const R N = K + 1.0, h = N * g.th + g.V * g.V, r0 = g.rho * M[0];
+  gb.rho += M[0] * W0b[0] + M[1] * W0b[1] + g.V * M[0] * W0b[2] + 0.5 * (M[2] + h * M[0]) * W0b[3];
+  gb.V += r0 * (W0b[2] + g.V * W0b[3]);
+  gb.th += 0.5 * N * r0 * W0b[3];
+  sb.M[0] += g.rho * (W0b[0] + g.V * W0b[2] + 0.5 * h * W0b[3]);
+  sb.M[1] += g.rho * W0b[1];
+  sb.M[2] += 0.5 * g.rho * W0b[3];
+  Grad xb = grad_zero(), yb = grad_zero(), tb = grad_zero();
+  half_side_adj(g, N, 2.0 * f.sl * f.sl, f.x, f.y, f.t, f.s, sb, gb, xb, yb, tb);
+  cons_rate_adj(g, 0.5 * K + 1.0, f.t, f.Wq, Wqb, 0.0, gb, tb);
+  prim_rate_adj(g, gm1, f.x, f.y, tb, gb, xb, yb);
+  prim_grad_adj(g, gm1, D, f.x, xb, gb, Db);
+  prim_grad_adj(g, gm1, Dt, f.y, yb, gb, Dtb);
+  half_moments_adj(g, sign, f.sl, M, sb.M, gb);
+  gas_state_adj(W, gm1, g, gb, Wb);
+}
+
+// heat flux of the energy flux relative to (U0, V0), x-normal:
 // adds hb times its partial derivatives to Fb, Wb, U0b, V0b
 FD_HD void heat_flux_x_adj(const R F[4], const R W[4], R U0, R V0, R hb, R Fb[4], R Wb[4], R& U0b, R& V0b) {
   Fb[3] += hb;
@@ -594,18 +637,6 @@ FD_HD void heat_flux_x_adj(const R F[4], const R W[4], R U0, R V0, R hb, R Fb[4]
   U0b += hb * (-W[3] - F[1] + 3.0 * U0 * W[1] + V0 * W[2] - 0.5 * (3.0 * U0 * U0 + V0 * V0) * W[0]);
   V0b += hb * (-F[2] + V0 * W[1] + U0 * W[2] - U0 * V0 * W[0]);
 }
-FD_HD void heat_flux_y_adj(const R G[4], const R W[4], R U0, R V0, R hb, R Gb[4], R Wb[4], R& U0b, R& V0b) {
-  Gb[3] += hb;
-  Wb[3] -= V0 * hb;
-  Gb[2] -= V0 * hb;
-  Gb[1] -= U0 * hb;
-  Wb[2] += (1.5 * V0 * V0 + 0.5 * U0 * U0) * hb;
-  Wb[1] += U0 * V0 * hb;
-  Wb[0] -= 0.5 * V0 * (U0 * U0 + V0 * V0) * hb;
-  V0b += hb * (-W[3] - G[2] + 3.0 * V0 * W[2] + U0 * W[1] - 0.5 * (3.0 * V0 * V0 + U0 * U0) * W[0]);
-  U0b += hb * (-G[1] + U0 * W[2] + V0 * W[1] - U0 * V0 * W[0]);
-}
-
 // time coefficients of the interface distribution (time_coef): the adjoints
 // of cn[6], ct[6], E, e1 -> d/dtau
 FD_HD R time_coef_adj(R tau, R dt, R inv_dt, const R cnb_in[6], const R ctb_in[6], R Eb, R e1b) {
@@ -651,291 +682,115 @@ FD_HD R time_coef_adj(R tau, R dt, R inv_dt, const R cnb_in[6], const R ctb_in[6
 FD_HD void iface_solve_x_adj(const GasK<R>& gas, const R Wl[4], const R Wr[4], const R Wln[4], const R Wrn[4],
                              const R Wt[4], bool want_n, const IfaceOut<R>& ob, R Wlb[4], R Wrb[4], R Wlnb[4],
                              R Wrnb[4], R Wtb[4]) {
-  const R K = gas.K, c4K = gas.c4K, gm1 = gas.gm1;
+  const R K = gas.K, gm1 = gas.gm1, N = K + 1.0, hN = 0.5 * K + 1.0;
   // ---- forward ----
-  const Maxw<R> gl = maxw_from_W(Wl, gm1), gr = maxw_from_W(Wr, gm1);
-  Tab<R> Tl, Tr, Tlp, Trn;
-  tab_full(gl, K, Tl);
-  tab_full(gr, K, Tr);
-  tab_half(gl, +1, Tl, Tlp);
-  tab_half(gr, -1, Tr, Trn);
-  R W0[4], pl0[4], pr0[4];
-  mpsi<0, 0, 0>(Tlp, pl0);
-  mpsi<0, 0, 0>(Trn, pr0);
-  for (int k = 0; k < 4; ++k) W0[k] = gl.rho * pl0[k] + gr.rho * pr0[k];
-  const Maxw<R> g0 = maxw_from_W(W0, gm1);
-  Tab<R> T0;
-  tab_full(g0, K, T0);
-  R ral[4], rbl[4], rar[4], rbr[4], ra0[4], rb0[4];
-  for (int k = 0; k < 4; ++k) {
-    ral[k] = Wln[k] * gl.ir;
-    rbl[k] = Wt[k] * gl.ir;
-    rar[k] = Wrn[k] * gr.ir;
-    rbr[k] = Wt[k] * gr.ir;
-    ra0[k] = 0.5 * (Wln[k] + Wrn[k]) * g0.ir;
-    rb0[k] = Wt[k] * g0.ir;
+  SideFwd l, r;
+  side_fwd(Wl, Wln, Wt, +1, K, gm1, l);
+  side_fwd(Wr, Wrn, Wt, -1, K, gm1, r);
+  R W0[4], x1[4], W0q[4], rt0, FE[4], FQ[4], FS[4];
+  {
+    const R ml = l.g.rho * l.s.M[0], mr = r.g.rho * r.s.M[0];
+    W0[0] = ml + mr;
+    W0[1] = l.g.rho * l.s.M[1] + r.g.rho * r.s.M[1];
+    W0[2] = l.g.V * ml + r.g.V * mr;
+    W0[3] = 0.5 * (l.g.rho * (l.s.M[2] + N * l.g.th * l.s.M[0] + l.g.V * l.g.V * l.s.M[0]) +
+                   r.g.rho * (r.s.M[2] + N * r.g.th * r.s.M[0] + r.g.V * r.g.V * r.s.M[0]));
   }
-  R al[4], bl[4], ar[4], br[4], a0[4], b0[4];
-  slope_solve(gl, K, c4K, ral, al);
-  slope_solve(gl, K, c4K, rbl, bl);
-  slope_solve(gr, K, c4K, rar, ar);
-  slope_solve(gr, K, c4K, rbr, br);
-  slope_solve(g0, K, c4K, ra0, a0);
-  slope_solve(g0, K, c4K, rb0, b0);
-  R rl[4], rr[4], r0[4], Al[4], Ar[4], A0[4], x1[4], x2[4];
-  mslope<1, 0>(Tl, al, x1);
-  mslope<0, 1>(Tl, bl, x2);
-  for (int k = 0; k < 4; ++k) rl[k] = -(x1[k] + x2[k]);
-  slope_solve(gl, K, c4K, rl, Al);
-  mslope<1, 0>(Tr, ar, x1);
-  mslope<0, 1>(Tr, br, x2);
-  for (int k = 0; k < 4; ++k) rr[k] = -(x1[k] + x2[k]);
-  slope_solve(gr, K, c4K, rr, Ar);
-  mslope<1, 0>(T0, a0, x1);
-  mslope<0, 1>(T0, b0, x2);
-  for (int k = 0; k < 4; ++k) r0[k] = -(x1[k] + x2[k]);
-  slope_solve(g0, K, c4K, r0, A0);
-  const R ip0 = 2.0 * g0.lam * g0.ir;
-  const R dp = gl.p - gr.p, sp = gl.p + gr.p;
+  const Gas g0 = gas_state(W0, gm1);
+  for (int k = 0; k < 4; ++k) x1[k] = 0.5 * (Wln[k] + Wrn[k]);
+  const Grad gx = prim_grad(g0, gm1, x1), gy = prim_grad(g0, gm1, Wt), gt = prim_rate(g0, gm1, gx, gy);
+  cons_rate(g0, hN, gt, W0q, rt0);
+  euler_flux(g0, W0, FE);
+  euler_flux_rate(g0, W0, gt, W0q, rt0, FQ);
+  stress_flux(g0, K, gm1, gx, gy, FS);
+  const R ip0 = 1.0 / g0.p, dp = l.g.p - r.g.p, sp = l.g.p + r.g.p;
   const R tau = gas.c1 * gas.dt + gas.mu * ip0 + gas.c2 * gas.dt * s_abs(dp) / sp;
   const TimeCoef<R> tc = time_coef(tau, gas.dt, gas.inv_dt);
-  // the six basis terms' flux (mf) and W (mw) moment vectors
-  R mf[6][4], mw[6][4], y1[4], y2[4];
-  mpsi<1, 0, 0>(T0, mf[0]);
-  mpsi<0, 0, 0>(T0, mw[0]);
-  for (int k = 0; k < 4; ++k) { mf[0][k] *= g0.rho; mw[0][k] *= g0.rho; }
-  mslope<2, 0>(T0, a0, x1);
-  mslope<1, 1>(T0, b0, x2);
-  for (int k = 0; k < 4; ++k) { mf[1][k] = g0.rho * (x1[k] + x2[k]); mw[1][k] = -g0.rho * r0[k]; }
-  mslope<1, 0>(T0, A0, x1);
-  for (int k = 0; k < 4; ++k) { mf[2][k] = g0.rho * x1[k]; mw[2][k] = g0.rho * r0[k]; }
-  mpsi<1, 0, 0>(Tlp, x1);
-  mpsi<1, 0, 0>(Trn, x2);
-  for (int k = 0; k < 4; ++k) { mf[3][k] = gl.rho * x1[k] + gr.rho * x2[k]; mw[3][k] = W0[k]; }
-  mslope<2, 0>(Tlp, al, x1);
-  mslope<1, 1>(Tlp, bl, x2);
-  mslope<2, 0>(Trn, ar, y1);
-  mslope<1, 1>(Trn, br, y2);
-  for (int k = 0; k < 4; ++k) mf[4][k] = gl.rho * (x1[k] + x2[k]) + gr.rho * (y1[k] + y2[k]);
-  mslope<1, 0>(Tlp, al, x1);
-  mslope<0, 1>(Tlp, bl, x2);
-  mslope<1, 0>(Trn, ar, y1);
-  mslope<0, 1>(Trn, br, y2);
-  for (int k = 0; k < 4; ++k) mw[4][k] = gl.rho * (x1[k] + x2[k]) + gr.rho * (y1[k] + y2[k]);
-  mslope<1, 0>(Tlp, Al, x1);
-  mslope<1, 0>(Trn, Ar, y1);
-  mslope<0, 0>(Tlp, Al, x2);
-  mslope<0, 0>(Trn, Ar, y2);
-  for (int k = 0; k < 4; ++k) { mf[5][k] = gl.rho * x1[k] + gr.rho * y1[k]; mw[5][k] = gl.rho * x2[k] + gr.rho * y2[k]; }
-  R F[4], Ftt[4], We[4], Wet[4];
-  for (int k = 0; k < 4; ++k) {
-    F[k] = Ftt[k] = We[k] = Wet[k] = 0.0;
-    for (int kk = 0; kk < 6; ++kk) {
-      F[k] += tc.cn[kk] * mf[kk][k];
-      Ftt[k] += tc.ct[kk] * mf[kk][k];
-      We[k] += tc.cn[kk] * mw[kk][k];
-      Wet[k] += tc.ct[kk] * mw[kk][k];
-    }
-  }
   const R E = tc.E, e1 = tc.e1;
 
   // ---- reverse ----
-  MaxwB glb = maxw_zero(), grb = maxw_zero(), g0b = maxw_zero();
-  TabB Tlb = tab_zero(), Trb = tab_zero(), Tlpb = tab_zero(), Trnb = tab_zero(), T0b = tab_zero();
-  R Fb[4], Fttb[4], Web[4], Wetb[4], rlb[4], rrb[4], r0b[4], Eb = 0.0, e1b = 0.0;
-  for (int k = 0; k < 4; ++k) {
-    rlb[k] = rrb[k] = r0b[k] = 0.0;
-    // o.Ft = Ftt; o.Wlt = e1 Wet + E rho_l rl; o.Wrt = e1 Wet + E rho_r rr
-    Fttb[k] = ob.Ft[k];
-    Wetb[k] = e1 * (ob.Wlt[k] + ob.Wrt[k]);
-    e1b += Wet[k] * (ob.Wlt[k] + ob.Wrt[k]);
-    Eb += gl.rho * rl[k] * ob.Wlt[k] + gr.rho * rr[k] * ob.Wrt[k];
-    glb.rho += E * rl[k] * ob.Wlt[k];
-    grb.rho += E * rr[k] * ob.Wrt[k];
-    rlb[k] += E * gl.rho * ob.Wlt[k];
-    rrb[k] += E * gr.rho * ob.Wrt[k];
-    Fb[k] = Web[k] = 0.0;
-    if (want_n) {
-      // o.F = F; o.Wl = e1 We + E Wl; o.Wr = e1 We + E Wr
-      Fb[k] = ob.F[k];
-      Web[k] = e1 * (ob.Wl[k] + ob.Wr[k]);
-      e1b += We[k] * (ob.Wl[k] + ob.Wr[k]);
-      Eb += Wl[k] * ob.Wl[k] + Wr[k] * ob.Wr[k];
-      Wlb[k] += E * ob.Wl[k];
-      Wrb[k] += E * ob.Wr[k];
-    }
-  }
-  // Prandtl correction F3 += prfix q(F, We), Ftt3 likewise (F, Ftt above are
-  // the sums before the correction; only the energy components change)
-  heat_flux_x_adj(F, We, g0.U, g0.V, gas.prfix * Fb[3], Fb, Web, g0b.U, g0b.V);
-  heat_flux_x_adj(Ftt, Wet, g0.U, g0.V, gas.prfix * Fttb[3], Fttb, Wetb, g0b.U, g0b.V);
-  // accumulation F = sum cn mf, ... -> adjoints of mf, mw and of the coefficients
-  R cnb[6], ctb[6], mfb[6][4], mwb[6][4];
-  for (int kk = 0; kk < 6; ++kk) {
-    cnb[kk] = ctb[kk] = 0.0;
+  HalfSide<R> lb, rb;
+  half_side_zero(lb);
+  half_side_zero(rb);
+  Gas g0b = gas_zero();
+  R W0b[4] = {0.0, 0.0, 0.0, 0.0}, W0qb[4] = {0.0, 0.0, 0.0, 0.0};
+  R FEb[4] = {0.0, 0.0, 0.0, 0.0}, FQb[4] = {0.0, 0.0, 0.0, 0.0}, FSb[4] = {0.0, 0.0, 0.0, 0.0};
+  R cnb[6] = {0, 0, 0, 0, 0, 0}, ctb[6] = {0, 0, 0, 0, 0, 0}, Eb = 0.0, e1b = 0.0, Wlqb[4], Wrqb[4];
+  // set 0: the values (cn), set 1: the time derivatives (ct)
+  for (int set = want_n ? 0 : 1; set < 2; ++set) {
+    const R* c = set ? tc.ct : tc.cn;
+    R* cb = set ? ctb : cnb;
+    const R kq = c[2] - c[1];
+    R F[4], We[4], Fb[4], Web[4];
     for (int k = 0; k < 4; ++k) {
-      mfb[kk][k] = tc.cn[kk] * Fb[k] + tc.ct[kk] * Fttb[k];
-      mwb[kk][k] = tc.cn[kk] * Web[k] + tc.ct[kk] * Wetb[k];
-      cnb[kk] += mf[kk][k] * Fb[k] + mw[kk][k] * Web[k];
-      ctb[kk] += mf[kk][k] * Fttb[k] + mw[kk][k] * Wetb[k];
+      F[k] = c[0] * FE[k] + kq * FQ[k] + c[1] * FS[k];
+      We[k] = c[0] * W0[k] + kq * W0q[k];
     }
-  }
-  R W0b[4] = {0.0, 0.0, 0.0, 0.0};
-  R alb[4] = {0, 0, 0, 0}, blb[4] = {0, 0, 0, 0}, arb[4] = {0, 0, 0, 0}, brb[4] = {0, 0, 0, 0};
-  R a0b[4] = {0, 0, 0, 0}, b0b[4] = {0, 0, 0, 0}, Alb[4] = {0, 0, 0, 0}, Arb[4] = {0, 0, 0, 0};
-  R A0b[4] = {0, 0, 0, 0};
-  R t[4];
-  // term 0: rho0 <u psi>_0, rho0 <psi>_0
-  mpsi<1, 0, 0>(T0, x1);
-  mpsi<0, 0, 0>(T0, x2);
-  for (int k = 0; k < 4; ++k) g0b.rho += x1[k] * mfb[0][k] + x2[k] * mwb[0][k];
-  for (int k = 0; k < 4; ++k) t[k] = g0.rho * mfb[0][k];
-  mpsi_adj<1, 0, 0>(T0, t, T0b);
-  for (int k = 0; k < 4; ++k) t[k] = g0.rho * mwb[0][k];
-  mpsi_adj<0, 0, 0>(T0, t, T0b);
-  // term 1: rho0 (<a0 u u psi> + <b0 u v psi>), -rho0 r0
-  mslope<2, 0>(T0, a0, x1);
-  mslope<1, 1>(T0, b0, x2);
-  for (int k = 0; k < 4; ++k) {
-    g0b.rho += (x1[k] + x2[k]) * mfb[1][k] - r0[k] * mwb[1][k];
-    r0b[k] -= g0.rho * mwb[1][k];
-    t[k] = g0.rho * mfb[1][k];
-  }
-  mslope_adj<2, 0>(T0, a0, t, T0b, a0b);
-  mslope_adj<1, 1>(T0, b0, t, T0b, b0b);
-  // term 2: rho0 <A0 u psi>, rho0 r0
-  mslope<1, 0>(T0, A0, x1);
-  for (int k = 0; k < 4; ++k) {
-    g0b.rho += x1[k] * mfb[2][k] + r0[k] * mwb[2][k];
-    r0b[k] += g0.rho * mwb[2][k];
-    t[k] = g0.rho * mfb[2][k];
-  }
-  mslope_adj<1, 0>(T0, A0, t, T0b, A0b);
-  // term 3: rho_l <u psi>_{u>0} + rho_r <u psi>_{u<0}, W0
-  mpsi<1, 0, 0>(Tlp, x1);
-  mpsi<1, 0, 0>(Trn, x2);
-  for (int k = 0; k < 4; ++k) {
-    glb.rho += x1[k] * mfb[3][k];
-    grb.rho += x2[k] * mfb[3][k];
-    W0b[k] += mwb[3][k];
-  }
-  for (int k = 0; k < 4; ++k) t[k] = gl.rho * mfb[3][k];
-  mpsi_adj<1, 0, 0>(Tlp, t, Tlpb);
-  for (int k = 0; k < 4; ++k) t[k] = gr.rho * mfb[3][k];
-  mpsi_adj<1, 0, 0>(Trn, t, Trnb);
-  // term 4: the one-sided (a u + b v) terms
-  {
-    R f1[4], f2[4], f3[4], f4[4], w1[4], w2[4], w3[4], w4[4];
-    mslope<2, 0>(Tlp, al, f1);
-    mslope<1, 1>(Tlp, bl, f2);
-    mslope<2, 0>(Trn, ar, f3);
-    mslope<1, 1>(Trn, br, f4);
-    mslope<1, 0>(Tlp, al, w1);
-    mslope<0, 1>(Tlp, bl, w2);
-    mslope<1, 0>(Trn, ar, w3);
-    mslope<0, 1>(Trn, br, w4);
+    half_flux(l.s, c[3], c[4], c[5], F, We);
+    half_flux(r.s, c[3], c[4], c[5], F, We);
     for (int k = 0; k < 4; ++k) {
-      glb.rho += (f1[k] + f2[k]) * mfb[4][k] + (w1[k] + w2[k]) * mwb[4][k];
-      grb.rho += (f3[k] + f4[k]) * mfb[4][k] + (w3[k] + w4[k]) * mwb[4][k];
+      // o.F = F, o.W(l,r) = e1 We + E W(l,r); for set 1 o.Ft, o.W(l,r)t with W(l,r)_t
+      const R ol = set ? ob.Wlt[k] : ob.Wl[k], orr = set ? ob.Wrt[k] : ob.Wr[k];
+      Fb[k] = set ? ob.Ft[k] : ob.F[k];
+      Web[k] = e1 * (ol + orr);
+      e1b += We[k] * (ol + orr);
+      if (set) {
+        Eb += l.Wq[k] * ol + r.Wq[k] * orr;
+        Wlqb[k] = E * ol;
+        Wrqb[k] = E * orr;
+      } else {
+        Eb += Wl[k] * ol + Wr[k] * orr;
+        Wlb[k] += E * ol;
+        Wrb[k] += E * orr;
+      }
     }
-    for (int k = 0; k < 4; ++k) t[k] = gl.rho * mfb[4][k];
-    mslope_adj<2, 0>(Tlp, al, t, Tlpb, alb);
-    mslope_adj<1, 1>(Tlp, bl, t, Tlpb, blb);
-    for (int k = 0; k < 4; ++k) t[k] = gr.rho * mfb[4][k];
-    mslope_adj<2, 0>(Trn, ar, t, Trnb, arb);
-    mslope_adj<1, 1>(Trn, br, t, Trnb, brb);
-    for (int k = 0; k < 4; ++k) t[k] = gl.rho * mwb[4][k];
-    mslope_adj<1, 0>(Tlp, al, t, Tlpb, alb);
-    mslope_adj<0, 1>(Tlp, bl, t, Tlpb, blb);
-    for (int k = 0; k < 4; ++k) t[k] = gr.rho * mwb[4][k];
-    mslope_adj<1, 0>(Trn, ar, t, Trnb, arb);
-    mslope_adj<0, 1>(Trn, br, t, Trnb, brb);
-  }
-  // term 5: the one-sided A terms
-  {
-    R f1[4], f3[4], w1[4], w3[4];
-    mslope<1, 0>(Tlp, Al, f1);
-    mslope<1, 0>(Trn, Ar, f3);
-    mslope<0, 0>(Tlp, Al, w1);
-    mslope<0, 0>(Trn, Ar, w3);
+    // Prandtl correction F3 += prfix q(F, We) (F above is the sum before it)
+    if (gas.prfix != 0.0) heat_flux_x_adj(F, We, g0.U, g0.V, gas.prfix * Fb[3], Fb, Web, g0b.U, g0b.V);
+    R kqb = 0.0;
     for (int k = 0; k < 4; ++k) {
-      glb.rho += f1[k] * mfb[5][k] + w1[k] * mwb[5][k];
-      grb.rho += f3[k] * mfb[5][k] + w3[k] * mwb[5][k];
+      cb[0] += FE[k] * Fb[k] + W0[k] * Web[k];
+      cb[1] += FS[k] * Fb[k];
+      kqb += FQ[k] * Fb[k] + W0q[k] * Web[k];
+      FEb[k] += c[0] * Fb[k];
+      FQb[k] += kq * Fb[k];
+      FSb[k] += c[1] * Fb[k];
+      W0b[k] += c[0] * Web[k];
+      W0qb[k] += kq * Web[k];
     }
-    for (int k = 0; k < 4; ++k) t[k] = gl.rho * mfb[5][k];
-    mslope_adj<1, 0>(Tlp, Al, t, Tlpb, Alb);
-    for (int k = 0; k < 4; ++k) t[k] = gr.rho * mfb[5][k];
-    mslope_adj<1, 0>(Trn, Ar, t, Trnb, Arb);
-    for (int k = 0; k < 4; ++k) t[k] = gl.rho * mwb[5][k];
-    mslope_adj<0, 0>(Tlp, Al, t, Tlpb, Alb);
-    for (int k = 0; k < 4; ++k) t[k] = gr.rho * mwb[5][k];
-    mslope_adj<0, 0>(Trn, Ar, t, Trnb, Arb);
+    cb[1] -= kqb;
+    cb[2] += kqb;
+    half_flux_adj(l.s, c + 3, Fb, Web, lb, cb + 3);
+    half_flux_adj(r.s, c + 3, Fb, Web, rb, cb + 3);
   }
   // time coefficients and the collision time
+  Gas glb = gas_zero(), grb = gas_zero();
   {
     const R taub = time_coef_adj(tau, gas.dt, gas.inv_dt, cnb, ctb, Eb, e1b);
-    const R ip0b = gas.mu * taub;
-    g0b.lam += 2.0 * g0.ir * ip0b;
-    g0b.ir += 2.0 * g0.lam * ip0b;
+    g0b.p -= gas.mu * ip0 * ip0 * taub;
     // |dp| / sp with d|x|/dx = sign(x), 0 at x = 0
-    const R s = sgn0(dp), adp = s_abs(dp);
-    const R c = gas.c2 * gas.dt * taub / (sp * sp);
+    const R s = sgn0(dp), adp = s_abs(dp), c = gas.c2 * gas.dt * taub / (sp * sp);
     glb.p += c * (s * sp - adp);
     grb.p += c * (-s * sp - adp);
   }
-  // time slopes A = slope_solve(g, -<(a u + b v) psi>)
-  slope_solve_adj(g0, K, c4K, r0, A0, A0b, g0b, r0b);
-  for (int k = 0; k < 4; ++k) t[k] = -r0b[k];
-  mslope_adj<1, 0>(T0, a0, t, T0b, a0b);
-  mslope_adj<0, 1>(T0, b0, t, T0b, b0b);
-  slope_solve_adj(gr, K, c4K, rr, Ar, Arb, grb, rrb);
-  for (int k = 0; k < 4; ++k) t[k] = -rrb[k];
-  mslope_adj<1, 0>(Tr, ar, t, Trb, arb);
-  mslope_adj<0, 1>(Tr, br, t, Trb, brb);
-  slope_solve_adj(gl, K, c4K, rl, Al, Alb, glb, rlb);
-  for (int k = 0; k < 4; ++k) t[k] = -rlb[k];
-  mslope_adj<1, 0>(Tl, al, t, Tlb, alb);
-  mslope_adj<0, 1>(Tl, bl, t, Tlb, blb);
-  // spatial slopes from r = dW / rho
+  // equilibrium state: stress, Euler flux and its time derivative, gradients
   {
-    R rb_[4];
-    for (int k = 0; k < 4; ++k) rb_[k] = 0.0;
-    slope_solve_adj(g0, K, c4K, rb0, b0, b0b, g0b, rb_);
-    for (int k = 0; k < 4; ++k) { Wtb[k] += rb_[k] * g0.ir; g0b.ir += rb_[k] * Wt[k]; rb_[k] = 0.0; }
-    slope_solve_adj(g0, K, c4K, ra0, a0, a0b, g0b, rb_);
+    Grad xb = grad_zero(), yb = grad_zero(), tb = grad_zero();
+    R rtb = 0.0, x1b[4] = {0.0, 0.0, 0.0, 0.0};
+    stress_flux_adj(g0, K, gm1, gx, gy, FSb, g0b, xb, yb);
+    euler_flux_rate_adj(g0, W0, gt, W0q, rt0, FQb, g0b, W0b, tb, W0qb, rtb);
+    euler_flux_adj(g0, W0, FEb, g0b, W0b);
+    cons_rate_adj(g0, hN, gt, W0q, W0qb, rtb, g0b, tb);
+    prim_rate_adj(g0, gm1, gx, gy, tb, g0b, xb, yb);
+    prim_grad_adj(g0, gm1, x1, gx, xb, g0b, x1b);
+    prim_grad_adj(g0, gm1, Wt, gy, yb, g0b, Wtb);
+    gas_state_adj(W0, gm1, g0, g0b, W0b);
     for (int k = 0; k < 4; ++k) {
-      Wlnb[k] += 0.5 * rb_[k] * g0.ir;
-      Wrnb[k] += 0.5 * rb_[k] * g0.ir;
-      g0b.ir += rb_[k] * 0.5 * (Wln[k] + Wrn[k]);
-      rb_[k] = 0.0;
+      Wlnb[k] += 0.5 * x1b[k];
+      Wrnb[k] += 0.5 * x1b[k];
     }
-    slope_solve_adj(gr, K, c4K, rbr, br, brb, grb, rb_);
-    for (int k = 0; k < 4; ++k) { Wtb[k] += rb_[k] * gr.ir; grb.ir += rb_[k] * Wt[k]; rb_[k] = 0.0; }
-    slope_solve_adj(gr, K, c4K, rar, ar, arb, grb, rb_);
-    for (int k = 0; k < 4; ++k) { Wrnb[k] += rb_[k] * gr.ir; grb.ir += rb_[k] * Wrn[k]; rb_[k] = 0.0; }
-    slope_solve_adj(gl, K, c4K, rbl, bl, blb, glb, rb_);
-    for (int k = 0; k < 4; ++k) { Wtb[k] += rb_[k] * gl.ir; glb.ir += rb_[k] * Wt[k]; rb_[k] = 0.0; }
-    slope_solve_adj(gl, K, c4K, ral, al, alb, glb, rb_);
-    for (int k = 0; k < 4; ++k) { Wlnb[k] += rb_[k] * gl.ir; glb.ir += rb_[k] * Wln[k]; }
   }
-  // equilibrium state W0 = rho_l <psi>_{u>0} + rho_r <psi>_{u<0} and its Maxwellian
-  tab_full_adj(g0, K, T0, T0b, g0b);
-  maxw_from_W_adj(W0, gm1, g0, g0b, W0b);
-  for (int k = 0; k < 4; ++k) {
-    glb.rho += pl0[k] * W0b[k];
-    grb.rho += pr0[k] * W0b[k];
-    t[k] = gl.rho * W0b[k];
-  }
-  mpsi_adj<0, 0, 0>(Tlp, t, Tlpb);
-  for (int k = 0; k < 4; ++k) t[k] = gr.rho * W0b[k];
-  mpsi_adj<0, 0, 0>(Trn, t, Trnb);
-  // one-sided tables and the Maxwellians of the two sides
-  tab_half_adj(gl, +1, Tlp, Tlpb, Tlb, glb);
-  tab_half_adj(gr, -1, Trn, Trnb, Trb, grb);
-  tab_full_adj(gl, K, Tl, Tlb, glb);
-  tab_full_adj(gr, K, Tr, Trb, grb);
-  maxw_from_W_adj(Wl, gm1, gl, glb, Wlb);
-  maxw_from_W_adj(Wr, gm1, gr, grb, Wrb);
+  side_adj(Wl, Wln, Wt, +1, K, gm1, l, lb, Wlqb, W0b, glb, Wlb, Wlnb, Wtb);
+  side_adj(Wr, Wrn, Wt, -1, K, gm1, r, rb, Wrqb, W0b, grb, Wrb, Wrnb, Wtb);
 }
 
 // any normal: the x <-> y transposition of iface_solve, transposed
@@ -961,94 +816,71 @@ FD_HD void iface_solve_adj(const GasK<R>& gas, int normal, const R Wl[4], const 
 // ---------------------------------------------------------------------------
 // nodal flux (Sec. 2.1): adjoints of F, G, F_t, G_t -> of W, W_x, W_y (added)
 // ---------------------------------------------------------------------------
+// the x <-> y transposition of a state and of a gradient (its own inverse)
+FD_HD Gas swap_gas(const Gas& g) { return Gas{g.rho, g.ir, g.V, g.U, g.p, g.th, g.en}; }
+FD_HD Grad swap_grad(const Grad& q) { return Grad{q.d, q.v, q.u, q.t}; }
+
+// x-flux and its time derivative: Fb, Ftb -> the adjoints of the state, W, the
+// gradients, W_t and rho theta_t
+FD_HD void nodal_dir_adj(R K, R gm1, R prfix, R tau, const Gas& g, const R W[4], const Grad& x, const Grad& y,
+                         const Grad& t, const R Wq[4], R rt, const R Fb[4], const R Ftb[4], Gas& gb, R Wb[4], Grad& xb,
+                         Grad& yb, Grad& tb, R Wqb[4], R& rtb, R& taub) {
+  const R c = prfix * (0.5 * K + 2.0);
+  // Ft = Euler rate, Ft3 += c p U_t
+  euler_flux_rate_adj(g, W, t, Wq, rt, Ftb, gb, Wb, tb, Wqb, rtb);
+  gb.p += c * t.u * Ftb[3];
+  tb.u += c * g.p * Ftb[3];
+  // F = Euler - tau S, S3 += c p theta_x
+  euler_flux_adj(g, W, Fb, gb, Wb);
+  R S[4], Sb[4];
+  stress_flux(g, K, gm1, x, y, S);
+  S[3] += c * g.p * x.t;
+  for (int k = 0; k < 4; ++k) {
+    taub -= S[k] * Fb[k];
+    Sb[k] = -tau * Fb[k];
+  }
+  stress_flux_adj(g, K, gm1, x, y, Sb, gb, xb, yb);
+  gb.p += c * x.t * Sb[3];
+  xb.t += c * g.p * Sb[3];
+}
+
 FD_HD void nodal_flux_adj(const GasK<R>& gas, const R W[4], const R Wx[4], const R Wy[4], const R Fb_in[4],
                           const R Gb_in[4], const R Ftb_in[4], const R Gtb_in[4], R Wb[4], R Wxb[4], R Wyb[4]) {
-  const R K = gas.K, c4K = gas.c4K;
-  const Maxw<R> g = maxw_from_W(W, gas.gm1);
-  Tab<R> T;
-  tab_full(g, K, T);
-  R rx[4], ry[4], a[4], b[4], r[4], A[4], x1[4], x2[4], Wt[4];
-  for (int k = 0; k < 4; ++k) { rx[k] = Wx[k] * g.ir; ry[k] = Wy[k] * g.ir; }
-  slope_solve(g, K, c4K, rx, a);
-  slope_solve(g, K, c4K, ry, b);
-  mslope<1, 0>(T, a, x1);
-  mslope<0, 1>(T, b, x2);
-  for (int k = 0; k < 4; ++k) r[k] = -(x1[k] + x2[k]);
-  slope_solve(g, K, c4K, r, A);
-  for (int k = 0; k < 4; ++k) Wt[k] = g.rho * r[k];
-  const R tau = gas.c1_r * gas.dt_r + gas.mu_r * (2.0 * g.lam * g.ir);
-  R e0x[4], eax[4], ebx[4], eAx[4], e0y[4], eay[4], eby[4], eAy[4];
-  mpsi<1, 0, 0>(T, e0x);
-  mslope<2, 0>(T, a, eax);
-  mslope<1, 1>(T, b, ebx);
-  mslope<1, 0>(T, A, eAx);
-  mpsi<0, 1, 0>(T, e0y);
-  mslope<1, 1>(T, a, eay);
-  mslope<0, 2>(T, b, eby);
-  mslope<0, 1>(T, A, eAy);
-  R F[4], G[4], Ft[4], Gt[4];   // before the Prandtl correction
+  const R K = gas.K, gm1 = gas.gm1, hN = 0.5 * K + 1.0;
+  const Gas g = gas_state(W, gm1);
+  const Grad x = prim_grad(g, gm1, Wx), y = prim_grad(g, gm1, Wy), t = prim_rate(g, gm1, x, y);
+  R Wq[4], rt;
+  cons_rate(g, hN, t, Wq, rt);
+  const R ip = 1.0 / g.p, tau = gas.c1_r * gas.dt_r + gas.mu_r * ip;
+  Gas gb = gas_zero(), sgb = gas_zero();
+  Grad xb = grad_zero(), yb = grad_zero(), tb = grad_zero(), sxb = grad_zero(), syb = grad_zero(), stb = grad_zero();
+  R Wqb[4] = {0, 0, 0, 0}, sWqb[4] = {0, 0, 0, 0}, sWb[4] = {0, 0, 0, 0}, rtb = 0.0, taub = 0.0;
+  nodal_dir_adj(K, gm1, gas.prfix, tau, g, W, x, y, t, Wq, rt, Fb_in, Ftb_in, gb, Wb, xb, yb, tb, Wqb, rtb, taub);
+  const R sW[4] = {W[0], W[2], W[1], W[3]}, sWq[4] = {Wq[0], Wq[2], Wq[1], Wq[3]};
+  const R sG[4] = {Gb_in[0], Gb_in[2], Gb_in[1], Gb_in[3]}, sGt[4] = {Gtb_in[0], Gtb_in[2], Gtb_in[1], Gtb_in[3]};
+  nodal_dir_adj(K, gm1, gas.prfix, tau, swap_gas(g), sW, swap_grad(y), swap_grad(x), swap_grad(t), sWq, rt, sG, sGt,
+                sgb, sWb, syb, sxb, stb, sWqb, rtb, taub);
+  const int sw[4] = {0, 2, 1, 3};
   for (int k = 0; k < 4; ++k) {
-    F[k] = g.rho * (e0x[k] - tau * (eax[k] + ebx[k] + eAx[k]));
-    Ft[k] = g.rho * eAx[k];
-    G[k] = g.rho * (e0y[k] - tau * (eay[k] + eby[k] + eAy[k]));
-    Gt[k] = g.rho * eAy[k];
+    Wb[k] += sWb[sw[k]];
+    Wqb[k] += sWqb[sw[k]];
   }
-  // ---- reverse ----
-  MaxwB gb = maxw_zero();
-  TabB Tb = tab_zero();
-  R Fb[4], Gb[4], Ftb[4], Gtb[4], Wtb[4] = {0, 0, 0, 0};
-  for (int k = 0; k < 4; ++k) { Fb[k] = Fb_in[k]; Gb[k] = Gb_in[k]; Ftb[k] = Ftb_in[k]; Gtb[k] = Gtb_in[k]; }
-  heat_flux_x_adj(F, W, g.U, g.V, gas.prfix * Fb[3], Fb, Wb, gb.U, gb.V);
-  heat_flux_y_adj(G, W, g.U, g.V, gas.prfix * Gb[3], Gb, Wb, gb.U, gb.V);
-  heat_flux_x_adj(Ft, Wt, g.U, g.V, gas.prfix * Ftb[3], Ftb, Wtb, gb.U, gb.V);
-  heat_flux_y_adj(Gt, Wt, g.U, g.V, gas.prfix * Gtb[3], Gtb, Wtb, gb.U, gb.V);
-  R e0b[4], sb[4], eAb[4], taub = 0.0, ab[4] = {0, 0, 0, 0}, bb[4] = {0, 0, 0, 0}, Ab[4] = {0, 0, 0, 0};
-  // x-flux: F = rho (e0 - tau (ea + eb + eA)), Ft = rho eA
-  for (int k = 0; k < 4; ++k) {
-    gb.rho += (e0x[k] - tau * (eax[k] + ebx[k] + eAx[k])) * Fb[k] + eAx[k] * Ftb[k];
-    taub -= g.rho * (eax[k] + ebx[k] + eAx[k]) * Fb[k];
-    e0b[k] = g.rho * Fb[k];
-    sb[k] = -g.rho * tau * Fb[k];
-    eAb[k] = sb[k] + g.rho * Ftb[k];
-  }
-  mpsi_adj<1, 0, 0>(T, e0b, Tb);
-  mslope_adj<2, 0>(T, a, sb, Tb, ab);
-  mslope_adj<1, 1>(T, b, sb, Tb, bb);
-  mslope_adj<1, 0>(T, A, eAb, Tb, Ab);
-  for (int k = 0; k < 4; ++k) {
-    gb.rho += (e0y[k] - tau * (eay[k] + eby[k] + eAy[k])) * Gb[k] + eAy[k] * Gtb[k];
-    taub -= g.rho * (eay[k] + eby[k] + eAy[k]) * Gb[k];
-    e0b[k] = g.rho * Gb[k];
-    sb[k] = -g.rho * tau * Gb[k];
-    eAb[k] = sb[k] + g.rho * Gtb[k];
-  }
-  mpsi_adj<0, 1, 0>(T, e0b, Tb);
-  mslope_adj<1, 1>(T, a, sb, Tb, ab);
-  mslope_adj<0, 2>(T, b, sb, Tb, bb);
-  mslope_adj<0, 1>(T, A, eAb, Tb, Ab);
-  // tau = c1 dt + mu (2 lam ir)
-  gb.lam += gas.mu_r * 2.0 * g.ir * taub;
-  gb.ir += gas.mu_r * 2.0 * g.lam * taub;
-  // Wt = rho r, A = slope_solve(g, r), r = -(<a u psi> + <b v psi>)
-  R rb[4];
-  for (int k = 0; k < 4; ++k) {
-    gb.rho += r[k] * Wtb[k];
-    rb[k] = g.rho * Wtb[k];
-  }
-  slope_solve_adj(g, K, c4K, r, A, Ab, gb, rb);
-  for (int k = 0; k < 4; ++k) rb[k] = -rb[k];
-  mslope_adj<1, 0>(T, a, rb, Tb, ab);
-  mslope_adj<0, 1>(T, b, rb, Tb, bb);
-  R rxb[4] = {0, 0, 0, 0}, ryb[4] = {0, 0, 0, 0};
-  slope_solve_adj(g, K, c4K, ry, b, bb, gb, ryb);
-  slope_solve_adj(g, K, c4K, rx, a, ab, gb, rxb);
-  for (int k = 0; k < 4; ++k) {
-    Wxb[k] += rxb[k] * g.ir;
-    Wyb[k] += ryb[k] * g.ir;
-    gb.ir += rxb[k] * Wx[k] + ryb[k] * Wy[k];
-  }
-  tab_full_adj(g, K, T, Tb, gb);
-  maxw_from_W_adj(W, gas.gm1, g, gb, Wb);
+  auto addg = [](Grad& a, const Grad& b) { a.d += b.d; a.u += b.v; a.v += b.u; a.t += b.t; };
+  addg(xb, sxb);
+  addg(yb, syb);
+  addg(tb, stb);
+  gb.rho += sgb.rho;
+  gb.ir += sgb.ir;
+  gb.U += sgb.V;
+  gb.V += sgb.U;
+  gb.p += sgb.p - gas.mu_r * ip * ip * taub;   // tau = c1 dt + mu/p
+  gb.th += sgb.th;
+  gb.en += sgb.en;
+  cons_rate_adj(g, hN, t, Wq, Wqb, rtb, gb, tb);
+  prim_rate_adj(g, gm1, x, y, tb, gb, xb, yb);
+  prim_grad_adj(g, gm1, Wx, x, xb, gb, Wxb);
+  prim_grad_adj(g, gm1, Wy, y, yb, gb, Wyb);
+  gas_state_adj(W, gm1, g, gb, Wb);
 }
 
 }  // namespace rev
