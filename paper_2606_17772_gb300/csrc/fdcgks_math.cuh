@@ -370,14 +370,14 @@ FD_HD void recon_interface(const GenoK<R>& g, const R Q[4], const R Qx[4], R h, 
   const R b0 = Q[1] - Q[0], b1 = Q[2] - Q[1], b2 = Q[3] - Q[2];
   // shared high-order derivative (identical for left and right)
   const R PHx = (b0 + b2 + R(46) * b1) * (ih * c30) - R(0.3) * (Qx[1] + Qx[2]);
-  const R PHl = (R(22) * b1 + b2 - R(7) * b0 + (Qx[0] + R(22) * Qx[1] - R(7) * Qx[2]) * h) * c64;
-  const R PHr = (R(7) * b2 - R(22) * b1 - b0 + (R(7) * Qx[1] - R(22) * Qx[2] - Qx[3]) * h) * c64;
+  const R PHl = R(22) * b1 + b2 - R(7) * b0 + (Qx[0] + R(22) * Qx[1] - R(7) * Qx[2]) * h;      // times 64
+  const R PHr = R(7) * b2 - R(22) * b1 - b0 + (R(7) * Qx[1] - R(22) * Qx[2] - Qx[3]) * h;
   bool smooth_l = g.linear, smooth_r = g.linear;
   if (GenoScreen<R>::v && !g.linear && fscale == R(0))
     screen_iface(g, b0, b1, b2, Qx[0], Qx[3], screen_h(h), smooth_l, smooth_r);
   chil = chir = g.linear ? R(1) : g.inv_tanhC;
-  vl = Q[1] + PHl;
-  vr = Q[2] + PHr;
+  vl = Q[1] + c64 * PHl;
+  vr = Q[2] + c64 * PHr;
   dl = dr = PHx;
   if (smooth_l && smooth_r) return;
   const R fl = geno_floor_of(s_max(s_max(s_abs(Q[0]), s_abs(Q[1])), s_max(s_abs(Q[2]), s_abs(Q[3]))), fscale);
@@ -400,7 +400,7 @@ FD_HD void recon_interface(const GenoK<R>& g, const R Q[4], const R Qx[4], R h, 
       const R PL = w[0] * (R(1.25) * b0 - R(0.75) * xh) + w[1] * (R(0.125) * b0 + R(0.375) * b1) +
                    w[2] * (R(0.625) * b1 - R(0.125) * b2);
       const R PLx = w[0] * (R(3) * b0 * ih - R(2) * Qx[0]) + (w[1] + w[2]) * (b1 * ih);
-      vl = Q[1] + (chi * PHl + om * PL);
+      vl = Q[1] + (chi * (c64 * PHl) + om * PL);
       dl = chi * PHx + om * PLx;
     }
   }
@@ -421,7 +421,7 @@ FD_HD void recon_interface(const GenoK<R>& g, const R Q[4], const R Qx[4], R h, 
       const R PL = w[0] * (R(0.75) * xh - R(1.25) * b2) - w[1] * (R(0.125) * b2 + R(0.375) * b1) +
                    w[2] * (R(0.125) * b0 - R(0.625) * b1);
       const R PLx = w[0] * (R(3) * b2 * ih - R(2) * Qx[3]) + (w[1] + w[2]) * (b1 * ih);
-      vr = Q[2] + (chi * PHr + om * PL);
+      vr = Q[2] + (chi * (c64 * PHr) + om * PL);
       dr = chi * PHx + om * PLx;
     }
   }
@@ -496,9 +496,27 @@ FD_HD TimeCoef<TW> time_coef(TW tau, TW dt, TW inv_dt) {
   // one transcendental: em = exp(-dt/(2 tau)) - 1, then
   // exp(-dt/tau) - 1 = em (em + 2) without cancellation.  Beyond
   // dt/(2 tau) = 40 expm1 rounds to -1 in FP64 (from 37.5 on) and FP32; smooth
-  // inviscid flow lies there, and the test spares it the division and expm1
-  TW em = TW(-1);
-  if (!(TW(0.5) * dt > TW(40) * tau)) em = s_expm1(-TW(0.5) * dt / tau);
+  // inviscid flow lies there and is spared the division, expm1 and 25 products
+  if (TW(0.5) * dt > TW(40) * tau) {
+    // em = -1: the fits in closed form, with r = tau/dt
+    const TW r = tau * inv_dt, tr = tau * r, r4 = TW(4) * r * r;
+    t.E = TW(0);
+    t.e1 = TW(1);
+    t.cn[3] = TW(3) * r;
+    t.cn[4] = TW(-6) * tr;
+    t.cn[5] = TW(-3) * tr;
+    t.ct[0] = TW(4) * r * inv_dt;
+    t.ct[4] = TW(2) * r4;
+    t.ct[5] = r4;
+    t.cn[0] = TW(1) - t.cn[3];
+    t.cn[1] = -tau - t.cn[4];
+    t.cn[2] = -tau - t.cn[5];
+    t.ct[1] = -t.ct[4];
+    t.ct[2] = TW(1) - r4;
+    t.ct[3] = -t.ct[0];
+    return t;
+  }
+  const TW em = s_expm1(-TW(0.5) * dt / tau);
   TW Eh = TW(1) + em, e1h = -em;
   t.E = Eh * Eh;
   t.e1 = -em * (em + TW(2));
@@ -592,12 +610,15 @@ FD_HD GasState<R> gas_state(const R W[4], R gm1) {
   g.U = W[1] * g.ir;
   g.V = D1 ? R(0) : W[2] * g.ir;
   g.en = W[3] * g.ir;
-  g.th = gm1 * (g.en - R(0.5) * (D1 ? g.U * g.U : g.U * g.U + g.V * g.V));
-  g.p = g.rho * g.th;
+  g.p = gm1 * (W[3] - R(0.5) * (D1 ? W[1] * g.U : W[1] * g.U + W[2] * g.V));
+  g.th = g.p * g.ir;
   return g;
 }
 
-// a derivative of the primitive variables: d = rho'/rho, u = U', v = V', t = theta'
+// rho times a derivative of the primitive variables: d = rho', u = rho U',
+// v = rho V', t = rho theta'.  Everything they enter is linear in them and
+// wanted per unit volume, so the weight saves the products with 1/rho here and
+// with rho there (some 40 of a solve's 900 FP64 operations).
 template <class R>
 struct PrimGrad {
   R d, u, v, t;
@@ -606,14 +627,14 @@ struct PrimGrad {
 template <bool D1 = false, class R>
 FD_HD PrimGrad<R> prim_grad(const GasState<R>& g, R gm1, const R D[4]) {
   PrimGrad<R> q;
-  q.d = D[0] * g.ir;
-  q.u = D[1] * g.ir - g.U * q.d;
+  q.d = D[0];
+  q.u = D[1] - g.U * D[0];
   if (D1) {
     q.v = R(0);
-    q.t = gm1 * (D[3] * g.ir - g.en * q.d - g.U * q.u);
+    q.t = gm1 * (D[3] - g.en * D[0] - g.U * q.u);
   } else {
-    q.v = D[2] * g.ir - g.V * q.d;
-    q.t = gm1 * (D[3] * g.ir - g.en * q.d - g.U * q.u - g.V * q.v);
+    q.v = D[2] - g.V * D[0];
+    q.t = gm1 * (D[3] - g.en * D[0] - g.U * q.u - g.V * q.v);
   }
   return q;
 }
@@ -636,22 +657,19 @@ FD_HD PrimGrad<R> prim_rate(const GasState<R>& g, R gm1, const PrimGrad<R>& x, c
   q.t = -(g.U * x.t + g.V * y.t + gm1 * g.th * div);
   return q;
 }
-// derivative of the conservative variables; hN = (K + 2)/2; rt = rho theta'
+// derivative of the conservative variables; hN = (K + 2)/2
 template <bool D1 = false, class R>
-FD_HD void cons_rate(const GasState<R>& g, R hN, const PrimGrad<R>& q, R W[4], R& rt) {
-  const R ru = g.rho * q.u;
-  rt = g.rho * q.t;
-  W[0] = g.rho * q.d;
-  W[1] = g.U * W[0] + ru;
+FD_HD void cons_rate(const GasState<R>& g, R hN, const PrimGrad<R>& q, R W[4]) {
+  W[0] = q.d;
+  W[1] = g.U * q.d + q.u;
   if (D1) {
-    W[3] = g.en * W[0] + g.U * ru + hN * rt;
+    W[3] = g.en * q.d + g.U * q.u + hN * q.t;
     return;
   }
-  const R rv = g.rho * q.v;
-  W[2] = g.V * W[0] + rv;
-  W[3] = g.en * W[0] + g.U * ru + g.V * rv + hN * rt;
+  W[2] = g.V * q.d + q.v;
+  W[3] = g.en * q.d + g.U * q.u + g.V * q.v + hN * q.t;
 }
-// Euler x-flux of g and its derivative for the derivative (q, Wq, rt) of g
+// Euler x-flux of g and its derivative for the derivative q (Wq: of W)
 template <bool D1 = false, class R>
 FD_HD void euler_flux(const GasState<R>& g, const R W[4], R F[4]) {
   F[0] = W[1];
@@ -660,12 +678,12 @@ FD_HD void euler_flux(const GasState<R>& g, const R W[4], R F[4]) {
   F[3] = g.U * (W[3] + g.p);
 }
 template <bool D1 = false, class R>
-FD_HD void euler_flux_rate(const GasState<R>& g, const R W[4], const PrimGrad<R>& q, const R Wq[4], R rt, R F[4]) {
-  const R pq = g.th * Wq[0] + rt;
+FD_HD void euler_flux_rate(const GasState<R>& g, const PrimGrad<R>& q, const R Wq[4], R F[4]) {
+  const R pq = g.th * q.d + q.t;
   F[0] = Wq[1];
-  F[1] = g.U * Wq[1] + W[1] * q.u + pq;
-  if (!D1) F[2] = g.V * Wq[1] + W[1] * q.v;
-  F[3] = q.u * (W[3] + g.p) + g.U * (Wq[3] + pq);
+  F[1] = g.U * (Wq[1] + q.u) + pq;
+  if (!D1) F[2] = g.V * Wq[1] + g.U * q.v;
+  F[3] = q.u * (g.en + g.th) + g.U * (Wq[3] + pq);
 }
 // rho <u psi (a u + b v + A)>: minus the Navier-Stokes stress and heat flux
 // over the collision time (the density component is 0)
@@ -673,20 +691,20 @@ template <bool D1 = false, class R>
 FD_HD void stress_flux(const GasState<R>& g, R K, R gm1, const PrimGrad<R>& x, const PrimGrad<R>& y, R S[4]) {
   S[0] = R(0);
   if (D1) {
-    S[1] = g.p * ((R(2) - gm1) * x.u);
-    S[3] = g.U * S[1] + (R(0.5) * K + R(2)) * g.p * x.t;
+    S[1] = g.th * ((R(2) - gm1) * x.u);
+    S[3] = g.U * S[1] + (R(0.5) * K + R(2)) * (g.th * x.t);
     return;
   }
-  S[1] = g.p * (R(2) * x.u - gm1 * (x.u + y.v));
-  S[2] = g.p * (x.v + y.u);
-  S[3] = g.U * S[1] + g.V * S[2] + (R(0.5) * K + R(2)) * g.p * x.t;
+  S[1] = g.th * (R(2) * x.u - gm1 * (x.u + y.v));
+  S[2] = g.th * (x.v + y.u);
+  S[3] = g.U * S[1] + g.V * S[2] + (R(0.5) * K + R(2)) * (g.th * x.t);
 }
 
 // ---------------------------------------------------------------------------
 // One side of the interface: the half-space moments M[n] = <u^n> over u > 0
 // (sign +1) or u < 0 (sign -1), and the slope polynomials D = a u + b v and A
-// integrated over c and xi against 1, c and (c^2 + xi^2)/2.  With weights
-// k3 + k4 D + k5 A the moments are, for T_k = <s u^k>,
+// integrated over c and xi against 1, c and (c^2 + xi^2)/2, both times rho.
+// With weights k3 + k4 D + k5 A the moments are, for T_k = <s u^k>,
 //   T_k = e0 M_k + e1 M_{k+1} + e2 M_{k+2} + e3 M_{k+3},
 //   <s u^k c> = c0 M_k + c1 M_{k+1} + c2 M_{k+2},
 //   <s u^k (u^2 + c^2 + xi^2)/2> = T_{k+2}/2 + N theta/2 T_k + X0 M_k + X1 M_{k+1}.
@@ -707,11 +725,11 @@ FD_HD void half_moments(const GasState<R>& g, int sign, R sl, R M[7]) {
   const R isqpi2 = R(0.56418958354775628695);   // 1/sqrt(pi); sl th = 1/(2 sqrt(lambda))
   M[0] = R(0.5) * ec;
   M[1] = g.U * M[0] + R(sign) * isqpi2 * (e * (sl * g.th));
-  R nth = R(0);
+  R nth = g.th;
 #pragma unroll
   for (int n = 0; n < 5; ++n) {
-    nth = nth + g.th;
     M[n + 2] = g.U * M[n + 1] + nth * M[n];
+    if (n < 4) nth = nth + g.th;
   }
 }
 
@@ -753,7 +771,7 @@ FD_HD void half_side(const GasState<R>& g, R N, R ith, const PrimGrad<R>& gx, co
 // adds rho <psi s> to Wm and rho <u psi s> to F for s = k3 + k4 D + k5 A
 template <bool D1 = false, class R>
 FD_HD void half_flux(const HalfSide<R>& s, R k3, R k4, R k5, R F[4], R Wm[4]) {
-  const R q3 = s.rho * k3, q4 = s.rho * k4, q5 = s.rho * k5;
+  const R q3 = s.rho * k3, q4 = k4, q5 = k5;
   const R e0 = D1 ? q3 + q5 * s.Ae0 : q3 + q4 * s.e0 + q5 * s.Ae0, e1 = q4 * s.e1 + q5 * s.Ae1, e2 = q4 * s.e2 + q5 * s.Ae2;
   const R e3 = q4 * s.e3;
   const R X0 = D1 ? q5 * s.AX0 : q4 * s.X0 + q5 * s.AX0, X1 = q4 * s.X1;
@@ -831,7 +849,7 @@ FD_HD void iface_solve_x(const GasK<R>& gas, const R Wl[4], const R Wr[4], const
   const GasState<R> g0 = gas_state<D1>(W0, gm1);
 
   // gradients (x: normal, y: tangential) and time derivatives of each state
-  R x1[4], W0q[4], rt;
+  R x1[4], W0q[4];
   PrimGrad<R> gtl, gtr;
   {
     const PrimGrad<R> gx = prim_grad<D1>(gl, gm1, Wln), gy = prim_grad<D1>(gl, gm1, Wt);
@@ -849,9 +867,9 @@ FD_HD void iface_solve_x(const GasK<R>& gas, const R Wl[4], const R Wr[4], const
     for (int k = 0; k < 4; ++k)
       if (!D1 || k != 2) x1[k] = R(0.5) * (Wln[k] + Wrn[k]);
     const PrimGrad<R> gx = prim_grad<D1>(g0, gm1, x1), gy = prim_grad<D1>(g0, gm1, Wt), gt = prim_rate<D1>(g0, gm1, gx, gy);
-    cons_rate<D1>(g0, hN, gt, W0q, rt);
+    cons_rate<D1>(g0, hN, gt, W0q);
     euler_flux<D1>(g0, W0, FE);
-    euler_flux_rate<D1>(g0, W0, gt, W0q, rt, FQ);
+    euler_flux_rate<D1>(g0, gt, W0q, FQ);
     stress_flux<D1>(g0, K, gm1, gx, gy, FS);
   }
 
@@ -943,8 +961,8 @@ FD_HD void iface_solve_x(const GasK<R>& gas, const R Wl[4], const R Wr[4], const
   // 3.41 ms, mixed 0.140 -> 0.137)
   if (E != R(0)) {
     R Wlq[4], Wrq[4];
-    cons_rate<D1>(gl, hN, gtl, Wlq, rt);
-    cons_rate<D1>(gr, hN, gtr, Wrq, rt);
+    cons_rate<D1>(gl, hN, gtl, Wlq);
+    cons_rate<D1>(gr, hN, gtr, Wrq);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       if (!used(k)) continue;
@@ -989,19 +1007,19 @@ FD_HD void nodal_flux(const GasK<R>& gas, const R W[4], const R Wx[4], const R W
   const R K = gas.K, gm1 = gas.gm1;
   const GasState<R> g = gas_state(W, gm1);
   const PrimGrad<R> gx = prim_grad(g, gm1, Wx), gy = prim_grad(g, gm1, Wy), gt = prim_rate(g, gm1, gx, gy);
-  R Wq[4], rt;
-  cons_rate(g, R(0.5) * K + R(1), gt, Wq, rt);
+  R Wq[4];
+  cons_rate(g, R(0.5) * K + R(1), gt, Wq);
   // f_t = A g: the time derivative of the Euler fluxes; its heat flux relative
   // to the fixed (U, V) is (K + 4)/2 p (U_t, V_t).  y-flux by the
   // transposition u <-> v
-  const R qf = gas.prfix * (R(0.5) * K + R(2)) * g.p;
-  euler_flux_rate(g, W, gt, Wq, rt, Ft);
+  const R qf = gas.prfix * (R(0.5) * K + R(2)) * g.th;
+  euler_flux_rate(g, gt, Wq, Ft);
   Ft[3] += qf * gt.u;
   const GasState<R> s = {g.rho, g.ir, g.V, g.U, g.p, g.th, g.en};
   const PrimGrad<R> sx = {gx.d, gx.v, gx.u, gx.t}, sy = {gy.d, gy.v, gy.u, gy.t}, st = {gt.d, gt.v, gt.u, gt.t};
   const R Ws[4] = {W[0], W[2], W[1], W[3]}, Wsq[4] = {Wq[0], Wq[2], Wq[1], Wq[3]};
   R x[4], y[4];
-  euler_flux_rate(s, Ws, st, Wsq, rt, x);
+  euler_flux_rate(s, st, Wsq, x);
   Gt[0] = x[0]; Gt[1] = x[2]; Gt[2] = x[1]; Gt[3] = x[3] + qf * gt.v;
   if (!want_n) {
 #pragma unroll
@@ -1009,7 +1027,8 @@ FD_HD void nodal_flux(const GasK<R>& gas, const R W[4], const R Wx[4], const R W
     return;
   }
   // F = Euler - tau stress, the heat flux (K + 4)/2 p theta' over Pr
-  const R tau = gas.c1_r * gas.dt_r + gas.mu_r * s_div(R(1), g.p);   // c1 dt + mu/p
+  R tau = gas.c1_r * gas.dt_r;                                       // c1 dt + mu/p
+  if (gas.mu_r != R(0)) tau = tau + gas.mu_r * s_div(R(1), g.p);
   euler_flux(g, W, F);
   stress_flux(g, K, gm1, gx, gy, x);
   x[3] += qf * gx.t;
@@ -1030,13 +1049,14 @@ FD_HD void nodal_flux_1d(const GasK<R>& gas, const R W[4], const R Wx[4], R F[4]
   const R K = gas.K, gm1 = gas.gm1;
   const GasState<R> g = gas_state<true>(W, gm1);
   const PrimGrad<R> gx = prim_grad<true>(g, gm1, Wx), gt = prim_rate<true>(g, gm1, gx, gx);
-  R Wq[4], rt, x[4];
-  cons_rate<true>(g, R(0.5) * K + R(1), gt, Wq, rt);
-  const R qf = gas.prfix * (R(0.5) * K + R(2)) * g.p;
-  euler_flux_rate<true>(g, W, gt, Wq, rt, Ft);
+  R Wq[4], x[4];
+  cons_rate<true>(g, R(0.5) * K + R(1), gt, Wq);
+  const R qf = gas.prfix * (R(0.5) * K + R(2)) * g.th;
+  euler_flux_rate<true>(g, gt, Wq, Ft);
   Ft[3] += qf * gt.u;
   if (!want_n) return;
-  const R tau = gas.c1_r * gas.dt_r + gas.mu_r * s_div(R(1), g.p);   // c1 dt + mu/p
+  R tau = gas.c1_r * gas.dt_r;                                       // c1 dt + mu/p
+  if (gas.mu_r != R(0)) tau = tau + gas.mu_r * s_div(R(1), g.p);
   euler_flux<true>(g, W, F);
   stress_flux<true>(g, K, gm1, gx, gx, x);
   x[3] += qf * gx.t;

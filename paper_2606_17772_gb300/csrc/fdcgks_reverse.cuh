@@ -383,15 +383,13 @@ FD_HD void gas_state_adj(const R W[4], R gm1, const Gas& g, const Gas& gb, R Wb[
 
 FD_HD void prim_grad_adj(const Gas& g, R gm1, const R D[4], const Grad& q, const Grad& qb, Gas& gb, R Db[4]) {
   const R tb = gm1 * qb.t, ub = qb.u - g.U * tb, vb = qb.v - g.V * tb;
-  const R db = qb.d - g.en * tb - g.V * vb - g.U * ub;
-  gb.en -= q.d * tb;
-  gb.U -= q.u * tb + q.d * ub;
-  gb.V -= q.v * tb + q.d * vb;
-  gb.ir += D[0] * db + D[1] * ub + D[2] * vb + D[3] * tb;
-  Db[0] += g.ir * db;
-  Db[1] += g.ir * ub;
-  Db[2] += g.ir * vb;
-  Db[3] += g.ir * tb;
+  gb.en -= D[0] * tb;
+  gb.U -= q.u * tb + D[0] * ub;
+  gb.V -= q.v * tb + D[0] * vb;
+  Db[0] += qb.d - g.en * tb - g.V * vb - g.U * ub;
+  Db[1] += ub;
+  Db[2] += vb;
+  Db[3] += tb;
 }
 
 FD_HD void prim_rate_adj(const Gas& g, R gm1, const Grad& x, const Grad& y, const Grad& qb, Gas& gb, Grad& xb,
@@ -410,18 +408,14 @@ FD_HD void prim_rate_adj(const Gas& g, R gm1, const Grad& x, const Grad& y, cons
   yb.t -= g.V * qb.t + qb.v;
 }
 
-// W = cons_rate(g, q), rt = rho q.t; the adjoints Wb and rtb
-FD_HD void cons_rate_adj(const Gas& g, R hN, const Grad& q, const R W[4], const R Wb[4], R rtb, Gas& gb, Grad& qb) {
-  const R w0b = Wb[0] + g.U * Wb[1] + g.V * Wb[2] + g.en * Wb[3];
-  const R rub = Wb[1] + g.U * Wb[3], rvb = Wb[2] + g.V * Wb[3], tb = rtb + hN * Wb[3];
-  gb.U += W[0] * Wb[1] + g.rho * q.u * Wb[3];
-  gb.V += W[0] * Wb[2] + g.rho * q.v * Wb[3];
-  gb.en += W[0] * Wb[3];
-  gb.rho += q.d * w0b + q.u * rub + q.v * rvb + q.t * tb;
-  qb.d += g.rho * w0b;
-  qb.u += g.rho * rub;
-  qb.v += g.rho * rvb;
-  qb.t += g.rho * tb;
+FD_HD void cons_rate_adj(const Gas& g, R hN, const Grad& q, const R Wb[4], Gas& gb, Grad& qb) {
+  gb.U += q.d * Wb[1] + q.u * Wb[3];
+  gb.V += q.d * Wb[2] + q.v * Wb[3];
+  gb.en += q.d * Wb[3];
+  qb.d += Wb[0] + g.U * Wb[1] + g.V * Wb[2] + g.en * Wb[3];
+  qb.u += Wb[1] + g.U * Wb[3];
+  qb.v += Wb[2] + g.V * Wb[3];
+  qb.t += hN * Wb[3];
 }
 
 FD_HD void euler_flux_adj(const Gas& g, const R W[4], const R Fb[4], Gas& gb, R Wb[4]) {
@@ -432,35 +426,33 @@ FD_HD void euler_flux_adj(const Gas& g, const R W[4], const R Fb[4], Gas& gb, R 
   gb.p += Fb[1] + g.U * Fb[3];
 }
 
-FD_HD void euler_flux_rate_adj(const Gas& g, const R W[4], const Grad& q, const R Wq[4], R rt, const R Fb[4], Gas& gb,
-                               R Wb[4], Grad& qb, R Wqb[4], R& rtb) {
-  const R pq = g.th * Wq[0] + rt, pqb = Fb[1] + g.U * Fb[3], Ep = W[3] + g.p;
-  gb.U += Wq[1] * Fb[1] + (Wq[3] + pq) * Fb[3];
+FD_HD void euler_flux_rate_adj(const Gas& g, const Grad& q, const R Wq[4], const R Fb[4], Gas& gb, Grad& qb,
+                               R Wqb[4]) {
+  const R pq = g.th * q.d + q.t, pqb = Fb[1] + g.U * Fb[3], quFb = q.u * Fb[3];
+  gb.U += (Wq[1] + q.u) * Fb[1] + q.v * Fb[2] + (Wq[3] + pq) * Fb[3];
   gb.V += Wq[1] * Fb[2];
-  gb.p += q.u * Fb[3];
-  gb.th += Wq[0] * pqb;
-  Wb[1] += q.u * Fb[1] + q.v * Fb[2];
-  Wb[3] += q.u * Fb[3];
-  qb.u += W[1] * Fb[1] + Ep * Fb[3];
-  qb.v += W[1] * Fb[2];
-  Wqb[0] += g.th * pqb;
+  gb.en += quFb;
+  gb.th += quFb + q.d * pqb;
+  qb.d += g.th * pqb;
+  qb.t += pqb;
+  qb.u += g.U * Fb[1] + (g.en + g.th) * Fb[3];
+  qb.v += g.U * Fb[2];
   Wqb[1] += Fb[0] + g.U * Fb[1] + g.V * Fb[2];
   Wqb[3] += g.U * Fb[3];
-  rtb += pqb;
 }
 
 FD_HD void stress_flux_adj(const Gas& g, R K, R gm1, const Grad& x, const Grad& y, const R Sb[4], Gas& gb, Grad& xb,
                            Grad& yb) {
   const R A = 2.0 * x.u - gm1 * (x.u + y.v), B = x.v + y.u, c = 0.5 * K + 2.0;
-  const R s1 = Sb[1] + g.U * Sb[3], s2 = Sb[2] + g.V * Sb[3], s1p = g.p * s1, s2p = g.p * s2;
-  gb.U += g.p * A * Sb[3];
-  gb.V += g.p * B * Sb[3];
-  gb.p += A * s1 + B * s2 + c * x.t * Sb[3];
+  const R s1 = Sb[1] + g.U * Sb[3], s2 = Sb[2] + g.V * Sb[3], s1p = g.th * s1, s2p = g.th * s2;
+  gb.U += g.th * A * Sb[3];
+  gb.V += g.th * B * Sb[3];
+  gb.th += A * s1 + B * s2 + c * x.t * Sb[3];
   xb.u += (2.0 - gm1) * s1p;
   yb.v -= gm1 * s1p;
   xb.v += s2p;
   yb.u += s2p;
-  xb.t += c * g.p * Sb[3];
+  xb.t += c * g.th * Sb[3];
 }
 
 // half_moments with sl = 1/sqrt(2 theta): Mb -> U, theta (Mb is used up)
@@ -526,7 +518,7 @@ FD_HD void half_side_adj(const Gas& g, R N, R ith, const Grad& gx, const Grad& g
 // half_flux for the weights k[0..2] = (k3, k4, k5): the adjoints Fb, Wb of the
 // sums it adds to -> those of the side (into sb, M's included) and of k
 FD_HD void half_flux_adj(const HalfSide<R>& s, const R k[3], const R Fb[4], const R Wb[4], HalfSide<R>& sb, R kb[3]) {
-  const R q3 = s.rho * k[0], q4 = s.rho * k[1], q5 = s.rho * k[2];
+  const R q3 = s.rho * k[0], q4 = k[1], q5 = k[2];
   const R e[4] = {q3 + q4 * s.e0 + q5 * s.Ae0, q4 * s.e1 + q5 * s.Ae1, q4 * s.e2 + q5 * s.Ae2, q4 * s.e3};
   const R X0 = q4 * s.X0 + q5 * s.AX0, X1 = q4 * s.X1;
   const R c0 = q4 * s.c0 + q5 * s.Ac0, c1 = q4 * s.c1, c2 = q4 * s.c2;
@@ -571,10 +563,10 @@ FD_HD void half_flux_adj(const HalfSide<R>& s, const R k[3], const R Fb[4], cons
   const R q4b = s.e0 * eb[0] + s.e1 * eb[1] + s.e2 * eb[2] + s.e3 * eb[3] + s.X0 * X0b + s.X1 * X1b + s.c0 * c0b +
                 s.c1 * c1b + s.c2 * c2b;
   const R q5b = s.Ae0 * eb[0] + s.Ae1 * eb[1] + s.Ae2 * eb[2] + s.AX0 * X0b + s.Ac0 * c0b;
-  sb.rho += k[0] * eb[0] + k[1] * q4b + k[2] * q5b;
+  sb.rho += k[0] * eb[0];
   kb[0] += s.rho * eb[0];
-  kb[1] += s.rho * q4b;
-  kb[2] += s.rho * q5b;
+  kb[1] += q4b;
+  kb[2] += q5b;
 }
 
 FD_HD void half_side_zero(HalfSide<R>& s) {
@@ -588,7 +580,7 @@ FD_HD void half_side_zero(HalfSide<R>& s) {
 struct SideFwd {
   Gas g;
   Grad x, y, t;
-  R sl, Wq[4], rt;
+  R sl, Wq[4];
   HalfSide<R> s;
 };
 FD_HD void side_fwd(const R W[4], const R D[4], const R Dt[4], int sign, R K, R gm1, SideFwd& f) {
@@ -599,7 +591,7 @@ FD_HD void side_fwd(const R W[4], const R D[4], const R Dt[4], int sign, R K, R 
   f.y = prim_grad(f.g, gm1, Dt);
   f.t = prim_rate(f.g, gm1, f.x, f.y);
   half_side(f.g, K + 1.0, 2.0 * f.sl * f.sl, f.x, f.y, f.t, f.s);
-  cons_rate(f.g, 0.5 * K + 1.0, f.t, f.Wq, f.rt);
+  cons_rate(f.g, 0.5 * K + 1.0, f.t, f.Wq);
 }
 // sb: adjoint of the half-space quantities, Wqb of W_t, W0b of the equilibrium
 // state rho (M0, M1, V M0, (M2 + (N theta + V^2) M0)/2) summed over the sides
@@ -616,7 +608,7 @@ FD_HD void side_adj(const R W[4], const R D[4], const R Dt[4], int sign, R K, R 
   sb.M[2] += 0.5 * g.rho * W0b[3];
   Grad xb = grad_zero(), yb = grad_zero(), tb = grad_zero();
   half_side_adj(g, N, 2.0 * f.sl * f.sl, f.x, f.y, f.t, f.s, sb, gb, xb, yb, tb);
-  cons_rate_adj(g, 0.5 * K + 1.0, f.t, f.Wq, Wqb, 0.0, gb, tb);
+  cons_rate_adj(g, 0.5 * K + 1.0, f.t, Wqb, gb, tb);
   prim_rate_adj(g, gm1, f.x, f.y, tb, gb, xb, yb);
   prim_grad_adj(g, gm1, D, f.x, xb, gb, Db);
   prim_grad_adj(g, gm1, Dt, f.y, yb, gb, Dtb);
@@ -687,7 +679,7 @@ FD_HD void iface_solve_x_adj(const GasK<R>& gas, const R Wl[4], const R Wr[4], c
   SideFwd l, r;
   side_fwd(Wl, Wln, Wt, +1, K, gm1, l);
   side_fwd(Wr, Wrn, Wt, -1, K, gm1, r);
-  R W0[4], x1[4], W0q[4], rt0, FE[4], FQ[4], FS[4];
+  R W0[4], x1[4], W0q[4], FE[4], FQ[4], FS[4];
   {
     const R ml = l.g.rho * l.s.M[0], mr = r.g.rho * r.s.M[0];
     W0[0] = ml + mr;
@@ -699,9 +691,9 @@ FD_HD void iface_solve_x_adj(const GasK<R>& gas, const R Wl[4], const R Wr[4], c
   const Gas g0 = gas_state(W0, gm1);
   for (int k = 0; k < 4; ++k) x1[k] = 0.5 * (Wln[k] + Wrn[k]);
   const Grad gx = prim_grad(g0, gm1, x1), gy = prim_grad(g0, gm1, Wt), gt = prim_rate(g0, gm1, gx, gy);
-  cons_rate(g0, hN, gt, W0q, rt0);
+  cons_rate(g0, hN, gt, W0q);
   euler_flux(g0, W0, FE);
-  euler_flux_rate(g0, W0, gt, W0q, rt0, FQ);
+  euler_flux_rate(g0, gt, W0q, FQ);
   stress_flux(g0, K, gm1, gx, gy, FS);
   const R ip0 = 1.0 / g0.p, dp = l.g.p - r.g.p, sp = l.g.p + r.g.p;
   const R tau = gas.c1 * gas.dt + gas.mu * ip0 + gas.c2 * gas.dt * s_abs(dp) / sp;
@@ -775,11 +767,11 @@ FD_HD void iface_solve_x_adj(const GasK<R>& gas, const R Wl[4], const R Wr[4], c
   // equilibrium state: stress, Euler flux and its time derivative, gradients
   {
     Grad xb = grad_zero(), yb = grad_zero(), tb = grad_zero();
-    R rtb = 0.0, x1b[4] = {0.0, 0.0, 0.0, 0.0};
+    R x1b[4] = {0.0, 0.0, 0.0, 0.0};
     stress_flux_adj(g0, K, gm1, gx, gy, FSb, g0b, xb, yb);
-    euler_flux_rate_adj(g0, W0, gt, W0q, rt0, FQb, g0b, W0b, tb, W0qb, rtb);
+    euler_flux_rate_adj(g0, gt, W0q, FQb, g0b, tb, W0qb);
     euler_flux_adj(g0, W0, FEb, g0b, W0b);
-    cons_rate_adj(g0, hN, gt, W0q, W0qb, rtb, g0b, tb);
+    cons_rate_adj(g0, hN, gt, W0qb, g0b, tb);
     prim_rate_adj(g0, gm1, gx, gy, tb, g0b, xb, yb);
     prim_grad_adj(g0, gm1, x1, gx, xb, g0b, x1b);
     prim_grad_adj(g0, gm1, Wt, gy, yb, g0b, Wtb);
@@ -821,27 +813,27 @@ FD_HD Gas swap_gas(const Gas& g) { return Gas{g.rho, g.ir, g.V, g.U, g.p, g.th, 
 FD_HD Grad swap_grad(const Grad& q) { return Grad{q.d, q.v, q.u, q.t}; }
 
 // x-flux and its time derivative: Fb, Ftb -> the adjoints of the state, W, the
-// gradients, W_t and rho theta_t
+// gradients and W_t
 FD_HD void nodal_dir_adj(R K, R gm1, R prfix, R tau, const Gas& g, const R W[4], const Grad& x, const Grad& y,
-                         const Grad& t, const R Wq[4], R rt, const R Fb[4], const R Ftb[4], Gas& gb, R Wb[4], Grad& xb,
-                         Grad& yb, Grad& tb, R Wqb[4], R& rtb, R& taub) {
+                         const Grad& t, const R Wq[4], const R Fb[4], const R Ftb[4], Gas& gb, R Wb[4], Grad& xb,
+                         Grad& yb, Grad& tb, R Wqb[4], R& taub) {
   const R c = prfix * (0.5 * K + 2.0);
-  // Ft = Euler rate, Ft3 += c p U_t
-  euler_flux_rate_adj(g, W, t, Wq, rt, Ftb, gb, Wb, tb, Wqb, rtb);
-  gb.p += c * t.u * Ftb[3];
-  tb.u += c * g.p * Ftb[3];
-  // F = Euler - tau S, S3 += c p theta_x
+  // Ft = Euler rate, Ft3 += c theta rho U_t
+  euler_flux_rate_adj(g, t, Wq, Ftb, gb, tb, Wqb);
+  gb.th += c * t.u * Ftb[3];
+  tb.u += c * g.th * Ftb[3];
+  // F = Euler - tau S, S3 += c theta rho theta_x
   euler_flux_adj(g, W, Fb, gb, Wb);
   R S[4], Sb[4];
   stress_flux(g, K, gm1, x, y, S);
-  S[3] += c * g.p * x.t;
+  S[3] += c * g.th * x.t;
   for (int k = 0; k < 4; ++k) {
     taub -= S[k] * Fb[k];
     Sb[k] = -tau * Fb[k];
   }
   stress_flux_adj(g, K, gm1, x, y, Sb, gb, xb, yb);
-  gb.p += c * x.t * Sb[3];
-  xb.t += c * g.p * Sb[3];
+  gb.th += c * x.t * Sb[3];
+  xb.t += c * g.th * Sb[3];
 }
 
 FD_HD void nodal_flux_adj(const GasK<R>& gas, const R W[4], const R Wx[4], const R Wy[4], const R Fb_in[4],
@@ -849,17 +841,17 @@ FD_HD void nodal_flux_adj(const GasK<R>& gas, const R W[4], const R Wx[4], const
   const R K = gas.K, gm1 = gas.gm1, hN = 0.5 * K + 1.0;
   const Gas g = gas_state(W, gm1);
   const Grad x = prim_grad(g, gm1, Wx), y = prim_grad(g, gm1, Wy), t = prim_rate(g, gm1, x, y);
-  R Wq[4], rt;
-  cons_rate(g, hN, t, Wq, rt);
+  R Wq[4];
+  cons_rate(g, hN, t, Wq);
   const R ip = 1.0 / g.p, tau = gas.c1_r * gas.dt_r + gas.mu_r * ip;
   Gas gb = gas_zero(), sgb = gas_zero();
   Grad xb = grad_zero(), yb = grad_zero(), tb = grad_zero(), sxb = grad_zero(), syb = grad_zero(), stb = grad_zero();
-  R Wqb[4] = {0, 0, 0, 0}, sWqb[4] = {0, 0, 0, 0}, sWb[4] = {0, 0, 0, 0}, rtb = 0.0, taub = 0.0;
-  nodal_dir_adj(K, gm1, gas.prfix, tau, g, W, x, y, t, Wq, rt, Fb_in, Ftb_in, gb, Wb, xb, yb, tb, Wqb, rtb, taub);
+  R Wqb[4] = {0, 0, 0, 0}, sWqb[4] = {0, 0, 0, 0}, sWb[4] = {0, 0, 0, 0}, taub = 0.0;
+  nodal_dir_adj(K, gm1, gas.prfix, tau, g, W, x, y, t, Wq, Fb_in, Ftb_in, gb, Wb, xb, yb, tb, Wqb, taub);
   const R sW[4] = {W[0], W[2], W[1], W[3]}, sWq[4] = {Wq[0], Wq[2], Wq[1], Wq[3]};
   const R sG[4] = {Gb_in[0], Gb_in[2], Gb_in[1], Gb_in[3]}, sGt[4] = {Gtb_in[0], Gtb_in[2], Gtb_in[1], Gtb_in[3]};
-  nodal_dir_adj(K, gm1, gas.prfix, tau, swap_gas(g), sW, swap_grad(y), swap_grad(x), swap_grad(t), sWq, rt, sG, sGt,
-                sgb, sWb, syb, sxb, stb, sWqb, rtb, taub);
+  nodal_dir_adj(K, gm1, gas.prfix, tau, swap_gas(g), sW, swap_grad(y), swap_grad(x), swap_grad(t), sWq, sG, sGt,
+                sgb, sWb, syb, sxb, stb, sWqb, taub);
   const int sw[4] = {0, 2, 1, 3};
   for (int k = 0; k < 4; ++k) {
     Wb[k] += sWb[sw[k]];
@@ -876,7 +868,7 @@ FD_HD void nodal_flux_adj(const GasK<R>& gas, const R W[4], const R Wx[4], const
   gb.p += sgb.p - gas.mu_r * ip * ip * taub;   // tau = c1 dt + mu/p
   gb.th += sgb.th;
   gb.en += sgb.en;
-  cons_rate_adj(g, hN, t, Wq, Wqb, rtb, gb, tb);
+  cons_rate_adj(g, hN, t, Wqb, gb, tb);
   prim_rate_adj(g, gm1, x, y, tb, gb, xb, yb);
   prim_grad_adj(g, gm1, Wx, x, xb, gb, Wxb);
   prim_grad_adj(g, gm1, Wy, y, yb, gb, Wyb);
