@@ -470,7 +470,7 @@ KArgs<double> stage_args(const Work& w, double dt, int stage) {
   a.flux_variant = w.v.p.flux_variant;
   a.grad_base = w.v.p.grad_base;
   a.want_n = stage == 0 ? 1 : 0;
-  a.dt = dt;
+  set_dt(a, dt);
   a.flag = w.flag;
   a.Sn = w.Sn;
   a.Wacc = w.Wacc;

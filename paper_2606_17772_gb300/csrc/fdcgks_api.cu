@@ -479,7 +479,7 @@ static KArgs<R> make_args(fdcgks_t c, double dt, const double* S, double* Sout, 
   a.grad_base = c->p.grad_base;
   a.recon_vars = c->p.recon_vars;
   a.want_n = want_n;
-  a.dt = dt;
+  set_dt(a, dt);
   a.flag = c->flag;
   return a;
 }

@@ -287,14 +287,7 @@ __global__ void ens_dt_kernel(KArgs<R>* args, const MemberMeta* meta, const unsi
     last_dt[m] = 0.0;
     return;
   }
-  for (int s = 0; s < 2; ++s) {
-    KArgs<R>& a = args[2 * m + s];
-    a.dt = dt;
-    a.gas.dt = dt;
-    a.gas.inv_dt = 1.0 / dt;
-    a.gas.dt_r = (R)dt;
-    a.gas.inv_dt_r = (R)(1.0 / dt);
-  }
+  for (int s = 0; s < 2; ++s) set_dt(args[2 * m + s], dt);
   time[m] += dt;
   last_dt[m] = dt;
 }
@@ -587,7 +580,7 @@ void fill_args(fdcgks_ens_t e, int m, char* base, const std::vector<size_t>& off
     a.flux_variant = p.flux_variant;
     a.grad_base = p.grad_base;
     a.want_n = s == 0 ? 1 : 0;
-    a.dt = 1.0;
+    set_dt(a, 1.0);
     a.flag = e->mstat + m;
     if (e->precision == FDCGKS_MIXED) {
       float* Shi = (float*)(base + off[0]);

@@ -125,9 +125,25 @@ struct KArgs {
   int flux_variant, grad_base, want_n;
   int recon_vars;        // 0 conservative, 1 characteristic interface reconstruction
   double dt;
+  double dtk[4];         // dt/2, dt^2/8, dt^2/6, dt^2/3 (set_dt)
   int* flag;             // bit 0: non-physical state found
   double* op[8];         // operator outputs (Lp, Ltp, gbp, gtp, Ld, Ltd, gbd, gtd), interior layout
 };
+
+// the time-step fields of an argument block (a division by 6 or 3 in every
+// thread of the update would cost it 18 slots of the FP64 pipe)
+template <class R>
+FD_HD void set_dt(KArgs<R>& a, double dt) {
+  a.dt = dt;
+  a.dtk[0] = 0.5 * dt;
+  a.dtk[1] = 0.125 * dt * dt;
+  a.dtk[2] = dt * dt / 6.0;
+  a.dtk[3] = dt * dt / 3.0;
+  a.gas.dt = dt;
+  a.gas.inv_dt = 1.0 / dt;
+  a.gas.dt_r = (R)dt;
+  a.gas.inv_dt_r = (R)(1.0 / dt);
+}
 
 // Ghost layers of one grid g of a padded state (W, x- and y-gradients), as the
 // adjoint folds them back (the forward fill is ghost_fill below):

@@ -651,13 +651,13 @@ __device__ __forceinline__ void update_body(const KArgs<R>& a, int mode, int g, 
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const double dL = (double)o.L[c], dLt = (double)o.Lt[c];
-        Wnew[c] = Wn[c] + 0.5 * dt * dL + 0.125 * dt * dt * dLt;
-        Ag[(long)c * P + c0] = Wn[c] + dt * dL + dt * dt / 6.0 * dLt;
+        Wnew[c] = Wn[c] + a.dtk[0] * dL + a.dtk[1] * dLt;
+        Ag[(long)c * P + c0] = Wn[c] + dt * dL + a.dtk[2] * dLt;
       }
 #pragma unroll
       for (int f = 0; f < 8; ++f) {
         Bg[(long)f * P + c0] = Gb[f];
-        Gnew[f] = Gb[f] + 0.5 * dt * (double)(f < 4 ? o.gtx[f] : o.gty[f - 4]);
+        Gnew[f] = Gb[f] + a.dtk[0] * (double)(f < 4 ? o.gtx[f] : o.gty[f - 4]);
       }
     } else {
 #pragma unroll
@@ -665,7 +665,7 @@ __device__ __forceinline__ void update_body(const KArgs<R>& a, int mode, int g, 
 #pragma unroll
       for (int f = 0; f < 8; ++f) Gnew[f] = Bg[(long)f * P + c0];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) Wnew[c] = Wnew[c] + dt * dt / 3.0 * (double)o.Lt[c];
+      for (int c = 0; c < 4; ++c) Wnew[c] = Wnew[c] + a.dtk[3] * (double)o.Lt[c];
 #pragma unroll
       for (int f = 0; f < 8; ++f) Gnew[f] = Gnew[f] + dt * (double)(f < 4 ? o.gtx[f] : o.gty[f - 4]);
     }
@@ -681,9 +681,9 @@ __device__ __forceinline__ void update_body(const KArgs<R>& a, int mode, int g, 
     for (int c = 0; c < 4; ++c) Og[(long)c * P + c0] = Wnew[c];
 #pragma unroll
     for (int f = 0; f < 8; ++f) Og[(long)(4 + f) * P + c0] = Gnew[f];
-    // positivity of density and pressure (no trap: a flag the host reads)
-    double p = Wnew[3] - 0.5 * (Wnew[1] * Wnew[1] + Wnew[2] * Wnew[2]) / Wnew[0];
-    if (!(Wnew[0] > 0.0) || !(p > 0.0)) atomicOr(a.flag, 1);
+    // positivity of density and pressure (no trap: a flag the host reads), p > 0
+    // as 2 E rho > m^2, without a division
+    if (!(Wnew[0] > 0.0) || !(2.0 * Wnew[3] * Wnew[0] > Wnew[1] * Wnew[1] + Wnew[2] * Wnew[2])) atomicOr(a.flag, 1);
   }
 }
 

@@ -178,7 +178,7 @@ __device__ void line_update(const LineArgs<R>& a, int mode, int stage, double dt
                             const double* Bin, double* Bout, double* A, int line, int* flag) {
   const int ni = a.n + 3, nn = a.n + 2;
   const R ih = (R)a.ih;
-  const double dt26 = dt * dt / 6.0, dt23 = dt * dt / 3.0;
+  const double dt26 = dt * dt * (1.0 / 6.0), dt23 = 2.0 * dt26;
   for (int j = lt_index(a); j < a.n; j += lt_count(a)) {
     const R chip = P[18 * ni + j + 2], chim = P[18 * ni + j + 1];
     double L[3], Lt[3], gb[3], gt[3];
@@ -227,8 +227,8 @@ __device__ void line_update(const LineArgs<R>& a, int mode, int stage, double dt
       }
       Bout[c * a.np + GH + j] = W[c];
     }
-    const double p = W[2] - 0.5 * W[1] * W[1] / W[0];
-    if (!(W[0] > 0.0) || !(p > 0.0)) atomicOr(flag, 1);
+    // p > 0 as 2 E rho > m^2
+    if (!(W[0] > 0.0) || !(2.0 * W[2] * W[0] > W[1] * W[1])) atomicOr(flag, 1);
   }
 }
 

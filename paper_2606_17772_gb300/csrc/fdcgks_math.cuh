@@ -839,7 +839,7 @@ FD_HD void iface_solve_x(const GasK<R>& gas, const R Wl[4], const R Wr[4], const
     W0[1] = gl.rho * sl.M[1] + gr.rho * sr.M[1];
     if (D1) {
       W0[2] = R(0);
-      W0[3] = R(0.5) * (gl.rho * (sl.M[2] + N * gl.th * sl.M[0]) + gr.rho * (sr.M[2] + N * gr.th * sr.M[0]));
+      W0[3] = R(0.5) * (gl.rho * sl.M[2] + gr.rho * sr.M[2] + N * (gl.p * sl.M[0] + gr.p * sr.M[0]));
     } else {
       W0[2] = gl.V * ml + gr.V * mr;
       W0[3] = R(0.5) * (gl.rho * sl.M[2] + gr.rho * sr.M[2] + (ml * (gl.V * gl.V) + mr * (gr.V * gr.V)) +
