@@ -610,8 +610,13 @@ FD_HD GasState<R> gas_state(const R W[4], R gm1) {
   g.U = W[1] * g.ir;
   g.V = D1 ? R(0) : W[2] * g.ir;
   g.en = W[3] * g.ir;
-  g.p = gm1 * (W[3] - R(0.5) * (D1 ? W[1] * g.U : W[1] * g.U + W[2] * g.V));
-  g.th = g.p * g.ir;
+  if (IsF32<R>::v) {   // squares of one factor: every kernel contracts them alike, so their results agree
+    g.th = gm1 * (g.en - R(0.5) * (D1 ? g.U * g.U : g.U * g.U + g.V * g.V));
+    g.p = g.rho * g.th;
+  } else {
+    g.p = gm1 * (W[3] - R(0.5) * (D1 ? W[1] * g.U : W[1] * g.U + W[2] * g.V));
+    g.th = g.p * g.ir;
+  }
   return g;
 }
 
