@@ -15,13 +15,12 @@
 //                  update and nodal kernels (the FP64 kernels are FP64-pipe bound and
 //                  are left uncapped).  1024^2 vortex, ms per mixed step:
 //                  update 4, 5, 6, 8 gave 0.448, 0.411, 0.382, 0.437; nodal
-//                  5, 6, 8, 10, 12, 16 gave 0.303, 0.264, 0.234, 0.221, 0.225,
-//                  0.332
+//                  (its loads issued together) 5, 6 give 0.116, 0.115
 #ifndef FDK_UPDATE_MINB_F32
 #define FDK_UPDATE_MINB_F32 6
 #endif
 #ifndef FDK_NODAL_MINB_F32
-#define FDK_NODAL_MINB_F32 10
+#define FDK_NODAL_MINB_F32 6
 #endif
 // FDK_STAGE_THREADS_F64  block size of the FP64 stage kernel (below; 32 and 128:
 //                  33^2 0.213 and 0.227 ms per step, 512^2 4.73 and 4.78)
@@ -72,19 +71,33 @@ template <> struct PointTune<float> {
 // node, 1/2 its x neighbours -/+, 3/4 its y neighbours -/+); st(k, v): output
 // k (F[4], G[4], F_t[4], G_t[4]); want_n = false (second S2O4 stage): F_t and
 // G_t only, F and G are neither computed nor stored.
+// FP32: bound by the latency of its 44 loads (DRAM 16 % busy), so all of them
+// are issued before the first component's branches: 1024^2 mixed 0.160 -> 0.115
+// ms per step (one component ahead 0.123), 512^2 0.0458 -> 0.0392.  FP64 is
+// bound by its pipe and keeps the registers.
 template <class R, class LD, class ST>
 FD_HD void nodal_compute(const GenoK<R>& geno, const GasK<R>& gas, const R h[2], const R ih[2], LD ld, ST st,
                          bool want_n = true) {
-  R W[4], Wx[4], Wy[4];
+  constexpr int AHEAD = IsF32<R>::v ? 4 : 1;   // components loaded at once
+  R W[4], Wx[4], Wy[4], qx[AHEAD][3], gx[AHEAD][3], qy[AHEAD][3], gy[AHEAD][3];
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
-    W[c] = ld(0, c);
-    R qx[3] = {ld(1, c), W[c], ld(2, c)};
-    R gxv[3] = {ld(1, 4 + c), ld(0, 4 + c), ld(2, 4 + c)};
-    Wx[c] = recon_node(geno, qx, gxv, h[0], ih[0]);
-    R qy[3] = {ld(3, c), W[c], ld(4, c)};
-    R gyv[3] = {ld(3, 8 + c), ld(0, 8 + c), ld(4, 8 + c)};
-    Wy[c] = recon_node(geno, qy, gyv, h[1], ih[1]);
+    if (c % AHEAD == 0) {
+#pragma unroll
+      for (int k = 0; k < AHEAD; ++k)
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {   // the lower neighbour, the node, the upper one
+          const int ex = e == 1 ? 0 : e == 0 ? 1 : 2, ey = e == 1 ? 0 : e == 0 ? 3 : 4;
+          qx[k][e] = ld(ex, c + k);
+          gx[k][e] = ld(ex, 4 + c + k);
+          qy[k][e] = e == 1 ? qx[k][1] : ld(ey, c + k);
+          gy[k][e] = ld(ey, 8 + c + k);
+        }
+    }
+    const int k = c % AHEAD;
+    W[c] = qx[k][1];
+    Wx[c] = recon_node(geno, qx[k], gx[k], h[0], ih[0]);
+    Wy[c] = recon_node(geno, qy[k], gy[k], h[1], ih[1]);
   }
   R F[4], G[4], Ft[4], Gt[4];
   nodal_flux(gas, W, Wx, Wy, F, G, Ft, Gt, want_n);
