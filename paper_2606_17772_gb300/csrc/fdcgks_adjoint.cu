@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(128) update_adj_kernel(KArgs<double> a, int st
   const long P = L.plane, c0 = cell(L, i, j), pp = L.pplane;
   const double dt = a.dt;
   const bool want_n = stage == 0;
-  NodeOp<double> o;
+  NodeOp o;
   node_operator(a, g, i, j, want_n, o);
   const double* Ao = Aout + (long)g * NFLD * P;
   double Wb[4], Gb[8];

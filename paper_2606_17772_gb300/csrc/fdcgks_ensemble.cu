@@ -63,13 +63,16 @@ struct PhaseQ {
 // tile width of the points phase in the pair form (two lanes per point, so
 // ENS_THREADS / 2 points per tile): 2^min(lbx, 6)
 __host__ __device__ inline int ens_points_lbx(int lbx) { return lbx < 6 ? lbx : 6; }
+// tile width of the mixed update (update_block<4>: 32 lanes of 4 rows, so
+// ENS_THREADS nodes at most 32 wide)
+__host__ __device__ inline int ens_update_lbx(bool mixed, int lbx) { return mixed && lbx > 5 ? 5 : lbx; }
 
 template <class R, int PH> struct EnsMinB { static constexpr int v = 1; };
 template <class R> struct EnsMinB<R, PH_NODAL> { static constexpr int v = PointTune<R>::nodal_minb; };
 template <class R> struct EnsMinB<R, PH_POINTS> {
   static constexpr int v = PointTune<R>::pair_minb;
 };
-template <class R> struct EnsMinB<R, PH_UPDATE> { static constexpr int v = PointTune<R>::update_minb; };
+template <class R> struct EnsMinB<R, PH_UPDATE> { static constexpr int v = IsF32<R>::v ? UpdRows<4>::minb : 1; };
 
 template <class R>
 __device__ __forceinline__ void copy_args(KArgs<R>& dst, const KArgs<R>* src) {
@@ -94,6 +97,7 @@ template <class R, int PH, int PERSIST>
 __global__ void __launch_bounds__(ENS_THREADS, (EnsMinB<R, PH>::v)) ens_phase_kernel(const KArgs<R>* args, PhaseQ q) {
   __shared__ KArgs<R> sa;
   __shared__ int s_tile;
+  __shared__ float sw[PH == PH_UPDATE && IsF32<R>::v ? 4 : 1][4][32];
   for (int iter = 0;; ++iter) {
     const int t = next_tile<PERSIST>(q, iter, &s_tile);
     if (t >= q.ntiles) break;
@@ -119,8 +123,16 @@ __global__ void __launch_bounds__(ENS_THREADS, (EnsMinB<R, PH>::v)) ens_phase_ke
         const int pi_x = (tl.z << lbp) + (pi & ((1 << lbp) - 1));
         const int pj = tl.w * ((ENS_THREADS / 2) >> lbp) + (pi >> lbp);
         point_pair_body<R, false>(sa, tl.y, pi_x - 2, pj - 2, threadIdx.x & 1);
-      } else {
-        update_body(sa, q.stage == 0 ? UPD_STAGE1 : UPD_STAGE2, tl.y, i, j);
+      } else if constexpr (PH == PH_UPDATE) {
+        const int mode = q.stage == 0 ? UPD_STAGE1 : UPD_STAGE2;
+        if constexpr (IsF32<R>::v) {
+          const int lb = ens_update_lbx(true, q.lbx), lane = threadIdx.x & 31;
+          update_block<4>(sa, mode, tl.y,
+                          make_int2((tl.z << lb) + (lane & ((1 << lb) - 1)),
+                                    tl.w * (ENS_THREADS >> lb) + 4 * (lane >> lb)), sw);
+        } else {
+          update_body(sa, mode, tl.y, i, j);
+        }
       }
     }
     __syncthreads();   // sa and s_tile are rewritten by the next tile
@@ -411,7 +423,7 @@ fdcgks_status build_tiles(fdcgks_ens_t e) {
               for (int tx = 0; tx < (w + bx - 1) / bx; ++tx) t.push_back(make_int4(m, g, tx, ty));
             break;
           }
-          case PH_UPDATE: rect(m, g, nxg, nyg, e->cfg.lbx[2]); break;
+          case PH_UPDATE: rect(m, g, nxg, nyg, ens_update_lbx(e->precision == FDCGKS_MIXED, e->cfg.lbx[2])); break;
           case PH_CFL: {
             const long nn = (long)nxg * nyg;
             for (long k = 0; k < nn; k += CFL_TILE) t.push_back(make_int4(m, g, (int)k, 0));

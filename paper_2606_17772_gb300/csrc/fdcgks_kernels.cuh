@@ -10,15 +10,10 @@
 #include "fdcgks_internal.cuh"
 
 // Tuning knobs of the interface-point kernel (defaults are the tuned values):
-// FDK_UPDATE_MINB_F32, FDK_NODAL_MINB_F32  minimum resident blocks per SM in
-//                  the launch bounds (caps registers per thread) of the FP32
-//                  update and nodal kernels (the FP64 kernels are FP64-pipe bound and
-//                  are left uncapped).  1024^2 vortex, ms per mixed step:
-//                  update 4, 5, 6, 8 gave 0.448, 0.411, 0.382, 0.437; nodal
-//                  (its loads issued together) 5, 6 give 0.116, 0.115
-#ifndef FDK_UPDATE_MINB_F32
-#define FDK_UPDATE_MINB_F32 6
-#endif
+// FDK_NODAL_MINB_F32  minimum resident blocks per SM in the launch bounds (caps
+//                  registers per thread) of the FP32 nodal kernel (the FP64
+//                  kernels are FP64-pipe bound and are left uncapped).  1024^2
+//                  vortex, ms per mixed step: 5, 6 give 0.116, 0.115
 #ifndef FDK_NODAL_MINB_F32
 #define FDK_NODAL_MINB_F32 6
 #endif
@@ -52,12 +47,10 @@ namespace fdk {
 
 template <class R> struct PointTune;
 template <> struct PointTune<double> {
-  static constexpr int update_minb = 1;
   static constexpr int nodal_minb = 1;
   static constexpr int pair_minb = FDK_POINT_PAIR_MINB_F64;
 };
 template <> struct PointTune<float> {
-  static constexpr int update_minb = FDK_UPDATE_MINB_F32;
   static constexpr int nodal_minb = FDK_NODAL_MINB_F32;
   static constexpr int pair_minb = FDK_POINT_PAIR_MINB_F32;
 };
@@ -436,13 +429,12 @@ __global__ void __launch_bounds__(StageTune<R>::threads, PointTune<R>::pair_minb
 // one node's stage operator: L, dL/dt (per component), the averaged gradients
 // re-evaluated from the interface solution (node's own side) and their time
 // derivatives
-template <class R>
 struct NodeOp {
-  R L[4], Lt[4], gbx[4], gby[4], gtx[4], gty[4];
+  double L[4], Lt[4], gbx[4], gby[4], gtx[4], gty[4];
 };
 
-template <class R>
-__device__ __forceinline__ void node_operator(const KArgs<R>& a, int g, int i, int j, bool want_n, NodeOp<R>& o) {
+__device__ __forceinline__ void node_operator(const KArgs<double>& a, int g, int i, int j, bool want_n, NodeOp& o) {
+  using R = double;
   const Layout& L = a.L;
   const long pp = L.pplane;
   // x-interface k+1/2 of this grid's row and y-interface k+1/2 of its column
@@ -458,11 +450,9 @@ __device__ __forceinline__ void node_operator(const KArgs<R>& a, int g, int i, i
   const long ym2 = yi(j - 2), ym1 = yi(j - 1), y0 = yi(j), yp1 = yi(j + 1);
   const R chixm = PX[PO_CHI * pp + xm1], chix0 = PX[PO_CHI * pp + x0];
   const R chiym = PY[PO_CHI * pp + ym1], chiy0 = PY[PO_CHI * pp + y0];
-  if constexpr (!IsF32<R>::v) {
-    // FP64, bound by the FP64 pipe: the short form of the flux difference where
-    // all four interfaces are smooth (1024^2 vortex: 2.77 -> 1.39 ms per step).
-    // The FP32 kernel below is bound by memory; there the second copy of the
-    // loads costs registers and 18 % of its time
+  // bound by the FP64 pipe: the short form of the flux difference where all
+  // four interfaces are smooth (1024^2 vortex: 2.77 -> 1.39 ms per step)
+  {
     auto components = [&](auto sm) {
       constexpr bool SMOOTH = decltype(sm)::value;
 #pragma unroll
@@ -488,39 +478,6 @@ __device__ __forceinline__ void node_operator(const KArgs<R>& a, int g, int i, i
     };
     if (chixm == R(1) && chix0 == R(1) && chiym == R(1) && chiy0 == R(1)) components(std::true_type());
     else components(std::false_type());
-  } else {
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const R* nF = NF + (long)c * L.plane;
-      const R* nG = NF + (long)(4 + c) * L.plane;
-      const R* nFt = NF + (long)(8 + c) * L.plane;
-      const R* nGt = NF + (long)(12 + c) * L.plane;
-      const R* pF = PX + (long)(PO_F + c) * pp;
-      const R* pFt = PX + (long)(PO_FT + c) * pp;
-      const R* qF = PY + (long)(PO_F + c) * pp;
-      const R* qFt = PY + (long)(PO_FT + c) * pp;
-      {
-        R fp = compact_flux(fv, chix0, pFt[xm1], pFt[x0], pFt[xp1], nFt[cN], nFt[cN + 1]);
-        R fm = compact_flux(fv, chixm, pFt[xm2], pFt[xm1], pFt[x0], nFt[cN - 1], nFt[cN]);
-        R gp = compact_flux(fv, chiy0, qFt[ym1], qFt[y0], qFt[yp1], nGt[cN], nGt[cN + L.pitch]);
-        R gm = compact_flux(fv, chiym, qFt[ym2], qFt[ym1], qFt[y0], nGt[cN - L.pitch], nGt[cN]);
-        o.Lt[c] = -(fp - fm) * ihx - (gp - gm) * ihy;
-      }
-      o.L[c] = R(0);
-      o.gbx[c] = R(0);
-      o.gby[c] = R(0);
-      if (want_n) {
-        R fp = compact_flux(fv, chix0, pF[xm1], pF[x0], pF[xp1], nF[cN], nF[cN + 1]);
-        R fm = compact_flux(fv, chixm, pF[xm2], pF[xm1], pF[x0], nF[cN - 1], nF[cN]);
-        R gp = compact_flux(fv, chiy0, qF[ym1], qF[y0], qF[yp1], nG[cN], nG[cN + L.pitch]);
-        R gm = compact_flux(fv, chiym, qF[ym2], qF[ym1], qF[y0], nG[cN - L.pitch], nG[cN]);
-        o.L[c] = -(fp - fm) * ihx - (gp - gm) * ihy;
-        o.gbx[c] = (PX[(PO_WL + c) * pp + x0] - PX[(PO_WR + c) * pp + xm1]) * ihx;
-        o.gby[c] = (PY[(PO_WL + c) * pp + y0] - PY[(PO_WR + c) * pp + ym1]) * ihy;
-      }
-      o.gtx[c] = (PX[(PO_WLT + c) * pp + x0] - PX[(PO_WRT + c) * pp + xm1]) * ihx;
-      o.gty[c] = (PY[(PO_WLT + c) * pp + y0] - PY[(PO_WRT + c) * pp + ym1]) * ihy;
-    }
   }
 }
 
@@ -539,12 +496,11 @@ __device__ __forceinline__ void ff_add(float& hi, float& lo, float b) {
   lo = e - (hi - s);
 }
 
-template <class R>
-__device__ __forceinline__ void update_body(const KArgs<R>& a, int mode, int g, int i, int j) {
+__device__ __forceinline__ void update_body(const KArgs<double>& a, int mode, int g, int i, int j) {
   const Layout& L = a.L;
   const int nxg = g == 0 ? L.nx : L.nxd, nyg = g == 0 ? L.ny : L.nyd;
   if (i < 0 || j < 0 || i >= nxg || j >= nyg) return;
-  NodeOp<R> o;
+  NodeOp o;
   node_operator(a, g, i, j, mode != UPD_STAGE2, o);
   const long c0 = cell(L, i, j);
   if (mode == UPD_OPERATOR) {
@@ -567,93 +523,15 @@ __device__ __forceinline__ void update_body(const KArgs<R>& a, int mode, int g, 
   const bool ywall = g == 1 && ((a.bc[2] == 3 && j == 0) || (a.bc[3] == 3 && j == nyg - 1));
   const long P = L.plane;
 
-  if constexpr (IsF32<R>::v) {
-    // mixed path: state and accumulators are float-float pairs; increments are
-    // formed in FP32 and added exactly (two_sum) to the pairs
-    const float dtr = a.gas.dt_r;
-    float Wh[4], Wl[4], Gh[8], Gl[8];
-    const float* Snh = a.Sn_hi + (long)g * NFLD * P;
-    const float* Snl = a.Sn_lo + (long)g * NFLD * P;
-    float* Ah = a.Acc_hi + (long)g * 4 * P;
-    float* Al = a.Acc_lo + (long)g * 4 * P;
-    float* Bh = a.Gb_hi + (long)g * 8 * P;
-    float* Bl = a.Gb_lo + (long)g * 8 * P;
-    // every input pair is loaded before the first store, so that the loads
-    // are issued together (the stores could alias them for the compiler)
-    if (mode == UPD_STAGE1) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        Wh[c] = Snh[(long)c * P + c0];
-        Wl[c] = Snl[(long)c * P + c0];
-      }
-#pragma unroll
-      for (int f = 0; f < 8; ++f) {
-        Gh[f] = a.grad_base ? Snh[(long)(4 + f) * P + c0] : (f < 4 ? o.gbx[f] : o.gby[f - 4]);
-        Gl[f] = a.grad_base ? Snl[(long)(4 + f) * P + c0] : 0.0f;
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const float wh = Wh[c], wl = Wl[c];
-        ff_add(Wh[c], Wl[c], 0.5f * dtr * o.L[c] + 0.125f * dtr * dtr * o.Lt[c]);
-        float ah = wh, al = wl;
-        ff_add(ah, al, dtr * o.L[c] + dtr * dtr * (1.0f / 6.0f) * o.Lt[c]);
-        Ah[(long)c * P + c0] = ah;
-        Al[(long)c * P + c0] = al;
-      }
-      // the gradient base: re-evaluated gradients are FP32 values (low part 0,
-      // not stored); a base taken from the state keeps its low part
-#pragma unroll
-      for (int f = 0; f < 8; ++f) {
-        Bh[(long)f * P + c0] = Gh[f];
-        if (a.grad_base) Bl[(long)f * P + c0] = Gl[f];
-        ff_add(Gh[f], Gl[f], 0.5f * dtr * (f < 4 ? o.gtx[f] : o.gty[f - 4]));
-      }
-    } else {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        Wh[c] = Ah[(long)c * P + c0];
-        Wl[c] = Al[(long)c * P + c0];
-      }
-#pragma unroll
-      for (int f = 0; f < 8; ++f) {
-        Gh[f] = Bh[(long)f * P + c0];
-        Gl[f] = a.grad_base ? Bl[(long)f * P + c0] : 0.0f;
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) ff_add(Wh[c], Wl[c], dtr * dtr * (1.0f / 3.0f) * o.Lt[c]);
-#pragma unroll
-      for (int f = 0; f < 8; ++f) ff_add(Gh[f], Gl[f], dtr * (f < 4 ? o.gtx[f] : o.gty[f - 4]));
-    }
-    if (xwall || ywall) {
-      float ke = 0.5f * (Wh[1] * Wh[1] + Wh[2] * Wh[2]) / Wh[0];
-      Wh[1] = Wl[1] = Wh[2] = Wl[2] = 0.0f;
-      ff_add(Wh[3], Wl[3], -ke);
-    }
-    if (xwall) { Gh[5] = Gl[5] = Gh[6] = Gl[6] = 0.0f; }   // y-gradients of rho U, rho V
-    if (ywall) { Gh[1] = Gl[1] = Gh[2] = Gl[2] = 0.0f; }   // x-gradients of rho U, rho V
-    float* Oh = a.Out_hi + (long)g * NFLD * P;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) Oh[(long)c * P + c0] = Wh[c];
-#pragma unroll
-    for (int f = 0; f < 8; ++f) Oh[(long)(4 + f) * P + c0] = Gh[f];
-    if (a.Out_lo) {
-      float* Ol = a.Out_lo + (long)g * NFLD * P;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) Ol[(long)c * P + c0] = Wl[c];
-#pragma unroll
-      for (int f = 0; f < 8; ++f) Ol[(long)(4 + f) * P + c0] = Gl[f];
-    }
-    float pr = Wh[3] - 0.5f * (Wh[1] * Wh[1] + Wh[2] * Wh[2]) / Wh[0];
-    if (!(Wh[0] > 0.0f) || !(pr > 0.0f)) atomicOr(a.flag, 1);
-  } else {
-    // FP64 path
+  {
     const double dt = a.dt;
     const double* Sng = a.Sn + (long)g * NFLD * P;
     double* Og = a.Sout + (long)g * NFLD * P;
     double* Ag = a.Wacc + (long)g * 4 * P;
     double* Bg = a.gB + (long)g * 8 * P;
     double Wnew[4], Gnew[8];
-    // inputs first, then the stores (see the mixed branch)
+    // every input is loaded before the first store, so that the loads are
+    // issued together (the stores could alias them for the compiler)
     if (mode == UPD_STAGE1) {
       double Wn[4], Gb[8];
 #pragma unroll
@@ -700,9 +578,238 @@ __device__ __forceinline__ void update_body(const KArgs<R>& a, int mode, int g, 
   }
 }
 
-template <class R>
-__global__ void __launch_bounds__(128, PointTune<R>::update_minb) update_kernel(KArgs<R> a, int mode) {
+static __global__ void __launch_bounds__(128) update_kernel(KArgs<double> a, int mode) {
   update_body(a, mode, blockIdx.z, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y);
+}
+
+// ---------------------------------------------------------------------------
+// The mixed update: one thread per component and column of ROWS nodes, the
+// component the index of the warp in its block of four, which covers 32 ROWS
+// nodes.  It is bound by the latency and number of its loads (148 a node, DRAM
+// 46 % busy), not by arithmetic: a thread of one component needs few enough
+// registers to have a column's loads in flight together, and its rows share
+// the interfaces between them (20 loads a component and node of 4 rows where
+// one node takes 28).  ms per step of the update against one thread per node
+// with all four components:
+//             33^2    128^2   512^2   1024^2
+//   by node   0.0195  0.0215  0.104   0.345
+//   1 row     0.0147  0.0166  0.126   0.447   (40 registers: 0.106, 0.363)
+//   2 rows    0.0188  0.0204  0.0988  0.325   (40 registers; 64: 0.0996, 0.334)
+//   4 rows    0.0198  0.0216  0.0964  0.312   (64 registers; 48: 0.1135, 0.369)
+//   8 rows    0.0376  0.0358  0.147   0.438   (80 registers)
+// ---------------------------------------------------------------------------
+// Rows a thread: 1 where the whole grid is then one wave of blocks (12 an SM,
+// 152 SMs, two grids in blocks of 32 nodes), 4 where it fills the GPU anyway
+// (the table above), 2 between (200^2 nodes, step: 1, 2, 4 rows 0.0742, 0.0692,
+// 0.0700 ms; 256^2 0.0966, 0.0946, 0.0944).
+template <int ROWS> struct UpdRows { static constexpr int minb = 12; };
+template <> struct UpdRows<4> { static constexpr int minb = 8; };
+const long UPD_SMALL_NODES = 29000, UPD_LARGE_NODES = 100000;
+
+// what one component of one node of the mixed update hands to its second half
+struct CompOut {
+  float Wh, Wl, gxh, gxl, gyh, gyl;
+};
+
+// component c of rows j..j + ROWS - 1 of column i, `rows` >= 1 of which exist
+template <int ROWS>
+__device__ __forceinline__ void update_comp(const KArgs<float>& a, int mode, int g, int c, int i, int j, int rows,
+                                            CompOut o[ROWS]) {
+  const Layout& L = a.L;
+  const long pp = L.pplane, P = L.plane;
+  const bool want_n = mode != UPD_STAGE2;
+  const int fv = a.flux_variant;
+  const float ihx = a.ih[0], ihy = a.ih[1];
+  const long xc = g == 0 ? pcell(L, i, j) : pcell(L, i, j - 1), yc = g == 0 ? pcell(L, i, j) : pcell(L, i - 1, j);
+  const float* PX = (g == 0 ? a.PA : a.PB + NPS * pp) + xc;
+  const float* PY = (g == 0 ? a.PB : a.PA + NPS * pp) + yc;
+  const float* PXc = PX + (long)c * pp;
+  const float* PYc = PY + (long)c * pp;
+  const long c0 = cell(L, i, j);
+  const float* NF = a.NF + ((long)g * NNF + c) * P + c0;
+  const int sp = L.ppitch, sn = L.pitch;
+  auto rr = [&](int r) { return ROWS > 1 ? min(r, rows - 1) : r; };   // rows past the grid: its last one
+  float chx[2 * ROWS], chy[ROWS + 1];
+#pragma unroll
+  for (int r = 0; r < ROWS; ++r) {
+    chx[2 * r] = PX[PO_CHI * pp + rr(r) * sp - 1];
+    chx[2 * r + 1] = PX[PO_CHI * pp + rr(r) * sp];
+  }
+#pragma unroll
+  for (int r = 0; r <= ROWS; ++r) chy[r] = PY[PO_CHI * pp + (ROWS > 1 ? min(r, rows) - 1 : r - 1) * sp];
+  // compact_flux with its roundings spelled out, as every sum of products below:
+  // the kernels that inline this for other ROWS give the same bits
+  auto flux = [&](float chi, float Fm, float F0, float Fp, float N0, float N1) {
+    const float hi = __fmul_rn(__fmaf_rn(-9.0f, N0 + N1, __fmaf_rn(46.0f, F0, Fm) + Fp), 1.0f / 30.0f);
+    const float lo = fv == 62 ? F0 : __fmul_rn(__fmaf_rn(8.0f, F0, -N0) - N1, 1.0f / 6.0f);
+    return __fmaf_rn(chi, hi, __fmul_rn(1.0f - chi, lo));
+  };
+  float Ll[2][ROWS];
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {   // F_t, then F
+    if (d == 1 && !want_n) {
+#pragma unroll
+      for (int r = 0; r < ROWS; ++r) Ll[1][r] = 0.0f;
+      continue;
+    }
+    const int po = d == 0 ? PO_FT : PO_F, no = d == 0 ? 8 : 0;
+    const float* f = PXc + po * pp;
+    const float* q = PYc + po * pp;
+    const float* n = NF + no * P;
+    const float* m = NF + (no + 4) * P;
+    float y[ROWS + 3], ny[ROWS + 2];
+#pragma unroll
+    for (int r = 0; r < ROWS + 3; ++r) y[r] = q[(ROWS > 1 ? min(r, rows + 2) - 2 : r - 2) * sp];
+#pragma unroll
+    for (int r = 0; r < ROWS + 2; ++r) ny[r] = m[(ROWS > 1 ? min(r, rows + 1) - 1 : r - 1) * sn];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+      const float* fr = f + rr(r) * sp;
+      const float* nr = n + rr(r) * sn;
+      const float x0 = fr[-2], x1 = fr[-1], x2 = fr[0], x3 = fr[1], n0 = nr[-1], n1 = nr[0], n2 = nr[1];
+      const float fp = flux(chx[2 * r + 1], x1, x2, x3, n1, n2);
+      const float fm = flux(chx[2 * r], x0, x1, x2, n0, n1);
+      const float gp = flux(chy[r + 1], y[r + 1], y[r + 2], y[r + 3], ny[r + 1], ny[r + 2]);
+      const float gm = flux(chy[r], y[r], y[r + 1], y[r + 2], ny[r], ny[r + 1]);
+      Ll[d][r] = __fmaf_rn(gm - gp, ihy, __fmul_rn(fm - fp, ihx));
+    }
+  }
+  float gbx[ROWS], gby[ROWS], gtx[ROWS], gty[ROWS];
+#pragma unroll
+  for (int r = 0; r < ROWS; ++r) {
+    const float* x = PXc + rr(r) * sp;
+    const float* y = PYc + rr(r) * sp;
+    gtx[r] = __fmul_rn(x[PO_WLT * pp] - x[PO_WRT * pp - 1], ihx);
+    gty[r] = __fmul_rn(y[PO_WLT * pp] - y[PO_WRT * pp - sp], ihy);
+    gbx[r] = gby[r] = 0.0f;
+    if (want_n && (!a.grad_base || mode == UPD_OPERATOR)) {
+      gbx[r] = __fmul_rn(x[PO_WL * pp] - x[PO_WR * pp - 1], ihx);
+      gby[r] = __fmul_rn(y[PO_WL * pp] - y[PO_WR * pp - sp], ihy);
+    }
+  }
+  if (mode == UPD_OPERATOR) {
+    const int nxg = g == 0 ? L.nx : L.nxd, nyg = g == 0 ? L.ny : L.nyd;
+    const long NN = (long)nxg * nyg, oi = (long)j * nxg + i;
+    double* const* op = a.op + 4 * g;
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+      if (r >= rows) break;
+      const long k = oi + (long)r * nxg;
+      op[0][c * NN + k] = (double)Ll[1][r];
+      op[1][c * NN + k] = (double)Ll[0][r];
+      op[2][c * NN + k] = (double)gbx[r];
+      op[2][(4 + c) * NN + k] = (double)gby[r];
+      op[3][c * NN + k] = (double)gtx[r];
+      op[3][(4 + c) * NN + k] = (double)gty[r];
+    }
+    return;
+  }
+  // state and accumulators are float-float pairs; increments are formed in
+  // FP32 and added exactly (two_sum) to the pairs
+  const float dtr = a.gas.dt_r;
+  const long sc = ((long)g * NFLD + c) * P + c0, ac = ((long)g * 4 + c) * P + c0, bc = ((long)g * 8 + c) * P + c0;
+#pragma unroll
+  for (int r = 0; r < ROWS; ++r) {
+    if (r >= rows) break;
+    CompOut& v = o[r];
+    const long k = (long)r * sn;
+    if (mode == UPD_STAGE1) {
+      v.Wh = a.Sn_hi[sc + k];
+      v.Wl = a.Sn_lo[sc + k];
+      v.gxh = gbx[r]; v.gxl = 0.0f;
+      v.gyh = gby[r]; v.gyl = 0.0f;
+      if (a.grad_base) {
+        v.gxh = a.Sn_hi[sc + 4 * P + k]; v.gxl = a.Sn_lo[sc + 4 * P + k];
+        v.gyh = a.Sn_hi[sc + 8 * P + k]; v.gyl = a.Sn_lo[sc + 8 * P + k];
+      }
+      float ah = v.Wh, al = v.Wl;
+      ff_add(v.Wh, v.Wl, __fmaf_rn(0.125f * dtr * dtr, Ll[0][r], __fmul_rn(0.5f * dtr, Ll[1][r])));
+      ff_add(ah, al, __fmaf_rn(dtr * dtr * (1.0f / 6.0f), Ll[0][r], __fmul_rn(dtr, Ll[1][r])));
+      a.Acc_hi[ac + k] = ah;
+      a.Acc_lo[ac + k] = al;
+      // the gradient base: re-evaluated gradients are FP32 values (low part 0,
+      // not stored); a base taken from the state keeps its low part
+      a.Gb_hi[bc + k] = v.gxh;
+      a.Gb_hi[bc + 4 * P + k] = v.gyh;
+      if (a.grad_base) {
+        a.Gb_lo[bc + k] = v.gxl;
+        a.Gb_lo[bc + 4 * P + k] = v.gyl;
+      }
+      ff_add(v.gxh, v.gxl, __fmul_rn(0.5f * dtr, gtx[r]));
+      ff_add(v.gyh, v.gyl, __fmul_rn(0.5f * dtr, gty[r]));
+    } else {
+      v.Wh = a.Acc_hi[ac + k];
+      v.Wl = a.Acc_lo[ac + k];
+      v.gxh = a.Gb_hi[bc + k];
+      v.gyh = a.Gb_hi[bc + 4 * P + k];
+      v.gxl = a.grad_base ? a.Gb_lo[bc + k] : 0.0f;
+      v.gyl = a.grad_base ? a.Gb_lo[bc + 4 * P + k] : 0.0f;
+      ff_add(v.Wh, v.Wl, __fmul_rn(dtr * dtr * (1.0f / 3.0f), Ll[0][r]));
+      ff_add(v.gxh, v.gxl, __fmul_rn(dtr, gtx[r]));
+      ff_add(v.gyh, v.gyl, __fmul_rn(dtr, gty[r]));
+    }
+  }
+}
+
+// second half: the walls, the stores and the positivity flag; W[comp] are the
+// four components' high parts of the node (before the walls)
+__device__ __forceinline__ void update_comp_store(const KArgs<float>& a, int g, int c, int i, int j, CompOut v,
+                                                  float w0, float w1, float w2) {
+  const Layout& L = a.L;
+  const int nxg = g == 0 ? L.nx : L.nxd, nyg = g == 0 ? L.ny : L.nyd;
+  // dual nodes on a no-slip wall: velocity set to zero (internal energy kept),
+  // and, as U = V = 0 along the whole wall, the momentum gradients along it too
+  const bool xwall = g == 1 && ((a.bc[0] == 3 && i == 0) || (a.bc[1] == 3 && i == nxg - 1));
+  const bool ywall = g == 1 && ((a.bc[2] == 3 && j == 0) || (a.bc[3] == 3 && j == nyg - 1));
+  if (xwall || ywall) {
+    if (c == 3) ff_add(v.Wh, v.Wl, __fmul_rn(-0.5f, __fmaf_rn(w2, w2, __fmul_rn(w1, w1))) / w0);
+    if (c == 1 || c == 2) {
+      v.Wh = v.Wl = 0.0f;
+      if (xwall) v.gyh = v.gyl = 0.0f;   // y-gradients of rho U, rho V
+      if (ywall) v.gxh = v.gxl = 0.0f;   // x-gradients of rho U, rho V
+    }
+    w1 = w2 = 0.0f;
+  }
+  const long k = ((long)g * NFLD + c) * L.plane + cell(L, i, j);
+  a.Out_hi[k] = v.Wh;
+  a.Out_hi[k + 4 * L.plane] = v.gxh;
+  a.Out_hi[k + 8 * L.plane] = v.gyh;
+  if (a.Out_lo) {
+    a.Out_lo[k] = v.Wl;
+    a.Out_lo[k + 4 * L.plane] = v.gxl;
+    a.Out_lo[k + 8 * L.plane] = v.gyl;
+  }
+  if (c == 3) {
+    const float pr = v.Wh - 0.5f * (w1 * w1 + w2 * w2) / w0;
+    if (!(w0 > 0.0f) || !(pr > 0.0f)) atomicOr(a.flag, 1);
+  }
+}
+
+// A block's nodes: lane l takes ROWS rows from column and row `at`.  The
+// components meet in shared memory for the walls and the positivity test.
+template <int ROWS>
+__device__ __forceinline__ void update_block(const KArgs<float>& a, int mode, int g, int2 at, float (*sw)[4][32]) {
+  const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nxg = g == 0 ? a.L.nx : a.L.nxd, nyg = g == 0 ? a.L.ny : a.L.nyd;
+  const bool in = at.x < nxg && at.y < nyg;
+  CompOut o[ROWS];
+  if (in) {
+    update_comp<ROWS>(a, mode, g, c, at.x, at.y, nyg - at.y, o);
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) sw[r][c][lane] = o[r].Wh;
+  }
+  if (mode == UPD_OPERATOR) return;
+  __syncthreads();
+  if (!in) return;
+#pragma unroll
+  for (int r = 0; r < ROWS; ++r)
+    if (at.y + r < nyg) update_comp_store(a, g, c, at.x, at.y + r, o[r], sw[r][0][lane], sw[r][1][lane], sw[r][2][lane]);
+}
+
+template <int ROWS>
+__global__ void __launch_bounds__(128, UpdRows<ROWS>::minb) update_comp_kernel(KArgs<float> a, int mode) {
+  __shared__ float sw[ROWS][4][32];
+  update_block<ROWS>(a, mode, blockIdx.z, make_int2(blockIdx.x * 32 + (threadIdx.x & 31), blockIdx.y * ROWS), sw);
 }
 
 // ---------------------------------------------------------------------------
@@ -754,9 +861,16 @@ cudaError_t launch_points(const KArgs<R>& a, bool nodal, cudaStream_t s) {
 
 template <class R>
 cudaError_t launch_update(const KArgs<R>& a, int mode, cudaStream_t s) {
-  dim3 b(32, 4);
-  int mx = a.L.nx > a.L.nxd ? a.L.nx : a.L.nxd, my = a.L.ny > a.L.nyd ? a.L.ny : a.L.nyd;
-  update_kernel<R><<<grid2(mx, my, b, 2), b, 0, s>>>(a, mode);
+  const int mx = a.L.nx > a.L.nxd ? a.L.nx : a.L.nxd, my = a.L.ny > a.L.nyd ? a.L.ny : a.L.nyd;
+  if constexpr (IsF32<R>::v) {
+    const long nn = (long)mx * my;
+    if (nn > UPD_LARGE_NODES) update_comp_kernel<4><<<grid2(mx, my, dim3(32, 4), 2), 128, 0, s>>>(a, mode);
+    else if (nn > UPD_SMALL_NODES) update_comp_kernel<2><<<grid2(mx, my, dim3(32, 2), 2), 128, 0, s>>>(a, mode);
+    else update_comp_kernel<1><<<grid2(mx, my, dim3(32, 1), 2), 128, 0, s>>>(a, mode);
+  } else {
+    const dim3 b(32, 4);
+    update_kernel<<<grid2(mx, my, b, 2), b, 0, s>>>(a, mode);
+  }
   return cudaGetLastError();
 }
 
