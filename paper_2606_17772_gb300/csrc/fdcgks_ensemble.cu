@@ -70,7 +70,7 @@ __host__ __device__ inline int ens_update_lbx(bool mixed, int lbx) { return mixe
 template <class R, int PH> struct EnsMinB { static constexpr int v = 1; };
 template <class R> struct EnsMinB<R, PH_NODAL> { static constexpr int v = PointTune<R>::nodal_minb; };
 template <class R> struct EnsMinB<R, PH_POINTS> {
-  static constexpr int v = PointTune<R>::pair_minb;
+  static constexpr int v = PointTune<R>::alone_minb;   // mixed_40, ms per step: 4 and 5 blocks 2.085, 2.005
 };
 template <class R> struct EnsMinB<R, PH_UPDATE> { static constexpr int v = IsF32<R>::v ? UpdRows<4>::minb : 1; };
 

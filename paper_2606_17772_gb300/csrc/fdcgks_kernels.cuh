@@ -22,8 +22,18 @@
 // FDK_POINT_PAIR_MINB_F32 / _F64  minimum resident blocks per SM of the pair
 //                  kernel (FP32 without preload: 2, 3, 4, 5 gave 1.43, 1.06,
 //                  0.915, 0.903 ms; with preload 4 and 5 give 0.822 and 0.840)
+// FDK_POINT_ALONE_MINB_F32  the same for the FP32 stage kernel of points alone
+//                  and conservative reconstruction, whose 20 live registers
+//                  more spill little: 4 and 5 give 0.495 and 0.467 ms at
+//                  1024^2 (6: 0.480), tube 1000x500 0.488 and 0.479 a step;
+//                  with the nodes merged in 5 loses (128^2 step 0.0478 ->
+//                  0.0505), and so does the characteristic form (960x240
+//                  0.289 -> 0.292)
 #ifndef FDK_POINT_PAIR_MINB_F32
 #define FDK_POINT_PAIR_MINB_F32 4
+#endif
+#ifndef FDK_POINT_ALONE_MINB_F32
+#define FDK_POINT_ALONE_MINB_F32 5
 #endif
 #ifndef FDK_POINT_PAIR_MINB_F64
 #define FDK_POINT_PAIR_MINB_F64 1
@@ -48,11 +58,11 @@ namespace fdk {
 template <class R> struct PointTune;
 template <> struct PointTune<double> {
   static constexpr int nodal_minb = 1;
-  static constexpr int pair_minb = FDK_POINT_PAIR_MINB_F64;
+  static constexpr int pair_minb = FDK_POINT_PAIR_MINB_F64, alone_minb = pair_minb;
 };
 template <> struct PointTune<float> {
   static constexpr int nodal_minb = FDK_NODAL_MINB_F32;
-  static constexpr int pair_minb = FDK_POINT_PAIR_MINB_F32;
+  static constexpr int pair_minb = FDK_POINT_PAIR_MINB_F32, alone_minb = FDK_POINT_ALONE_MINB_F32;
 };
 
 // ---------------------------------------------------------------------------
@@ -381,7 +391,9 @@ template <> struct StageTune<double> { static constexpr int threads = FDK_STAGE_
 template <> struct StageTune<float> { static constexpr int threads = 128; };
 
 template <class R, bool CHAR, bool NODAL>
-__global__ void __launch_bounds__(StageTune<R>::threads, PointTune<R>::pair_minb * 128 / StageTune<R>::threads)
+__global__ void __launch_bounds__(StageTune<R>::threads,
+                                  (CHAR || NODAL ? PointTune<R>::pair_minb : PointTune<R>::alone_minb) * 128 /
+                                      StageTune<R>::threads)
     stage_kernel(KArgs<R> a, StageGrid G) {
   const int T = StageTune<R>::threads;
   if constexpr (IsF32<R>::v) {
