@@ -585,8 +585,10 @@ __device__ __forceinline__ void update_body(const KArgs<double>& a, int mode, in
 #pragma unroll
     for (int f = 0; f < 8; ++f) Og[(long)(4 + f) * P + c0] = Gnew[f];
     // positivity of density and pressure (no trap: a flag the host reads), p > 0
-    // as 2 E rho > m^2, without a division
-    if (!(Wnew[0] > 0.0) || !(2.0 * Wnew[3] * Wnew[0] > Wnew[1] * Wnew[1] + Wnew[2] * Wnew[2])) atomicOr(a.flag, 1);
+    // as 2 E rho > m^2, without a division unless it fails (products out of range)
+    const double m2 = Wnew[1] * Wnew[1] + Wnew[2] * Wnew[2];
+    if (!(Wnew[0] > 0.0) || (!(2.0 * Wnew[3] * Wnew[0] > m2) && !(Wnew[3] - 0.5 * m2 / Wnew[0] > 0.0)))
+      atomicOr(a.flag, 1);
   }
 }
 

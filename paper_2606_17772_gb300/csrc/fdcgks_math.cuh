@@ -813,11 +813,12 @@ FD_HD void half_flux(const HalfSide<R>& s, R k3, R k4, R k5, R F[4], R Wm[4]) {
 // The distribution is g0 (k0 + k1 (a0 u + b0 v) + k2 A0) on the whole space
 // plus g (k3 + k4 (a u + b v) + k5 A) on each half, k = cn for the value and
 // ct for the time slope; each set's polynomial is formed first, so a side's
-// moments are taken once per set instead of once per basis term: 981 flops
-// instead of the 1667 of moment tables and moment-system solves, and 117
-// instead of 402 for the nodal flux below (GB300, vortex 512^2, ms per step:
-// FP64 points 7.80 -> 5.55, nodal 1.63 -> 1.24; mixed points 0.223 -> 0.174,
-// nodal 0.062 -> 0.051).  The FP64 kernels are bound by the FP64 pipe, which
+// moments are taken once per set instead of once per basis term: 855 flops
+// instead of the 1667 of moment tables and moment-system solves, and 114
+// instead of 402 for the nodal flux below (GB300, vortex 512^2, ms per step,
+// this form alone: FP64 points 7.80 -> 5.55, nodal 1.63 -> 1.24; mixed points
+// 0.223 -> 0.174, nodal 0.062 -> 0.051; with rho-weighted gradients FP64 points
+// 3.41 -> 3.15).  The FP64 kernels are bound by the FP64 pipe, which
 // takes 16 clocks of an SM per warp instruction whatever the occupancy, the
 // FP32 ones by instruction issue: fewer operations is what both need.
 // ---------------------------------------------------------------------------
