@@ -850,10 +850,11 @@ def main():
         equiv["cfl"] = 5
         kf = kernel_fractions(work, pms, pn, equiv, peaks, hbm)
         # measured DRAM bytes per launch (profiles/dram_traffic.json) beside the
-        # algorithmic bytes per launch (a step launches 4 point, 2 nodal, 2 update kernels)
+        # algorithmic bytes per launch (a profiled step launches 2 of each: both
+        # point types in one, the nodes apart)
         rt = "double" if name == "fp64" else "float"
-        for cls, kname, per_step in (("points", "point_pair_kernel<%s>" % rt, 4), ("nodal", "nodal_kernel<%s>" % rt, 2),
-                                     ("update", "update_kernel<%s>" % rt, 2)):
+        for cls, kname, per_step in (("points", "stage_kernel<%s>" % rt, 2), ("nodal", "nodal_kernel<%s>" % rt, 2),
+                                     ("update", "update_kernel" if name == "fp64" else "update_comp_kernel", 2)):
             if cls in kf:
                 kf[cls]["algorithmic_bytes_per_launch"] = work[cls][2] / per_step
                 kf[cls]["dram_bytes_per_launch"] = profiled_traffic(kname, n)
@@ -866,8 +867,8 @@ def main():
     step_ms = {k: v for k, v in fp["prof_ms"].items() if k != "cfl"}
     pk = fp["kernels"]["points"]
     roof = {"bound": "alu", "achieved": pk["achieved_tflops"], "peak": peaks["fp64"], "unit": "TFLOP/s",
-            "frac": pk["alu_frac"], "traffic": profiled_traffic("point_pair_kernel<double>", n),
-            "kernel": "point_kernel<double> (Type A + B interface points)",
+            "frac": pk["alu_frac"], "traffic": profiled_traffic("stage_kernel<double>", n),
+            "kernel": "stage_kernel<double> (Type A + B interface points)",
             "peak_source": "measured FP64 FMA pipe (csrc/pipe_peak.cu), this run",
             "step_share": step_ms["points"] / max(sum(step_ms.values()), 1e-9)}
 

@@ -134,7 +134,8 @@ fdcgks_status fdcgks_steps(fdcgks_t ctx, double dt, int nsteps);
  * lets the scheme's grid-scale diagonal modes grow slowly (visible over
  * thousands of steps, first in mixed precision); cfl 0.2 is stable.
  * Evaluated in FP64 (on the joined float-float pairs in a mixed context) at
- * the nodes that can hold the maxima: a first pass takes FP32 estimates of
+ * every node of a small grid, in one pass.  On larger grids only at the nodes
+ * that can hold the maxima: a first pass takes FP32 estimates of
  * every node's rates, a second evaluates the FP64 rates only where the
  * estimate is unreliable or within a relative 5e-5 of the largest estimate,
  * which is more than twice the estimates' error; the result equals the
@@ -163,9 +164,10 @@ fdcgks_status fdcgks_stage_operator(fdcgks_t ctx, double dt, double* Lp, double*
 
 /* Kernel-class timing: with profiling enabled, every stage records CUDA
  * events on the context stream around its ghost fill, nodal kernel, point
- * kernels (Type A and B) and update kernel, and fdcgks_cfl_dt /
- * fdcgks_cfl_dt_sum around their reduction kernel (with the float-float to
- * FP64 join of the state on mixed contexts).  fdcgks_get_profile waits for
+ * kernel (both types) and update kernel, and fdcgks_cfl_dt /
+ * fdcgks_cfl_dt_sum around their reduction.  Nodes and points, which share a
+ * launch otherwise (FP64, and mixed grids of up to 100,000 nodes), are then
+ * launched apart, to be timed apart.  fdcgks_get_profile waits for
  * the recorded events, returns the summed milliseconds and the number of
  * launch groups per class in ms[5] / count[5] (order: ghost, nodal, points,
  * update, cfl; either may be NULL), clears the record, and returns in
