@@ -130,6 +130,7 @@ static size_t rsize(const fdcgks_params& p) { return p.precision == FDCGKS_MIXED
 // ---------------------------------------------------------------------------
 template <class T, class KINDS>
 __global__ void ghost_kernel(T* S, Layout L, KINDS K) {
+  if constexpr (IsF32<T>::v) step_begin();
   ghost_fill(S, L, K, blockIdx.z, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -162,13 +163,12 @@ static cudaError_t fill_ghosts(fdcgks_t c, T* S, double t) {
   const Layout& L = c->L;
   const dim3 grid((ghost_count(std::max(L.nx, L.nxd), std::max(L.ny, L.nyd)) + 127) / 128, 1, 2);
   if (c->has_sides) {
-    ghost_kernel<<<grid, 128, 0, c->stream>>>(S, L, ghost_sides(c, t));
+    return launch_step(IsF32<T>::v, ghost_kernel<T, GhostSides>, grid, dim3(128), c->stream, S, L, ghost_sides(c, t));
   } else {
     GhostPlain K;
     for (int k = 0; k < 4; ++k) K.bc[k] = c->p.bc[k];
-    ghost_kernel<<<grid, 128, 0, c->stream>>>(S, L, K);
+    return launch_step(IsF32<T>::v, ghost_kernel<T, GhostPlain>, grid, dim3(128), c->stream, S, L, K);
   }
-  return cudaGetLastError();
 }
 
 // mixed path: FP64 state <-> float-float pairs (whole padded planes)
@@ -344,6 +344,7 @@ __device__ __forceinline__ void block_max2(T& a, T& b, T* sa, T* sb) {
 // (cfl_estimate_f) of the rate and of nu.
 template <class ST>
 __global__ void cfl_screen_kernel(ST S, CflGrid G, int items, float2* est) {
+  step_begin();
   __shared__ float sa[32], sb[32];
   float mr = 0.0f, mn = 0.0f;
   const long P = G.L.plane;
@@ -375,6 +376,7 @@ struct CflRes {
 };
 template <class ST, bool ALL>
 __global__ void cfl_kernel(ST S, CflGrid G, int items, const float2* est, int nest, CflRes* res, double* out) {
+  step_begin();
   __shared__ float fa[32], fb[32];
   __shared__ double sa[32], sb[32];
   const long P = G.L.plane;
@@ -583,17 +585,17 @@ template <class ST>
 static cudaError_t launch_cfl(fdcgks_t c, const ST& st, const CflGrid& G, int items) {
   const int blocks = std::min(items, c->red_blocks);
   const Layout& L = c->L;
+  const bool overlap = c->p.precision == FDCGKS_MIXED;
   if ((long)L.nx * L.ny + (long)L.nxd * L.nyd <= CFL_ALL_NODES) {
-    cfl_kernel<ST, true><<<blocks, 256, 0, c->stream>>>(st, G, items, nullptr, 0, c->res, c->res_host);
     c->launches += 1;
-    return cudaGetLastError();
+    return launch_step(overlap, cfl_kernel<ST, true>, dim3(blocks), dim3(256), c->stream, st, G, items, nullptr, 0,
+                       c->res, c->res_host);
   }
-  cfl_screen_kernel<<<blocks, 256, 0, c->stream>>>(st, G, items, c->est);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_step(overlap, cfl_screen_kernel<ST>, dim3(blocks), dim3(256), c->stream, st, G, items, c->est);
   if (e != cudaSuccess) return e;
-  cfl_kernel<ST, false><<<blocks, 256, 0, c->stream>>>(st, G, items, c->est, blocks, c->res, c->res_host);
   c->launches += 2;
-  return cudaGetLastError();
+  return launch_step(overlap, cfl_kernel<ST, false>, dim3(blocks), dim3(256), c->stream, st, G, items, c->est, blocks,
+                     c->res, c->res_host);
 }
 
 // ---------------------------------------------------------------------------

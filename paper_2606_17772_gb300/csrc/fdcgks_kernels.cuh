@@ -135,6 +135,7 @@ __device__ __forceinline__ void nodal_body(const KArgs<R>& a, int g, int i, int 
 
 template <class R>
 __global__ void __launch_bounds__(128, PointTune<R>::nodal_minb) nodal_kernel(KArgs<R> a) {
+  if constexpr (IsF32<R>::v) step_begin();
   nodal_body(a, blockIdx.z, blockIdx.x * blockDim.x + threadIdx.x - 1, blockIdx.y * blockDim.y + threadIdx.y - 1);
 }
 
@@ -395,6 +396,7 @@ __global__ void __launch_bounds__(StageTune<R>::threads,
                                   (CHAR || NODAL ? PointTune<R>::pair_minb : PointTune<R>::alone_minb) * 128 /
                                       StageTune<R>::threads)
     stage_kernel(KArgs<R> a, StageGrid G) {
+  if constexpr (IsF32<R>::v) step_begin();
   const int T = StageTune<R>::threads;
   if constexpr (IsF32<R>::v) {
     int b = blockIdx.x;
@@ -817,12 +819,14 @@ __device__ __forceinline__ void update_block(const KArgs<float>& a, int mode, in
   if (!in) return;
 #pragma unroll
   for (int r = 0; r < ROWS; ++r)
-    if (at.y + r < nyg) update_comp_store(a, g, c, at.x, at.y + r, o[r], sw[r][0][lane], sw[r][1][lane], sw[r][2][lane]);
+    if (at.y + r < nyg)
+      update_comp_store(a, g, c, at.x, at.y + r, o[r], sw[r][0][lane], sw[r][1][lane], sw[r][2][lane]);
 }
 
 template <int ROWS>
 __global__ void __launch_bounds__(128, UpdRows<ROWS>::minb) update_comp_kernel(KArgs<float> a, int mode) {
   __shared__ float sw[ROWS][4][32];
+  step_begin();
   update_block<ROWS>(a, mode, blockIdx.z, make_int2(blockIdx.x * 32 + (threadIdx.x & 31), blockIdx.y * ROWS), sw);
 }
 
@@ -837,8 +841,7 @@ template <class R>
 cudaError_t launch_nodal(const KArgs<R>& a, cudaStream_t s) {
   dim3 b(32, 4);
   int mx = (a.L.nx > a.L.nxd ? a.L.nx : a.L.nxd) + 2, my = (a.L.ny > a.L.nyd ? a.L.ny : a.L.nyd) + 2;
-  nodal_kernel<R><<<grid2(mx, my, b, 2), b, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_step(IsF32<R>::v, nodal_kernel<R>, grid2(mx, my, b, 2), b, s, a);
 }
 
 // interface points, with the nodal work in the same launch if nodal is set
@@ -863,14 +866,9 @@ cudaError_t launch_points(const KArgs<R>& a, bool nodal, cudaStream_t s) {
     const long np = (2L * G.nA + 2L * G.nB + 31) / 32 * 32;
     blocks = (np + (nodal ? (long)G.nN0 + G.nN1 : 0) + T - 1) / T;
   }
-  if (a.recon_vars) {
-    if (nodal) stage_kernel<R, true, true><<<(unsigned)blocks, T, 0, s>>>(a, G);
-    else stage_kernel<R, true, false><<<(unsigned)blocks, T, 0, s>>>(a, G);
-  } else {
-    if (nodal) stage_kernel<R, false, true><<<(unsigned)blocks, T, 0, s>>>(a, G);
-    else stage_kernel<R, false, false><<<(unsigned)blocks, T, 0, s>>>(a, G);
-  }
-  return cudaGetLastError();
+  auto kernel = a.recon_vars ? (nodal ? stage_kernel<R, true, true> : stage_kernel<R, true, false>)
+                             : (nodal ? stage_kernel<R, false, true> : stage_kernel<R, false, false>);
+  return launch_step(IsF32<R>::v, kernel, dim3((unsigned)blocks), dim3(T), s, a, G);
 }
 
 template <class R>
@@ -878,14 +876,14 @@ cudaError_t launch_update(const KArgs<R>& a, int mode, cudaStream_t s) {
   const int mx = a.L.nx > a.L.nxd ? a.L.nx : a.L.nxd, my = a.L.ny > a.L.nyd ? a.L.ny : a.L.nyd;
   if constexpr (IsF32<R>::v) {
     const long nn = (long)mx * my;
-    if (nn > UPD_LARGE_NODES) update_comp_kernel<4><<<grid2(mx, my, dim3(32, 4), 2), 128, 0, s>>>(a, mode);
-    else if (nn > UPD_SMALL_NODES) update_comp_kernel<2><<<grid2(mx, my, dim3(32, 2), 2), 128, 0, s>>>(a, mode);
-    else update_comp_kernel<1><<<grid2(mx, my, dim3(32, 1), 2), 128, 0, s>>>(a, mode);
+    const int rows = nn > UPD_LARGE_NODES ? 4 : nn > UPD_SMALL_NODES ? 2 : 1;
+    auto kernel = rows == 4 ? update_comp_kernel<4> : rows == 2 ? update_comp_kernel<2> : update_comp_kernel<1>;
+    return launch_step(true, kernel, grid2(mx, my, dim3(32, rows), 2), dim3(128), s, a, mode);
   } else {
     const dim3 b(32, 4);
     update_kernel<<<grid2(mx, my, b, 2), b, 0, s>>>(a, mode);
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
