@@ -155,8 +155,12 @@ def step_counts(case, state, dt, precision=0, nsample=4000, seed=0):
         upd1 = comb((cflux, 32), (glue(4 * (18 + 14 + 32) + 6, 0), 1))
         upd2 = comb((cflux, 16), (glue(4 * (9 + 7 + 24) + 6, 0), 1))
     else:
-        upd1 = comb((cflux, 32), (glue(4 * 18, 4 * 19 + 6), 1))
-        upd2 = comb((cflux, 16), (glue(4 * 9, 4 * 8 + 6), 1))
+        # FP64: the short difference of a pair of faces that smooth nodes take (5
+        # additions, 3 products; it holds the glue's subtraction of the faces)
+        diff = comb()
+        diff["fp64"]["add"], diff["fp64"]["mul"] = 5.0, 3.0
+        upd1 = comb((diff, 16), (glue(4 * 14, 4 * 19 + 6), 1))
+        upd2 = comb((diff, 8), (glue(4 * 7, 4 * 8 + 6), 1))
     # per node pair per step: 2 points + 2 nodes + 2 updates in each stage
     pair = comb((point1, 2), (point2, 2), (node, 2), (node2, 2), (upd1, 2), (upd2, 2))
     per_node = {p: {k: pair[p][k] / 2.0 for k in KINDS} for p in ("fp64", "fp32")}
