@@ -625,8 +625,15 @@ extern "C" fdcgks_status fdcgks_vjp_steps(fdcgks_t ctx, double dt, int nsteps, i
     // adjoint of the final state
     double* Aout = w.A0;
     double* Ain = w.A1;
-    const DenseState seed{{const_cast<double*>(aWp), const_cast<double*>(aWd)},
-                          {const_cast<double*>(aGp), const_cast<double*>(aGd)}};
+    DenseState seed{{const_cast<double*>(aWp), const_cast<double*>(aWd)},
+                    {const_cast<double*>(aGp), const_cast<double*>(aGd)}};
+    const DenseState grad{{gWp, gWd}, {gGp, gGd}};
+    const DenseState staged = dense_areas(w.P1A, L);   // free between steps
+    if (!kernel_reaches(seed)) {
+      if ((r = copy_dense(staged, seed, L, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
+        return afail(ctx, FDCGKS_ERR_CUDA, "adjoint seed", r);
+      seed = staged;
+    }
     if ((r = launch_load(seed, L, 0.0, Aout, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s)) != cudaSuccess)
       return afail(ctx, FDCGKS_ERR_CUDA, "adjoint seed", r);
     // reverse sweep, one checkpoint segment at a time
@@ -644,8 +651,10 @@ extern "C" fdcgks_status fdcgks_vjp_steps(fdcgks_t ctx, double dt, int nsteps, i
         std::swap(Aout, Ain);
       }
     }
-    if ((r = launch_store(DenseState{{gWp, gWd}, {gGp, gGd}}, L, Aout, nullptr, nullptr, s)) != cudaSuccess)
-      return afail(ctx, FDCGKS_ERR_CUDA, "gradient copy", r);
+    const bool direct = kernel_reaches(grad);
+    r = launch_store(direct ? grad : staged, L, Aout, nullptr, nullptr, s);
+    if (r == cudaSuccess && !direct) r = copy_dense(grad, staged, L, cudaMemcpyDeviceToDevice, s);
+    if (r != cudaSuccess) return afail(ctx, FDCGKS_ERR_CUDA, "gradient copy", r);
     if (mixed && (fs = ctx_load_padded(ctx, w.fin)) != FDCGKS_OK) return fs;
     if ((r = cudaStreamSynchronize(s)) != cudaSuccess) return afail(ctx, FDCGKS_ERR_CUDA, "adjoint", r);
     return FDCGKS_OK;

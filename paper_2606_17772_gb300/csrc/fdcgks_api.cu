@@ -707,38 +707,19 @@ fdcgks_status fdcgks_dims(fdcgks_t c, int* nx, int* ny, int* nxd, int* nyd) {
   return FDCGKS_OK;
 }
 
-// The state at host pointers as a dense state on the device: four contiguous
-// areas in the point-output buffer, which is free between steps (192 bytes a
-// primary and dual node pair against its 200 or 400 bytes a point).
-// Contiguous copies run at the host link's full rate where per-row (pitched)
-// copies do not.
-static DenseState staged(fdcgks_t c) {
-  const long N0 = (long)c->L.nx * c->L.ny, N1 = (long)c->L.nxd * c->L.nyd;
-  double* st = (double*)c->PA;
-  return DenseState{{st, st + NFLD * N0}, {st + 4 * N0, st + NFLD * N0 + 4 * N1}};
-}
-
-static cudaError_t host_state_copy(fdcgks_t c, double* const* host, bool to_dev) {
-  const Layout& L = c->L;
-  const DenseState d = staged(c);
-  double* const dev[4] = {d.W[0], d.G[0], d.W[1], d.G[1]};
-  const long N0 = (long)L.nx * L.ny, N1 = (long)L.nxd * L.nyd, len[4] = {4 * N0, 8 * N0, 4 * N1, 8 * N1};
-  cudaError_t e = cudaSuccess;
-  for (int k = 0; k < 4 && e == cudaSuccess; ++k)
-    e = to_dev ? cudaMemcpyAsync(dev[k], host[k], sizeof(double) * len[k], cudaMemcpyHostToDevice, c->stream)
-               : cudaMemcpyAsync(host[k], dev[k], sizeof(double) * len[k], cudaMemcpyDeviceToHost, c->stream);
-  return e;
-}
+// Where the state of arrays that no kernel of this device reaches is staged: the
+// point-output buffer, which is free between steps (192 bytes a primary and
+// dual node pair against its 200 or 400 bytes a point).
+static DenseState staged(fdcgks_t c) { return dense_areas((double*)c->PA, c->L); }
 
 fdcgks_status fdcgks_set_state(fdcgks_t c, const double* Wp, const double* Gp, const double* Wd, const double* Gd,
                                int on_device) {
   if (!c) return fail(nullptr, FDCGKS_ERR_ARG, "ctx is NULL");
   if (!Wp || !Gp || !Wd || !Gd) return fail(c, FDCGKS_ERR_ARG, "NULL state pointer");
-  double* const src[4] = {const_cast<double*>(Wp), const_cast<double*>(Gp), const_cast<double*>(Wd),
-                          const_cast<double*>(Gd)};
-  DenseState d{{src[0], src[2]}, {src[1], src[3]}};
-  if (!on_device) {
-    CUDA_TRY(c, host_state_copy(c, src, true));
+  DenseState d{{const_cast<double*>(Wp), const_cast<double*>(Wd)}, {const_cast<double*>(Gp), const_cast<double*>(Gd)}};
+  if (!on_device || !kernel_reaches(d)) {
+    CUDA_TRY(c, copy_dense(staged(c), d, c->L, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
+                           c->stream));
     d = staged(c);
   }
   volatile int* bad = (volatile int*)(c->res_host + 2);
@@ -758,13 +739,13 @@ fdcgks_status fdcgks_get_state(fdcgks_t c, double* Wp, double* Gp, double* Wd, d
   if (!c) return fail(nullptr, FDCGKS_ERR_ARG, "ctx is NULL");
   if (!c->has_state) return fail(c, FDCGKS_ERR_STATE, "no state loaded");
   if (!Wp || !Gp || !Wd || !Gd) return fail(c, FDCGKS_ERR_ARG, "NULL state pointer");
-  double* const dst[4] = {Wp, Gp, Wd, Gd};
-  const DenseState d = on_device ? DenseState{{Wp, Wd}, {Gp, Gd}} : staged(c);
-  CUDA_TRY(c, launch_store(d, c->L, c->S, c->Sf, c->Slo, c->stream));
-  if (!on_device) {
-    CUDA_TRY(c, host_state_copy(c, dst, false));
-    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  }
+  const DenseState d{{Wp, Wd}, {Gp, Gd}};
+  const bool direct = on_device && kernel_reaches(d);
+  CUDA_TRY(c, launch_store(direct ? d : staged(c), c->L, c->S, c->Sf, c->Slo, c->stream));
+  if (!direct)
+    CUDA_TRY(c, copy_dense(d, staged(c), c->L, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                           c->stream));
+  if (!on_device) CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   return FDCGKS_OK;
 }
 

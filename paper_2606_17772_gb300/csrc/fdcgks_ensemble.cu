@@ -340,7 +340,7 @@ struct fdcgks_ens {
   unsigned* mxf = nullptr;
   int* heads = nullptr;
   int* vflag = nullptr;                   // pinned host memory: set_state's verdict, written by the device
-  double* staging = nullptr;              // room for the largest member's dense state (host copies)
+  double* staging = nullptr;              // room for the largest member's dense state (staged)
   // per member: padded FP64 state S (FP64 path) or the float-float pair (mixed)
   std::vector<double*> S;
   std::vector<float*> Shi, Slo;
@@ -723,26 +723,8 @@ fdcgks_status time_config(fdcgks_ens_t e, int steps, double* ms) {
 // ---------------------------------------------------------------------------
 extern "C" {
 
-// member m's dense state at host pointers, staged on the device in four
-// contiguous areas
-static DenseState staged(fdcgks_ens_t e, int m) {
-  const long N0 = (long)e->L[m].nx * e->L[m].ny, N1 = (long)e->L[m].nxd * e->L[m].nyd;
-  double* st = e->staging;
-  return DenseState{{st, st + NFLD * N0}, {st + 4 * N0, st + NFLD * N0 + 4 * N1}};
-}
-static cudaError_t host_copy(fdcgks_ens_t e, int m, const DenseState& h, bool to_dev) {
-  const DenseState d = staged(e, m);
-  cudaError_t r = cudaSuccess;
-  for (int g = 0; g < 2 && r == cudaSuccess; ++g) {
-    const Layout& L = e->L[m];
-    const size_t b = sizeof(double) * 4 * (g == 0 ? (size_t)L.nx * L.ny : (size_t)L.nxd * L.nyd);
-    const cudaMemcpyKind k = to_dev ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost;
-    r = cudaMemcpyAsync(to_dev ? d.W[g] : h.W[g], to_dev ? h.W[g] : d.W[g], b, k, e->stream);
-    if (r == cudaSuccess)
-      r = cudaMemcpyAsync(to_dev ? d.G[g] : h.G[g], to_dev ? h.G[g] : d.G[g], 2 * b, k, e->stream);
-  }
-  return r;
-}
+// where member m's arrays that no kernel of this device reaches are staged
+static DenseState staged(fdcgks_ens_t e, int m) { return dense_areas(e->staging, e->L[m]); }
 
 void fdcgks_ens_destroy(fdcgks_ens_t e) {
   if (!e) return;
@@ -899,9 +881,13 @@ fdcgks_status fdcgks_ens_set_state(fdcgks_ens_t e, int m, const double* Wp, cons
   const bool mixed = e->precision == FDCGKS_MIXED;
   e->has_state[m] = 0;
   DenseState d{{const_cast<double*>(Wp), const_cast<double*>(Wd)}, {const_cast<double*>(Gp), const_cast<double*>(Gd)}};
-  if (!on_device) ENS_TRY(e, host_copy(e, m, d, true));
+  if (!on_device || !kernel_reaches(d)) {
+    ENS_TRY(e, copy_dense(staged(e, m), d, L, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
+                          e->stream));
+    d = staged(e, m);
+  }
   *(volatile int*)e->vflag = 0;
-  ENS_TRY(e, launch_load(on_device ? d : staged(e, m), L, e->p[m].gamma, mixed ? nullptr : e->S[m],
+  ENS_TRY(e, launch_load(d, L, e->p[m].gamma, mixed ? nullptr : e->S[m],
                          mixed ? e->Shi[m] : nullptr, mixed ? e->Slo[m] : nullptr, e->vflag, e->mstat + m, e->time + m,
                          e->last_dt + m, e->stream));
   ENS_TRY(e, cudaStreamSynchronize(e->stream));
@@ -919,9 +905,12 @@ fdcgks_status fdcgks_ens_get_state(fdcgks_ens_t e, int m, double* Wp, double* Gp
   if (!Wp || !Gp || !Wd || !Gd) return efail(e, FDCGKS_ERR_ARG, "NULL state pointer");
   const bool mixed = e->precision == FDCGKS_MIXED;
   const DenseState d{{Wp, Wd}, {Gp, Gd}};
-  ENS_TRY(e, launch_store(on_device ? d : staged(e, m), e->L[m], e->S[m], mixed ? e->Shi[m] : nullptr,
+  const bool direct = on_device && kernel_reaches(d);
+  ENS_TRY(e, launch_store(direct ? d : staged(e, m), e->L[m], e->S[m], mixed ? e->Shi[m] : nullptr,
                           mixed ? e->Slo[m] : nullptr, e->stream));
-  if (!on_device) ENS_TRY(e, host_copy(e, m, d, false));
+  if (!direct)
+    ENS_TRY(e, copy_dense(d, staged(e, m), e->L[m], on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                          e->stream));
   ENS_TRY(e, cudaStreamSynchronize(e->stream));
   return FDCGKS_OK;
 }

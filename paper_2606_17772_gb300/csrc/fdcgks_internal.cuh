@@ -388,8 +388,49 @@ struct DenseState {
   double* G[2];
 };
 
+// the same in four contiguous areas of a staging buffer of 12 entries a node
+inline DenseState dense_areas(double* st, const Layout& L) {
+  const long N0 = (long)L.nx * L.ny, N1 = (long)L.nxd * L.nyd;
+  return DenseState{{st, st + NFLD * N0}, {st + 4 * N0, st + NFLD * N0 + 4 * N1}};
+}
+
+// copy of a dense state, one contiguous copy an array: contiguous copies run at
+// the host link's full rate where per-row (pitched) copies do not
+inline cudaError_t copy_dense(const DenseState& dst, const DenseState& src, const Layout& L, cudaMemcpyKind kind,
+                              cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  for (int g = 0; g < 2 && e == cudaSuccess; ++g) {
+    const size_t b = sizeof(double) * 4 * (g == 0 ? (size_t)L.nx * L.ny : (size_t)L.nxd * L.nyd);
+    e = cudaMemcpyAsync(dst.W[g], src.W[g], b, kind, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dst.G[g], src.G[g], 2 * b, kind, s);
+  }
+  return e;
+}
+
+// Whether a kernel on `device` may dereference a caller's device array: memory
+// of that device, or managed memory.  Any other array (of a second device,
+// which need not be mapped here, or pinned host memory) is reached by the copy
+// engine, which takes all of them and answers a bad pointer with an error code.
+inline bool kernel_reaches(const cudaPointerAttributes& a, int device) {
+  return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == device);
+}
+inline bool kernel_reaches(const DenseState& d) {
+  int device = 0;
+  if (cudaGetDevice(&device) != cudaSuccess) return false;
+  const void* p[] = {d.W[0], d.W[1], d.G[0], d.G[1]};
+  for (const void* q : p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, q) != cudaSuccess) {
+      cudaGetLastError();   // not an error of this call: the copy reports it
+      return false;
+    }
+    if (!kernel_reaches(a, device)) return false;
+  }
+  return true;
+}
+
 // whole-state helpers of the host runtime (fdcgks_api.cu), on stream s.
-// launch_load: a dense state into the padded layout, as FP64 (S, unless null)
+// launch_load: a dense state (kernel_reaches) into the padded layout, as FP64 (S, unless null)
 // and/or as float-float pairs (hi, lo, unless null), in one pass.  With
 // `bad` given, every node is checked (positive finite density and pressure,
 // finite gradients) and *bad is set to 1 where one fails; *clear, *t0 and *t1
