@@ -83,8 +83,12 @@ typedef struct {
                                  2: linear reconstruction and flux (chi = 1) */
   int grad_base;              /* Eq. eq-interface-update base: 0 = re-evaluated from the
                                  interface solution at t^n (default), 1 = stored gradient */
-  int precision;              /* fdcgks_precision: FP64, or MIXED (FP32 reconstruction and
-                                 flux arithmetic, FP64 state, accumulation and time coefficients) */
+  int precision;              /* fdcgks_precision: FP64, or MIXED: FP32 reconstruction and flux
+                                 arithmetic; state and accumulation as float-float pairs (FP64 in
+                                 the line solver); the interface solution's time coefficients
+                                 in FP32 where dt/tau > 4, where their terms do not cancel,
+                                 below in FP64 (1 < dt/tau) or float-float, each coefficient
+                                 then rounded once to FP32 */
   double tau_c1, tau_c2;      /* collision time tau = c1 dt + mu/p + c2 dt |pl - pr|/(pl + pr)
                                  at interfaces, c1 dt + mu/p at nodes (paper App. A cites the
                                  GKS literature for tau; these constants are run parameters) */

@@ -26,7 +26,7 @@
 // FP64 lines of 400 nodes, 10 steps, bound by the FP64 pipe: 22.3 -> 17.3 ms;
 // one 200-node line, 21 steps: 3.26 -> 2.87 ms).  The compute type R is FP64, or FP32 (the
 // mixed path: reconstruction, kinetic solves and compact fluxes in FP32 with
-// the 2-D mixed path's FP64 time coefficients, the interface and nodal
+// the 2-D mixed path's time coefficients, the interface and nodal
 // outputs stored in FP32); the state, its stage copy and the S2O4
 // accumulation are FP64 in both.
 #include <cmath>

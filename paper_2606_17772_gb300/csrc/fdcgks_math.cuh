@@ -202,8 +202,8 @@ struct GasK {
 };
 
 // dt/tau above which the time coefficients show no cancellation and the FP32
-// path evaluates them in FP32 (e^{-dt/tau} < 0.02); at or below it they are
-// computed in FP64 with expm1
+// path evaluates them in FP32 (e^{-dt/tau} < 0.02); from 1 to it they are
+// computed in FP64 with expm1, up to 1 by float-float series (time_coef_small)
 const double TIME_COEF_FP32_RATIO = 4.0;
 
 template <class R> FD_HD R rpow(R x, int r) { return r == 3 ? x * x * x : x * x; }
@@ -472,7 +472,8 @@ FD_HD R heat_flux_x(const R F[4], const R W[4], R U0, R V0) {
 // ---------------------------------------------------------------------------
 // Time coefficients of the interface distribution, integrated over
 // [0, delta] for delta = dt/2 and dt and fitted to f^n + t f_t^n (App. A1).
-// Always FP64: the coefficients cancel when dt/tau is small.
+// The terms cancel where dt/tau is small: TW is FP64 there, unless the series
+// of time_coef_small replace this form.
 // ---------------------------------------------------------------------------
 template <class TW>
 struct TimeCoef {
@@ -540,46 +541,140 @@ FD_HD TimeCoef<TW> time_coef(TW tau, TW dt, TW inv_dt) {
   return t;
 }
 
-// The same for x = dt/tau <= 1, for the FP32 path without FP64: inserting
-// exp(-y) = sum (-y)^n/n! in the integrals, every term that cancels drops out
-// and four power series in x remain,
-//   cn0 = x^2 p0,  cn1 = dt x p1,  cn2 = -dt x p0,
-//   ct0 = x (1 - x r0)/dt,  ct1 = x s0,  ct2 = x r0,
-//   p0 = sum_{n>=3} (-1)^n (4/2^n - 1)/n! x^(n-3),  p1 the same times (n - 2),
-//   r0 = -sum_{n>=3} (-1)^n 4 (1 - 2/2^n)/n! x^(n-3),  s0 = -r0's terms times (n - 2),
-// each dominated by its first term, so that Horner's rule keeps them within
-// about an ulp of FP32; terms to n = 11 (the next is below 1e-8 of the sum).
+// Float-float numbers h + l (|l| a few ulp of h at most, so that l l' counts for
+// nothing): sums and products of some 44 bits from FP32 operations (Dekker 1971,
+// Knuth's TwoSum).  add_rn and mul_rn are rounded by themselves, never fused.
+FD_HD float add_rn(float a, float b) {
+#if defined(__CUDA_ARCH__)
+  return __fadd_rn(a, b);
+#else
+  volatile float r = a + b;
+  return r;
+#endif
+}
+FD_HD float mul_rn(float a, float b) {
+#if defined(__CUDA_ARCH__)
+  return __fmul_rn(a, b);
+#else
+  volatile float r = a * b;
+  return r;
+#endif
+}
+FD_HD float s_fma(float a, float b, float c) { return fmaf(a, b, c); }
+template <class R> FD_HD R add_rn(R a, R b) { return a + b; }   // other scalar types
+template <class R> FD_HD R mul_rn(R a, R b) { return a * b; }
+template <class R> FD_HD R s_fma(R a, R b, R c) { return a * b + c; }
+
 template <class R>
-FD_HD TimeCoef<R> time_coef_small(R x, R tau, R dt, R inv_dt) {
-  const int NC = 9;   // n = 3..11
-  R p0 = R(0), p1 = R(0), r0 = R(0), s0 = R(0);
+struct FF {
+  R h, l;
+};
+template <class R> FD_HD FF<R> ff_neg(FF<R> a) { return {-a.h, -a.l}; }
+template <class R> FD_HD FF<R> ff_scale(FF<R> a, R k) { return {a.h * k, a.l * k}; }   // k a power of two
+template <class R> FD_HD R ff_round(FF<R> a) { return add_rn(a.h, a.l); }
+template <class R>
+FD_HD FF<R> ff_quick(R a, R b) {   // a + b exactly, |a| >= |b|
+  const R s = add_rn(a, b);
+  return {s, add_rn(b, -add_rn(s, -a))};
+}
+template <class R>
+FD_HD FF<R> ff_sum(R a, R b) {     // a + b exactly
+  const R s = add_rn(a, b), v = add_rn(s, -a);
+  return {s, add_rn(add_rn(a, -add_rn(s, -v)), add_rn(b, -v))};
+}
+template <class R>
+FD_HD FF<R> ff_add(FF<R> a, FF<R> b) {   // |a| >= |b|
+  const FF<R> s = ff_quick(a.h, b.h);
+  return {s.h, add_rn(s.l, add_rn(a.l, b.l))};
+}
+template <class R>
+FD_HD FF<R> ff_mul(FF<R> a, FF<R> b) {
+  const R p = mul_rn(a.h, b.h);
+  return {p, s_fma(a.h, b.l, s_fma(a.l, b.h, s_fma(a.h, b.h, -p)))};
+}
+template <class R>
+FD_HD FF<R> ff_div(FF<R> a, FF<R> b) {
+  const R i = s_div(R(1), b.h), q = mul_rn(a.h, i);
+  return {q, mul_rn(add_rn(s_fma(-q, b.h, a.h), s_fma(-q, b.l, a.l)), i)};
+}
+template <class R> FD_HD FF<R> ff_one_less(FF<R> a) { return ff_add(FF<R>{R(1), R(0)}, ff_neg(a)); }
+// an FP64 value to 46 bits or more: one slot of the FP64 pipe
+template <class R> FD_HD FF<R> ff_split(double v) { return {R(v), R(0)}; }
+template <>
+FD_HD FF<float> ff_split<float>(double v) {
+  const float h = est_f32(v);
+  return {h, est_f32(v - f32_to_f64(h))};
+}
+
+// The same for q = tau/dt >= 1, for the FP32 path without FP64's pipe: inserting
+// exp(-y) = sum (-y)^n/n! in the integrals, with x = 1/q, every term that
+// cancels drops out and two power series in x remain,
+//   p = sum_{n>=3} (-1)^n (4/2^n - 1)/n! x^(n-3),
+//   r = -sum_{n>=3} (-1)^n 4 (1 - 2/2^n)/n! x^(n-3),
+// from which, with w = 1 - x r and m = w/4 - 2 p,
+//   cn0 = x^2 p,  cn1 = dt x m,  cn2 = -dt x p,
+//   ct0 = x w/dt,  ct1 = 2 (x r - x^2 p) - 3/2 x w,  ct2 = x r,
+//   1 - E = x (1 - x^2 p - x w/2).
+// The series' terms to n = 8 are summed by a compensated Horner rule (Graillat,
+// Langlois and Louvet 2005), those to n = 16 (below 2^-14 of the sum, the next
+// below 2^-42) in FP32 in front of it, and the rest is float-float, so that a
+// coefficient is its exact value rounded once: the error is at most 0.500 ulp
+// of FP32, which the FP64 form reaches for x > 1e-2 (0.54 at 1e-3, 13 at 1e-4:
+// its terms cancel to third order), where four plain FP32 series were 4 to 9 ulp
+// off.  Viscous tube 1000x500, five steps with loading and reading: 2.49 ms with
+// those series, 2.67 so; the FP64 form took 1.20 of a step's ms alone.
+template <class R>
+FD_HD TimeCoef<R> time_coef_small(FF<R> q, FF<R> dt, FF<R> inv_dt) {
+  const int FIRST = 3, SPLIT = 8, LAST = 16;
+  const FF<R> x = ff_div(FF<R>{R(1), R(0)}, q);
+  R ps = R(0), rs = R(0), pe = R(0), re = R(0);   // the sums and their errors
+  auto step = [&](R& s, R& e, double c) {
+    const R ch = R((float)c), cl = R((float)(c - (double)(float)c)), t = mul_rn(s, x.h);
+    const FF<R> u = ff_quick(ch, t);
+    e = s_fma(e, x.h, s_fma(s, x.l, add_rn(s_fma(s, x.h, -t), add_rn(u.l, cl))));
+    s = u.h;
+  };
 #pragma unroll
-  for (int n = NC + 2; n >= 3; --n) {
+  for (int n = LAST; n >= FIRST; --n) {
     double f = 1.0, h = 1.0;   // n!, 2^-n
     for (int k = 1; k <= n; ++k) { f *= k; h *= 0.5; }
-    const double sg = n % 2 ? -1.0 : 1.0, a = sg * (4.0 * h - 1.0) / f, b = sg * 4.0 * (1.0 - 2.0 * h) / f;
-    p0 = p0 * x + R(a);
-    p1 = p1 * x + R(a * (n - 2));
-    r0 = r0 * x + R(-b);
-    s0 = s0 * x + R(b * (n - 2));
+    const double sg = n % 2 ? -1.0 : 1.0, a = sg * (4.0 * h - 1.0) / f, b = -sg * 4.0 * (1.0 - 2.0 * h) / f;
+    if (n > SPLIT) {
+      ps = s_fma(ps, x.h, R(a));
+      rs = s_fma(rs, x.h, R(b));
+    } else {
+      step(ps, pe, a);
+      step(rs, re, b);
+    }
   }
+  const FF<R> p = {ps, pe}, r = {rs, re};
+  const FF<R> xp = ff_mul(x, p), xr = ff_mul(x, r), xxp = ff_mul(x, xp), w = ff_one_less(xr), xw = ff_mul(x, w);
+  const FF<R> xm = ff_mul(x, ff_add(ff_scale(w, R(0.25)), ff_scale(p, R(-2))));
   TimeCoef<R> t;
-  const R xdt = x * dt, q0 = R(1) - x * r0;
-  t.cn[0] = x * x * p0;
-  t.cn[1] = xdt * p1;
-  t.cn[2] = -xdt * p0;
-  t.ct[0] = x * q0 * inv_dt;
-  t.ct[1] = x * s0;
-  t.ct[2] = x * r0;
-  t.cn[3] = R(1) - t.cn[0];
+  t.cn[0] = ff_round(xxp);
+  t.cn[1] = ff_round(ff_mul(dt, xm));
+  t.cn[2] = -ff_round(ff_mul(dt, xp));
+  t.ct[0] = ff_round(ff_mul(inv_dt, xw));
+  t.ct[1] = -ff_round(ff_add(ff_add(xw, ff_scale(xw, R(0.5))), ff_scale(ff_add(xr, ff_neg(xxp)), R(-2))));
+  t.ct[2] = ff_round(xr);
+  t.cn[3] = ff_round(ff_one_less(xxp));
   t.ct[3] = -t.ct[0];
-  t.cn[4] = -tau - t.cn[1];
+  t.cn[4] = -ff_round(ff_mul(dt, ff_add(q, xm)));
   t.ct[4] = -t.ct[1];
-  t.cn[5] = -tau - t.cn[2];
-  t.ct[5] = q0;
-  t.e1 = -s_expm1(-x);
-  t.E = R(1) - t.e1;
+  t.cn[5] = -ff_round(ff_mul(dt, ff_add(q, ff_neg(xp))));
+  t.ct[5] = ff_round(w);
+  const FF<R> e1 = ff_mul(x, ff_one_less(ff_add(ff_scale(xw, R(0.5)), xxp)));
+  t.e1 = ff_round(e1);
+  t.E = ff_round(ff_one_less(e1));
   return t;
+}
+// for plain arguments; x = dt/tau
+template <class R>
+FD_HD TimeCoef<R> time_coef_small(R x, R tau, R dt, R inv_dt) {
+  (void)x;
+  const FF<R> d = {dt, R(0)};
+  (void)inv_dt;
+  return time_coef_small(ff_div(FF<R>{tau, R(0)}, d), d, ff_div(FF<R>{R(1), R(0)}, d));
 }
 
 // ---------------------------------------------------------------------------
@@ -881,8 +976,9 @@ FD_HD void iface_solve_x(const GasK<R>& gas, const R Wl[4], const R Wr[4], const
 
   // collision time and time coefficients: FP64 with expm1 where they cancel
   // (dt/tau small); in the FP32 path FP32 where dt/tau > 4, where they do not,
-  // and where dt/tau <= 1, from series that do not (viscous runs lie there: the
-  // 85 slots of the FP64 pipe cost more than the rest of the FP32 solve)
+  // and where dt/tau <= 1 float-float, as exact as FP64's when rounded to FP32
+  // (viscous runs lie there: the FP64 form's 85 slots of the FP64 pipe cost
+  // more than the rest of the FP32 solve)
   typedef typename Wide<R>::T TW;
   R cn[6], ct[6], E, e1;
   R ip0r = R(0);                               // 1/p0, needed with viscosity only
@@ -895,7 +991,17 @@ FD_HD void iface_solve_x(const GasK<R>& gas, const R Wl[4], const R Wr[4], const
     E = tc.E;
     e1 = tc.e1;
   } else if (IsF32<R>::v && !(gas.dt_r > taur)) {
-    TimeCoef<R> tc = time_coef_small(s_div(gas.dt_r, taur), taur, gas.dt_r, gas.inv_dt_r);
+    // tau/dt = c1 + c2 |pl - pr|/(pl + pr) + (mu/dt)/p0
+    FF<R> dp = ff_sum(gl.p, -gr.p);
+    if (dp.h < R(0)) dp = ff_neg(dp);
+    const FF<R> qj = ff_mul(ff_split<R>(gas.c2), ff_div(dp, ff_sum(gl.p, gr.p))), q1 = ff_split<R>(gas.c1);
+    FF<R> q = ff_sum(q1.h, qj.h);
+    q.l = q.l + (q1.l + qj.l);
+    if (gas.mu_r != R(0)) {
+      const FF<R> qm = ff_mul(ff_split<R>(gas.mu * gas.inv_dt), FF<R>{ip0r, R(0)}), s = ff_sum(q.h, qm.h);
+      q = {s.h, s.l + (q.l + qm.l)};
+    }
+    TimeCoef<R> tc = time_coef_small(q, ff_split<R>(gas.dt), ff_split<R>(gas.inv_dt));
 #pragma unroll
     for (int k = 0; k < 6; ++k) { cn[k] = tc.cn[k]; ct[k] = tc.ct[k]; }
     E = tc.E;
