@@ -8,6 +8,7 @@
 #pragma once
 
 #include <math.h>
+#include <string.h>
 
 #include "fdcgks_gauss_table.h"
 
@@ -95,20 +96,58 @@ FD_HD double s_erfc_e(double x, double ex2) {
 }
 FD_HD float s_erfc_e(float x, float ex2) { (void)ex2; return erfcf(x); }
 
+// the words of an FP64 value and the bits of an FP32 one
+FD_HD void words_of(double x, unsigned& hi, unsigned& lo) {
+#if defined(__CUDA_ARCH__)
+  hi = (unsigned)__double2hiint(x);
+  lo = (unsigned)__double2loint(x);
+#else
+  unsigned long long b;
+  memcpy(&b, &x, sizeof(b));
+  hi = (unsigned)(b >> 32);
+  lo = (unsigned)b;
+#endif
+}
+FD_HD double of_words(unsigned hi, unsigned lo) {
+#if defined(__CUDA_ARCH__)
+  return __hiloint2double((int)hi, (int)lo);
+#else
+  const unsigned long long b = (unsigned long long)hi << 32 | lo;
+  double x;
+  memcpy(&x, &b, sizeof(x));
+  return x;
+#endif
+}
+FD_HD unsigned bits_of(float x) {
+#if defined(__CUDA_ARCH__)
+  return __float_as_uint(x);
+#else
+  unsigned b;
+  memcpy(&b, &x, sizeof(b));
+  return b;
+#endif
+}
+FD_HD float of_bits(unsigned b) {
+#if defined(__CUDA_ARCH__)
+  return __uint_as_float(b);
+#else
+  float x;
+  memcpy(&x, &b, sizeof(x));
+  return x;
+#endif
+}
+
 // FP32 copy of an FP64 value, rounded toward zero (for estimates and small terms):
 // shifts of its words, which cost the integer pipe 5 operations where a
 // conversion takes a slot of the FP64 pipe.  Zero below 2^-126, infinite from
 // 2^128 on; NaN becomes infinite.
 FD_HD float est_f32(double x) {
-#if defined(__CUDA_ARCH__)
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  unsigned hi, lo;
+  words_of(x, hi, lo);
   const unsigned a = hi & 0x7fffffffu;
-  unsigned m = __funnelshift_l(lo, a - 0x38000000u, 3);
+  unsigned m = (a - 0x38000000u) << 3 | lo >> 29;
   m = a < 0x38100000u ? 0u : a >= 0x47f00000u ? 0x7f800000u : m;
-  return __uint_as_float(m | (hi & 0x80000000u));
-#else
-  return (float)x;
-#endif
+  return of_bits(m | (hi & 0x80000000u));
 }
 
 // exp(-y^2) and erfc(y), which the half-space moments take together.
@@ -133,14 +172,11 @@ FD_HD void exp_erfc(R y, R& e, R& ec) {
 FDK_GAUSS_TABLE(static __device__, gauss_table_dev)
 #endif
 FDK_GAUSS_TABLE(static, gauss_table_host)
-// FP32 to FP64 by shifts, off the FP64 pipe (a zero becomes 2^-127)
+// FP32 to FP64 by shifts, off the FP64 pipe (exact for normal numbers; below
+// 2^-126 the result is off by at most 2^-127, a zero becomes 2^-127)
 FD_HD double f32_to_f64(float x) {
-#if defined(__CUDA_ARCH__)
-  const unsigned b = __float_as_uint(x);
-  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
-#else
-  return (double)x;
-#endif
+  const unsigned b = bits_of(x);
+  return of_words((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u), b << 29);
 }
 FD_HD void exp_erfc(double y, double& e, double& ec) {
   const double a = fabs(y);
@@ -151,16 +187,16 @@ FD_HD void exp_erfc(double y, double& e, double& ec) {
   }
   const double magic = 6755399441055744.0;   // 1.5 * 2^52: adds round to an integer in the low word
   const double s = a * FDK_GAUSS_STEPS + magic;
+  unsigned sh, k;
+  words_of(s, sh, k);
 #if defined(__CUDA_ARCH__)
-  const int k = __double2loint(s);
   const double E = gauss_table_dev[k][0], C = gauss_table_dev[k][1];
 #else
-  const int k = (int)(s - magic);
   const double E = gauss_table_host[k][0], C = gauss_table_host[k][1];
 #endif
   const double x = (s - magic) * (1.0 / FDK_GAUSS_STEPS), d = a - x;
   // FP32: q = p_4 + p_5 d + p_6 d^2, r = p_4/5 + p_5 d/6
-  const float xf = (float)k * (1.0f / FDK_GAUSS_STEPS), df = est_f32(d), wf = xf * xf;
+  const float xf = (float)(int)k * (1.0f / FDK_GAUSS_STEPS), df = est_f32(d), wf = xf * xf;
   const float f2 = 2.0f * wf - 1.0f, f3 = xf * (2.0f - (4.0f / 3.0f) * wf);
   const float f4 = -0.5f * (xf * f3 + f2), f5 = -0.4f * (xf * f4 + f3), f6 = (-1.0f / 3.0f) * (xf * f5 + f4);
   const double q = f32_to_f64(f4 + df * (f5 + df * f6)), r = f32_to_f64(0.2f * f4 + df * ((1.0f / 6.0f) * f5));
