@@ -388,7 +388,13 @@ FD_HD void screen_iface(const GenoK<R>&, R, R, R, R, R, float, bool&, bool&) {}
 template <class R>
 FD_HD bool screen_node(const GenoK<R>&, R, R, R, R, float) { return false; }
 template <class R> FD_HD float screen_h(R) { return 0.0f; }
-FD_HD float screen_h(double h) { return (float)h; }
+// the spacing for the screen: infinite, which fails every test, where FP32 does not
+// hold it (subnormal) or where the gradients that est_f32 flushes (below 2^-126)
+// would count, h 2^-126 against the root of eps_a (3e-8): from 2^80 on, 2^-46
+FD_HD float screen_h(double h) {
+  const float hf = (float)h;
+  return hf >= 1.17549435e-38f && hf < 1.2089258e24f ? hf : INFINITY;
+}
 
 // left and right states at the interface between Q[1] and Q[2] of a 4-point
 // line, with averaged gradients Qx[0..3] of the same 4 nodes (Sec. 3.1 Eq.
