@@ -314,9 +314,28 @@ FD_HD R geno_chi(const GenoK<R>& g, R IS0, R IS1, R IS2, R floor = R(0)) {
   return s_tanh(z) * g.inv_tanhC;
 }
 
+// Scales four numbers by 2^-512 where the last, the sum of the others, is finite and
+// above 2^864 (1e260): in their exponents, which all exceed 2^-510 then, so that it
+// costs no slot of the FP64 pipe and no branch.
+FD_HD void scale_vast(double w[3], double& sum) {
+  unsigned hi, lo;
+  words_of(sum, hi, lo);
+  const unsigned first = (1023u + 864u) << 20, inf = 0x7ff00000u;
+  const unsigned down = hi - first < inf - first ? 512u << 20 : 0u;
+  sum = of_words(hi - down, lo);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    words_of(w[k], hi, lo);
+    w[k] = of_words(hi - down, lo);
+  }
+}
+template <class R> FD_HD void scale_vast(R[3], R&) {}   // other scalar types
+
 // Weights of the three sub-stencils up to the factor returned (FP64: the
 // reciprocal of their sum, which is applied once to what they weight; FP32:
-// 1, the weights are normalised, which keeps their range).
+// 1, the weights are normalised, which keeps their range).  In FP64 they reach
+// the eighth power of the data's differences, and times a ninth would overflow
+// from differences of 1e34 on: the largest are scaled down.
 template <class R>
 FD_HD R geno_weights(const GenoK<R>& g, const R d[3], R IS0, R IS1, R IS2, R w[3]) {
   R e0 = IS0 + g.eps_w, e1 = IS1 + g.eps_w, e2 = IS2 + g.eps_w;
@@ -333,7 +352,9 @@ FD_HD R geno_weights(const GenoK<R>& g, const R d[3], R IS0, R IS1, R IS2, R w[3
   w[0] = d[0] * (s1 * s2);
   w[1] = d[1] * (s0 * s2);
   w[2] = d[2] * (s0 * s1);
-  return R(1) / (w[0] + (w[1] + w[2]));
+  R sum = w[0] + (w[1] + w[2]);
+  scale_vast(w, sum);
+  return R(1) / sum;
 }
 
 // The floor of an FP64 evaluation: (fscale max|Q|)^2 when fscale is given
