@@ -340,10 +340,10 @@ struct fdcgks_ens {
   unsigned* mxf = nullptr;
   int* heads = nullptr;
   int* vflag = nullptr;                   // pinned host memory: set_state's verdict, written by the device
-  double* staging = nullptr;              // room for the largest member's dense state (staged)
   // per member: padded FP64 state S (FP64 path) or the float-float pair (mixed)
   std::vector<double*> S;
   std::vector<float*> Shi, Slo;
+  std::vector<double*> PA;                // Type A point outputs: also the staging room, free between steps
   // tile lists
   TileCfg cfg;
   int4* tiles = nullptr;
@@ -723,14 +723,15 @@ fdcgks_status time_config(fdcgks_ens_t e, int steps, double* ms) {
 // ---------------------------------------------------------------------------
 extern "C" {
 
-// where member m's arrays that no kernel of this device reaches are staged
-static DenseState staged(fdcgks_ens_t e, int m) { return dense_areas(e->staging, e->L[m]); }
+// where member m's arrays that no kernel of this device reaches are staged: its
+// own point-output buffer, which has the room (as the single run's)
+static DenseState staged(fdcgks_ens_t e, int m) { return dense_areas(e->PA[m], e->L[m]); }
 
 void fdcgks_ens_destroy(fdcgks_ens_t e) {
   if (!e) return;
   drop_graphs(e);
   void* bufs[] = {e->arena, e->args, e->meta, e->mstat, e->time, e->last_dt, e->fixed_dt, e->cfl,
-                  e->mx, e->mxf, e->heads, e->staging, e->tiles};
+                  e->mx, e->mxf, e->heads, e->tiles};
   for (void* b : bufs)
     if (b) cudaFree(b);
   if (e->vflag) cudaFreeHost(e->vflag);
@@ -777,14 +778,12 @@ fdcgks_status fdcgks_ens_create(const fdcgks_params* params, int count, fdcgks_e
   // member layouts and the arena plan
   std::vector<std::vector<size_t>> offs(count);
   size_t total = 0;
-  long max_plane = 0;
   for (int m = 0; m < count; ++m) {
     const fdcgks_params& p = params[m];
     Layout L = make_layout(p);
     e->L.push_back(L);
     e->hx.push_back((p.x1 - p.x0) / p.nx);
     e->hy.push_back((p.y1 - p.y0) / p.ny);
-    if (L.plane > max_plane) max_plane = L.plane;
     std::vector<size_t> sizes;
     if (mixed) {
       const size_t fp = sizeof(float) * L.plane;
@@ -819,7 +818,6 @@ fdcgks_status fdcgks_ens_create(const fdcgks_params* params, int count, fdcgks_e
       {(void**)&e->mx, sizeof(unsigned long long) * 2 * count},
       {(void**)&e->mxf, sizeof(unsigned) * 2 * count},
       {(void**)&e->heads, sizeof(int) * N_COUNTERS},
-      {(void**)&e->staging, sizeof(double) * 2 * NFLD * max_plane},
   };
   for (auto& a : allocs) {
     if (!a.bytes) continue;
@@ -848,6 +846,7 @@ fdcgks_status fdcgks_ens_create(const fdcgks_params* params, int count, fdcgks_e
       e->Shi.push_back(nullptr);
       e->Slo.push_back(nullptr);
     }
+    e->PA.push_back((double*)(e->arena + offs[m][offs[m].size() - 2]));
   }
   e->has_state.assign(count, 0);
   r = cudaMemsetAsync(e->arena, 0, total, e->stream);
