@@ -43,6 +43,7 @@ struct fdcgks_ctx {
   double* res_host = nullptr;     // pinned host memory the device writes: the two maxima, set_state's verdict
   int red_blocks = 0;             // most blocks of the CFL reduction
   bool has_state = false;
+  bool overlap = false;       // programmatic dependent launches (mixed contexts)
   // kernel-class timing with CUDA events on the context stream (optional)
   int profiling = 0;
   cudaEvent_t* ev = nullptr;  // event pool
@@ -163,11 +164,11 @@ static cudaError_t fill_ghosts(fdcgks_t c, T* S, double t) {
   const Layout& L = c->L;
   const dim3 grid((ghost_count(std::max(L.nx, L.nxd), std::max(L.ny, L.nyd)) + 127) / 128, 1, 2);
   if (c->has_sides) {
-    return launch_step(IsF32<T>::v, ghost_kernel<T, GhostSides>, grid, dim3(128), c->stream, S, L, ghost_sides(c, t));
+    return launch_step(c->overlap, ghost_kernel<T, GhostSides>, grid, dim3(128), c->stream, S, L, ghost_sides(c, t));
   } else {
     GhostPlain K;
     for (int k = 0; k < 4; ++k) K.bc[k] = c->p.bc[k];
-    return launch_step(IsF32<T>::v, ghost_kernel<T, GhostPlain>, grid, dim3(128), c->stream, S, L, K);
+    return launch_step(c->overlap, ghost_kernel<T, GhostPlain>, grid, dim3(128), c->stream, S, L, K);
   }
 }
 
@@ -483,6 +484,7 @@ static KArgs<R> make_args(fdcgks_t c, double dt, const double* S, double* Sout, 
   a.want_n = want_n;
   set_dt(a, dt);
   a.flag = c->flag;
+  a.overlap = c->overlap;
   return a;
 }
 
@@ -585,7 +587,7 @@ template <class ST>
 static cudaError_t launch_cfl(fdcgks_t c, const ST& st, const CflGrid& G, int items) {
   const int blocks = std::min(items, c->red_blocks);
   const Layout& L = c->L;
-  const bool overlap = c->p.precision == FDCGKS_MIXED;
+  const bool overlap = c->overlap;
   if ((long)L.nx * L.ny + (long)L.nxd * L.nyd <= CFL_ALL_NODES) {
     c->launches += 1;
     return launch_step(overlap, cfl_kernel<ST, true>, dim3(blocks), dim3(256), c->stream, st, G, items, nullptr, 0,
@@ -643,6 +645,7 @@ fdcgks_status fdcgks_create(const fdcgks_params* p, fdcgks_t* out) {
   c->hx = (p->x1 - p->x0) / p->nx;
   c->hy = (p->y1 - p->y0) / p->ny;
   c->L = make_layout(*p);
+  c->overlap = p->precision == FDCGKS_MIXED;
   const Layout& L = c->L;
   const size_t rs = rsize(*p);
   const bool mixed = p->precision == FDCGKS_MIXED;
@@ -864,6 +867,12 @@ fdcgks_status fdcgks_set_time(fdcgks_t c, double t) {
 fdcgks_status fdcgks_get_time(fdcgks_t c, double* t) {
   if (!c || !t) return fail(c, FDCGKS_ERR_ARG, "NULL argument");
   *t = c->t;
+  return FDCGKS_OK;
+}
+
+int fdk_set_overlap(fdcgks_t c, int on) {
+  if (!c) return FDCGKS_ERR_ARG;
+  c->overlap = on != 0 && c->p.precision == FDCGKS_MIXED;
   return FDCGKS_OK;
 }
 

@@ -127,6 +127,7 @@ struct KArgs {
   double dt;
   double dtk[4];         // dt/2, dt^2/8, dt^2/6, dt^2/3 (set_dt)
   int* flag;             // bit 0: non-physical state found
+  int overlap;           // host only: launch as a programmatic dependent (launch_step)
   double* op[8];         // operator outputs (Lp, Ltp, gbp, gtp, Ld, Ltd, gbd, gtd), interior layout
 };
 
@@ -317,6 +318,11 @@ cudaError_t launch_step(bool overlap, void (*kernel)(P...), dim3 grid, dim3 bloc
 #endif
 
 enum { UPD_STAGE1 = 0, UPD_STAGE2 = 1, UPD_OPERATOR = 2 };
+
+// Whether the mixed steps of one context are launched as programmatic dependents
+// (on at creation).  The kernels and their results are the same either way;
+// tests compare the two.  Exported, but no part of the interface.
+extern "C" int fdk_set_overlap(fdcgks_t ctx, int on);
 
 // message returned by fdcgks_last_error(NULL)
 void set_global_error(const char* msg);

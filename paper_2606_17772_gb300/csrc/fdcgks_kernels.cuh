@@ -841,7 +841,7 @@ template <class R>
 cudaError_t launch_nodal(const KArgs<R>& a, cudaStream_t s) {
   dim3 b(32, 4);
   int mx = (a.L.nx > a.L.nxd ? a.L.nx : a.L.nxd) + 2, my = (a.L.ny > a.L.nyd ? a.L.ny : a.L.nyd) + 2;
-  return launch_step(IsF32<R>::v, nodal_kernel<R>, grid2(mx, my, b, 2), b, s, a);
+  return launch_step(a.overlap, nodal_kernel<R>, grid2(mx, my, b, 2), b, s, a);
 }
 
 // interface points, with the nodal work in the same launch if nodal is set
@@ -868,7 +868,7 @@ cudaError_t launch_points(const KArgs<R>& a, bool nodal, cudaStream_t s) {
   }
   auto kernel = a.recon_vars ? (nodal ? stage_kernel<R, true, true> : stage_kernel<R, true, false>)
                              : (nodal ? stage_kernel<R, false, true> : stage_kernel<R, false, false>);
-  return launch_step(IsF32<R>::v, kernel, dim3((unsigned)blocks), dim3(T), s, a, G);
+  return launch_step(a.overlap, kernel, dim3((unsigned)blocks), dim3(T), s, a, G);
 }
 
 template <class R>
@@ -878,7 +878,7 @@ cudaError_t launch_update(const KArgs<R>& a, int mode, cudaStream_t s) {
     const long nn = (long)mx * my;
     const int rows = nn > UPD_LARGE_NODES ? 4 : nn > UPD_SMALL_NODES ? 2 : 1;
     auto kernel = rows == 4 ? update_comp_kernel<4> : rows == 2 ? update_comp_kernel<2> : update_comp_kernel<1>;
-    return launch_step(true, kernel, grid2(mx, my, dim3(32, rows), 2), dim3(128), s, a, mode);
+    return launch_step(a.overlap, kernel, grid2(mx, my, dim3(32, rows), 2), dim3(128), s, a, mode);
   } else {
     const dim3 b(32, 4);
     update_kernel<<<grid2(mx, my, b, 2), b, 0, s>>>(a, mode);
