@@ -462,10 +462,10 @@ KArgs<double> stage_args(const Work& w, double dt, int stage) {
   a.L = w.v.L;
   a.geno = make_geno<double>(w.v.p.geno_variant);
   a.gas = make_gas<double>(w.v.p, dt);
-  a.hd[0] = a.h[0] = w.v.hx;
-  a.hd[1] = a.h[1] = w.v.hy;
-  a.ihd[0] = a.ih[0] = 1.0 / w.v.hx;
-  a.ihd[1] = a.ih[1] = 1.0 / w.v.hy;
+  a.h[0] = w.v.hx;
+  a.h[1] = w.v.hy;
+  a.ih[0] = 1.0 / w.v.hx;
+  a.ih[1] = 1.0 / w.v.hy;
   for (int k = 0; k < 4; ++k) a.bc[k] = w.v.p.bc[k];
   a.flux_variant = w.v.p.flux_variant;
   a.grad_base = w.v.p.grad_base;

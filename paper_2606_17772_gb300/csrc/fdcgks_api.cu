@@ -470,8 +470,6 @@ static KArgs<R> make_args(fdcgks_t c, double dt, const double* S, double* Sout, 
   a.PB = (R*)c->PB;
   a.geno = make_geno<R>(c->p.geno_variant);
   a.gas = make_gas<R>(c->p, dt);
-  a.hd[0] = c->hx; a.hd[1] = c->hy;
-  a.ihd[0] = 1.0 / c->hx; a.ihd[1] = 1.0 / c->hy;
   a.h[0] = (R)c->hx; a.h[1] = (R)c->hy;
   a.ih[0] = (R)(1.0 / c->hx); a.ih[1] = (R)(1.0 / c->hy);
   // the no-slip wall reset reads bc: an unsplit side's kind, else a non-wall kind

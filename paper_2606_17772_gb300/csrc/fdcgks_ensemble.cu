@@ -580,10 +580,6 @@ void fill_args(fdcgks_ens_t e, int m, char* base, const std::vector<size_t>& off
     a.L = e->L[m];
     a.geno = make_geno<R>(p.geno_variant);
     a.gas = make_gas<R>(p, 1.0);   // dt fields are written on the device every step
-    a.hd[0] = e->hx[m];
-    a.hd[1] = e->hy[m];
-    a.ihd[0] = 1.0 / e->hx[m];
-    a.ihd[1] = 1.0 / e->hy[m];
     a.h[0] = (R)e->hx[m];
     a.h[1] = (R)e->hy[m];
     a.ih[0] = (R)(1.0 / e->hx[m]);

@@ -120,7 +120,6 @@ struct KArgs {
   GenoK<R> geno;
   GasK<R> gas;
   R h[2], ih[2];
-  double hd[2], ihd[2];
   int bc[4];
   int flux_variant, grad_base, want_n;
   int recon_vars;        // 0 conservative, 1 characteristic interface reconstruction

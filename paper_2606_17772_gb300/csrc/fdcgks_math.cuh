@@ -208,11 +208,12 @@ FD_HD void exp_erfc(double y, double& e, double& ec) {
   ec = y >= 0.0 ? c : 2.0 - c;
 }
 
-// value at which tanh(z) rounds to exactly 1 in the compute type
+// value at which tanh(z) rounds to exactly 1 in FP32
 template <class R> struct TanhSat;
-template <> struct TanhSat<double> { static constexpr double z = 19.5; };
 template <> struct TanhSat<float> { static constexpr float z = 9.5f; };
-// and, in FP64, the value from which it does: e^(-2z) = 2^-54, z = 27 ln 2
+// FP64: the value from which (1 - e)/(1 + e), e = e^(-2z), rounds to 1: e = 2^-54,
+// z = 27 ln 2.  tanh itself rounds to 1 from 27.5 ln 2 = 19.0615 on; between the
+// two chi is 1 where it is 1 - 2^-53 rounded, an ulp of a weight.
 const double GENO_SAT64 = 18.715;
 
 // ---------------------------------------------------------------------------
@@ -266,7 +267,7 @@ FD_HD R geno_floor(R qmax) {
   return R(0);
 }
 
-// Sufficient test for tanh(C alpha) rounding to 1, which smooth data pass:
+// Sufficient test for chi = 1 (TanhSat, GENO_SAT64), which smooth data pass:
 // alpha = 2 aH/(aH + aL) with aH >= 1, so C alpha > z wherever
 // aL = 1 + (tau/(ISL + eps))^r < 2C/z - 1.  C = 20; the bounds on
 // tau/(ISL + eps) are the r-th roots of 2C/z - 2 (0.13732 in FP64, where z =
@@ -286,13 +287,15 @@ FD_HD R geno_chi(const GenoK<R>& g, R IS0, R IS1, R IS2, R floor = R(0)) {
   R ISH = s_max(IS0, s_max(IS1, IS2));
   R tau = s_abs(R(0.5) * (IS1 + IS2) - IS0);
   if (geno_smooth(tau, ISL, g.eps_a + floor, g.r)) return g.inv_tanhC;
-  R alpha;
-  if (IsF32<R>::v) {
+  if constexpr (IsF32<R>::v) {
     // FP32: quotient form (the product form could overflow for large IS)
     const R ea = g.eps_a + floor;
     R aH = R(1) + rpow(s_div(tau, ISH + ea), g.r);
     R aL = R(1) + rpow(s_div(tau, ISL + ea), g.r);
-    alpha = s_div(R(2) * aH, aH + aL);
+    const R z = g.C * s_div(R(2) * aH, aH + aL);
+    // tanh(z) is exactly 1 in this precision above the saturation point
+    if (z > R(TanhSat<R>::z)) return g.inv_tanhC;
+    return s_tanh(z) * g.inv_tanhC;
   } else {
     // tanh(C alpha) with alpha = 2 aH/(aH + aL), aH = 1 + (tau/h)^r, aL = 1 +
     // (tau/l)^r, over the common denominator h^r l^r; tanh z as
@@ -308,10 +311,6 @@ FD_HD R geno_chi(const GenoK<R>& g, R IS0, R IS1, R IS2, R floor = R(0)) {
     const R e = s_exp(R(-2) * z);
     return (R(1) - e) * (R(1) / (R(1) + e));
   }
-  R z = g.C * alpha;
-  // tanh(z) is exactly 1 in this precision above the saturation point
-  if (z > R(TanhSat<R>::z)) return g.inv_tanhC;
-  return s_tanh(z) * g.inv_tanhC;
 }
 
 // Scales four numbers by 2^-512 where the last, the sum of the others, is finite and

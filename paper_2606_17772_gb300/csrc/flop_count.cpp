@@ -143,7 +143,6 @@ inline CF s_erfc_e(CF x, CF e) { (void)e; return s_erfc(x); }
 #include "fdcgks_math.cuh"
 
 namespace fdk {
-template <> struct TanhSat<CD> { static constexpr double z = 19.5; };
 template <> struct IsF32<CF> { static constexpr bool v = true; };
 template <> struct TanhSat<CF> { static constexpr float z = 9.5f; };
 template <> struct Wide<CD> { typedef CD T; };
