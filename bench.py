@@ -885,6 +885,9 @@ def main():
                       "hbm_source": hbm_src, "fp64_derived": FP64_DERIVED_TFLOPS,
                       "fp32_derived": FP32_DERIVED_TFLOPS},
             "kernels": {"fp64": fp["kernels"]},
+            "kernels_note": "class times of a separate run of the same steps with class timing on, whose stages launch "
+                            "nodes and points apart, as differently compiled kernels; a timed FP64 step (and a mixed one "
+                            "of up to 100,000 nodes) launches them together",
             "flops_per_node_update": {"fp64": fp["cnt"]["per_node_update_total"]}}
 
     if "mixed" in results:

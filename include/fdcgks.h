@@ -171,7 +171,8 @@ fdcgks_status fdcgks_stage_operator(fdcgks_t ctx, double dt, double* Lp, double*
  * kernel (both types) and update kernel, and fdcgks_cfl_dt /
  * fdcgks_cfl_dt_sum around their reduction.  Nodes and points, which share a
  * launch otherwise (FP64, and mixed grids of up to 100,000 nodes), are then
- * launched apart, to be timed apart.  fdcgks_get_profile waits for
+ * launched apart, to be timed apart: other kernels of the same arithmetic, whose
+ * results can differ from an ordinary run's in the last bits.  fdcgks_get_profile waits for
  * the recorded events, returns the summed milliseconds and the number of
  * launch groups per class in ms[5] / count[5] (order: ghost, nodal, points,
  * update, cfl; either may be NULL), clears the record, and returns in

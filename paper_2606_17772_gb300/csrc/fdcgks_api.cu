@@ -20,7 +20,8 @@ struct fdcgks_ctx {
   Layout L;
   double hx, hy;
   cudaStream_t stream;
-  double* S = nullptr;      // state [2][12][plane] (FP64 path; staging of set/get_state in the mixed path)
+  double* S = nullptr;      // state [2][12][plane] (FP64 path; mixed path: the loaded state, for the adjoint's sweep,
+                            // and its steps' FP64 buffer; stepping and get_state do not read it)
   double* S2 = nullptr;     // stage state (FP64 path)
   // mixed path: the state as float-float pairs (high parts with ghost layers,
   // read by the nodal/point kernels), the stage state (high parts) and the

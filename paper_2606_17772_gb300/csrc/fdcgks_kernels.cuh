@@ -9,46 +9,45 @@
 
 #include "fdcgks_internal.cuh"
 
-// Tuning knobs of the interface-point kernel (defaults are the tuned values):
+// Tuning knobs (defaults are the tuned values).  Figures: ms per step of a fixed
+// time loop, all builds of this source; points and nodal are the class's time.
 // FDK_NODAL_MINB_F32  minimum resident blocks per SM in the launch bounds (caps
 //                  registers per thread) of the FP32 nodal kernel (the FP64
-//                  kernels are FP64-pipe bound and are left uncapped).  1024^2
-//                  vortex, ms per mixed step: 5, 6 give 0.116, 0.115
+//                  kernels are FP64-pipe bound and are left uncapped): 5, 6, 8
+//                  give 0.111, 0.106, 0.108 (nodal, 1024^2 vortex)
 #ifndef FDK_NODAL_MINB_F32
 #define FDK_NODAL_MINB_F32 6
 #endif
-// FDK_STAGE_THREADS_F64  block size of the FP64 stage kernel (below; 32 and 128:
-//                  33^2 0.213 and 0.227 ms per step, 512^2 4.73 and 4.78)
-// FDK_POINT_PAIR_MINB_F32 / _F64  minimum resident blocks per SM of the pair
-//                  kernel (FP32 without preload: 2, 3, 4, 5 gave 1.43, 1.06,
-//                  0.915, 0.903 ms; with preload 4 and 5 give 0.822 and 0.840)
-// FDK_POINT_ALONE_MINB_F32  the same for the FP32 stage kernel of points alone
-//                  and conservative reconstruction, whose 20 live registers
-//                  more spill little: 4 and 5 give 0.495 and 0.467 ms at
-//                  1024^2 (6: 0.480), tube 1000x500 0.488 and 0.479 a step;
-//                  with the nodes merged in 5 loses (128^2 step 0.0478 ->
-//                  0.0505), and so does the characteristic form (960x240
-//                  0.289 -> 0.292)
+// FDK_POINT_PAIR_MINB_F32 / _F64  the same for the stage kernel in its forms with
+//                  the nodes or with characteristic reconstruction: FP32 3, 4, 5
+//                  give 0.0363, 0.0342, 0.0350 (128^2 vortex) and 0.296, 0.277,
+//                  0.279 (double Mach 960x240, characteristic); FP64 holds 8
+//                  one-warp blocks at its 248 registers
 #ifndef FDK_POINT_PAIR_MINB_F32
 #define FDK_POINT_PAIR_MINB_F32 4
-#endif
-#ifndef FDK_POINT_ALONE_MINB_F32
-#define FDK_POINT_ALONE_MINB_F32 5
 #endif
 #ifndef FDK_POINT_PAIR_MINB_F64
 #define FDK_POINT_PAIR_MINB_F64 1
 #endif
-// FDK_PAIR_PRELOAD_F32  1: a pair-kernel thread loads its line's 32 values (4
-//                  entries x W and the gradient along the line) into registers
-//                  before the first reconstruction, so the loads are not issued
-//                  between the reconstructions.  The reconstruction is inlined:
-//                  with its arithmetic in differences and no indicators on
-//                  smooth data it is short enough (512^2 vortex, point phase per
-//                  step: mixed 0.153 -> 0.146 ms, FP64 4.25 -> 4.20 ms against
-//                  one out-of-line copy per kernel)
+// FDK_POINT_ALONE_MINB_F32  the same for the FP32 stage kernel of points alone and
+//                  conservative reconstruction, which needs fewer registers and
+//                  spills 36 bytes at 96: 4, 5, 6 give 0.912, 0.878, 0.886
+//                  (1024^2 vortex) and 0.517, 0.509, 0.516 (tube 1000x500)
+#ifndef FDK_POINT_ALONE_MINB_F32
+#define FDK_POINT_ALONE_MINB_F32 5
+#endif
+// FDK_STAGE_THREADS_F64  block size of the FP64 stage kernel: 32 and 128 give 0.177
+//                  and 0.190 (33^2), 0.458 and 0.454 (128^2), 3.90 and 3.94 (512^2)
 #ifndef FDK_STAGE_THREADS_F64
 #define FDK_STAGE_THREADS_F64 32
 #endif
+// FDK_PAIR_PRELOAD_F32  1: a thread of the FP32 stage kernel loads its line's 32
+//                  values (4 entries x W and the gradient along the line) into
+//                  registers before the first reconstruction, so the loads are
+//                  not issued between the reconstructions: 0 and 1 give points
+//                  0.570 and 0.480 (1024^2 vortex).  The reconstruction is inlined:
+//                  in differences and without indicators on smooth data it is
+//                  short enough
 #ifndef FDK_PAIR_PRELOAD_F32
 #define FDK_PAIR_PRELOAD_F32 1
 #endif

@@ -373,6 +373,9 @@ class Solver:
         return bool(out.value)
 
     def set_profiling(self, enable=True):
+        """Class timing (fdcgks_set_profiling): launches nodes and points apart,
+        as differently compiled kernels, so a timed run differs from an ordinary
+        one of FP64, or of a small mixed grid, in its last bits."""
         _check(load().fdcgks_set_profiling(self._h, int(bool(enable))), self._h)
 
     def get_profile(self):
