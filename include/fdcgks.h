@@ -23,6 +23,8 @@
  *     Dual-grid arrays use (nyd, nxd) from fdcgks_dims().
  *   - "on_device" selects device pointers (stream-ordered on the context's
  *     stream) or host pointers (the call returns after the copy completed).
+ *     Arrays of another GPU, and pinned host memory given as device pointers,
+ *     are copied through the context's own memory.
  *   - The caller owns every pointer it passes; the library never frees or
  *     retains caller memory.  The context owns its device buffers.
  *   - All work is issued on params.stream (a cudaStream_t; NULL = legacy
