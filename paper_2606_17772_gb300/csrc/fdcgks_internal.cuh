@@ -419,19 +419,22 @@ inline cudaError_t copy_dense(const DenseState& dst, const DenseState& src, cons
 inline bool kernel_reaches(const cudaPointerAttributes& a, int device) {
   return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == device);
 }
-inline bool kernel_reaches(const DenseState& d) {
+inline bool kernel_reaches(const void* const* p, int n) {
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess) return false;
-  const void* p[] = {d.W[0], d.W[1], d.G[0], d.G[1]};
-  for (const void* q : p) {
+  for (int k = 0; k < n; ++k) {
     cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, q) != cudaSuccess) {
+    if (cudaPointerGetAttributes(&a, p[k]) != cudaSuccess) {
       cudaGetLastError();   // not an error of this call: the copy reports it
       return false;
     }
     if (!kernel_reaches(a, device)) return false;
   }
   return true;
+}
+inline bool kernel_reaches(const DenseState& d) {
+  const void* p[] = {d.W[0], d.W[1], d.G[0], d.G[1]};
+  return kernel_reaches(p, 4);
 }
 
 // whole-state helpers of the host runtime (fdcgks_api.cu), on stream s.

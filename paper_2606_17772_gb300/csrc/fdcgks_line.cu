@@ -585,9 +585,11 @@ fdcgks_status fdcgks_line_set_state(fdcgks_line_t c, const double* W, const doub
   if (!W || !Wx) return lfail(c, FDCGKS_ERR_ARG, "W or Wx is NULL");
   const long total = 3L * c->p.n * c->p.batch;
   const double *w = W, *wx = Wx;
-  if (!on_device) {
-    LINE_TRY(c, cudaMemcpyAsync(c->stage, W, total * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-    LINE_TRY(c, cudaMemcpyAsync(c->stage + total, Wx, total * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+  const void* arrays[] = {W, Wx};
+  if (!on_device || !kernel_reaches(arrays, 2)) {
+    const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    LINE_TRY(c, cudaMemcpyAsync(c->stage, W, total * sizeof(double), kind, c->stream));
+    LINE_TRY(c, cudaMemcpyAsync(c->stage + total, Wx, total * sizeof(double), kind, c->stream));
     w = c->stage;
     wx = c->stage + total;
   }
@@ -604,16 +606,19 @@ fdcgks_status fdcgks_line_get_state(fdcgks_line_t c, double* W, double* Wx, int 
   if (!c) return lfail(nullptr, FDCGKS_ERR_ARG, "ctx is NULL");
   if (!W || !Wx) return lfail(c, FDCGKS_ERR_ARG, "W or Wx is NULL");
   const long total = 3L * c->p.n * c->p.batch;
-  double* w = on_device ? W : c->stage;
-  double* wx = on_device ? Wx : c->stage + total;
+  const void* arrays[] = {W, Wx};
+  const bool direct = on_device && kernel_reaches(arrays, 2);
+  double* w = direct ? W : c->stage;
+  double* wx = direct ? Wx : c->stage + total;
   const int blocks = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
   line_gather_kernel<<<blocks, 256, 0, c->stream>>>(c->a.S, w, wx, c->p.n, c->a.np, total);
   LINE_TRY(c, cudaGetLastError());
-  if (!on_device) {
-    LINE_TRY(c, cudaMemcpyAsync(W, w, total * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    LINE_TRY(c, cudaMemcpyAsync(Wx, wx, total * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    LINE_TRY(c, cudaStreamSynchronize(c->stream));
+  if (!direct) {
+    const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+    LINE_TRY(c, cudaMemcpyAsync(W, w, total * sizeof(double), kind, c->stream));
+    LINE_TRY(c, cudaMemcpyAsync(Wx, wx, total * sizeof(double), kind, c->stream));
   }
+  if (!on_device) LINE_TRY(c, cudaStreamSynchronize(c->stream));
   return FDCGKS_OK;
 }
 

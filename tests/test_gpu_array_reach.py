@@ -78,6 +78,23 @@ def test_adjoint(precision):
         assert (a.cpu() - b).abs().max() <= 1e-12 * a.abs().max().cpu()
 
 
+@pytest.mark.parametrize("precision", PRECISIONS)
+def test_lines(precision):
+    case = inputs.lax_strip(30, 1)
+    W, Wx = (torch.from_numpy(a).contiguous() for a in inputs.line_state(case))
+    lib = fdcgks.load()
+    with fdcgks.Lines.from_case(case, precision=precision) as L:
+        L.set_state(W.cuda()[None], Wx.cuda()[None])
+        L.steps(1e-3, 2)
+        ref = L.get_state()
+        pin = [W.pin_memory(), Wx.pin_memory()]
+        assert lib.fdcgks_line_set_state(L._h, *ptrs(pin), 1) == 0
+        L.steps(1e-3, 2)
+        out = [torch.empty_like(a, device="cpu").pin_memory() for a in ref]
+        assert lib.fdcgks_line_get_state(L._h, *ptrs(out), 1) == 0
+        assert same(ref, out)
+
+
 def test_get_state_is_captured():
     case = inputs.vortex(16)
     dev, _ = state(case)
