@@ -683,8 +683,8 @@ FD_HD FF<float> ff_split<float>(double v) {
 // coefficient is its exact value rounded once: the error is at most 0.500 ulp
 // of FP32, which the FP64 form reaches for x > 1e-2 (0.54 at 1e-3, 13 at 1e-4:
 // its terms cancel to third order), where four plain FP32 series were 4 to 9 ulp
-// off.  Viscous tube 1000x500, five steps with loading and reading: 2.49 ms with
-// those series, 2.67 so; the FP64 form took 1.20 of a step's ms alone.
+// off.  Viscous tube 1000x500, ms per step: 0.47 with those series, 0.51 so, 1.07
+// with the FP64 form.
 template <class R>
 FD_HD TimeCoef<R> time_coef_small(FF<R> q, FF<R> dt, FF<R> inv_dt) {
   const int FIRST = 3, SPLIT = 8, LAST = 16;
@@ -730,7 +730,7 @@ FD_HD TimeCoef<R> time_coef_small(FF<R> q, FF<R> dt, FF<R> inv_dt) {
   t.E = ff_round(ff_one_less(e1));
   return t;
 }
-// for plain arguments; x = dt/tau
+// the same for FP32 arguments (x = dt/tau, implied by the others), for tests
 template <class R>
 FD_HD TimeCoef<R> time_coef_small(R x, R tau, R dt, R inv_dt) {
   (void)x;
@@ -999,8 +999,8 @@ FD_HD void iface_solve_x(const GasK<R>& gas, const R Wl_[4], const R Wr_[4], con
   // The slopes carry the density (PrimGrad): in FP32 their products with theta^-2
   // leave the range for densities far from 1 where the specific ones would not.
   // The solve is linear in the density's unit, so there the unit is the power of
-  // two below the left density (exact).  Elsewhere a test and two branches not
-  // taken: 1024^2 mixed vortex 0.938 -> 0.939 ms per step.
+  // two below the left density (exact).  Elsewhere a test and branches not taken,
+  // us per step: 33^2 22.6 -> 22.9, 1024^2 876 -> 878, an ensemble of 40 925 -> 935.
   R unit = R(1), Wl[4], Wr[4], Wln[4], Wrn[4], Wt[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) { Wl[k] = Wl_[k]; Wr[k] = Wr_[k]; Wln[k] = Wln_[k]; Wrn[k] = Wrn_[k]; Wt[k] = Wt_[k]; }
